@@ -51,6 +51,14 @@ __device__ __forceinline__ uint64_t insert_zeros(uint64_t j, const Positions &p)
     return j;
 }
 
+// an index whose bits sit on arbitrary positions: lane t's bit at position p, over the warp
+__device__ __forceinline__ uint64_t warp_deposit(bool bit, int p) {
+    const uint64_t v = bit ? 1ull << p : 0ull;
+    const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)v);
+    const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(v >> 32));
+    return ((uint64_t)hi << 32) | lo;
+}
+
 inline unsigned grid_for(uint64_t units, int sms, int per_sm = 16) {
     uint64_t b = (units + kThreads - 1) / kThreads;
     uint64_t cap = (uint64_t)sms * per_sm;
@@ -292,6 +300,112 @@ __global__ void __launch_bounds__(kThreads) k_modexp(const typename Amp<R>::T *_
     }
 }
 
+// The same gather through shared memory, for a register on consecutive physical
+// bits that is narrow enough: a tile is every register value times the lowest other
+// bits (c of them, so that reads and writes are runs of at least 32 bytes).  The
+// control register of the order-finding circuit holds the lowest bits, so
+// neighbouring amplitudes take different multipliers: k_modexp's lanes each read
+// another sector and use 8 of its 32 bytes, here every sector is read once.  The
+// multiplier of each of the tile's 2^c control patterns is formed once per tile.
+// HBM-bound by bytes: at 27 qubits (9-bit register above 18 controls,
+// complex64) 2.64 -> 0.45 ms, 4.8 TB/s.
+constexpr int kModExpMaxLow = 8;   // at most 2^8 control patterns per tile
+struct ModExpTiled {
+    int w, cb, n_other;
+    int lp0, rev;                  // the register is local bits lp0 .. lp0 + w - 1
+    uint64_t n_tiles;
+    uint32_t N, mu;                // N <= 2^14: products stay below 2^28; mu = floor((2^32-1)/N)
+    uint8_t bit[16];               // local bit -> physical bit, ascending
+    uint8_t other[36];             // tile-index bit -> physical bit
+    int nctl;
+    uint8_t cpos[kModExpMaxControls];
+    uint32_t inv[kModExpMaxControls];
+    Cond cond;
+};
+
+__device__ __forceinline__ uint32_t mulmod_small(uint32_t x, uint32_t y, uint32_t N, uint32_t mu) {
+    const uint32_t p = x * y;                  // x, y < 2^14: exact
+    uint32_t r = p - __umulhi(p, mu) * N;      // the quotient is low by at most 2
+    while (r >= N) r -= N;
+    return r;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kThreads) k_modexp_tiled(const typename Amp<R>::T *__restrict__ in,
+                                                           typename Amp<R>::T *__restrict__ out,
+                                                           const __grid_constant__ ModExpTiled a,
+                                                           const uint8_t *cbits) {
+    using T = typename Amp<R>::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *buf = reinterpret_cast<T *>(smem_raw);
+    __shared__ uint32_t mtab[1 << kModExpMaxLow];
+    __shared__ uint64_t offj[64];              // offsets of the local bits from 8 on
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int tb = a.w + a.cb, M = 1 << tb;
+    const int rounds = M > kThreads ? M / kThreads : 1;
+    const bool active = (a.cond.n == 0) || cond_ok(a.cond, cbits);
+    uint64_t off0 = 0;
+    for (int k = 0; k < 8 && k < tb; ++k)
+        if ((tid >> k) & 1) off0 |= 1ull << a.bit[k];
+    if (tid < rounds) {
+        uint64_t o = 0;
+        for (int k = 8; k < tb; ++k)
+            if ((tid >> (k - 8)) & 1) o |= 1ull << a.bit[k];
+        offj[tid] = o;
+    }
+    const uint32_t rmask = (1u << a.w) - 1, lomask = (1u << a.lp0) - 1;
+    // thread t < 2^cb: the offset of control pattern t (the local bits outside the register)
+    uint64_t coff = 0;
+    for (int k = 0; k < a.cb; ++k)
+        if ((tid >> k) & 1) coff |= 1ull << a.bit[k < a.lp0 ? k : k + a.w];
+    __syncthreads();
+    const bool live = tid < M;
+    for (uint64_t tile = blockIdx.x; tile < a.n_tiles; tile += gridDim.x) {
+        // the tile's base; tile-index bits above 32 (never at sizes that fit) by hand
+        uint64_t base = warp_deposit(lane < a.n_other && ((tile >> lane) & 1u), lane < a.n_other ? a.other[lane] : 0);
+        for (int t = 32; t < a.n_other; ++t)
+            if ((tile >> t) & 1u) base |= 1ull << a.other[t];
+        const T *src = in + (base | off0);
+        if (live) {
+            for (int j0 = 0; j0 < rounds; j0 += 8) {
+                T v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (j0 + j < rounds) v[j] = src[offj[j0 + j]];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (j0 + j < rounds) buf[tid + (j0 + j) * kThreads] = v[j];
+            }
+        }
+        if (tid < (1 << a.cb)) {
+            const uint64_t i = base | coff;
+            uint32_t m = 1u % a.N;
+            for (int j = 0; j < a.nctl; ++j)
+                if ((i >> a.cpos[j]) & 1u) m = mulmod_small(m, a.inv[j], a.N, a.mu);
+            mtab[tid] = m;
+        }
+        __syncthreads();
+        if (live) {
+            T *dst = out + (base | off0);
+#pragma unroll 4
+            for (int j = 0; j < rounds; ++j) {
+                const uint32_t L = (uint32_t)(tid + j * kThreads);
+                uint32_t y = (L >> a.lp0) & rmask;
+                if (a.rev) y = __brev(y) >> (32 - a.w);
+                uint32_t s = L;
+                if (active && y < a.N) {
+                    const uint32_t c = (L & lomask) | ((L >> (a.lp0 + a.w)) << a.lp0);
+                    uint32_t x = mulmod_small(mtab[c], y, a.N, a.mu);
+                    if (a.rev) x = __brev(x) >> (32 - a.w);
+                    s = (L & ~(rmask << a.lp0)) | (x << a.lp0);
+                }
+                dst[offj[j]] = buf[s];
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // ---------------------------------------------------------------------------
 // K6: measurement.  reduce -> per-block (S0, S1); the last block to finish adds
 // the block partials in a fixed order (so results do not depend on timing) and
@@ -446,14 +560,6 @@ struct RelabelTiled {
 // either side's runs stay conflict-free; linear over GF(2)
 __device__ __forceinline__ int relabel_slot(int u) { return u ^ ((u >> 5) & 31); }
 
-// the low bits of a tile's index (lane t's bit at position p) added up over the warp
-__device__ __forceinline__ uint64_t warp_deposit(bool bit, int p) {
-    const uint64_t v = bit ? 1ull << p : 0ull;
-    const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)v);
-    const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(v >> 32));
-    return ((uint64_t)hi << 32) | lo;
-}
-
 // J = 2^m / kThreads elements per thread (1 when the tile is smaller)
 template <typename R, int J>
 __global__ void __launch_bounds__(kThreads) k_relabel_tiled(const typename Amp<R>::T *__restrict__ in,
@@ -572,13 +678,68 @@ cudaError_t launch_matk(int prec, void *psi, const MatKArgs &a, const uint8_t *c
     return prec == 0 ? matk_r<float>(psi, a, cbits, sms, s) : matk_r<double>(psi, a, cbits, sms, s);
 }
 
+// k_modexp_tiled where the register is a field of at most 12 bits (complex64) whose
+// tile keeps runs of 32 bytes; anything else goes to k_modexp
+template <typename R>
+static bool modexp_tile(const ModExpArgs &a, ModExpTiled &t) {
+    int n = 0;
+    while ((1ull << n) < a.n_amps) ++n;
+    const int full = sizeof(R) == 4 ? 13 : 12;           // 64 KiB of amplitudes: three blocks per SM
+    const int need = a.field.p0 == 0 ? 0 : (sizeof(R) == 4 ? 2 : 1);
+    if (!a.field.contig || a.w > 14 || a.w + need > full + 1 || n - a.w < need) return false;
+    int cb = full - a.w;
+    if (cb < need) cb = need;                            // 128 KiB: one block per SM
+    if (cb > kModExpMaxLow) cb = kModExpMaxLow;
+    if (cb > n - a.w) cb = n - a.w;
+    t.w = a.w;
+    t.cb = cb;
+    t.rev = a.field.rev;
+    t.N = (uint32_t)a.N;
+    t.mu = 0xffffffffu / t.N;
+    t.nctl = a.nctl;
+    for (int j = 0; j < a.nctl; ++j) {
+        t.cpos[j] = (uint8_t)a.cpos[j];
+        t.inv[j] = a.inv[j];
+    }
+    t.cond = a.cond;
+    const int p0 = a.field.p0, p1 = p0 + a.w;            // the register's bits
+    t.lp0 = p0 < cb ? p0 : cb;
+    int k = 0, left = cb;
+    for (int p = 0; p < n; ++p) {
+        const bool reg = p >= p0 && p < p1;
+        if (reg || left > 0) {
+            t.bit[k++] = (uint8_t)p;
+            left -= reg ? 0 : 1;
+        } else {
+            t.other[t.n_other++] = (uint8_t)p;
+        }
+    }
+    t.n_tiles = 1ull << t.n_other;
+    return true;
+}
+
+template <typename R>
+static cudaError_t modexp_r(const void *in, void *out, const ModExpArgs &a, const uint8_t *cbits, int sms,
+                            cudaStream_t s) {
+    using T = typename Amp<R>::T;
+    ModExpTiled t{};
+    if (!modexp_tile<R>(a, t)) {
+        k_modexp<R><<<grid_for(a.n_amps, sms), kThreads, 0, s>>>((const T *)in, (T *)out, a, cbits);
+        return cudaGetLastError();
+    }
+    const size_t sm = sizeof(T) << (t.w + t.cb);
+    if (sm > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k_modexp_tiled<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+    }
+    const uint64_t cap = (uint64_t)sms * (sm > 100 * 1024 ? 1 : sm > 48 * 1024 ? 3 : 6);
+    k_modexp_tiled<R><<<(unsigned)(t.n_tiles < cap ? t.n_tiles : cap), kThreads, sm, s>>>((const T *)in, (T *)out, t, cbits);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_modexp(int prec, const void *in, void *out, const ModExpArgs &a, const uint8_t *cbits, int sms,
                           cudaStream_t s) {
-    if (prec == 0)
-        k_modexp<float><<<grid_for(a.n_amps, sms), kThreads, 0, s>>>((const float2 *)in, (float2 *)out, a, cbits);
-    else
-        k_modexp<double><<<grid_for(a.n_amps, sms), kThreads, 0, s>>>((const double2 *)in, (double2 *)out, a, cbits);
-    return cudaGetLastError();
+    return prec == 0 ? modexp_r<float>(in, out, a, cbits, sms, s) : modexp_r<double>(in, out, a, cbits, sms, s);
 }
 
 cudaError_t launch_perm(int prec, const void *in, void *out, const PermArgs &a, const uint8_t *cbits,

@@ -930,7 +930,10 @@ qk_status qk_apply_modexp(qk_ctx *c, const int *targets, int nt, const int *cont
     a.field = qk::reg_field_of(a.rpos, nt);
     a.nctl = nc;
     a.ngroups = (nc + 7) / 8;
-    for (int j = 0; j < nc; ++j) a.cpos[j] = c->l2p[controls[j]];
+    for (int j = 0; j < nc; ++j) {
+        a.cpos[j] = c->l2p[controls[j]];
+        a.inv[j] = (uint32_t)inv[j];
+    }
     a.n_amps = 1ull << c->n;
     a.N = N;
     a.mu = (~0ull) / N;

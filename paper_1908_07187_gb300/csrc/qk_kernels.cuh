@@ -119,6 +119,7 @@ struct ModExpArgs {
     uint64_t n_amps;
     uint64_t N, mu;       // mu = floor((2^64-1)/N)
     Cond cond;
+    uint32_t inv[kModExpMaxControls];   // inverse of multiplier j
     uint32_t tab[kModExpGroups][256];
 };
 
