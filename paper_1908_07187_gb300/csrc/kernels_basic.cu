@@ -407,82 +407,196 @@ __global__ void __launch_bounds__(kThreads) k_modexp_tiled(const typename Amp<R>
 }
 
 // ---------------------------------------------------------------------------
-// K6: measurement.  reduce -> per-block (S0, S1); the last block to finish adds
-// the block partials in a fixed order (so results do not depend on timing) and
-// decides; collapse.  complex64 sums run in compensated FP32 (a float pair that
-// carries each addition's rounding error, about twice float's precision) and
-// reach FP64 once per thread: GB300 has 2 FP64 lanes per SM per clock.
+// K6: measurement, up to kMeasRound qubits per read of the state.  One qubit at a
+// time, P0 of the next qubit needs only sums of |a|^2 over the amplitudes that
+// match the outcomes so far, and the sums over every value of eight qubits give all
+// of those for eight decisions: one pass over 2^n amplitudes, then one over 2^(n-8),
+// instead of passes over 2^n, 2^(n-1), ... with a launch and a deciding block each.
+// A row is 2^L consecutive amplitudes, one 16-byte vector per lane, so measured bits
+// below L never mix across lanes and need no branch; a block sums rows of one value
+// of the round's higher bits.  The last block to finish (an atomic ticket, no
+// waiting) adds the block partials in a fixed order, so results do not depend on
+// timing.  complex64 sums run in compensated FP32 (a float pair that carries each
+// addition's rounding error, about twice float's precision) and reach FP64 once per
+// thread: GB300 has 2 FP64 lanes per SM per clock.  HBM-bound on large states,
+// launch-bound on small ones: 8 qubits of a 30-qubit complex64 state 2.90 -> 1.25 ms
+// (6.9 TB/s), 9 of 27 qubits 458 -> 194 us, 12 of 12 (complex128) 119 -> 24 us, one
+// qubit of 26 108 -> 101 us.
 // ---------------------------------------------------------------------------
-// prefix value of the decided outcomes: sum_j m_j << pos[j], j < k
+// prefix value of the decided outcomes: sum_j m_j << pos[j], j < k (whole warps)
 __device__ __forceinline__ uint64_t prefix_value(const MeasArgs &a, const MeasSlot *slots, int k) {
     uint64_t v = 0;
-    for (int j = 0; j < k; ++j) v |= (uint64_t)(slots[j].m & 1) << a.pos[j];
+    for (int j0 = 0; j0 < k; j0 += 32) {
+        const int j = j0 + (int)(threadIdx.x & 31);
+        v |= warp_deposit(j < k && (slots[j].m & 1), j < k ? a.pos[j] : 0);
+    }
     return v;
 }
 
-__device__ __forceinline__ uint64_t insert_bits(uint64_t j, const MeasArgs &a) {
-    for (int t = 0; t < a.nins; ++t) {
-        const uint64_t lo = j & ((1ull << a.ins[t]) - 1);
-        j = ((j - lo) << 1) | lo;
-    }
-    return j;
-}
+constexpr int kMeasThreads = 512;
 
 template <typename R>
-__global__ void __launch_bounds__(kThreads) k_meas_reduce(const typename Amp<R>::T *__restrict__ psi, MeasArgs a,
-                                                          const MeasSlot *slots, double *partials, Decide dec) {
-    __shared__ double sh[kThreads];
+__global__ void __launch_bounds__(kMeasThreads, 2)
+    k_meas_round(const typename Amp<R>::T *__restrict__ psi, const __grid_constant__ MeasArgs a, MeasSlot *slots,
+                 double *partials, unsigned *counter, uint8_t *cbits) {
+    constexpr bool kF = sizeof(R) == 4;
+    constexpr int L = meas_low_bits(kF ? 0 : 1), W = 1 << L, kWarps = kMeasThreads / 32;
+    __shared__ double sh[kWarps * W];
+    __shared__ unsigned s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint64_t pv = prefix_value(a, slots, a.k);
-    const int q = a.pos[a.k];
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool bit0_free = a.nins == 0 || a.ins[0] != 0;
+    uint64_t pm = 0;
+    for (int j = 0; j < a.k; ++j) pm |= 1ull << a.pos[j];
+    const uint32_t plm = (uint32_t)pm & (W - 1), plv = (uint32_t)pv & (W - 1);
+    const int hb = (int)(blockIdx.x / a.per_bin), p = (int)(blockIdx.x % a.per_bin);
+    uint64_t base = pv & ~(uint64_t)(W - 1);
+    for (int t = 0; t < a.bh; ++t) base |= (uint64_t)((hb >> t) & 1) << a.hpos[t];
+    // this lane's amplitudes of a row and whether the decided low bits let them in
+    const uint32_t i0 = kF ? 2 * lane : lane;
+    const uint32_t lim = a.n < L ? 1u << a.n : (uint32_t)W;
+    const bool in0 = i0 < lim && (i0 & plm) == plv, in1 = kF && i0 + 1 < lim && ((i0 + 1) & plm) == plv;
     double d0 = 0.0, d1 = 0.0;
-    if constexpr (sizeof(R) == 4) {
-        // complex64: |a|^2 in FP32, compensated FP32 running sums (FP64 only per thread)
+    if (in0 || in1) {
         FSum g0, g1;
-        if (bit0_free && a.n_units >= 2) {
-            // two adjacent amplitudes (one 16-byte vector) per unit
-            const uint64_t n_units = a.n_units >> 1;
-#pragma unroll 4
-            for (uint64_t u = tid; u < n_units; u += stride) {
-                const uint64_t i = insert_bits(u << 1, a) | pv;
-                const float4 v = *reinterpret_cast<const float4 *>(psi + i);
-                const float pa = v.x * v.x + v.y * v.y, pb = v.z * v.z + v.w * v.w;
-                if (q == 0) {
-                    g0.add(pa);
-                    g1.add(pb);
-                } else if ((i >> q) & 1u) {
-                    g1.add(pa + pb);
-                } else {
-                    g0.add(pa + pb);
+        const uint64_t stride = (uint64_t)a.per_bin * kWarps, r0 = (uint64_t)p * kWarps + warp;
+        // the free row bits count up around the fixed ones: a carry runs through the
+        // fixed bits when they are set for the addition
+        uint64_t fixed = 0, at = r0, step = stride;
+        for (int t = 0; t < a.nins; ++t) {
+            const uint64_t m = (1ull << a.ins[t]) - 1;
+            at += at & ~m;
+            step += step & ~m;
+            fixed |= m + 1;
+        }
+        at <<= L;
+        step <<= L;
+        fixed <<= L;
+        const typename Amp<R>::T *q = psi + (base | i0);
+        // several rows' loads in flight per lane before the first is added
+        constexpr int U = 8;
+        const int64_t todo = r0 < a.n_rows ? (int64_t)((a.n_rows - r0 + stride - 1) / stride) : 0;
+        for (int64_t left = todo; left > 0; left -= U) {
+            typename std::conditional<kF, float4, double2>::type v[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                v[k].x = v[k].y = 0;
+                if constexpr (kF) v[k].z = v[k].w = 0.f;
+                if (k < left) {
+                    if constexpr (kF) v[k] = *reinterpret_cast<const float4 *>(q + at);
+                    else v[k] = q[at];
+                    at = ((at | fixed) + step) & ~fixed;
                 }
             }
-        } else {
-            for (uint64_t u = tid; u < a.n_units; u += stride) {
-                const uint64_t i = insert_bits(u, a) | pv;
-                const typename Amp<R>::T v = psi[i];
-                const float pa = v.x * v.x + v.y * v.y;
-                if ((i >> q) & 1u) g1.add(pa); else g0.add(pa);
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                if constexpr (kF) {
+                    g0.add(v[k].x * v[k].x + v[k].y * v[k].y);
+                    g1.add(v[k].z * v[k].z + v[k].w * v[k].w);
+                } else {
+                    d0 += v[k].x * v[k].x + v[k].y * v[k].y;
+                }
             }
         }
-        d0 = g0.value();
-        d1 = g1.value();
-    } else {
-        for (uint64_t u = tid; u < a.n_units; u += stride) {
-            const uint64_t i = insert_bits(u, a) | pv;
-            const typename Amp<R>::T v = psi[i];
-            const double pa = (double)v.x * v.x + (double)v.y * v.y;
-            if ((i >> q) & 1u) d1 += pa; else d0 += pa;
+        if constexpr (kF) {
+            d0 = g0.value();
+            d1 = g1.value();
         }
     }
-    const double s0 = block_sum_w0(d0, sh);
-    const double s1 = block_sum_w0(d1, sh);
-    if (threadIdx.x == 0) {
-        partials[2 * blockIdx.x] = s0;
-        partials[2 * blockIdx.x + 1] = s1;
+    if constexpr (kF) {
+        sh[warp * W + 2 * lane] = in0 ? d0 : 0.0;
+        sh[warp * W + 2 * lane + 1] = in1 ? d1 : 0.0;
+    } else {
+        sh[warp * W + lane] = d0;
     }
-    last_block_decides(partials, dec);
+    __syncthreads();
+    const int bl = __popc(a.lmask);
+    if (warp == 0) {
+        // over the warps, then over the low bits that this round does not decide
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            s0 += sh[w * W + lane];
+            if (kF) s1 += sh[w * W + 32 + lane];
+        }
+        for (int k = 0; k < 5; ++k)
+            if (!((a.lmask >> k) & 1u)) {
+                s0 += __shfl_xor_sync(0xffffffffu, s0, 1 << k);
+                if (kF) s1 += __shfl_xor_sync(0xffffffffu, s1, 1 << k);
+            }
+        if (kF && !((a.lmask >> 5) & 1u)) s0 += s1;
+        if ((lane & ~a.lmask) == 0) {   // one lane per value of the round's low bits
+            int c = 0, k2 = 0;
+            for (int k = 0; k < 5; ++k)
+                if ((a.lmask >> k) & 1u) c |= ((lane >> k) & 1) << k2++;
+            double *out = partials + ((size_t)blockIdx.x << bl);
+            out[c] = s0;
+            if (kF && ((a.lmask >> 5) & 1u)) out[c | (1 << k2)] = s1;
+            __threadfence();            // the partials before the ticket
+        }
+        __syncwarp();
+        if (lane == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1 ? 1u : 0u;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // bin e holds the round's qubits in list order, the first as its highest bit:
+    // a tree of pair sums (node x of level j at sh[2^j + x]) gives every decision
+    const int bins = 1 << a.nb, parts = kMeasThreads >> a.nb;
+    {
+        const int e = tid & (bins - 1), part = tid >> a.nb;
+        int h = 0, c = 0;
+        for (int j = 0; j < a.nb; ++j) {
+            const int bit = (e >> (a.nb - 1 - j)) & 1, s = a.src[j];
+            if (s < 64) h |= bit << s;
+            else c |= bit << (s - 64);
+        }
+        const double *in = partials + ((size_t)h * a.per_bin << bl) + c;
+        double s = 0.0;
+#pragma unroll 4
+        for (int b = part; b < a.per_bin; b += parts) s += __ldcg(in + ((size_t)b << bl));
+        __syncthreads();
+        sh[tid] = s;                    // part-major: sh[part * bins + e]
+    }
+    for (int w = parts >> 1; w > 0; w >>= 1) {
+        __syncthreads();
+        if (tid < w * bins) sh[tid] += sh[tid + w * bins];
+    }
+    __syncthreads();
+    {
+        const double v = tid < bins ? sh[tid] : 0.0;
+        __syncthreads();
+        if (tid < bins) sh[bins + tid] = v;
+    }
+    for (int j = a.nb - 1; j >= 0; --j) {
+        __syncthreads();
+        if (tid < (1 << j)) sh[(1 << j) + tid] = sh[(2 << j) + 2 * tid] + sh[(2 << j) + 2 * tid + 1];
+    }
+    __syncthreads();
+    if (warp == 0) {
+        int node = 0;
+        double mine = 0.0, p0_mine = 1.0;
+        int m_mine = 0;
+        for (int j = 0; j < a.nb; ++j) {
+            const double s0 = sh[(2 << j) + 2 * node], s1 = sh[(2 << j) + 2 * node + 1];
+            const double tot = s0 + s1;
+            const double p0 = tot > 0.0 ? s0 / tot : 1.0;
+            const int m = (a.u[j] >= p0) ? 1 : 0;
+            if (lane == j) {
+                mine = m ? s1 : s0;
+                p0_mine = p0;
+                m_mine = m;
+            }
+            node = 2 * node + m;
+        }
+        if (lane < a.nb) {
+            MeasSlot *sl = slots + a.k + lane;
+            sl->p0 = p0_mine;
+            sl->m = m_mine;
+            sl->scale = mine > 0.0 ? 1.0 / sqrt(mine) : 0.0;
+            if (a.dest[lane] >= 0) cbits[a.dest[lane]] = (uint8_t)m_mine;
+        }
+        if (lane == 0) *counter = 0;
+    }
 }
 
 // Project onto the decided outcomes of every measured qubit and renormalise:
@@ -751,13 +865,45 @@ cudaError_t launch_perm(int prec, const void *in, void *out, const PermArgs &a, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_measure_reduce(int prec, const void *psi, int n, const MeasArgs &a, const MeasSlot *slots,
-                                  double *partials, int nblocks, const Decide &d, cudaStream_t s) {
-    if (n < 1) return cudaErrorInvalidValue;
+cudaError_t launch_measure_round(int prec, const void *psi, const MeasArgs &args, MeasSlot *slots, double *partials,
+                                 unsigned *counter, uint8_t *cbits, int sms, cudaStream_t s) {
+    MeasArgs a = args;
+    const int L = meas_low_bits(prec);
+    if (a.n < 1 || a.nb < 1 || a.nb > kMeasRound) return cudaErrorInvalidValue;
+    bool fixed[64] = {false};
+    a.bh = 0;
+    a.lmask = 0;
+    for (int j = 0; j < a.k + a.nb; ++j) {
+        const int q = a.pos[j];
+        if (q >= L) fixed[q] = true;
+        if (j < a.k) continue;
+        if (q >= L) {
+            a.src[j - a.k] = (uint8_t)a.bh;
+            a.hpos[a.bh++] = q;
+        } else {
+            a.lmask |= 1u << q;
+        }
+    }
+    for (int j = 0; j < a.nb; ++j) {   // a low qubit's rank among the round's low qubits
+        const int q = a.pos[a.k + j];
+        if (q < L) a.src[j] = (uint8_t)(64 + __builtin_popcount(a.lmask & ((1u << q) - 1)));
+    }
+    a.nins = 0;
+    for (int q = L; q < a.n; ++q)
+        if (fixed[q]) a.ins[a.nins++] = q - L;
+    a.n_rows = a.n > L ? 1ull << (a.n - L - a.nins) : 1;
+    // enough blocks to fill the device, no more than one row per warp
+    const int cap = sms * 2;
+    const uint64_t row_blocks = (a.n_rows + kMeasThreads / 32 - 1) / (kMeasThreads / 32);
+    int per = cap >> a.bh;
+    if (per < 1) per = 1;
+    if ((uint64_t)per > row_blocks) per = (int)row_blocks;
+    a.per_bin = per;
+    const unsigned grid = (unsigned)per << a.bh;
     if (prec == 0)
-        k_meas_reduce<float><<<nblocks, kThreads, 0, s>>>((const float2 *)psi, a, slots, partials, d);
+        k_meas_round<float><<<grid, kMeasThreads, 0, s>>>((const float2 *)psi, a, slots, partials, counter, cbits);
     else
-        k_meas_reduce<double><<<nblocks, kThreads, 0, s>>>((const double2 *)psi, a, slots, partials, d);
+        k_meas_round<double><<<grid, kMeasThreads, 0, s>>>((const double2 *)psi, a, slots, partials, counter, cbits);
     return cudaGetLastError();
 }
 

@@ -587,7 +587,8 @@ qk_status qk_create(qk_ctx **out, qk_precision precision, void *cuda_stream, con
     }
     c->pool_held = qk::pool_acquire(c->device) != nullptr;
     c->meas_blocks = c->sms * kMeasBlocksPerSM;
-    if (dalloc(c, (void **)&c->d_partials, sizeof(double) * 2 * c->meas_blocks) != cudaSuccess ||
+    if (dalloc(c, (void **)&c->d_partials,
+               sizeof(double) * std::max<size_t>(qk::meas_partials(c->sms), 2 * (size_t)c->meas_blocks)) != cudaSuccess ||
         dalloc(c, (void **)&c->d_err, sizeof(int)) != cudaSuccess ||
         dalloc(c, (void **)&c->d_counter, sizeof(unsigned)) != cudaSuccess ||
         cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned), c->stream) != cudaSuccess ||
@@ -1066,23 +1067,22 @@ qk_status qk_measure(qk_ctx *c, const int *qubits, int nq, const double *uniform
     if (s != QK_OK) return s;
     s = ensure_slots(c, nq);
     if (s != QK_OK) return s;
-    // decision k sums over the amplitudes that match decisions 0..k-1 (no
-    // collapse in between); one collapse pass projects onto all outcomes at the end
+    // a round decides up to kMeasRound qubits from one pass over the amplitudes that
+    // match the earlier rounds' outcomes (no collapse in between); one collapse pass
+    // projects onto all outcomes at the end
     qk::MeasArgs ma{};
+    ma.n = c->n;
     for (int a = 0; a < nq; ++a) ma.pos[a] = c->l2p[qubits[a]];
-    for (int k = 0; k < nq; ++k) {
+    for (int k = 0; k < nq; k += qk::kMeasRound) {
         ma.k = k;
-        ma.nins = k;
-        std::vector<int> ins(ma.pos, ma.pos + k);
-        std::sort(ins.begin(), ins.end());
-        for (int t = 0; t < k; ++t) ma.ins[t] = ins[t];
-        ma.n_units = 1ull << (c->n - k);
-        {
-            LaunchScope ls(c, 5, (double)c->amp * (double)ma.n_units);
-            const qk::Decide d{c->d_counter, uniforms[k], c->d_slots + k, c->d_cbits, dest ? dest[k] : -1};
-            CUDA_TRY(c, qk::launch_measure_reduce((int)c->prec, c->d_state, c->n, ma, c->d_slots, c->d_partials,
-                                                  c->meas_blocks, d, c->stream));
+        ma.nb = std::min(qk::kMeasRound, nq - k);
+        for (int j = 0; j < ma.nb; ++j) {
+            ma.u[j] = uniforms[k + j];
+            ma.dest[j] = dest ? dest[k + j] : -1;
         }
+        LaunchScope ls(c, 5, (double)c->amp * (double)(1ull << (c->n - k)));
+        CUDA_TRY(c, qk::launch_measure_round((int)c->prec, c->d_state, ma, c->d_slots, c->d_partials, c->d_counter,
+                                             c->d_cbits, c->sms, c->stream));
     }
     ma.k = nq;
     {

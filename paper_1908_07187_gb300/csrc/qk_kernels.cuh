@@ -218,17 +218,34 @@ __device__ __forceinline__ void last_block_decides(double *partials, const Decid
 }
 #endif
 
-// Measurement of a list of qubits, one decision at a time.  Decision k sums
-// |a_i|^2 over the indices whose earlier measured bits equal the outcomes
-// already decided (read from the slots on the device), split by bit pos[k].
+// Measurement of a list of qubits, up to kMeasRound decisions per round.  A round
+// sums |a_i|^2 over the indices whose earlier measured bits equal the outcomes
+// already decided (read from the slots on the device), into one bin per value of
+// the round's qubits; the decisions then follow one qubit at a time from the bins.
 constexpr int kMaxMeasure = 64;
+constexpr int kMeasRound = 8;
+// index bits below this are told apart by lane (and by the two amplitudes of a
+// lane's 16-byte vector in complex64); the bits above select rows
+__host__ __device__ constexpr int meas_low_bits(int prec) { return prec == 0 ? 6 : 5; }
 struct MeasArgs {
+    int n;
     int k;                // decisions already taken (prefix length); collapse: all decisions
-    int pos[40];          // physical bit of measured qubit j (list order), j < k and j == k
-    int nins;             // prefix bits sorted ascending, for enumeration
+    int nb;               // qubits decided in this round
+    int pos[64];          // physical bit of measured qubit j (list order), j < k + nb
+    int nins;             // row bits that are fixed (decided or a bin's), sorted ascending, for enumeration
     int ins[40];
-    uint64_t n_units;     // 2^(n-k) amplitudes match the prefix
+    uint64_t n_rows;      // rows per bin value of the high qubits
+    int bh;               // the round's qubits at or above the low bits: physical bit hpos[t] is
+    int hpos[kMeasRound]; // bit t of the high bin
+    uint32_t lmask;       // the round's qubits among the low bits
+    int per_bin;          // blocks per high bin
+    uint8_t src[kMeasRound];   // round qubit j: bit t of the high bin, or 64 + bit of the low bin
+    double u[kMeasRound];      // its uniform
+    int dest[kMeasRound];      // its destination cbit, -1: none
 };
+inline int meas_max_blocks(int sms) { return sms * 2 > (1 << kMeasRound) ? sms * 2 : 1 << kMeasRound; }
+// doubles of partial sums a round may need
+inline size_t meas_partials(int sms) { return (size_t)meas_max_blocks(sms) << 6; }
 
 // One fused Kitaev stage (kernels_kitaev.cu): control qubit at physical bit
 // cpos, register of w qubits at rpos[] (rpos[0] = MSB), permutation f given by
@@ -453,8 +470,8 @@ cudaError_t launch_modexp(int prec, const void *in, void *out, const ModExpArgs 
                           cudaStream_t s);
 cudaError_t launch_perm(int prec, const void *in, void *out, const PermArgs &a, const uint8_t *cbits,
                         int sms, cudaStream_t s);
-cudaError_t launch_measure_reduce(int prec, const void *psi, int n, const MeasArgs &a, const MeasSlot *slots,
-                                  double *partials, int nblocks, const Decide &d, cudaStream_t s);
+cudaError_t launch_measure_round(int prec, const void *psi, const MeasArgs &a, MeasSlot *slots, double *partials,
+                                 unsigned *counter, uint8_t *cbits, int sms, cudaStream_t s);
 cudaError_t launch_measure_collapse(int prec, void *psi, int n, const MeasArgs &a, const MeasSlot *slots, int sms,
                                     cudaStream_t s);
 cudaError_t launch_kitaev_reduce(int prec, const void *psi, const KitaevArgs &a, const uint8_t *cbits,
