@@ -24,6 +24,7 @@
 #include <cstdlib>
 #include <complex>
 #include <cstring>
+#include <deque>
 #include <vector>
 
 #include "qk_plan.h"
@@ -212,6 +213,510 @@ int local_of_tbit(int arr, int t) {
     if (t < 5) return arr == ARR_LO ? 5 + t : t;
     return arr == ARR_HI ? 5 + (t - 5) : 10 + (t - 5);
 }
+// The gates one pass takes from rem for a qubit set S: in order, each gate
+// that commutes with every gate left behind before it, whose 2x2 target is in
+// S (with grow, a target joins S while S has room) and whose classical
+// condition fits the condition table.  Counts only when tk is null.
+// Once every qubit carries a left-behind 2x2 gate, no later gate commutes with
+// them all, so the walk stops there (the rest is left behind as a whole).
+struct TakeLimits {
+    int tile_qubits, max_u2, max_ph;
+};
+void take_gates(const std::vector<POp> &rem, int n, const TakeLimits &lim, uint64_t S0, bool grow,
+                std::vector<Cond> &conds, std::vector<POp> *tk, std::vector<POp> *lf, uint64_t *S_out, int *n_u2_out,
+                int *n_ph_out) {
+    const uint64_t all_qubits = n >= 64 ? ~0ull : (1ull << n) - 1;
+    uint64_t S = S0;
+    int cnt = __builtin_popcountll(S0);
+    uint64_t ndb = 0, allb = 0;
+    int n_u2 = 0, n_ph = 0;
+    conds.clear();
+    for (auto it = rem.begin(); it != rem.end(); ++it) {
+        if (ndb == all_qubits) {
+            if (lf) lf->insert(lf->end(), it, rem.end());
+            break;
+        }
+        const POp &p = *it;
+        const bool is_u2 = p.op->kind == FusedOp::U2;
+        bool ok = (is_u2 ? n_u2 < lim.max_u2 : n_ph < lim.max_ph) && !(p.nd & allb) && !(p.all & ndb);
+        if (ok && is_u2) {
+            const uint64_t t = 1ull << p.op->q;
+            if (!(S & t)) {
+                if (grow && cnt < lim.tile_qubits) {
+                    S |= t;
+                    ++cnt;
+                } else {
+                    ok = false;
+                }
+            }
+        }
+        if (ok && p.op->cond.n) {
+            bool found = false;
+            for (const auto &cd : conds) found = found || same_cond(cd, p.op->cond);
+            if (!found) {
+                if ((int)conds.size() < kTileMaxConds) conds.push_back(p.op->cond);
+                else ok = false;
+            }
+        }
+        if (ok) {
+            if (tk) tk->push_back(p);
+            if (is_u2) ++n_u2; else ++n_ph;
+        } else {
+            if (lf) lf->push_back(p);
+            ndb |= p.nd;
+            allb |= p.all;
+        }
+    }
+    *S_out = S;
+    *n_u2_out = n_u2;
+    *n_ph_out = n_ph;
+}
+
+// S and its gates for one pass: the set that the greedy walk builds, or the low
+// contiguous qubits plus a window of consecutive qubits, whichever lets the pass take
+// the most 2x2 gates (then the most gates); a circuit whose gates spread along the
+// qubit line (layers of neighbour couplings) fills passes better with windows
+uint64_t choose_pass(const std::vector<POp> &rem, int n, const TakeLimits &lim, int contig, std::vector<Cond> &conds,
+                     std::vector<POp> &taken, std::vector<POp> &left, int *n_u2, int *n_ph) {
+    const uint64_t low = (1ull << contig) - 1;
+    uint64_t S = 0, best_S0 = low;
+    bool best_grow = true;
+    take_gates(rem, n, lim, low, true, conds, nullptr, nullptr, &S, n_u2, n_ph);
+    int best_u2 = *n_u2, best_all = *n_u2 + *n_ph;
+    const int wlen = lim.tile_qubits - contig;
+    for (int w = contig; w + wlen <= n; ++w) {
+        const uint64_t S0 = low | (((1ull << wlen) - 1) << w);
+        uint64_t Sw;
+        take_gates(rem, n, lim, S0, false, conds, nullptr, nullptr, &Sw, n_u2, n_ph);
+        if (*n_u2 > best_u2 || (*n_u2 == best_u2 && *n_u2 + *n_ph > best_all)) {
+            best_u2 = *n_u2;
+            best_all = *n_u2 + *n_ph;
+            best_S0 = S0;
+            best_grow = false;
+        }
+    }
+    left.clear();
+    taken.clear();
+    take_gates(rem, n, lim, best_S0, best_grow, conds, &taken, &left, &S, n_u2, n_ph);
+    int cnt = __builtin_popcountll(S);
+    // fill S up with the lowest unused qubits
+    for (int b = contig; b < n && cnt < lim.tile_qubits; ++b)
+        if (!((S >> b) & 1)) {
+            S |= 1ull << b;
+            ++cnt;
+        }
+    return S;
+}
+
+// ---------------------------------------------------------------------------
+// complex128 passes (Tile128Params in qk_kernels.cuh)
+// ---------------------------------------------------------------------------
+
+// Tile width by state size: wide tiles carry more gates per read and write of a state
+// in HBM; states that fit L2 are split over more CTAs instead, because one SM's two
+// FP64 lanes take 6 us for one gate on 2^12 amplitudes.  Measured on U3 / CZ / QFT
+// circuits (us at 8, 10 and 12 tile qubits): 12 qubits 263 / 384 / 879, 16 qubits 333 /
+// 412 / 924, 18 qubits 609 / 599 / 1003, 20 qubits 1831 / 1616 / 1676, 22 qubits 6691 /
+// 5677 / 5413.
+int tile128_qubits(int n) { return std::min(n, n <= 16 ? 8 : n <= 20 ? 10 : kTile128Max); }
+// Qubits that every tile holds, for runs of 128 bytes in HBM; none for states in L2.
+int tile128_contig(int n) { return n >= 18 ? 3 : 0; }
+
+// A diagonal term that is not yet in a program: f where (index & mask) == val.
+struct DTerm {
+    uint64_t mask, val;
+    cdm f;
+    const Cond *cond;
+    const FusedOp *src;      // the queued op that it is, if none of it became pending
+};
+
+// Builds one pass's program from its gates in order.  Single-qubit diagonal factors
+// never reach the device: F[q] is the pending complex factor of physical qubit q's |1>,
+// lam the one of every amplitude.  Diagonal terms on more qubits wait in terms until a
+// gate acts on one of their qubits and go out together there.
+struct Tile128Builder {
+    Tile128Params &P;
+    cdm *F;
+    cdm &lam;
+    int local_of[64], tile_of[64];
+    std::vector<DTerm> terms;
+    bool overflow = false;
+
+    Tile128Builder(Tile128Params &p, cdm *f, cdm &l) : P(p), F(f), lam(l) {}
+
+    Tile128Op *add(uint8_t kind, uint8_t q) {
+        if (P.nops >= kTile128Ops) {
+            overflow = true;
+            P.nops = 0;      // the program is thrown away
+        }
+        Tile128Op &o = P.ops[P.nops++];
+        std::memset(static_cast<void *>(&o), 0, sizeof o);
+        o.kind = kind;
+        o.q = q;
+        o.cond = kNoBit;
+        return &o;
+    }
+    // mask and value over physical bits as local and tile-index conditions
+    void conditions(Tile128Op &o, uint64_t mask, uint64_t val) {
+        for (uint64_t m = mask; m; m &= m - 1) {
+            const int b = __builtin_ctzll(m);
+            const uint32_t v = (uint32_t)(val >> b) & 1u;
+            if (local_of[b] >= 0) {
+                o.lmask |= (uint16_t)(1u << local_of[b]);
+                o.lval |= (uint16_t)(v << local_of[b]);
+            } else {
+                o.tmask |= 1u << tile_of[b];
+                o.tval |= v << tile_of[b];
+            }
+        }
+    }
+    uint8_t cond_index(const Cond &c) const {
+        for (int k = 0; k < P.n_conds; ++k)
+            if (same_cond(P.conds[k], c)) return (uint8_t)k;
+        return kNoBit;
+    }
+
+    // a term of the queue: single-qubit and constant parts become pending factors, a
+    // two-qubit term keeps only its (1, 1) pattern
+    void diagonal(const POp &p) {
+        const FusedOp &op = *p.op;
+        DTerm t{op.mask, op.val, op.f, op.cond.n ? &op.cond : nullptr, &op};
+        const int k = __builtin_popcountll(t.mask);
+        if (t.cond || k > 2) {
+            terms.push_back(t);
+            return;
+        }
+        if (k == 0) {
+            lam *= t.f;
+            return;
+        }
+        const int a = __builtin_ctzll(t.mask), b = 63 - __builtin_clzll(t.mask);
+        const int va = (int)(t.val >> a) & 1, vb = (int)(t.val >> b) & 1;
+        const cdm inv = 1.0 / t.f;
+        if (k == 1) {
+            if (va) F[a] *= t.f;
+            else {
+                lam *= t.f;
+                F[a] *= inv;
+            }
+            return;
+        }
+        if (va && !vb) F[a] *= t.f;
+        if (!va && vb) F[b] *= t.f;
+        if (!va && !vb) {
+            lam *= t.f;
+            F[a] *= inv;
+            F[b] *= inv;
+        }
+        if (t.val != t.mask) t.src = nullptr;
+        if (va != vb) t.f = inv;
+        t.val = t.mask;
+        terms.push_back(t);
+    }
+    static bool is_pair(const DTerm &t) { return !t.cond && t.val == t.mask && __builtin_popcountll(t.mask) == 2; }
+    static bool is_sign(const DTerm &t) { return t.f == cdm(-1.0, 0.0); }
+
+    void single_term(const DTerm &t) {
+        Tile128Op *o = add(D128_PH, kNoBit);
+        conditions(*o, t.mask, t.val);
+        if (t.cond) o->cond = cond_index(*t.cond);
+        o->c[0] = t.f.real();
+        o->c[1] = t.f.imag();
+    }
+    // an op on the amplitudes with physical bit b set: its local bit, or a tile-index condition
+    void on_bit(Tile128Op &o, int b) {
+        if (local_of[b] >= 0) o.q = (uint8_t)local_of[b];
+        else o.tval |= 1u << tile_of[b];
+    }
+    // factors fac[b] of the physical bits in bits, times c0, on the amplitudes with
+    // physical bit at set (at < 0: on all)
+    void table(int at, uint64_t bits, const cdm *fac, cdm c0) {
+        Tile128Op *o = add(D128_TABLE, kNoBit);
+        if (at >= 0) {
+            on_bit(*o, at);
+            o->tmask = o->tval;
+        }
+        o->first = (uint32_t)P.nfac;
+        o->c[0] = c0.real();
+        o->c[1] = c0.imag();
+        if (P.nfac + __builtin_popcountll(bits) > kTile128Facs) {
+            overflow = true;
+            return;
+        }
+        for (int pass = 0; pass < 2; ++pass)               // physical order is local and tile-index order
+            for (uint64_t m = bits; m; m &= m - 1) {
+                const int b = __builtin_ctzll(m);
+                if ((local_of[b] >= 0) != (pass == 0)) continue;
+                if (pass == 0) o->lmask |= (uint16_t)(1u << local_of[b]);
+                else o->tfac |= 1u << tile_of[b];
+                P.fac[P.nfac++] = make_double2(fac[b].real(), fac[b].imag());
+            }
+    }
+    // emit the waiting terms on physical qubit b.  Sign flips of pairs go to *sl, *st
+    // (local and tile-index parity masks of the other qubits), to an op of their own
+    // when these are null.
+    void emit_touching(int b, uint16_t *sl, uint32_t *st) {
+        uint64_t bits = 0, signs = 0;
+        cdm fac[64];
+        size_t w = 0;
+        const uint64_t bb = 1ull << b;
+        for (size_t i = 0; i < terms.size(); ++i) {
+            const DTerm &t = terms[i];
+            if (!(t.mask & bb)) {
+                terms[w++] = t;
+                continue;
+            }
+            if (!is_pair(t)) {
+                single_term(t);
+                continue;
+            }
+            const int d = __builtin_ctzll(t.mask & ~bb);
+            if (is_sign(t)) signs ^= 1ull << d;
+            else if ((bits >> d) & 1) fac[d] *= t.f;
+            else {
+                bits |= 1ull << d;
+                fac[d] = t.f;
+            }
+        }
+        terms.resize(w);
+        if (bits) table(b, bits, fac, cdm(1.0, 0.0));
+        if (!signs) return;
+        uint16_t l = 0;
+        uint32_t g = 0;
+        for (uint64_t m = signs; m; m &= m - 1) {
+            const int d = __builtin_ctzll(m);
+            if (local_of[d] >= 0) l |= (uint16_t)(1u << local_of[d]);
+            else g |= 1u << tile_of[d];
+        }
+        if (sl) {
+            *sl = l;
+            *st = g;
+            return;
+        }
+        Tile128Op *o = add(D128_SIGN, kNoBit);
+        on_bit(*o, b);
+        o->lmask = l;
+        o->tmask = g;
+    }
+    // every waiting term, grouped by the qubit that most pairs share
+    void emit_all() {
+        while (!terms.empty()) {
+            int cnt[64] = {0}, best = -1;
+            for (const DTerm &t : terms) {
+                if (!is_pair(t)) continue;
+                for (uint64_t m = t.mask; m; m &= m - 1) {
+                    const int b = __builtin_ctzll(m);
+                    if (best < 0 || ++cnt[b] > cnt[best]) best = b;
+                }
+            }
+            if (best < 0) best = __builtin_ctzll(terms[0].mask);
+            emit_touching(best, nullptr, nullptr);
+            if (overflow) return;
+        }
+    }
+    // the pending factor of qubit b onto the amplitudes
+    void materialise(int b) {
+        if (F[b] == cdm(1.0, 0.0)) return;
+        DTerm t{1ull << b, 1ull << b, F[b], nullptr, nullptr};
+        single_term(t);
+        F[b] = 1.0;
+    }
+
+    // A 2x2 gate on physical qubit op.q.  Uncontrolled: with M = W or X W (rows
+    // exchanged when that puts the larger entries on the diagonal) and F the pending
+    // factor, the outputs are W00 (y0 + a0 y1) and W11 F (y1 + a1 y0) with a0 = W01 F /
+    // W00, a1 = W10 / (W11 F), and a0 a1 = -r0 r1 is real for a unitary M.  Turning y1
+    // (or y0) by psi = arg a0 makes both updates real; of e^{i psi} = i^k cos(phi) (1 +
+    // i tan(phi)), |phi| <= pi/4, only i^k (1 + i tan) is applied and the cosine stays
+    // pending.  Updating one value from the other in place leaves s = 1 / (1 + r0 r1)
+    // on the second one.  Which value is turned and which is updated first is chosen so
+    // that the pending magnitude stays near 1.
+    void gate(const POp &p) {
+        const FusedOp &op = *p.op;
+        const int b = op.q;
+        const uint8_t q = (uint8_t)local_of[b];
+        const cdm *M = op.m;
+        const bool is_x = M[0] == 0.0 && M[3] == 0.0 && M[1] == 1.0 && M[2] == 1.0;
+        // the update form below takes a0 a1 for real, which a matrix defined with a loose
+        // tolerance need not have
+        const cdm pr = M[1] * M[2] * std::conj(M[0] * M[3]);
+        const bool unitary = std::abs(pr.imag()) <= 0x1p-50 * std::abs(pr) && pr.real() <= 0.0;
+        if (op.cmask || op.cond.n || !unitary) {
+            emit_touching(b, nullptr, nullptr);
+            materialise(b);
+            Tile128Op *o = add(is_x ? D128_X : D128_CU2, q);
+            conditions(*o, op.cmask, op.cmask);
+            if (op.cond.n) o->cond = cond_index(op.cond);
+            for (int e = 0; e < 4; ++e) {
+                o->c[2 * e] = M[e].real();
+                o->c[2 * e + 1] = M[e].imag();
+            }
+            return;
+        }
+        uint16_t sl = 0;
+        uint32_t sg = 0;
+        emit_touching(b, &sl, &sg);
+        Tile128Op *o = add(D128_U2, q);
+        o->lmask = sl;
+        o->tmask = sg;
+        cdm W[4] = {M[0], M[1], M[2], M[3]};
+        const bool sw = std::abs(W[0]) < std::abs(W[2]);
+        if (sw) {
+            std::swap(W[0], W[2]);
+            std::swap(W[1], W[3]);
+            o->flags |= kU2Swap;
+        }
+        const cdm f = F[b], a0 = W[1] * f / W[0], a1 = W[2] / (W[3] * f);
+        const double r0 = std::abs(a0), r1 = std::abs(a1), s = 1.0 / (1.0 + r0 * r1);
+        cdm p0 = W[0], p1 = W[3] * f;
+        if (r0 != 0.0 || r1 != 0.0) {
+            const double psi = std::arg(a0);
+            const int k = (int)std::lround(psi / (M_PI / 2));
+            const double phi = psi - k * (M_PI / 2), cs = std::cos(phi), tn = std::tan(phi);
+            const cdm e = std::polar(1.0, psi);
+            double best = 0.0;
+            int side = -1, first0 = 0;
+            for (int c = 0; c < 4; ++c) {                 // bit 0: y0 is turned; bit 1: y0 is updated first
+                double r = std::abs(p1 / p0) * ((c & 1) ? 1.0 / cs : cs) * ((c & 2) ? 1.0 / s : s);
+                if (sw) r = 1.0 / r;
+                r = std::abs(std::log(r));
+                if (side < 0 || r < best) {
+                    best = r;
+                    side = c & 1;
+                    first0 = c >> 1;
+                }
+            }
+            double b0, b1;
+            if (side == 0) {
+                b0 = r0 * cs;
+                b1 = -r1 / cs;
+                p1 *= std::conj(e) * cs;
+            } else {
+                b0 = r0 / cs;
+                b1 = -r1 * cs;
+                p0 *= e * cs;
+                o->flags |= kU2On0;
+            }
+            if (first0) {
+                b1 *= s;
+                p1 /= s;
+                o->flags |= kU2First0;
+            } else {
+                b0 *= s;
+                p0 /= s;
+            }
+            o->flags |= (uint8_t)((k & 3) | kU2Lift);
+            if (std::abs(tn) > 0x1p-55) o->flags |= kU2Phase;   // below: less than a rounding error
+            o->c[0] = tn;
+            o->c[1] = b0;
+            o->c[2] = b1;
+        }
+        if (sw) std::swap(p0, p1);
+        lam *= p0;
+        F[b] = p1 / p0;
+    }
+};
+
+}  // namespace
+
+qk_status plan_passes128(TilePlanner *planner, int n, const std::vector<FusedOp> &ops, const Pass128Sink &sink,
+                         const char **err) {
+    *err = "";
+    static thread_local std::vector<POp> rem, left, taken, next;
+    rem.clear();
+    for (const auto &op : ops) rem.push_back(classify(op));
+    const int m = tile128_qubits(n);
+    TakeLimits lim{m, kTile128Ops, 4096};
+    const int contig = std::min(tile128_contig(n), m);
+    std::vector<Cond> conds;
+    cdm F[64], lam = 1.0;
+    for (cdm &f : F) f = 1.0;
+    std::deque<FusedOp> rewritten;   // pair terms handed on without their single-qubit parts
+    while (!rem.empty()) {
+        int n_u2 = 0, n_ph = 0;
+        const uint64_t S = choose_pass(rem, n, lim, contig, conds, taken, left, &n_u2, &n_ph);
+        static thread_local Tile128Params P;
+        cdm F1[64], lam1 = lam;
+        std::copy(F, F + 64, F1);
+        Tile128Builder B(P, F1, lam1);
+        P.n = n;
+        P.m = m;
+        P.n_tiles = 1u << (n - m);
+        P.nfix = 0;
+        P.nops = P.nfac = 0;
+        for (int b = 0, lb = 0; b < 64; ++b) {
+            B.local_of[b] = B.tile_of[b] = -1;
+            if (b >= n) continue;
+            if ((S >> b) & 1) {
+                P.S[lb] = (int8_t)b;
+                B.local_of[b] = lb++;
+            } else {
+                P.fixed[P.nfix] = (int8_t)b;
+                B.tile_of[b] = P.nfix++;
+            }
+        }
+        P.n_conds = (int)conds.size();
+        for (int k = 0; k < P.n_conds; ++k) P.conds[k] = conds[k];
+        for (const POp &p : taken) {
+            if (p.op->kind == FusedOp::U2) B.gate(p);
+            else B.diagonal(p);
+            if (B.overflow) break;
+        }
+        // Terms that no gate of this pass called for go to the front of what is left:
+        // they commute with everything taken after them, and with what was left
+        // behind before them.  (Their single-qubit parts are pending already.)
+        if (!B.overflow && (left.empty() || n_u2 == 0)) B.emit_all();
+        if (!B.overflow && left.empty()) {
+            // the plan's last pass applies what is pending
+            uint64_t bits = 0;
+            for (int b = 0; b < n; ++b)
+                if (F1[b] != cdm(1.0, 0.0)) bits |= 1ull << b;
+            if (!B.overflow && (bits || lam1 != cdm(1.0, 0.0))) B.table(-1, bits, F1, lam1);
+        } else if (!B.overflow && !(std::abs(lam1) > 0x1p-200 && std::abs(lam1) < 0x1p200)) {
+            // a factor in [2^-1/2, 2] per gate: keep the stored amplitudes in range
+            B.table(-1, 0, F1, lam1);
+            lam1 = 1.0;
+        }
+        if (B.overflow) {
+            if (lim.max_u2 <= 1 && lim.max_ph <= 1) {
+                *err = "internal: tile program overflow";
+                return QK_EINVAL;
+            }
+            lim.max_u2 = std::max(1, lim.max_u2 / 2);
+            lim.max_ph = std::max(1, lim.max_ph / 2);
+            continue;
+        }
+        next.clear();
+        for (const DTerm &t : B.terms) {
+            if (t.src) {
+                next.push_back(classify(*t.src));
+                continue;
+            }
+            FusedOp o;
+            o.kind = FusedOp::PHASE;
+            o.mask = t.mask;
+            o.val = t.val;
+            o.f = t.f;
+            rewritten.push_back(o);
+            next.push_back(classify(rewritten.back()));
+        }
+        next.insert(next.end(), left.begin(), left.end());
+        if (planner->log)
+            std::fprintf(stderr, "[qk plan] c128 pass S=%#llx gates=%zu (u2 %d, phase %d) ops=%d factors=%d kept=%zu\n",
+                         (unsigned long long)S, taken.size(), n_u2, n_ph, P.nops, P.nfac, B.terms.size());
+        if (P.nops > 0) {
+            const qk_status st = sink(P);
+            if (st != QK_OK) return st;
+        }
+        std::copy(F1, F1 + 64, F);
+        lam = lam1;
+        rem.swap(next);
+        lim = TakeLimits{m, kTile128Ops, 4096};
+    }
+    return QK_OK;
+}
+
+namespace {
 }  // namespace
 
 qk_status plan_passes(TilePlanner *planner, int n, const std::vector<FusedOp> &ops, const PassSink &sink,
@@ -232,95 +737,11 @@ qk_status plan_passes(TilePlanner *planner, int n, const std::vector<FusedOp> &o
     double carry_mag[64];
     for (double &m : carry_mag) m = 1.0;
     double carry_u0 = 0.0, carry_lam = 1.0;
-    // The gates one pass takes from rem for a qubit set S: in order, each gate
-    // that commutes with every gate left behind before it, whose 2x2 target is in
-    // S (with grow, a target joins S while S has room) and whose classical
-    // condition fits the condition table.  Counts only when tk is null.
-    // Once every qubit carries a left-behind 2x2 gate, no later gate commutes with
-    // them all, so the walk stops there (the rest is left behind as a whole).
     std::vector<Cond> conds;
-    const uint64_t all_qubits = n >= 64 ? ~0ull : (1ull << n) - 1;
-    auto take = [&](uint64_t S0, bool grow, std::vector<POp> *tk, std::vector<POp> *lf, uint64_t *S_out,
-                    int *n_u2_out, int *n_ph_out) {
-        uint64_t S = S0;
-        int cnt = __builtin_popcountll(S0);
-        uint64_t ndb = 0, allb = 0;
-        int n_u2 = 0, n_ph = 0;
-        conds.clear();
-        for (auto it = rem.begin(); it != rem.end(); ++it) {
-            if (ndb == all_qubits) {
-                if (lf) lf->insert(lf->end(), it, rem.end());
-                break;
-            }
-            const POp &p = *it;
-            const bool is_u2 = p.op->kind == FusedOp::U2;
-            bool ok = (is_u2 ? n_u2 < max_u2 : n_ph < max_ph) && !(p.nd & allb) && !(p.all & ndb);
-            if (ok && is_u2) {
-                const uint64_t t = 1ull << p.op->q;
-                if (!(S & t)) {
-                    if (grow && cnt < kTileQubits) {
-                        S |= t;
-                        ++cnt;
-                    } else {
-                        ok = false;
-                    }
-                }
-            }
-            if (ok && p.op->cond.n) {
-                bool found = false;
-                for (const auto &cd : conds) found = found || same_cond(cd, p.op->cond);
-                if (!found) {
-                    if ((int)conds.size() < kTileMaxConds) conds.push_back(p.op->cond);
-                    else ok = false;
-                }
-            }
-            if (ok) {
-                if (tk) tk->push_back(p);
-                if (is_u2) ++n_u2; else ++n_ph;
-            } else {
-                if (lf) lf->push_back(p);
-                ndb |= p.nd;
-                allb |= p.all;
-            }
-        }
-        *S_out = S;
-        *n_u2_out = n_u2;
-        *n_ph_out = n_ph;
-    };
     while (!rem.empty()) {
-        // ---- choose S and the gates this pass takes: the set that the greedy
-        // walk builds, or the contiguous qubits plus a window of consecutive
-        // qubits, whichever lets the pass take the most 2x2 gates (then the most
-        // gates); a circuit whose gates spread along the qubit line (layers of
-        // neighbour couplings) fills passes better with windows
-        const uint64_t low = (1ull << kTileContig) - 1;
-        uint64_t S = 0, best_S0 = low;
-        bool best_grow = true;
         int n_u2 = 0, n_ph = 0;
-        take(low, true, nullptr, nullptr, &S, &n_u2, &n_ph);
-        int best_u2 = n_u2, best_all = n_u2 + n_ph;
-        const int wlen = kTileQubits - kTileContig;
-        for (int w = kTileContig; w + wlen <= n; ++w) {
-            const uint64_t S0 = low | (((1ull << wlen) - 1) << w);
-            uint64_t Sw;
-            take(S0, false, nullptr, nullptr, &Sw, &n_u2, &n_ph);
-            if (n_u2 > best_u2 || (n_u2 == best_u2 && n_u2 + n_ph > best_all)) {
-                best_u2 = n_u2;
-                best_all = n_u2 + n_ph;
-                best_S0 = S0;
-                best_grow = false;
-            }
-        }
-        left.clear();
-        taken.clear();
-        take(best_S0, best_grow, &taken, &left, &S, &n_u2, &n_ph);
-        int cnt = __builtin_popcountll(S);
-        // fill S up to 13 qubits with the lowest unused ones
-        for (int b = kTileContig; b < n && cnt < kTileQubits; ++b)
-            if (!((S >> b) & 1)) {
-                S |= 1ull << b;
-                ++cnt;
-            }
+        const uint64_t S = choose_pass(rem, n, TakeLimits{kTileQubits, max_u2, max_ph}, kTileContig, conds, taken, left,
+                                       &n_u2, &n_ph);
 
         static thread_local TileParams P;
         std::memset(static_cast<TileHead *>(&P), 0, sizeof(TileHead));
@@ -955,7 +1376,20 @@ qk_status plan_passes(TilePlanner *planner, int n, const std::vector<FusedOp> &o
 
 qk_status run_fused(TilePlanner *planner, qk_ctx *c, const std::vector<FusedOp> &ops) {
     const int n = ctx_n(c);
-    if (n < kTileQubits || ctx_prec(c) != 0) {
+    if (ctx_prec(c) != 0) {
+        const Pass128Sink launch = [&](Tile128Params &P) -> qk_status {
+            void *tok = nullptr;
+            ctx_launch_begin(c, 0, 2.0 * 16.0 * (double)(1ull << n), &tok);
+            const cudaError_t e = launch_tile128(ctx_state(c), P, ctx_cbits(c), ctx_stream(c));
+            ctx_launch_end(tok);
+            return e == cudaSuccess ? QK_OK : ctx_fail(c, QK_ECUDA, cudaGetErrorString(e));
+        };
+        const char *err = "";
+        const qk_status st = plan_passes128(planner, n, ops, launch, &err);
+        if (st != QK_OK && err[0]) return ctx_fail(c, st, err);
+        return st;
+    }
+    if (n < kTileQubits) {
         for (const auto &op : ops) {
             qk_status s = ctx_run_plain(c, op);
             if (s != QK_OK) return s;

@@ -33,8 +33,12 @@ void free_planner(TilePlanner *p);
 // On a planner error *err names it.
 using PassSink = std::function<qk_status(TileParams &)>;
 qk_status plan_passes(TilePlanner *p, int n, const std::vector<FusedOp> &ops, const PassSink &sink, const char **err);
-// plan_passes with each pass launched on the context's stream (n < 13 or
-// complex128: one plain launch per op)
+// the same for complex128 lists of any size (Tile128Params)
+using Pass128Sink = std::function<qk_status(Tile128Params &)>;
+qk_status plan_passes128(TilePlanner *p, int n, const std::vector<FusedOp> &ops, const Pass128Sink &sink,
+                         const char **err);
+// plan_passes or plan_passes128 with each pass launched on the context's stream
+// (complex64 with n < 13: one plain launch per op)
 qk_status run_fused(TilePlanner *p, qk_ctx *c, const std::vector<FusedOp> &ops);
 
 // context hooks implemented in qk_api.cu
