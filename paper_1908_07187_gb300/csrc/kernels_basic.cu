@@ -1,5 +1,5 @@
 // One-pass-per-gate kernels of libqk: 2x2 pair updates (K1), diagonal phases
-// (K2), dense k-qubit blocks, permutation gathers (K5), measurement (K6), and
+// (K2), permutation gathers (K5), measurement (K6), and
 // small helpers.  Every kernel streams the amplitudes it touches once, with
 // 16-byte vector accesses where the qubit layout allows.
 #include <cuda_runtime.h>
@@ -162,49 +162,6 @@ __global__ void __launch_bounds__(kThreads) k_phase(typename Amp<R>::T *psi, Pha
         } else {
             const uint64_t i = insert_zeros(u, a.ins) | a.val;
             psi[i] = cmul(psi[i], f);
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Dense k-qubit block.  Each block iteration handles 256 / 2^k groups with one
-// thread per output amplitude: the group vectors are staged in shared memory,
-// thread (g, r) forms row r of M v_g.  The matrix sits in shared memory too.
-// ---------------------------------------------------------------------------
-template <typename R>
-__global__ void __launch_bounds__(kThreads) k_matk(typename Amp<R>::T *psi, MatKArgs a, const uint8_t *cbits) {
-    using T = typename Amp<R>::T;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int K = a.k, G = 1 << K;
-    T *mat = reinterpret_cast<T *>(smem_raw);
-    T *vec = mat + G * G;
-    if (a.cond.n && !cond_ok(a.cond, cbits)) return;
-    const T *gm = reinterpret_cast<const T *>(a.mat);
-    for (int e = threadIdx.x; e < G * G; e += blockDim.x) mat[e] = gm[e];
-    const int gpb = kThreads >> K;          // groups per block iteration
-    const int g = threadIdx.x >> K, r = threadIdx.x & (G - 1);
-    uint64_t off = 0;                       // offset of register value r
-    for (int b = 0; b < K; ++b)
-        if ((r >> (K - 1 - b)) & 1) off |= 1ull << a.tpos[b];
-    for (uint64_t g0 = (uint64_t)blockIdx.x * gpb; g0 < a.n_groups; g0 += (uint64_t)gridDim.x * gpb) {
-        const uint64_t grp = g0 + g;
-        const bool live = grp < a.n_groups;
-        const uint64_t idx = live ? ((insert_zeros(grp, a.ins) | a.cmask) | off) : 0;
-        __syncthreads();
-        if (live) vec[threadIdx.x] = psi[idx];
-        __syncthreads();
-        if (live) {
-            T acc;
-            acc.x = 0;
-            acc.y = 0;
-            const T *row = mat + r * G;
-            const T *v = vec + g * G;
-            for (int c = 0; c < G; ++c) {
-                const T m = row[c], x = v[c];
-                acc.x += m.x * x.x - m.y * x.y;
-                acc.y += m.x * x.y + m.y * x.x;
-            }
-            psi[idx] = acc;
         }
     }
 }
@@ -769,27 +726,6 @@ cudaError_t launch_phase(int prec, void *psi, const PhaseArgs &a, const uint8_t 
         k_phase<double, 0><<<grid_for(a.n_units, sms), kThreads, 0, s>>>((double2 *)psi, a, cbits);
     }
     return cudaGetLastError();
-}
-
-template <typename R>
-static cudaError_t matk_r(void *psi, const MatKArgs &a, const uint8_t *cbits, int sms, cudaStream_t s) {
-    using T = typename Amp<R>::T;
-    if (a.k < 1 || a.k > 6) return cudaErrorInvalidValue;
-    const size_t sm = sizeof(T) * (((size_t)1 << (2 * a.k)) + kThreads);
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_matk<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
-    const uint64_t gpb = kThreads >> a.k;
-    uint64_t blocks = (a.n_groups + gpb - 1) / gpb;
-    if (blocks > (uint64_t)sms * 8) blocks = (uint64_t)sms * 8;
-    k_matk<R><<<(unsigned)blocks, kThreads, sm, s>>>((T *)psi, a, cbits);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_matk(int prec, void *psi, const MatKArgs &a, const uint8_t *cbits, int sms,
-                        cudaStream_t s) {
-    return prec == 0 ? matk_r<float>(psi, a, cbits, sms, s) : matk_r<double>(psi, a, cbits, sms, s);
 }
 
 // k_modexp_tiled where the register is a field of at most 12 bits (complex64) whose

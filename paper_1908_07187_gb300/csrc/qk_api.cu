@@ -129,7 +129,9 @@ struct qk_ctx {
     std::vector<GateDef> gates;
     void *d_swap_mat = nullptr;    // SWAP as a 4x4 matrix, for controlled SWAPs
 
-    std::vector<qk::FusedOp> pending;   // fused-mode queue (physical qubits)
+    // fused-mode queues (physical qubits); at most one of them holds gates
+    std::vector<qk::FusedOp> pending;
+    std::vector<qk::DenseItem> dense;
     qk::TilePlanner *planner = nullptr;
 
     uint64_t launches = 0, passes_x1000 = 0;
@@ -315,7 +317,25 @@ qk_status run_op_plain(qk_ctx *c, const qk::FusedOp &op) {
     return QK_OK;
 }
 
+// run the queued dense gates
+qk_status flush_dense(qk_ctx *c) {
+    if (c->dense.empty()) return QK_OK;
+    const qk_status st = qk::plan_dense(c->n, (int)c->prec, c->dense, [&](qk::DenseParams &P) -> qk_status {
+        double amps = 0.0;   // what the pass's gates touch, once
+        for (int i = 0; i < P.nops; ++i)
+            amps = std::max(amps, std::ldexp((double)P.n_tiles, P.ops[i].nfree + P.k + P.ops[i].ncs -
+                                                                    __builtin_popcount(P.ops[i].tmask)));
+        LaunchScope ls(c, 3, 2.0 * (double)c->amp * amps);
+        CUDA_TRY(c, qk::launch_dense((int)c->prec, c->d_state, P, c->d_cbits, c->sms, c->stream));
+        return QK_OK;
+    });
+    c->dense.clear();
+    return st;
+}
+
 qk_status flush(qk_ctx *c) {
+    const qk_status ds = flush_dense(c);
+    if (ds != QK_OK) return ds;
     if (c->pending.empty()) return QK_OK;
     qk_status st = QK_OK;
     if (c->opt.exec_mode == QK_EXEC_FUSED && c->planner) {
@@ -332,8 +352,30 @@ qk_status flush(qk_ctx *c) {
 
 qk_status enqueue(qk_ctx *c, const qk::FusedOp &op) {
     if (c->opt.exec_mode == QK_EXEC_PLAIN) return run_op_plain(c, op);
+    const qk_status ds = flush_dense(c);
+    if (ds != QK_OK) return ds;
     c->pending.push_back(op);
     if ((int)c->pending.size() >= c->opt.max_pending) return flush(c);
+    return QK_OK;
+}
+
+// Queue a dense k-qubit gate (plain mode: run it).
+qk_status apply_dense(qk_ctx *c, const void *mat, int k, const int *targets, uint64_t cmask, const qk::Cond &cond) {
+    if (!c->pending.empty()) {
+        const qk_status s = flush(c);
+        if (s != QK_OK) return s;
+    }
+    qk::DenseItem it;
+    it.k = k;
+    for (int t = 0; t < k; ++t) {
+        it.tpos[t] = c->l2p[targets[t]];
+        it.tmask |= 1ull << it.tpos[t];
+    }
+    it.cmask = cmask;
+    it.mat = mat;
+    it.cond = cond;
+    c->dense.push_back(it);
+    if (c->opt.exec_mode == QK_EXEC_PLAIN || (int)c->dense.size() >= c->opt.max_pending) return flush_dense(c);
     return QK_OK;
 }
 
@@ -789,22 +831,7 @@ qk_status qk_apply_gate(qk_ctx *c, int gate_id, const int *targets, int nt, cons
                 return s;
             }
             // controlled or classically conditioned SWAP: dense 4x4 block
-            qk_status s = flush(c);
-            if (s != QK_OK) return s;
-            qk::MatKArgs a{};
-            a.k = 2;
-            a.tpos[0] = c->l2p[targets[0]];
-            a.tpos[1] = c->l2p[targets[1]];
-            a.cmask = cmask;
-            std::vector<int> pos{a.tpos[0], a.tpos[1]};
-            for (int b = 0; b < nc; ++b) pos.push_back(c->l2p[controls[b]]);
-            set_positions(a.ins, pos);
-            a.n_groups = 1ull << (c->n - (int)pos.size());
-            a.mat = c->d_swap_mat;
-            a.cond = cond;
-            LaunchScope ls(c, 3, (double)2 * c->amp * (double)(a.n_groups << 2));
-            CUDA_TRY(c, qk::launch_matk((int)c->prec, c->d_state, a, c->d_cbits, c->sms, c->stream));
-            return QK_OK;
+            return apply_dense(c, c->d_swap_mat, 2, targets, cmask, cond);
         }
         return apply_1q(c, m, c->l2p[targets[0]], cmask, cond);
     }
@@ -841,10 +868,10 @@ qk_status qk_apply_gate(qk_ctx *c, int gate_id, const int *targets, int nt, cons
                 return QK_OK;
             }
         }
-        qk_status s = flush(c);
-        if (s != QK_OK) return s;
         if (g.k >= 3 && g.k <= 5 && c->n >= 5 && c->prec == QK_C64 && nc == 0 && ncc == 0 &&
             !c->opt.no_tensor_cores) {
+            qk_status s = flush(c);
+            if (s != QK_OK) return s;
             // targets elsewhere are first gathered onto the lowest physical qubits
             // (one relabelling pass), which costs far less than a CUDA-core block
             // pass; 3- and 4-qubit gates run as 5-qubit blocks U (x) I
@@ -854,22 +881,7 @@ qk_status qk_apply_gate(qk_ctx *c, int gate_id, const int *targets, int nt, cons
             for (int a = 0; a < g.k; ++a) key |= (uint32_t)c->l2p[targets[a]] << (3 * a);
             return apply_block_tc(c, gate_id, targets, key);
         }
-        qk::MatKArgs a{};
-        a.k = g.k;
-        std::vector<int> pos;
-        for (int t = 0; t < g.k; ++t) {
-            a.tpos[t] = c->l2p[targets[t]];
-            pos.push_back(a.tpos[t]);
-        }
-        for (int b = 0; b < nc; ++b) pos.push_back(c->l2p[controls[b]]);
-        set_positions(a.ins, pos);
-        a.cmask = cmask;
-        a.n_groups = 1ull << (c->n - (int)pos.size());
-        a.mat = g.d_mat;
-        a.cond = cond;
-        LaunchScope ls(c, 3, (double)2 * c->amp * (double)(a.n_groups << g.k));
-        CUDA_TRY(c, qk::launch_matk((int)c->prec, c->d_state, a, c->d_cbits, c->sms, c->stream));
-        return QK_OK;
+        return apply_dense(c, g.d_mat, g.k, targets, cmask, cond);
     }
     // permutation gates: out-of-place gather into scratch, then swap buffers
     qk_status s = flush(c);
@@ -1146,6 +1158,7 @@ qk_status qk_set_state(qk_ctx *c, const void *host_in, size_t bytes) {
     if (c->n == 0 || !host_in || bytes != c->state_bytes)
         return fail(c, QK_EINVAL, "set_state: need a buffer of exactly %zu bytes", c->state_bytes);
     c->pending.clear();
+    c->dense.clear();
     for (int q = 0; q < c->n; ++q) c->l2p[q] = q;
     CUDA_TRY(c, cudaMemcpyAsync(c->d_state, host_in, bytes, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
@@ -1156,6 +1169,7 @@ qk_status qk_reset(qk_ctx *c) {
     if (!c) return QK_EINVAL;
     if (c->n == 0) return fail(c, QK_ESTATE, "reset: no qubits");
     c->pending.clear();
+    c->dense.clear();
     for (int q = 0; q < c->n; ++q) c->l2p[q] = q;
     CUDA_TRY(c, cudaMemsetAsync(c->d_state, 0, c->state_bytes, c->stream));
     CUDA_TRY(c, qk::launch_set_basis((int)c->prec, c->d_state, 0, c->stream));

@@ -49,17 +49,6 @@ struct PhaseArgs {
     int rphase_idx[kMaxRphase];
 };
 
-// Dense k-qubit matrix on arbitrary targets with controls.
-struct MatKArgs {
-    int k;
-    int tpos[8];          // physical bit of register bit (k-1-a), a = list index; tpos[0] = MSB
-    uint64_t cmask;
-    Positions ins;        // targets and controls, sorted
-    uint64_t n_groups;
-    const void *mat;      // device matrix, 2^k x 2^k, row-major, amplitude type
-    Cond cond;
-};
-
 // Controlled permutation of a w-bit register, out-of-place gather.
 // A register whose qubits sit on consecutive physical bits p0 .. p0 + w - 1 is a bit
 // field of the index: its value is the field itself (first-listed qubit highest,
@@ -508,14 +497,53 @@ static_assert(sizeof(Tile128Params) <= 32764, "tile program must fit in the kern
 cudaError_t launch_tile128(void *psi, const Tile128Params &p, const uint8_t *cbits, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
+// dense k-qubit gates on CUDA cores (kernels_dense.cu): a pass keeps a tile of 2^m
+// amplitudes over m physical qubits S[0..m-1] (ascending) in shared memory and applies
+// a run of dense gates whose targets all lie in S.
+// ---------------------------------------------------------------------------
+constexpr int kDenseMaxK = 6;
+constexpr int kDenseOps = 48;
+constexpr int kDenseElems = 4096;    // matrix entries of one pass in shared memory
+constexpr int kDenseMaxBits = 13;
+// Shared-memory slot of local index i, linear over GF(2): index bits b, b + 4, b + 8 and
+// b + 12 fold onto bank bit b
+__host__ __device__ constexpr uint32_t dense_slot(uint32_t i) {
+    return i ^ ((i >> 4) & 15u) ^ ((i >> 8) & 15u) ^ ((i >> 12) & 15u);
+}
+struct DenseOp {
+    int8_t nfree;                // local bits that are neither targets nor local controls
+    uint8_t cond;                // index into conds, 0xff: none
+    uint16_t ls;                 // slot of the local control bits set
+    uint16_t ts[kDenseMaxK];     // slot of register bit b (b = 0: the last-listed target)
+    uint16_t fs[kDenseMaxBits];  // slots of the free bits; the first four on distinct banks where possible
+    // k = 2: a thread's 16 amplitudes are the register values times ncs column bits (slots
+    // cs); with pair set those are the next op's register bits, and both gates are applied
+    // while the amplitudes are in registers (that op is then skipped)
+    uint8_t pair, ncs;
+    uint16_t cs[2];
+    uint32_t tmask;              // tile-index control bits
+    const void *mat;             // device matrix, 2^k x 2^k, row-major, amplitude type
+};
+struct DenseParams {
+    uint64_t n_tiles;
+    uint64_t base;               // physical control bits that every tile has set (not in S, not enumerated)
+    int m, nfix;
+    int8_t S[16];
+    int8_t fixed[36];            // physical bits of the tile index, ascending
+    int nops, k;                 // every gate of a pass has the same k
+    int n_conds;
+    Cond conds[kTileMaxConds];
+    DenseOp ops[kDenseOps];
+};
+cudaError_t launch_dense(int prec, void *psi, const DenseParams &p, const uint8_t *cbits, int sms, cudaStream_t s);
+
+// ---------------------------------------------------------------------------
 // launchers (kernels_basic.cu); prec: 0 = complex64, 1 = complex128
 // ---------------------------------------------------------------------------
 cudaError_t launch_u2(int prec, void *psi, const U2Args &a, const uint8_t *cbits, int n, int sms,
                       cudaStream_t s);
 cudaError_t launch_phase(int prec, void *psi, const PhaseArgs &a, const uint8_t *cbits, int sms,
                          cudaStream_t s);
-cudaError_t launch_matk(int prec, void *psi, const MatKArgs &a, const uint8_t *cbits, int sms,
-                        cudaStream_t s);
 cudaError_t launch_modexp(int prec, const void *in, void *out, const ModExpArgs &a, const uint8_t *cbits, int sms,
                           cudaStream_t s);
 cudaError_t launch_perm(int prec, const void *in, void *out, const PermArgs &a, const uint8_t *cbits,

@@ -1374,6 +1374,134 @@ qk_status plan_passes(TilePlanner *planner, int n, const std::vector<FusedOp> &o
     return QK_OK;
 }
 
+// A dense pass: S starts as the lowest qubits (runs of 128 bytes in HBM, 32 for states in
+// L2) and takes the targets of every gate, in order, that commutes with the gates left
+// behind, has the first one's k and still fits.  A pass of one controlled gate enumerates only the tiles whose
+// control bits are set.  Fewer amplitudes per tile for small states, so that there are
+// tiles for all SMs.
+qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const DenseSink &sink) {
+    std::vector<const DenseItem *> rem, left, taken;
+    for (const DenseItem &it : ops) rem.push_back(&it);
+    while (!rem.empty()) {
+        left.clear();
+        taken.clear();
+        static thread_local DenseParams P;
+        std::memset(static_cast<void *>(&P), 0, offsetof(DenseParams, ops));
+        // complex64 gates of 5 and 6 qubits form 8 rows per thread, which takes 2^13
+        // amplitudes to give every thread columns
+        int m = prec != 0 ? 11 : rem[0]->k >= 5 ? 13 : 12;
+        if (n < 20) m = std::min(m, n >= 18 ? 11 : n >= 16 ? 10 : 9);
+        m = std::min(m, n);
+        const int contig = std::min(m, n >= 23 ? 4 : 2);
+        uint64_t S = 0, left_t = 0, left_all = 0;
+        int elems = 0;
+        const uint64_t low = (1ull << contig) - 1;
+        for (const DenseItem *it : rem) {
+            const uint64_t all = it->tmask | it->cmask;
+            bool ok = (int)taken.size() < kDenseOps && it->k == rem[0]->k &&
+                      elems + (1 << (2 * it->k)) <= kDenseElems &&
+                      !(it->tmask & left_all) && !(all & left_t);
+            // the first gate may use the room of the low qubits
+            if (ok && __builtin_popcountll(S | it->tmask | (taken.empty() ? 0 : low)) > m) ok = false;
+            int ci = -1;
+            if (ok && it->cond.n) {
+                for (int k = 0; k < P.n_conds; ++k)
+                    if (same_cond(P.conds[k], it->cond)) ci = k;
+                if (ci < 0 && P.n_conds >= kTileMaxConds) ok = false;
+                else if (ci < 0) {
+                    ci = P.n_conds++;
+                    P.conds[ci] = it->cond;
+                }
+            }
+            if (!ok) {
+                left.push_back(it);
+                left_t |= it->tmask;
+                left_all |= all;
+                continue;
+            }
+            S |= it->tmask;
+            elems += 1 << (2 * it->k);
+            taken.push_back(it);
+        }
+        const uint64_t lone = taken.size() == 1 ? taken[0]->cmask : 0;   // enumerated only where set
+        for (int b = 0; b < n && __builtin_popcountll(S) < m; ++b)
+            if (!((S | lone) >> b & 1)) S |= 1ull << b;
+        P.m = __builtin_popcountll(S);
+        P.base = lone;
+        int local_of[64], tile_of[64];
+        for (int b = 0, lb = 0; b < n; ++b) {
+            local_of[b] = tile_of[b] = -1;
+            if ((S >> b) & 1) {
+                P.S[lb] = (int8_t)b;
+                local_of[b] = lb++;
+            } else if (!((lone >> b) & 1)) {
+                P.fixed[P.nfix] = (int8_t)b;
+                tile_of[b] = P.nfix++;
+            }
+        }
+        P.n_tiles = 1ull << P.nfix;
+        P.k = rem[0]->k;
+        for (const DenseItem *const &it : taken) {
+            DenseOp &o = P.ops[P.nops++];
+            std::memset(static_cast<void *>(&o), 0, sizeof o);
+            uint32_t used = 0;
+            for (int b = 0; b < it->k; ++b) {
+                const int lb = local_of[it->tpos[it->k - 1 - b]];
+                o.ts[b] = (uint16_t)dense_slot(1u << lb);
+                used |= 1u << lb;
+            }
+            o.cond = 0xff;
+            if (it->cond.n)
+                for (int k = 0; k < P.n_conds; ++k)
+                    if (same_cond(P.conds[k], it->cond)) o.cond = (uint8_t)k;
+            for (uint64_t c = it->cmask & ~lone; c; c &= c - 1) {
+                const int b = __builtin_ctzll(c);
+                if (local_of[b] >= 0) {
+                    o.ls ^= (uint16_t)dense_slot(1u << local_of[b]);
+                    used |= 1u << local_of[b];
+                } else {
+                    o.tmask |= 1u << tile_of[b];
+                }
+            }
+            // two 2-qubit gates in a row on other qubits, both unconditional: one round trip
+            // through shared memory.  The first one's column bits are the second's register
+            // bits (or, for one gate alone, its last free bits).
+            const bool joined = P.nops >= 2 && P.ops[P.nops - 2].pair;
+            const bool free2 = it->k == 2 && !it->cmask && !it->cond.n;
+            o.pair = 0;
+            if (free2 && !joined && &it != &taken.back()) {
+                const DenseItem *nx = (&it)[1];
+                if (!nx->cmask && !nx->cond.n && !(nx->tmask & it->tmask)) {
+                    o.pair = 1;
+                    o.ncs = 2;
+                    for (int b = 0; b < 2; ++b) {
+                        const int lb = local_of[nx->tpos[1 - b]];
+                        o.cs[b] = (uint16_t)dense_slot(1u << lb);
+                        used |= 1u << lb;
+                    }
+                }
+            }
+            // free bits: lanes walk the first ones, so those go to distinct banks (bit mod 4)
+            uint32_t banks = 0, placed = used;
+            for (int pass = 0; pass < 2; ++pass)
+                for (int b = 0; b < P.m; ++b) {
+                    if ((placed >> b) & 1u) continue;
+                    if (pass == 0 && ((banks >> (b & 3)) & 1u)) continue;
+                    banks |= 1u << (b & 3);
+                    placed |= 1u << b;
+                    o.fs[o.nfree++] = (uint16_t)dense_slot(1u << b);
+                }
+            if (it->k == 2 && !o.pair)
+                while (o.ncs < 2 && o.nfree > 0) o.cs[o.ncs++] = o.fs[--o.nfree];
+            o.mat = it->mat;
+        }
+        const qk_status st = sink(P);
+        if (st != QK_OK) return st;
+        rem.swap(left);
+    }
+    return QK_OK;
+}
+
 qk_status run_fused(TilePlanner *planner, qk_ctx *c, const std::vector<FusedOp> &ops) {
     const int n = ctx_n(c);
     if (ctx_prec(c) != 0) {

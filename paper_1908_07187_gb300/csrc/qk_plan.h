@@ -25,6 +25,20 @@ struct FusedOp {
     Cond cond{};
 };
 
+// A queued dense k-qubit gate in physical qubits: 2^k x 2^k device matrix on targets
+// tpos[0..k-1] (tpos[0] = register MSB) where all cmask bits are 1.
+struct DenseItem {
+    int k = 0;
+    int tpos[kDenseMaxK];
+    uint64_t tmask = 0, cmask = 0;
+    const void *mat = nullptr;
+    Cond cond{};
+};
+// Group an ordered list of dense gates into passes (DenseParams); with one gate per
+// call (plain mode) the pass holds that gate.
+using DenseSink = std::function<qk_status(DenseParams &)>;
+qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const DenseSink &sink);
+
 struct TilePlanner;
 TilePlanner *make_planner();
 void free_planner(TilePlanner *p);
