@@ -1,17 +1,20 @@
-// Fused tile pass for complex128 states (Tile128Params in qk_kernels.cuh).
+// Fused pass over tiles in shared memory (SmemTileParams in qk_kernels.cuh): complex128
+// states, and complex64 states below 13 qubits.
 //
 // One CTA owns one tile of 2^m amplitudes in shared memory: it is read once, a
-// program of gates runs on it, and it is written back once.  With 2 FP64 lanes per SM
-// and clock a warp's FP64 instruction takes 16 cycles of the SM's FP64 unit, which is
-// the bound here (a gate's pair: 6 instructions, 96 cycles per warp, against 16 to 32
-// cycles of shared-memory traffic and about 10 of issue), so amplitudes stay in
-// shared memory between gates -- no register arrangements, no transposes -- and the
-// program does whatever it can by exchange, sign bit and index arithmetic.  The tile
-// width falls with the state (planner) so that small states still spread over the SMs.
-// Measured against one pass per gate: a 23-qubit circuit of 161 U3, 139 CZ and the QFT
-// 33.0 -> 10.7 ms (six passes; the FP64 unit's own time for its 5.2 G instructions per
-// lane is 8.3 ms), the 12-qubit circuit of 290 gates 1322 -> 333 us (bound by the
-// latency of one short op after another).
+// program of gates runs on it, and it is written back once.  In complex128, with 2
+// FP64 lanes per SM and clock, a warp's FP64 instruction takes 16 cycles of the SM's
+// FP64 unit, which is the bound (a gate's pair: 6 instructions, 96 cycles per warp,
+// against 16 to 32 cycles of shared-memory traffic and about 10 of issue), so
+// amplitudes stay in shared memory between gates -- no register arrangements, no
+// transposes -- and the program does whatever it can by exchange, sign bit and index
+// arithmetic.  The tile width falls with the state (planner) so that small states
+// still spread over the SMs.  Measured against one pass per gate: a 23-qubit
+// complex128 circuit of 161 U3, 139 CZ and the QFT 33.0 -> 10.7 ms (six passes; the
+// FP64 unit's own time for its 5.2 G instructions per lane is 8.3 ms), the 12-qubit
+// complex128 circuit of 290 gates 1322 -> 333 us (bound by the latency of one short op
+// after another), a 10-qubit complex64 circuit of 175 gates, viewed and measured, 828
+// -> 158 us.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -22,8 +25,20 @@ namespace {
 
 constexpr int kMaxThreads = 256;
 
-__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+template <typename R> struct Amp;
+template <> struct Amp<float> { using T = float2; };
+template <> struct Amp<double> { using T = double2; };
+__device__ __forceinline__ float2 pair(float x, float y) { return make_float2(x, y); }
+__device__ __forceinline__ double2 pair(double x, double y) { return make_double2(x, y); }
+// an op's coefficients and a program's factors in the working precision
+__device__ __forceinline__ const float *coef(const SmemTileOp &op, float) { return op.cf; }
+__device__ __forceinline__ const double *coef(const SmemTileOp &op, double) { return op.c; }
+__device__ __forceinline__ const float2 *factors(const SmemTileParams &P, float) { return P.facf; }
+__device__ __forceinline__ const double2 *factors(const SmemTileParams &P, double) { return P.fac; }
+
+template <typename T>
+__device__ __forceinline__ T cmul(T a, T b) {
+    return pair(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __device__ __forceinline__ uint32_t ins0(uint32_t j, int pos) {
     const uint32_t lo = j & ((1u << pos) - 1);
@@ -37,23 +52,20 @@ __device__ __forceinline__ uint32_t spread(uint32_t j, uint32_t mask) {
 __device__ __forceinline__ double flip(double x, uint32_t s) {   // s = 0 or 0x80000000
     return __hiloint2double(__double2hiint(x) ^ (int)s, __double2loint(x));
 }
-// i^k a
-__device__ __forceinline__ double2 quarter(double2 a, int k) {
-    const uint32_t sx = (k == 1 || k == 2) ? 0x80000000u : 0u, sy = (k & 2) ? 0x80000000u : 0u;
-    const bool sw = k & 1;
-    return make_double2(flip(sw ? a.y : a.x, sx), flip(sw ? a.x : a.y, sy));
-}
+__device__ __forceinline__ float flip(float x, uint32_t s) { return __uint_as_float(__float_as_uint(x) ^ s); }
 
-// One D128_U2 op.  The value that is turned and the one that is not are told apart by
+// One ST_U2 op.  The value that is turned and the one that is not are told apart by
 // their shared-memory slots, and the two orders of update are separate loops: as
 // branches inside one loop they became predicated instructions, which occupy the FP64
 // pipe (12 issued for the 6 that count).
-template <bool kFirst0, bool kPhase>
-__device__ __forceinline__ void u2_sweep(double2 *A, const Tile128Op &op, uint32_t tile, uint32_t half) {
+template <bool kFirst0, bool kPhase, typename T>
+__device__ __forceinline__ void u2_sweep(T *A, const SmemTileOp &op, uint32_t tile, uint32_t half) {
     const int fl = op.flags, q = op.q;
     const bool on0 = fl & kU2On0, lift = fl & kU2Lift, swap = fl & kU2Swap;
     const int k = on0 ? (4 - fl) & 3 : fl & 3;
-    const double t = on0 ? -op.c[0] : op.c[0], c0 = op.c[1], c1 = op.c[2];
+    using R = decltype(T().x);
+    const R *c = coef(op, R());
+    const R t = on0 ? -c[0] : c[0], c0 = c[1], c1 = c[2];
     const uint32_t smask = op.lmask, par = __popc(tile & op.tmask) & 1u, bit = 1u << q;
     // quarter turns: exchange of the parts, then signs
     const uint32_t kx = (k == 1 || k == 2) ? 0x80000000u : 0u, ky = (k & 2) ? 0x80000000u : 0u;
@@ -61,13 +73,13 @@ __device__ __forceinline__ void u2_sweep(double2 *A, const Tile128Op &op, uint32
     const bool turn0 = on0 && (k & 1), turn1 = !on0 && (k & 1);
     for (uint32_t p = threadIdx.x; p < half; p += blockDim.x) {
         const uint32_t i0 = ins0(p, q), i1 = i0 | bit;
-        const double2 v0 = A[i0], v1 = A[i1];
+        const T v0 = A[i0], v1 = A[i1];
         const uint32_t s = ((__popc(i0 & smask) + par) & 1u) << 31;
-        double2 z0 = make_double2(flip(turn0 ? v0.y : v0.x, x0), flip(turn0 ? v0.x : v0.y, y0s));
-        double2 z1 = make_double2(flip(turn1 ? v1.y : v1.x, x1 ^ s), flip(turn1 ? v1.x : v1.y, y1s ^ s));
+        T z0 = pair(flip(turn0 ? v0.y : v0.x, x0), flip(turn0 ? v0.x : v0.y, y0s));
+        T z1 = pair(flip(turn1 ? v1.y : v1.x, x1 ^ s), flip(turn1 ? v1.x : v1.y, y1s ^ s));
         if constexpr (kPhase) {
-            const double2 w = on0 ? z0 : z1;
-            const double2 r = make_double2(fma(-t, w.y, w.x), fma(t, w.x, w.y));
+            const T w = on0 ? z0 : z1;
+            const T r = pair(fma(-t, w.y, w.x), fma(t, w.x, w.y));
             if (on0) z0 = r;
             else z1 = r;
         }
@@ -89,29 +101,31 @@ __device__ __forceinline__ void u2_sweep(double2 *A, const Tile128Op &op, uint32
     }
 }
 
-// factors of a D128_TABLE op: lo[j] over local bits 0..5, hi[j] over the others times
+// factors of a ST_TABLE op: lo[j] over local bits 0..5, hi[j] over the others times
 // the constant and the tile-index bits' factors; built by doubling, a warp each.
 // Without factors on one side its table is left out (the constant goes to the other).
-__device__ __forceinline__ void build_tables(const Tile128Params &P, const Tile128Op &op, uint32_t tile, double2 *lo,
-                                             double2 *hi, int warp, int lane) {
+template <typename T>
+__device__ __forceinline__ void build_tables(const SmemTileParams &P, const SmemTileOp &op, uint32_t tile, T *lo, T *hi,
+                                             int warp, int lane) {
+    using R = decltype(T().x);
+    const T *fac = factors(P, R());
     const uint32_t lf = op.lmask;
     const bool use_hi = (lf >> 6) != 0;
     if (warp > 1) return;
-    double2 *tab = warp == 0 ? lo : hi;
+    T *tab = warp == 0 ? lo : hi;
     if (warp == 1 && !use_hi) return;
-    double2 c0 = make_double2(1.0, 0.0);
+    T c0 = pair(R(1), R(0));
     if ((warp == 1) == use_hi) {
         // the constant and the tile-index factors: one bit per lane, multiplied over the warp
         if (op.tfac) {
             if ((op.tfac >> lane) & (tile >> lane) & 1u)
-                c0 = P.fac[op.first + __popc(lf) + __popc(op.tfac & ((1u << lane) - 1))];
+                c0 = fac[op.first + __popc(lf) + __popc(op.tfac & ((1u << lane) - 1))];
             for (int o = 16; o > 0; o >>= 1) {
-                const double2 x = make_double2(__shfl_xor_sync(0xffffffffu, c0.x, o),
-                                               __shfl_xor_sync(0xffffffffu, c0.y, o));
+                const T x = pair(__shfl_xor_sync(0xffffffffu, c0.x, o), __shfl_xor_sync(0xffffffffu, c0.y, o));
                 c0 = cmul(c0, x);
             }
         }
-        c0 = cmul(c0, make_double2(op.c[0], op.c[1]));
+        c0 = cmul(c0, pair(coef(op, R())[0], coef(op, R())[1]));
     }
     const int b0 = warp == 0 ? 0 : 6, b1 = warp == 0 ? min(6, P.m) : P.m;
     if (lane == 0) tab[0] = c0;
@@ -119,19 +133,22 @@ __device__ __forceinline__ void build_tables(const Tile128Params &P, const Tile1
         __syncwarp();
         const int half = 1 << (b - b0);
         if (lane < half) {
-            double2 v = tab[lane];
-            if ((lf >> b) & 1u) v = cmul(v, P.fac[op.first + __popc(lf & ((1u << b) - 1))]);
+            T v = tab[lane];
+            if ((lf >> b) & 1u) v = cmul(v, fac[op.first + __popc(lf & ((1u << b) - 1))]);
             tab[half + lane] = v;
         }
     }
 }
 
-__global__ void __launch_bounds__(kMaxThreads)
-    k_tile128(double2 *__restrict__ psi, const __grid_constant__ Tile128Params P, const uint8_t *__restrict__ cbits) {
+template <typename R>
+__global__ void __launch_bounds__(kMaxThreads, 3)
+    k_smem_tile(typename Amp<R>::T *__restrict__ psi, const __grid_constant__ SmemTileParams P,
+                const uint8_t *__restrict__ cbits) {
+    using T = typename Amp<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2 *A = reinterpret_cast<double2 *>(smem_raw);
+    T *A = reinterpret_cast<T *>(smem_raw);
     const uint32_t dim = 1u << P.m, half = dim >> 1;
-    double2 *lo = A + dim, *hi = lo + 64;
+    T *lo = A + dim, *hi = lo + 64;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t tile = blockIdx.x;
 
@@ -151,7 +168,7 @@ __global__ void __launch_bounds__(kMaxThreads)
     const bool live = (uint32_t)tid < dim;
     if (live) {
         for (uint32_t j0 = 0; j0 < rounds; j0 += 4) {
-            double2 v[4];
+            T v[4];
             const uint64_t hi_off = ((j0 & 4) ? st[2] : 0) + ((j0 & 8) ? st[3] : 0);
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -170,10 +187,10 @@ __global__ void __launch_bounds__(kMaxThreads)
     __syncthreads();
 
     for (int o = 0; o < P.nops; ++o) {
-        const Tile128Op &op = P.ops[o];
+        const SmemTileOp &op = P.ops[o];
         const int q = op.q;
         switch (op.kind) {
-            case D128_U2: {
+            case ST_U2: {
                 if (op.flags & kU2First0) {
                     if (op.flags & kU2Phase) u2_sweep<true, true>(A, op, tile, half);
                     else u2_sweep<true, false>(A, op, tile, half);
@@ -183,58 +200,58 @@ __global__ void __launch_bounds__(kMaxThreads)
                 }
                 break;
             }
-            case D128_X:
-            case D128_CU2: {
+            case ST_X:
+            case ST_CU2: {
                 if ((tile & op.tmask) != op.tval || (op.cond != kNoBit && !((condok >> op.cond) & 1u))) continue;
                 const uint32_t bit = 1u << q, cm = op.lmask, cnt = half >> __popc(cm);
-                if (op.kind == D128_X) {
+                if (op.kind == ST_X) {
                     for (uint32_t u = tid; u < cnt; u += nt) {
                         const uint32_t i0 = spread(u, cm | bit) | op.lval, i1 = i0 | bit;
-                        const double2 a = A[i0], b = A[i1];
+                        const T a = A[i0], b = A[i1];
                         A[i0] = b;
                         A[i1] = a;
                     }
                 } else {
-                    const double2 m00 = make_double2(op.c[0], op.c[1]), m01 = make_double2(op.c[2], op.c[3]);
-                    const double2 m10 = make_double2(op.c[4], op.c[5]), m11 = make_double2(op.c[6], op.c[7]);
+                    const R *c = coef(op, R());
+                    const T m00 = pair(c[0], c[1]), m01 = pair(c[2], c[3]), m10 = pair(c[4], c[5]), m11 = pair(c[6], c[7]);
                     for (uint32_t u = tid; u < cnt; u += nt) {
                         const uint32_t i0 = spread(u, cm | bit) | op.lval, i1 = i0 | bit;
-                        const double2 a = A[i0], b = A[i1];
-                        A[i0] = make_double2(m00.x * a.x - m00.y * a.y + m01.x * b.x - m01.y * b.y,
-                                             m00.x * a.y + m00.y * a.x + m01.x * b.y + m01.y * b.x);
-                        A[i1] = make_double2(m10.x * a.x - m10.y * a.y + m11.x * b.x - m11.y * b.y,
-                                             m10.x * a.y + m10.y * a.x + m11.x * b.y + m11.y * b.x);
+                        const T a = A[i0], b = A[i1];
+                        A[i0] = pair(m00.x * a.x - m00.y * a.y + m01.x * b.x - m01.y * b.y,
+                                     m00.x * a.y + m00.y * a.x + m01.x * b.y + m01.y * b.x);
+                        A[i1] = pair(m10.x * a.x - m10.y * a.y + m11.x * b.x - m11.y * b.y,
+                                     m10.x * a.y + m10.y * a.x + m11.x * b.y + m11.y * b.x);
                     }
                 }
                 break;
             }
-            case D128_SIGN: {
+            case ST_SIGN: {
                 const uint32_t par = __popc(tile & op.tmask) & 1u;
                 const uint32_t n_at = q == kNoBit ? dim : half;
                 if (op.tval & ~tile) continue;   // the common bit is a tile-index bit that is 0
                 for (uint32_t p = tid; p < n_at; p += nt) {
                     const uint32_t i = q == kNoBit ? p : ins0(p, q) | (1u << q);
                     if (((__popc(i & op.lmask) + par) & 1u) == 0) continue;
-                    double2 a = A[i];
+                    T a = A[i];
                     a.x = flip(a.x, 0x80000000u);
                     a.y = flip(a.y, 0x80000000u);
                     A[i] = a;
                 }
                 break;
             }
-            case D128_PH: {
+            case ST_PH: {
                 if ((tile & op.tmask) != op.tval || (op.cond != kNoBit && !((condok >> op.cond) & 1u))) continue;
-                const double2 f = make_double2(op.c[0], op.c[1]);
+                const T f = pair(coef(op, R())[0], coef(op, R())[1]);
                 const uint32_t cnt = dim >> __popc(op.lmask);
                 for (uint32_t u = tid; u < cnt; u += nt) {
                     const uint32_t i = spread(u, op.lmask) | op.lval;
-                    if (f.x == -1.0 && f.y == 0.0) A[i] = quarter(A[i], 2);
-                    else if (f.y == 0.0) A[i] = make_double2(A[i].x * f.x, A[i].y * f.x);
+                    if (f.x == -1 && f.y == 0) A[i] = pair(-A[i].x, -A[i].y);
+                    else if (f.y == 0) A[i] = pair(A[i].x * f.x, A[i].y * f.x);
                     else A[i] = cmul(A[i], f);
                 }
                 break;
             }
-            default: {   // D128_TABLE
+            default: {   // ST_TABLE
                 if ((tile & op.tmask) != op.tval) continue;
                 build_tables(P, op, tile, lo, hi, warp, lane);
                 __syncthreads();
@@ -242,7 +259,7 @@ __global__ void __launch_bounds__(kMaxThreads)
                 const uint32_t n_at = q == kNoBit ? dim : half;
                 for (uint32_t p = tid; p < n_at; p += nt) {
                     const uint32_t i = q == kNoBit ? p : ins0(p, q) | (1u << q);
-                    const double2 f = use_lo ? (use_hi ? cmul(lo[i & 63], hi[i >> 6]) : lo[i & 63]) : hi[i >> 6];
+                    const T f = use_lo ? (use_hi ? cmul(lo[i & 63], hi[i >> 6]) : lo[i & 63]) : hi[i >> 6];
                     A[i] = cmul(A[i], f);
                 }
                 break;
@@ -264,17 +281,23 @@ __global__ void __launch_bounds__(kMaxThreads)
 
 }  // namespace
 
-cudaError_t launch_tile128(void *psi, const Tile128Params &p, const uint8_t *cbits, cudaStream_t s) {
-    if (p.m < 1 || p.m > kTile128Max || p.nops < 0 || p.nops > kTile128Ops || p.nfix > 31) return cudaErrorInvalidValue;
-    const uint32_t half = 1u << (p.m - 1);
-    const unsigned nt = half < 64 ? 64u : half > kMaxThreads ? (unsigned)kMaxThreads : half;
-    const size_t sm = sizeof(double2) * (((size_t)1 << p.m) + 128);
+template <typename R>
+static cudaError_t smem_tile_r(void *psi, const SmemTileParams &p, const uint8_t *cbits, unsigned nt, cudaStream_t s) {
+    using T = typename Amp<R>::T;
+    const size_t sm = sizeof(T) * (((size_t)1 << p.m) + 128);
     if (sm > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_tile128, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        const cudaError_t e = cudaFuncSetAttribute(k_smem_tile<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
     }
-    k_tile128<<<p.n_tiles, nt, sm, s>>>((double2 *)psi, p, cbits);
+    k_smem_tile<R><<<p.n_tiles, nt, sm, s>>>((T *)psi, p, cbits);
     return cudaGetLastError();
+}
+
+cudaError_t launch_smem_tile(int prec, void *psi, const SmemTileParams &p, const uint8_t *cbits, cudaStream_t s) {
+    if (p.m < 1 || p.m > kSmemTileMax || p.nops < 0 || p.nops > kSmemTileOps || p.nfix > 31) return cudaErrorInvalidValue;
+    const uint32_t half = 1u << (p.m - 1);
+    const unsigned nt = half < 64 ? 64u : half > kMaxThreads ? (unsigned)kMaxThreads : half;
+    return prec == 0 ? smem_tile_r<float>(psi, p, cbits, nt, s) : smem_tile_r<double>(psi, p, cbits, nt, s);
 }
 
 }  // namespace qk

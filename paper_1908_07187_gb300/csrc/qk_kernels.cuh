@@ -447,54 +447,64 @@ cudaError_t launch_tile_batch(const TileProg *progs, const uint32_t *first, int 
 bool tile_ops_need_general(const TileOp *ops, size_t n);
 
 // ---------------------------------------------------------------------------
-// fused tile pass in complex128 (kernels_tile128.cu).  A tile is 2^m amplitudes in
-// shared memory over m physical qubits S[0..m-1] (ascending); the other n - m bits
-// are the tile index.  GB300 does 2 FP64 lane operations per SM and clock, so a pass
-// is bound by its FP64 operations alone and the program is built to need few:
-//   D128_U2    an uncontrolled 2x2 gate on local bit q, left-multiplied by a diagonal
+// fused pass over tiles in shared memory (kernels_smem_tile.cu): complex128 states of
+// any size, and complex64 states below the register tile's 13 qubits.  A tile is 2^m
+// amplitudes over m physical qubits S[0..m-1] (ascending); the other n - m bits are the
+// tile index.  GB300 does 2 FP64 lane operations per SM and clock, so in complex128 a
+// pass is bound by its FP64 operations alone and the program is built to need few; in
+// complex64 the states are small and the time goes to the latency of one op after
+// another:
+//   ST_U2    an uncontrolled 2x2 gate on local bit q, left-multiplied by a diagonal
 //              that the planner keeps: y1 times i^k (1 + i t) (or y0 times its
 //              conjugate), then two real in-place updates of one value from the
 //              other: 6 FMAs per pair instead of the 16 operations of a complex 2x2
 //              product; controlled-Z terms on q are sign flips on the way in
-//   D128_X     exchange of the pair where the controls match (no arithmetic)
-//   D128_CU2   controlled or conditioned 2x2 gate, 16 operations per matching pair
-//   D128_SIGN  sign flips of the amplitudes with bit q set by a parity (no arithmetic)
-//   D128_PH    one diagonal term on the matching amplitudes
-//   D128_TABLE a product of factors, one per set local and tile-index bit, on the
+//   ST_X     exchange of the pair where the controls match (no arithmetic)
+//   ST_CU2   controlled or conditioned 2x2 gate, 16 operations per matching pair
+//   ST_SIGN  sign flips of the amplitudes with bit q set by a parity (no arithmetic)
+//   ST_PH    one diagonal term on the matching amplitudes
+//   ST_TABLE a product of factors, one per set local and tile-index bit, on the
 //              amplitudes with bit q set (q = kNoBit: on all): two tables of 64
 // ---------------------------------------------------------------------------
-constexpr int kTile128Max = 12;      // local qubits
-constexpr int kTile128Ops = 144;
-constexpr int kTile128Facs = 576;
+constexpr int kSmemTileMax = 12;      // local qubits
+constexpr int kSmemTileOps = 144;
+constexpr int kSmemTileFacs = 576;
 constexpr uint8_t kNoBit = 0xff;
-enum Tile128Kind : uint8_t { D128_U2 = 0, D128_X = 1, D128_CU2 = 2, D128_SIGN = 3, D128_PH = 4, D128_TABLE = 5 };
-// D128_U2 flags: quarter turns in bits 0..1, then
+enum SmemTileKind : uint8_t { ST_U2 = 0, ST_X = 1, ST_CU2 = 2, ST_SIGN = 3, ST_PH = 4, ST_TABLE = 5 };
+// ST_U2 flags: quarter turns in bits 0..1, then
 constexpr uint8_t kU2Phase = 4;      // t != 0
 constexpr uint8_t kU2On0 = 8;        // the phase goes on y0
 constexpr uint8_t kU2First0 = 16;    // y0 is updated first
 constexpr uint8_t kU2Swap = 32;      // the results are stored exchanged
 constexpr uint8_t kU2Lift = 64;      // b0, b1 not both zero
-struct Tile128Op {
+struct SmemTileOp {
     uint8_t kind, q, flags, cond;    // cond: index into conds, kNoBit: none
     uint16_t lmask, lval;            // local-bit condition; U2, SIGN: parity mask in lmask; TABLE: bits with a factor
     uint32_t tmask, tval;            // the same on the tile index (U2, SIGN: parity mask in tmask)
     uint32_t tfac;                   // TABLE: tile-index bits with a factor
     uint32_t first;                  // TABLE: its factors, local bits ascending, then tile-index bits
-    double c[8];                     // U2: t, b0, b1; CU2: matrix; PH, TABLE: factor (re, im)
+    union {                          // U2: t, b0, b1; CU2: matrix; PH, TABLE: factor (re, im)
+        double c[8];                 // (as the planner forms them, and in complex128 programs)
+        float cf[8];                 // in complex64 programs
+    };
 };
-struct Tile128Params {
+struct SmemTileParams {
     uint32_t n_tiles;
     int n, m, nfix;
-    int8_t S[kTile128Max + 4];
+    int8_t S[kSmemTileMax + 4];
     int8_t fixed[32];                // physical bits of the tile index, ascending
     int n_conds;
     Cond conds[kTileMaxConds];
     int nops, nfac;
-    Tile128Op ops[kTile128Ops];
-    double2 fac[kTile128Facs];
+    SmemTileOp ops[kSmemTileOps];
+    union {
+        double2 fac[kSmemTileFacs];
+        float2 facf[kSmemTileFacs];
+    };
+    SmemTileParams() {}
 };
-static_assert(sizeof(Tile128Params) <= 32764, "tile program must fit in the kernel parameter space");
-cudaError_t launch_tile128(void *psi, const Tile128Params &p, const uint8_t *cbits, cudaStream_t s);
+static_assert(sizeof(SmemTileParams) <= 32764, "tile program must fit in the kernel parameter space");
+cudaError_t launch_smem_tile(int prec, void *psi, const SmemTileParams &p, const uint8_t *cbits, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // dense k-qubit gates on CUDA cores (kernels_dense.cu): a pass keeps a tile of 2^m

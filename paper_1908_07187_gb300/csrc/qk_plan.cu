@@ -309,7 +309,7 @@ uint64_t choose_pass(const std::vector<POp> &rem, int n, const TakeLimits &lim, 
 }
 
 // ---------------------------------------------------------------------------
-// complex128 passes (Tile128Params in qk_kernels.cuh)
+// passes over tiles in shared memory (SmemTileParams in qk_kernels.cuh)
 // ---------------------------------------------------------------------------
 
 // Tile width by state size: wide tiles carry more gates per read and write of a state
@@ -317,10 +317,14 @@ uint64_t choose_pass(const std::vector<POp> &rem, int n, const TakeLimits &lim, 
 // FP64 lanes take 6 us for one gate on 2^12 amplitudes.  Measured on U3 / CZ / QFT
 // circuits (us at 8, 10 and 12 tile qubits): 12 qubits 263 / 384 / 879, 16 qubits 333 /
 // 412 / 924, 18 qubits 609 / 599 / 1003, 20 qubits 1831 / 1616 / 1676, 22 qubits 6691 /
-// 5677 / 5413.
-int tile128_qubits(int n) { return std::min(n, n <= 16 ? 8 : n <= 20 ? 10 : kTile128Max); }
+// 5677 / 5413.  complex64 (below 13 qubits, at 8, 9, 10 and 12 tile qubits): 10 qubits
+// 159 / 158 / 172 / 174, 12 qubits 182 / 170 / 184 / 231.
+int smem_tile_qubits(int n, int prec) {
+    if (prec == 0) return std::min(n, 9);
+    return std::min(n, n <= 16 ? 8 : n <= 20 ? 10 : kSmemTileMax);
+}
 // Qubits that every tile holds, for runs of 128 bytes in HBM; none for states in L2.
-int tile128_contig(int n) { return n >= 18 ? 3 : 0; }
+int smem_tile_contig(int n) { return n >= 18 ? 3 : 0; }
 
 // A diagonal term that is not yet in a program: f where (index & mask) == val.
 struct DTerm {
@@ -334,22 +338,22 @@ struct DTerm {
 // never reach the device: F[q] is the pending complex factor of physical qubit q's |1>,
 // lam the one of every amplitude.  Diagonal terms on more qubits wait in terms until a
 // gate acts on one of their qubits and go out together there.
-struct Tile128Builder {
-    Tile128Params &P;
+struct SmemTileBuilder {
+    SmemTileParams &P;
     cdm *F;
     cdm &lam;
     int local_of[64], tile_of[64];
     std::vector<DTerm> terms;
     bool overflow = false;
 
-    Tile128Builder(Tile128Params &p, cdm *f, cdm &l) : P(p), F(f), lam(l) {}
+    SmemTileBuilder(SmemTileParams &p, cdm *f, cdm &l) : P(p), F(f), lam(l) {}
 
-    Tile128Op *add(uint8_t kind, uint8_t q) {
-        if (P.nops >= kTile128Ops) {
+    SmemTileOp *add(uint8_t kind, uint8_t q) {
+        if (P.nops >= kSmemTileOps) {
             overflow = true;
             P.nops = 0;      // the program is thrown away
         }
-        Tile128Op &o = P.ops[P.nops++];
+        SmemTileOp &o = P.ops[P.nops++];
         std::memset(static_cast<void *>(&o), 0, sizeof o);
         o.kind = kind;
         o.q = q;
@@ -357,7 +361,7 @@ struct Tile128Builder {
         return &o;
     }
     // mask and value over physical bits as local and tile-index conditions
-    void conditions(Tile128Op &o, uint64_t mask, uint64_t val) {
+    void conditions(SmemTileOp &o, uint64_t mask, uint64_t val) {
         for (uint64_t m = mask; m; m &= m - 1) {
             const int b = __builtin_ctzll(m);
             const uint32_t v = (uint32_t)(val >> b) & 1u;
@@ -417,21 +421,21 @@ struct Tile128Builder {
     static bool is_sign(const DTerm &t) { return t.f == cdm(-1.0, 0.0); }
 
     void single_term(const DTerm &t) {
-        Tile128Op *o = add(D128_PH, kNoBit);
+        SmemTileOp *o = add(ST_PH, kNoBit);
         conditions(*o, t.mask, t.val);
         if (t.cond) o->cond = cond_index(*t.cond);
         o->c[0] = t.f.real();
         o->c[1] = t.f.imag();
     }
     // an op on the amplitudes with physical bit b set: its local bit, or a tile-index condition
-    void on_bit(Tile128Op &o, int b) {
+    void on_bit(SmemTileOp &o, int b) {
         if (local_of[b] >= 0) o.q = (uint8_t)local_of[b];
         else o.tval |= 1u << tile_of[b];
     }
     // factors fac[b] of the physical bits in bits, times c0, on the amplitudes with
     // physical bit at set (at < 0: on all)
     void table(int at, uint64_t bits, const cdm *fac, cdm c0) {
-        Tile128Op *o = add(D128_TABLE, kNoBit);
+        SmemTileOp *o = add(ST_TABLE, kNoBit);
         if (at >= 0) {
             on_bit(*o, at);
             o->tmask = o->tval;
@@ -439,7 +443,7 @@ struct Tile128Builder {
         o->first = (uint32_t)P.nfac;
         o->c[0] = c0.real();
         o->c[1] = c0.imag();
-        if (P.nfac + __builtin_popcountll(bits) > kTile128Facs) {
+        if (P.nfac + __builtin_popcountll(bits) > kSmemTileFacs) {
             overflow = true;
             return;
         }
@@ -493,7 +497,7 @@ struct Tile128Builder {
             *st = g;
             return;
         }
-        Tile128Op *o = add(D128_SIGN, kNoBit);
+        SmemTileOp *o = add(ST_SIGN, kNoBit);
         on_bit(*o, b);
         o->lmask = l;
         o->tmask = g;
@@ -544,7 +548,7 @@ struct Tile128Builder {
         if (op.cmask || op.cond.n || !unitary) {
             emit_touching(b, nullptr, nullptr);
             materialise(b);
-            Tile128Op *o = add(is_x ? D128_X : D128_CU2, q);
+            SmemTileOp *o = add(is_x ? ST_X : ST_CU2, q);
             conditions(*o, op.cmask, op.cmask);
             if (op.cond.n) o->cond = cond_index(op.cond);
             for (int e = 0; e < 4; ++e) {
@@ -556,7 +560,7 @@ struct Tile128Builder {
         uint16_t sl = 0;
         uint32_t sg = 0;
         emit_touching(b, &sl, &sg);
-        Tile128Op *o = add(D128_U2, q);
+        SmemTileOp *o = add(ST_U2, q);
         o->lmask = sl;
         o->tmask = sg;
         cdm W[4] = {M[0], M[1], M[2], M[3]};
@@ -619,26 +623,27 @@ struct Tile128Builder {
 
 }  // namespace
 
-qk_status plan_passes128(TilePlanner *planner, int n, const std::vector<FusedOp> &ops, const Pass128Sink &sink,
-                         const char **err) {
+qk_status plan_smem_passes(TilePlanner *planner, int n, int prec, const std::vector<FusedOp> &ops,
+                           const SmemPassSink &sink, const char **err) {
     *err = "";
     static thread_local std::vector<POp> rem, left, taken, next;
     rem.clear();
     for (const auto &op : ops) rem.push_back(classify(op));
-    const int m = tile128_qubits(n);
-    TakeLimits lim{m, kTile128Ops, 4096};
-    const int contig = std::min(tile128_contig(n), m);
+    const int m = smem_tile_qubits(n, prec);
+    TakeLimits lim{m, kSmemTileOps, 4096};
+    const int contig = std::min(smem_tile_contig(n), m);
     std::vector<Cond> conds;
+    const double far = prec == 0 ? 0x1p24 : 0x1p200;   // how far the stored amplitudes may drift from the true ones
     cdm F[64], lam = 1.0;
     for (cdm &f : F) f = 1.0;
     std::deque<FusedOp> rewritten;   // pair terms handed on without their single-qubit parts
     while (!rem.empty()) {
         int n_u2 = 0, n_ph = 0;
         const uint64_t S = choose_pass(rem, n, lim, contig, conds, taken, left, &n_u2, &n_ph);
-        static thread_local Tile128Params P;
+        static thread_local SmemTileParams P;
         cdm F1[64], lam1 = lam;
         std::copy(F, F + 64, F1);
-        Tile128Builder B(P, F1, lam1);
+        SmemTileBuilder B(P, F1, lam1);
         P.n = n;
         P.m = m;
         P.n_tiles = 1u << (n - m);
@@ -672,7 +677,7 @@ qk_status plan_passes128(TilePlanner *planner, int n, const std::vector<FusedOp>
             for (int b = 0; b < n; ++b)
                 if (F1[b] != cdm(1.0, 0.0)) bits |= 1ull << b;
             if (!B.overflow && (bits || lam1 != cdm(1.0, 0.0))) B.table(-1, bits, F1, lam1);
-        } else if (!B.overflow && !(std::abs(lam1) > 0x1p-200 && std::abs(lam1) < 0x1p200)) {
+        } else if (!B.overflow && !(std::abs(lam1) > 1.0 / far && std::abs(lam1) < far)) {
             // a factor in [2^-1/2, 2] per gate: keep the stored amplitudes in range
             B.table(-1, 0, F1, lam1);
             lam1 = 1.0;
@@ -704,6 +709,11 @@ qk_status plan_passes128(TilePlanner *planner, int n, const std::vector<FusedOp>
         if (planner->log)
             std::fprintf(stderr, "[qk plan] c128 pass S=%#llx gates=%zu (u2 %d, phase %d) ops=%d factors=%d kept=%zu\n",
                          (unsigned long long)S, taken.size(), n_u2, n_ph, P.nops, P.nfac, B.terms.size());
+        if (prec == 0) {   // coefficients and factors in the working precision
+            for (int i = 0; i < P.nops; ++i)
+                for (int e = 0; e < 8; ++e) P.ops[i].cf[e] = (float)P.ops[i].c[e];
+            for (int i = 0; i < P.nfac; ++i) P.facf[i] = make_float2((float)P.fac[i].x, (float)P.fac[i].y);
+        }
         if (P.nops > 0) {
             const qk_status st = sink(P);
             if (st != QK_OK) return st;
@@ -711,7 +721,7 @@ qk_status plan_passes128(TilePlanner *planner, int n, const std::vector<FusedOp>
         std::copy(F1, F1 + 64, F);
         lam = lam1;
         rem.swap(next);
-        lim = TakeLimits{m, kTile128Ops, 4096};
+        lim = TakeLimits{m, kSmemTileOps, 4096};
     }
     return QK_OK;
 }
@@ -1504,25 +1514,19 @@ qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const D
 
 qk_status run_fused(TilePlanner *planner, qk_ctx *c, const std::vector<FusedOp> &ops) {
     const int n = ctx_n(c);
-    if (ctx_prec(c) != 0) {
-        const Pass128Sink launch = [&](Tile128Params &P) -> qk_status {
+    const int prec = ctx_prec(c);
+    if (prec != 0 || n < kTileQubits) {
+        const SmemPassSink launch = [&](SmemTileParams &P) -> qk_status {
             void *tok = nullptr;
-            ctx_launch_begin(c, 0, 2.0 * 16.0 * (double)(1ull << n), &tok);
-            const cudaError_t e = launch_tile128(ctx_state(c), P, ctx_cbits(c), ctx_stream(c));
+            ctx_launch_begin(c, 0, (prec == 0 ? 2.0 * 8.0 : 2.0 * 16.0) * (double)(1ull << n), &tok);
+            const cudaError_t e = launch_smem_tile(prec, ctx_state(c), P, ctx_cbits(c), ctx_stream(c));
             ctx_launch_end(tok);
             return e == cudaSuccess ? QK_OK : ctx_fail(c, QK_ECUDA, cudaGetErrorString(e));
         };
         const char *err = "";
-        const qk_status st = plan_passes128(planner, n, ops, launch, &err);
+        const qk_status st = plan_smem_passes(planner, n, prec, ops, launch, &err);
         if (st != QK_OK && err[0]) return ctx_fail(c, st, err);
         return st;
-    }
-    if (n < kTileQubits) {
-        for (const auto &op : ops) {
-            qk_status s = ctx_run_plain(c, op);
-            if (s != QK_OK) return s;
-        }
-        return QK_OK;
     }
     const PassSink launch = [&](TileParams &P) -> qk_status {
         void *tok = nullptr;

@@ -47,12 +47,12 @@ void free_planner(TilePlanner *p);
 // On a planner error *err names it.
 using PassSink = std::function<qk_status(TileParams &)>;
 qk_status plan_passes(TilePlanner *p, int n, const std::vector<FusedOp> &ops, const PassSink &sink, const char **err);
-// the same for complex128 lists of any size (Tile128Params)
-using Pass128Sink = std::function<qk_status(Tile128Params &)>;
-qk_status plan_passes128(TilePlanner *p, int n, const std::vector<FusedOp> &ops, const Pass128Sink &sink,
-                         const char **err);
-// plan_passes or plan_passes128 with each pass launched on the context's stream
-// (complex64 with n < 13: one plain launch per op)
+// the same as programs for tiles in shared memory (SmemTileParams), any n >= 1
+using SmemPassSink = std::function<qk_status(SmemTileParams &)>;
+qk_status plan_smem_passes(TilePlanner *p, int n, int prec, const std::vector<FusedOp> &ops, const SmemPassSink &sink,
+                           const char **err);
+// one of them with each pass launched on the context's stream: register tiles for
+// complex64 from 13 qubits on, tiles in shared memory otherwise
 qk_status run_fused(TilePlanner *p, qk_ctx *c, const std::vector<FusedOp> &ops);
 
 // context hooks implemented in qk_api.cu
@@ -63,7 +63,6 @@ int ctx_sms(qk_ctx *c);
 int ctx_tile_qubits(qk_ctx *c);
 cudaStream_t ctx_stream(qk_ctx *c);
 const uint8_t *ctx_cbits(qk_ctx *c);
-qk_status ctx_run_plain(qk_ctx *c, const FusedOp &op);
 qk_status ctx_fail(qk_ctx *c, qk_status s, const char *msg);
 void ctx_launch_begin(qk_ctx *c, int cls, double bytes, void **token);
 void ctx_launch_end(void *token);
