@@ -12,17 +12,18 @@
 // transposing the tile through shared memory (three fixed arrangements, see
 // qk_kernels.cuh).
 //
-// Uncontrolled gates run in pivot form (LayerGate in qk_kernels.cuh): 8 FP32
-// FMAs per amplitude pair (in place) instead of the 16 operations of a complex
-// 2x2 product.  What the pivot form leaves over -- a real scale, the same for
-// every amplitude of the pass, and per-qubit factors -- stays pending.  The parts
-// that are the same for every thread are tracked by the planner and folded into
-// later gates' coefficients or the final flush; each thread only keeps the parts
-// that depend on its own bits
-// (diagonal terms coupling a register bit with a lane, warp or fixed bit), as six
-// 32-bit fixed-point phase sums (exact modulo one turn): one per register bit
-// and one for the whole thread.  A sum of exactly half a turn is a sign flip and
-// costs no phase factor.
+// Uncontrolled gates take 7 FP32 FMAs per amplitude pair in place (LayerGate in
+// qk_kernels.cuh).  What that leaves over -- a scale and phase, the same for every
+// amplitude, and one factor per qubit -- the planner keeps in FP64 and folds into later
+// gates or the final flush.  A diagonal term on two qubits waits in the planner until a
+// gate acts on one of them, and is applied there, once, on that gate's register bit: as
+// a sign, as a phase from the thread's own index bits (32-bit fixed point, exact modulo
+// one turn), or as a factor on two register bits.  So no phase is carried on the device
+// and a transpose has nothing to flush.  The pass is bound by FP32 issue and latency,
+// so threads in flight count: without carried phases the kernel fits 80 registers and
+// three CTAs share an SM.  Tile passes of the 30-qubit layered step: 100.1 ms with
+// carried phases, complex updates and two CTAs per SM (128 registers), 95.5 ms with the
+// terms applied once, 75.3 ms with the third CTA.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -39,7 +40,6 @@ constexpr uint32_t kHalfTurn = 0x80000000u;
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-__device__ __forceinline__ float2 conj2(float2 a) { return make_float2(a.x, -a.y); }
 __device__ __forceinline__ float2 splat(float x) { return make_float2(x, x); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -90,33 +90,6 @@ __device__ __forceinline__ float &im_of(Regs &v) {
     if constexpr (r & 1) return v.I[r >> 1].y;
     else return v.I[r >> 1].x;
 }
-
-// Thread-dependent pending phases: t(k) on register bit k = 1, t0 on the whole
-// thread.  The sums live in shared memory (word w of thread x at w * kTileThreads
-// + x, conflict-free), leaving the registers to the amplitudes; a register mask
-// says which sums may be nonzero, so a thread with nothing pending touches no
-// shared memory.
-struct DevPending {
-    uint32_t *p;   // word 0: t0, word 1 + k: t(k)
-    int mask;      // bit k: t(k) may be nonzero; bit 5: t0 may be nonzero
-    __device__ __forceinline__ uint32_t &w(int k) { return p[(k + 1) * kTileThreads]; }  // k = -1: t0
-    __device__ __forceinline__ void reset() { mask = 0; }
-    __device__ __forceinline__ uint32_t get(int k) { return (mask >> k) & 1 ? w(k) : 0u; }
-    __device__ __forceinline__ uint32_t get0() { return mask & 32 ? w(-1) : 0u; }
-    __device__ __forceinline__ void set(int k, uint32_t x) {
-        w(k) = x;
-        mask |= 1 << k;
-    }
-    __device__ __forceinline__ void set0(uint32_t x) {
-        w(-1) = x;
-        mask |= 32;
-    }
-    __device__ __forceinline__ void add(int k, uint32_t d) {  // k == 5: t0
-        if (k == 5) set0(get0() + d);
-        else set(k, get(k) + d);
-    }
-    __device__ __forceinline__ void clear(int k) { mask &= ~(1 << k); }
-};
 
 // Shared-memory slot (in floats, separate real and imaginary planes) of local
 // index L.  The map is linear over GF(2), so slot(thread part ^ register part)
@@ -179,26 +152,8 @@ __device__ __forceinline__ void transpose(Regs &v, float *sre, float *sim, int f
 }
 
 // ---------------------------------------------------------------------------
-// pending-phase flushes
+// diagonal factors
 // ---------------------------------------------------------------------------
-
-// Every sum is 0 or half a turn: amplitude r changes sign iff t0 + sum_k r_k t_k
-// is half a turn (sign bits combined by XOR, applied to the float sign bits).
-__device__ __forceinline__ void flush_signs(Regs &v, uint32_t t0, const uint32_t t[5]) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        uint32_t s = t0;
-        if (j & 1) s ^= t[1];
-        if (j & 2) s ^= t[2];
-        if (j & 4) s ^= t[3];
-        if (j & 8) s ^= t[4];
-        const uint32_t so = s ^ t[0];
-        v.R[j].x = xor_sign(v.R[j].x, s);
-        v.I[j].x = xor_sign(v.I[j].x, s);
-        v.R[j].y = xor_sign(v.R[j].y, so);
-        v.I[j].y = xor_sign(v.I[j].y, so);
-    }
-}
 
 // General diagonal D(r) = c0 * prod_{k in r} a_k on the 32 registers (any
 // magnitudes): per value of register bits 1, 2 the factor q = c0 a1^r1 a2^r2,
@@ -253,111 +208,123 @@ __device__ __forceinline__ void bit_factor_dispatch(int k, Regs &v, float2 f) {
     }
 }
 
-// Materialise the thread's pending phases (before a transpose moves amplitudes
-// between threads).
-__device__ __forceinline__ void flush_dev(Regs &v, DevPending &pd) {
-    if (pd.mask == 0) return;
-    uint32_t t[5];
+// amplitudes with register bit K set change sign
+template <int K>
+__device__ __forceinline__ void bit_negate(Regs &v) {
 #pragma unroll
-    for (int k = 0; k < 5; ++k) t[k] = pd.get(k);
-    const uint32_t t0 = pd.get0();
-    if (((t[0] | t[1] | t[2] | t[3] | t[4] | t0) & ~kHalfTurn) == 0u) {
-        flush_signs(v, t0, t);
-    } else {
-        float2 a[5];
-#pragma unroll
-        for (int k = 0; k < 5; ++k) a[k] = phase_of(t[k]);
-        apply_diagonal(v, phase_of(t0), a);
+    for (int j = 0; j < 16; ++j) {
+        if constexpr (K == 0) {
+            v.R[j].y = xor_sign(v.R[j].y, kHalfTurn);
+            v.I[j].y = xor_sign(v.I[j].y, kHalfTurn);
+        } else {
+            if (!(j & (1 << (K - 1)))) continue;
+            v.R[j].x = xor_sign(v.R[j].x, kHalfTurn);
+            v.R[j].y = xor_sign(v.R[j].y, kHalfTurn);
+            v.I[j].x = xor_sign(v.I[j].x, kHalfTurn);
+            v.I[j].y = xor_sign(v.I[j].y, kHalfTurn);
+        }
     }
-    pd.reset();
+}
+
+// turns of nt terms on thread bits and ni on tile-index bits (uniform over the CTA)
+__device__ __forceinline__ uint32_t sum_terms(const BitTerm *t, int nt, int ni, uint32_t tbits, uint32_t tidx) {
+    uint32_t acc = 0, uacc = 0;
+    const uint2 *w = reinterpret_cast<const uint2 *>(t);
+    for (int e = 0; e < nt; ++e) {
+        const uint2 x = w[e];
+        acc += ((tbits >> x.x) & 1u) * x.y;
+    }
+    for (int e = nt; e < nt + ni; ++e) {
+        const uint2 x = w[e];
+        uacc += ((tidx >> x.x) & 1u) * x.y;
+    }
+    return acc + uacc;
 }
 
 // ---------------------------------------------------------------------------
 // gates
 // ---------------------------------------------------------------------------
 
-// Pivot butterfly on register bit K >= 1 (see LayerGate): couples float2
-// registers (j, j | 2^(K-1)), two amplitude pairs per couple, in place in the
-// amplitudes' own registers.  ZF = 0: y1 += c1 y0, then y0 += c0 y1 with the new
-// y1; ZF = 1: y0 += c0 y1, then y1 += c1 y0 with the new y0.  8 packed FMAs per
-// couple.
-template <int K, int ZF>
-__device__ __forceinline__ void piv_packed(Regs &v, float2 c0r, float2 c0i, float2 nc0i, float2 c1r, float2 c1i,
-                                           float2 nc1i) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        if (j & (1 << (K - 1))) continue;
-        const int j1 = j | (1 << (K - 1));
-        float2 A = v.R[j], B = v.I[j], C = v.R[j1], D = v.I[j1];
-        if constexpr (ZF == 0) {
-            C = ffma2(nc1i, B, ffma2(c1r, A, C));
-            D = ffma2(c1i, A, ffma2(c1r, B, D));
-            A = ffma2(nc0i, D, ffma2(c0r, C, A));
-            B = ffma2(c0i, C, ffma2(c0r, D, B));
-        } else {
-            A = ffma2(nc0i, D, ffma2(c0r, C, A));
-            B = ffma2(c0i, C, ffma2(c0r, D, B));
-            C = ffma2(nc1i, B, ffma2(c1r, A, C));
-            D = ffma2(c1i, A, ffma2(c1r, B, D));
-        }
-        v.R[j] = A;
-        v.I[j] = B;
-        v.R[j1] = C;
-        v.I[j1] = D;
-    }
-}
-
-// Pivot butterfly on register bit 0: the pair is the two halves of one float2.
-template <int ZF>
-__device__ __forceinline__ void piv_bit0(Regs &v, float c0r, float c0i, float c1r, float c1i) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        float y0r = v.R[j].x, y0i = v.I[j].x, y1r = v.R[j].y, y1i = v.I[j].y;
-        if constexpr (ZF == 0) {
-            y1r = fmaf(-c1i, y0i, fmaf(c1r, y0r, y1r));
-            y1i = fmaf(c1i, y0r, fmaf(c1r, y0i, y1i));
-            y0r = fmaf(-c0i, y1i, fmaf(c0r, y1r, y0r));
-            y0i = fmaf(c0i, y1r, fmaf(c0r, y1i, y0i));
-        } else {
-            y0r = fmaf(-c0i, y1i, fmaf(c0r, y1r, y0r));
-            y0i = fmaf(c0i, y1r, fmaf(c0r, y1i, y0i));
-            y1r = fmaf(-c1i, y0i, fmaf(c1r, y0r, y1r));
-            y1i = fmaf(c1i, y0r, fmaf(c1r, y0i, y1i));
-        }
-        v.R[j] = make_float2(y0r, y1r);
-        v.I[j] = make_float2(y0i, y1i);
-    }
-}
-
-// One gate of a TOP_U2L layer on register bit K.  The planner folded every
-// pending factor that is the same for all threads into its coefficients C0, C1
-// and chose the stored bit order so that the pivot is the diagonal entry; the
-// thread's own pending phase e of bit K turns them into c0 = C0 e and
-// c1 = C1 conj(e), and leaves e pending on the bit.  zf: which value of the pair
-// is updated first (see LayerGate).
+// The |1> of register bit K turned by e^{i phi}, as three shears of (re, im) in place: h
+// = -tan(phi / 2), s = sin(phi).
 template <int K>
-__device__ __forceinline__ void layer_gate(Regs &v, DevPending &pd, const LayerGate &g, bool zf) {
-    float2 a0r = g.c[0], a0i = g.c[1], na0i = g.c[2], a1r = g.c[3], a1i = g.c[4], na1i = g.c[5];
-    const uint32_t tk = pd.get(K);
-    if (tk != 0u) {
-        if (tk == kHalfTurn) {
-            a0r = neg2(a0r); a0i = neg2(a0i); na0i = neg2(na0i);
-            a1r = neg2(a1r); a1i = neg2(a1i); na1i = neg2(na1i);
+__device__ __forceinline__ void turn(Regs &v, float2 h, float2 s) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        if constexpr (K == 0) {
+            v.R[j].y = fmaf(h.x, v.I[j].y, v.R[j].y);
+            v.I[j].y = fmaf(s.x, v.R[j].y, v.I[j].y);
+            v.R[j].y = fmaf(h.x, v.I[j].y, v.R[j].y);
         } else {
-            const float2 e = turns_to_phase(tk);
-            const float2 x0 = cmul(make_float2(a0r.x, a0i.x), e);
-            const float2 x1 = cmul(make_float2(a1r.x, a1i.x), conj2(e));
-            a0r = splat(x0.x); a0i = splat(x0.y); na0i = splat(-x0.y);
-            a1r = splat(x1.x); a1i = splat(x1.y); na1i = splat(-x1.y);
+            if (!(j & (1 << (K - 1)))) continue;
+            v.R[j] = ffma2(h, v.I[j], v.R[j]);
+            v.I[j] = ffma2(s, v.R[j], v.I[j]);
+            v.R[j] = ffma2(h, v.I[j], v.R[j]);
         }
     }
-    if constexpr (K == 0) {
-        if (zf) piv_bit0<1>(v, a0r.x, a0i.x, a1r.x, a1i.x);
-        else piv_bit0<0>(v, a0r.x, a0i.x, a1r.x, a1i.x);
-    } else {
-        if (zf) piv_packed<K, 1>(v, a0r, a0i, na0i, a1r, a1i, na1i);
-        else piv_packed<K, 0>(v, a0r, a0i, na0i, a1r, a1i, na1i);
+}
+
+// The two real updates of a pair (LayerGate), in place, two pairs per packed FMA.
+template <int K, int ZF>
+__device__ __forceinline__ void lift(Regs &v, float2 c0, float2 c1) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        if constexpr (K == 0) {
+            float y0r = v.R[j].x, y0i = v.I[j].x, y1r = v.R[j].y, y1i = v.I[j].y;
+            if constexpr (ZF == 0) {
+                y1r = fmaf(c1.x, y0r, y1r);
+                y1i = fmaf(c1.x, y0i, y1i);
+                y0r = fmaf(c0.x, y1r, y0r);
+                y0i = fmaf(c0.x, y1i, y0i);
+            } else {
+                y0r = fmaf(c0.x, y1r, y0r);
+                y0i = fmaf(c0.x, y1i, y0i);
+                y1r = fmaf(c1.x, y0r, y1r);
+                y1i = fmaf(c1.x, y0i, y1i);
+            }
+            v.R[j] = make_float2(y0r, y1r);
+            v.I[j] = make_float2(y0i, y1i);
+        } else {
+            if (j & (1 << (K - 1))) continue;
+            const int j1 = j | (1 << (K - 1));
+            float2 A = v.R[j], B = v.I[j], C = v.R[j1], D = v.I[j1];
+            if constexpr (ZF == 0) {
+                C = ffma2(c1, A, C);
+                D = ffma2(c1, B, D);
+                A = ffma2(c0, C, A);
+                B = ffma2(c0, D, B);
+            } else {
+                A = ffma2(c0, C, A);
+                B = ffma2(c0, D, B);
+                C = ffma2(c1, A, C);
+                D = ffma2(c1, B, D);
+            }
+            v.R[j] = A;
+            v.I[j] = B;
+            v.R[j1] = C;
+            v.I[j1] = D;
+        }
     }
+}
+
+// One gate of a TOP_U2L layer on register bit K.  w: the op's flags for the gate (see
+// TOP_U2L), already shifted to bit 0.
+template <int K>
+__device__ __forceinline__ void layer_gate(Regs &v, const LayerGate &g, const BitTerm *bt, int zf, int on, int sign,
+                                           int terms, uint32_t tbits, uint32_t tidx) {
+    if ((sign | terms) & 1) {
+        bool neg = false;
+        if (sign & 1) neg = ((__popc(tbits & g.ts) + __popc(tidx & g.fs)) & 1) != 0;
+        if (terms & 1) {
+            const uint32_t t = sum_terms(bt + g.first, g.nt, g.ni, tbits, tidx);
+            if (t == kHalfTurn) neg = !neg;
+            else if (t != 0u) bit_factor<K>(v, turns_to_phase(t));
+        }
+        if (neg) bit_negate<K>(v);
+    }
+    if (on & 1) turn<K>(v, g.h, g.s);
+    if (zf & 1) lift<K, 1>(v, g.c0, g.c1);
+    else lift<K, 0>(v, g.c0, g.c1);
 }
 
 // General 2x2 gate on register bit K >= 1 where the register bits in rmask are 1
@@ -443,16 +410,6 @@ __device__ __forceinline__ void pair_pat(Regs &v, float2 f) {
         pair_all<K, L, PAT>(v, f, std::make_integer_sequence<int, 32>{});
     }
 }
-template <int K, int L>
-__device__ __forceinline__ void pair_factor(Regs &v, float2 f, int pat) {
-    switch (pat) {
-        case 0: pair_pat<K, L, 0>(v, f); break;
-        case 1: pair_pat<K, L, 1>(v, f); break;
-        case 2: pair_pat<K, L, 2>(v, f); break;
-        default: pair_pat<K, L, 3>(v, f); break;
-    }
-}
-
 template <int K, int L, int r>
 __device__ __forceinline__ void pair_neg_one(Regs &v) {
     if constexpr (((r >> K) & 1) && ((r >> L) & 1)) {
@@ -496,24 +453,7 @@ __device__ __forceinline__ void pair_neg(Regs &v, int code) {
     }
 }
 
-// pair factor on register bits (code k | l << 3), pattern pat of the two bits
-__device__ __forceinline__ void pair_dispatch(Regs &v, int code, float2 f, int pat) {
-    switch (code) {
-        case 0 | (1 << 3): pair_factor<0, 1>(v, f, pat); break;
-        case 0 | (2 << 3): pair_factor<0, 2>(v, f, pat); break;
-        case 0 | (3 << 3): pair_factor<0, 3>(v, f, pat); break;
-        case 0 | (4 << 3): pair_factor<0, 4>(v, f, pat); break;
-        case 1 | (2 << 3): pair_factor<1, 2>(v, f, pat); break;
-        case 1 | (3 << 3): pair_factor<1, 3>(v, f, pat); break;
-        case 1 | (4 << 3): pair_factor<1, 4>(v, f, pat); break;
-        case 2 | (3 << 3): pair_factor<2, 3>(v, f, pat); break;
-        case 2 | (4 << 3): pair_factor<2, 4>(v, f, pat); break;
-        default: pair_factor<3, 4>(v, f, pat); break;
-    }
-}
-
-// TOP_PAIRU: the pattern is always (1, 1) (the planner moves the other patterns'
-// constant and single-bit parts into its uniform phases)
+// factor on the amplitudes whose register bits k and l are both 1 (code k | l << 3)
 __device__ __forceinline__ void pair11_dispatch(Regs &v, int code, float2 f) {
     switch (code) {
         case 0 | (1 << 3): pair_pat<0, 1, 3>(v, f); break;
@@ -588,73 +528,41 @@ __device__ __forceinline__ uint64_t tile_base(const Head &P, uint64_t tile) {
     return b;
 }
 
-// The op kinds a layered circuit rarely needs: controlled / conditioned 2x2
-// gates, conditioned or complex pair factors, direct diagonal factors.
+// The op kinds a layered circuit rarely needs: controlled or conditioned 2x2 gates,
+// phase terms before them, direct diagonal factors.
 template <typename Off>
-__device__ __forceinline__ void general_op(Regs &v, DevPending &pd, const TileOp &op, int tbits, Off base,
-                                           unsigned condok) {
-    if (op.kind == TOP_U2) {   // uniform part of the target's pending factor, in every thread
-        pd.add(op.k, op.hturns);
-        if (op.hmag != 1.f) bit_factor_dispatch(op.k, v, make_float2(op.hmag, 0.f));
-    }
-    if (!op_applies<Off>(op, tbits, base, condok)) return;
-    if (op.kind == TOP_PAIR) {
-        pair_dispatch(v, op.k, make_float2(op.ph.re, op.ph.im), op.rval);
+__device__ __forceinline__ void general_op(Regs &v, const TileOp &op, const BitTerm *bt, int tbits, uint32_t tidx,
+                                           Off base, unsigned condok) {
+    if (op.kind == TOP_PHQ) {
+        const uint32_t t = sum_terms(bt + op.first, op.count, op.count2, (uint32_t)tbits, tidx);
+        if (t != 0u) bit_factor_dispatch(op.k, v, phase_of(t));
         return;
     }
+    if (!op_applies<Off>(op, tbits, base, condok)) return;
     if (op.kind == TOP_U2) {
-        float2 m00 = make_float2(op.m[0], op.m[1]), m01 = make_float2(op.m[2], op.m[3]);
-        float2 m10 = make_float2(op.m[4], op.m[5]), m11 = make_float2(op.m[6], op.m[7]);
-        const int k = op.k;
-        const uint32_t tk = pd.get(k);
-        if (tk != 0u) {
-            const float2 ak = phase_of(tk);
-            if (op.rmask == 0) {  // fold diag(1, a_k) into the gate: U * diag(1, a_k)
-                m01 = cmul(m01, ak);
-                m11 = cmul(m11, ak);
-            } else {
-                bit_factor_dispatch(k, v, ak);
-            }
+        const float2 m00 = make_float2(op.m[0], op.m[1]), m01 = make_float2(op.m[2], op.m[3]);
+        const float2 m10 = make_float2(op.m[4], op.m[5]), m11 = make_float2(op.m[6], op.m[7]);
+        switch (op.k) {
+            case 0: u2_bit0(v, m00, m01, m10, m11, op.rmask, op.rval); break;
+            case 1: u2_packed<1>(v, m00, m01, m10, m11, op.rmask, op.rval); break;
+            case 2: u2_packed<2>(v, m00, m01, m10, m11, op.rmask, op.rval); break;
+            case 3: u2_packed<3>(v, m00, m01, m10, m11, op.rmask, op.rval); break;
+            default: u2_packed<4>(v, m00, m01, m10, m11, op.rmask, op.rval); break;
         }
-        pd.clear(k);
-        if (k == 0) {
-            u2_bit0(v, m00, m01, m10, m11, op.rmask, op.rval);
-        } else {
-            switch (k) {
-                case 1: u2_packed<1>(v, m00, m01, m10, m11, op.rmask, op.rval); break;
-                case 2: u2_packed<2>(v, m00, m01, m10, m11, op.rmask, op.rval); break;
-                case 3: u2_packed<3>(v, m00, m01, m10, m11, op.rmask, op.rval); break;
-                default: u2_packed<4>(v, m00, m01, m10, m11, op.rmask, op.rval); break;
-            }
-        }
-    } else if (op.kind == TOP_PHASE) {  // factor where (register index & rmask) == rval
-        const int rm = op.rmask;
-        const int pc = __popc(rm);
-        if (pc == 0) {
-            pd.add(5, op.ph.turns);
-        } else if (pc == 1) {
-            const int k = __ffs(rm) - 1;
-            if (op.rval) {
-                pd.add(k, op.ph.turns);
-            } else {  // f on bit k = 0:  f * (f^-1 on bit k = 1)
-                pd.add(5, op.ph.turns);
-                pd.add(k, 0u - op.ph.turns);
-            }
-        } else {
-            const int rv = op.rval;
-            const float2 f = make_float2(op.ph.re, op.ph.im);
+    } else {  // TOP_PHASE: factor where (register index & rmask) == rval
+        const int rm = op.rmask, rv = op.rval;
+        const float2 f = make_float2(op.ph.re, op.ph.im);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                if (((2 * j) & rm) == rv) {
-                    const float xr = v.R[j].x, xi = v.I[j].x;
-                    v.R[j].x = xr * f.x - xi * f.y;
-                    v.I[j].x = xr * f.y + xi * f.x;
-                }
-                if (((2 * j + 1) & rm) == rv) {
-                    const float xr = v.R[j].y, xi = v.I[j].y;
-                    v.R[j].y = xr * f.x - xi * f.y;
-                    v.I[j].y = xr * f.y + xi * f.x;
-                }
+        for (int j = 0; j < 16; ++j) {
+            if (((2 * j) & rm) == rv) {
+                const float xr = v.R[j].x, xi = v.I[j].x;
+                v.R[j].x = xr * f.x - xi * f.y;
+                v.I[j].x = xr * f.y + xi * f.x;
+            }
+            if (((2 * j + 1) & rm) == rv) {
+                const float xr = v.R[j].y, xi = v.I[j].y;
+                v.R[j].y = xr * f.x - xi * f.y;
+                v.I[j].y = xr * f.y + xi * f.x;
             }
         }
     }
@@ -667,17 +575,17 @@ struct ParamProg {
     __device__ __forceinline__ const TileHead &head() const { return P; }
     __device__ __forceinline__ const TileOp &op(int i) const { return P.ops[i]; }
     __device__ __forceinline__ const LayerGate &lg(int i) const { return P.lg[i]; }
-    __device__ __forceinline__ const LinTerm &lin(int i) const { return P.lin[i]; }
+    __device__ __forceinline__ const BitTerm *bt() const { return P.bt; }
 };
 struct PoolProg {
     const TileProg &h;
     const TileOp *ops;
     const LayerGate *lgs;
-    const LinTerm *lins;
+    const BitTerm *bts;
     __device__ __forceinline__ const TileProg &head() const { return h; }
     __device__ __forceinline__ const TileOp &op(int i) const { return ops[h.op0 + i]; }
     __device__ __forceinline__ const LayerGate &lg(int i) const { return lgs[h.lg0 + i]; }
-    __device__ __forceinline__ const LinTerm &lin(int i) const { return lins[h.lin0 + i]; }
+    __device__ __forceinline__ const BitTerm *bt() const { return bts + h.bt0; }
 };
 
 // The fields of a TileOp that the common op kinds read (its first 16 bytes),
@@ -688,12 +596,12 @@ struct OpHead {
     uint32_t w0, w1, w2, w3;
     __device__ __forceinline__ int kind() const { return (int)(w0 & 0xffu); }
     __device__ __forceinline__ int k() const { return (int)((w0 >> 8) & 0xffu); }
-    __device__ __forceinline__ int rmask() const { return (int)((w0 >> 16) & 0xffu); }   // TOP_U2L: zf mask
+    __device__ __forceinline__ int rmask() const { return (int)((w0 >> 16) & 0xffu); }
     __device__ __forceinline__ int rval() const { return (int)(w0 >> 24); }
     __device__ __forceinline__ int count() const { return (int)(w2 >> 16); }
     __device__ __forceinline__ int first() const { return (int)(w3 & 0xffffu); }
     __device__ __forceinline__ int czmask() const { return (int)(w1 & 0x3ffu); }   // TOP_U2L: tmask
-    __device__ __forceinline__ int count2() const { return (int)(w3 >> 16); }
+    __device__ __forceinline__ int tval() const { return (int)(w1 >> 16); }
 };
 __device__ __forceinline__ OpHead load_head(const TileOp &op) {
     const uint2 *p = reinterpret_cast<const uint2 *>(&op);
@@ -702,18 +610,17 @@ __device__ __forceinline__ OpHead load_head(const TileOp &op) {
 }
 
 // One tile of one pass: load, run the program, final flush, store.  GEN: the
-// program may hold general ops (controlled or conditioned 2x2 gates, conditioned
-// pair factors, direct diagonal factors); without them the kernel leaves their
+// program may hold general ops (controlled or conditioned 2x2 gates and what comes
+// before them, direct diagonal factors); without them the kernel leaves their
 // code out, which measured about 4 % faster on layer circuits (about 40 % less
 // code in the op loop).
 template <typename Off, bool GEN, typename Prog>
 __device__ __forceinline__ void tile_body(const Prog &pr, float2 *__restrict__ psi, uint64_t tile,
                                           const uint8_t *__restrict__ cbits) {
     const auto &P = pr.head();
-    // 2 x 2^13 floats (64 KiB) for transposes, then per thread six pending words
+    // 2 x 2^13 floats (64 KiB) for transposes
     extern __shared__ __align__(16) float smf[];
     float *sre = smf, *sim = smf + (1 << kTileQubits);
-    uint32_t *spd = reinterpret_cast<uint32_t *>(smf + (2 << kTileQubits));     // pending sums
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int tbits = (warp << 5) | lane;
     // lanes run over local qubits 0..4 in the load and store arrangements
@@ -747,9 +654,6 @@ __device__ __forceinline__ void tile_body(const Prog &pr, float2 *__restrict__ p
         }
         __syncthreads();
 
-        DevPending pd;
-        pd.p = spd + threadIdx.x;
-        pd.reset();
         int cur = ARR_IO;
         const uint32_t tidx = (uint32_t)tile;
         OpHead nh{0u, 0u, 0u, 0u};
@@ -759,83 +663,43 @@ __device__ __forceinline__ void tile_body(const Prog &pr, float2 *__restrict__ p
             if (i + 1 < P.nops) nh = load_head(pr.op(i + 1));
             switch (h.kind()) {
                 case TOP_U2L: {
-                    const LayerGate *lg = &pr.lg(h.first());
-                    const int bits = h.k(), zf = h.rmask();
-                    if (bits & 1) layer_gate<0>(v, pd, *lg++, zf & 1);
-                    if (bits & 2) layer_gate<1>(v, pd, *lg++, zf & 2);
-                    if (bits & 4) layer_gate<2>(v, pd, *lg++, zf & 4);
-                    if (bits & 8) layer_gate<3>(v, pd, *lg++, zf & 8);
-                    if (bits & 16) layer_gate<4>(v, pd, *lg, zf & 16);
                     if (h.czmask()) cz_mask(v, h.czmask());
+                    const LayerGate *lg = &pr.lg(h.first());
+                    const BitTerm *bt = pr.bt();
+                    const int bits = h.k(), zf = h.rmask(), on = h.rval(), sg = h.tval(), tm = h.count();
+                    if (bits & 1) layer_gate<0>(v, *lg++, bt, zf, on, sg, tm, tbits, tidx);
+                    if (bits & 2) layer_gate<1>(v, *lg++, bt, zf >> 1, on >> 1, sg >> 1, tm >> 1, tbits, tidx);
+                    if (bits & 4) layer_gate<2>(v, *lg++, bt, zf >> 2, on >> 2, sg >> 2, tm >> 2, tbits, tidx);
+                    if (bits & 8) layer_gate<3>(v, *lg++, bt, zf >> 3, on >> 3, sg >> 3, tm >> 3, tbits, tidx);
+                    if (bits & 16) layer_gate<4>(v, *lg, bt, zf >> 4, on >> 4, sg >> 4, tm >> 4, tbits, tidx);
                     break;
                 }
                 case TOP_PAIRNEG:
                     pair_neg(v, h.k());
                     break;
-                case TOP_PHASEL: {
-                    uint32_t acc = 0;
-                    const int end = h.first() + h.count();
-                    for (int e = h.first(); e < end; ++e) {
-                        const LinTerm &L = pr.lin(e);
-                        const bool ok = ((tbits & L.tmask) == L.tval) && ((tidx & L.fmask) == L.fval);
-                        acc += ok ? L.turns : 0u;
-                    }
-                    if (acc) {
-                        if (h.rval()) {  // the term's qubit is stored flipped: on bit k = 0
-                            pd.add(5, acc);
-                            pd.add(h.k(), 0u - acc);
-                        } else {
-                            pd.add(h.k(), acc);
-                        }
-                    }
-                    break;
-                }
-                case TOP_PHASEB: {
-                    const uint2 *t = reinterpret_cast<const uint2 *>(&pr.lin(0)) + h.first();
-                    const int nt = h.count(), nf = h.count2();
-                    uint32_t acc = 0, uacc = 0;
-                    for (int e = 0; e < nt; ++e) {
-                        const uint2 w = t[e];
-                        acc += (((uint32_t)tbits >> w.x) & 1u) * w.y;
-                    }
-                    for (int e = nt; e < nt + nf; ++e) {
-                        const uint2 w = t[e];
-                        uacc += ((tidx >> w.x) & 1u) * w.y;
-                    }
-                    acc += uacc;
-                    if (acc) {
-                        if (h.rval()) {
-                            pd.add(5, acc);
-                            pd.add(h.k(), 0u - acc);
-                        } else {
-                            pd.add(h.k(), acc);
-                        }
-                    }
-                    break;
-                }
                 case TOP_PAIRU: {
                     const float2 f = *reinterpret_cast<const float2 *>(&pr.op(i).ph.re);
                     pair11_dispatch(v, h.k(), f);
                     break;
                 }
                 case TOP_XPOSE:
-                    flush_dev(v, pd);
                     transpose(v, sre, sim, cur, h.k(), lane, warp);
                     cur = h.k();
                     break;
                 default:
-                    if constexpr (GEN) general_op<Off>(v, pd, pr.op(i), tbits, base, condok);
+                    if constexpr (GEN) general_op<Off>(v, pr.op(i), pr.bt(), tbits, tidx, base, condok);
                     break;
             }
         }
 
-        // final flush: the thread's own pending phases plus the planner's uniform
-        // factors (register bits, and lane / warp bits as a thread constant; each a
-        // phase and a magnitude) and the pass's real scale.  The store arrangement is ARR_IO or ARR_HI: lanes =
-        // local 0..4 in both; registers local 5..9 / 8..12, warps local 10..12 / 5..7.
+        // final flush: the planner's uniform factors (register bits, and lane / warp /
+        // tile-index bits as a thread constant; each a phase and a magnitude), the
+        // pass's scale, and the diagonal terms that no gate called for.  The store
+        // arrangement is ARR_IO or ARR_HI: lanes = local 0..4 in both; registers local
+        // 5..9 / 8..12, warps local 10..12 / 5..7.
         {
             const int rb = cur == ARR_IO ? 5 : 8, wb = cur == ARR_IO ? 10 : 5;
-            uint32_t t0 = pd.get0() + P.fin_turns[13];
+            uint32_t t0 = P.fin_turns[13];
             float mg = P.fin_scale;   // the thread's constant magnitude
             for (uint64_t fm = P.fin_fixed_mask; fm; fm &= fm - 1) {
                 const int b = __ffsll((long long)fm) - 1;
@@ -843,6 +707,11 @@ __device__ __forceinline__ void tile_body(const Prog &pr, float2 *__restrict__ p
                     t0 += P.fin_fixed[b];
                     mg *= P.fin_fixed_mag[b];
                 }
+            }
+            const uint64_t x = (uint64_t)tbits | ((uint64_t)tidx << 8);
+            for (int e = 0; e < P.fin2_n; ++e) {
+                const BitTerm w = pr.bt()[P.fin2_first + e];
+                t0 += (uint32_t)((x >> (w.bit & 0xffu)) & (x >> (w.bit >> 8)) & 1u) * w.turns;
             }
 #pragma unroll
             for (int j = 0; j < 5; ++j)
@@ -860,7 +729,8 @@ __device__ __forceinline__ void tile_body(const Prog &pr, float2 *__restrict__ p
             bool any = t0 != 0u || mg != 1.f;
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
-                const uint32_t tk = pd.get(k) + P.fin_turns[rb + k];
+                const uint32_t tk = P.fin_turns[rb + k] +
+                                    sum_terms(pr.bt() + P.fin_first[k], P.fin_nt[k], P.fin_ni[k], (uint32_t)tbits, tidx);
                 const float mk = P.fin_mag[rb + k];
                 any = any || tk != 0u || mk != 1.f;
                 const float2 e = phase_of(tk);
@@ -895,7 +765,7 @@ __device__ __forceinline__ void tile_body(const Prog &pr, float2 *__restrict__ p
 // one tile per CTA (a grid-stride loop would keep the tile's addressing state
 // live across iterations and push the kernel into spills)
 template <typename Off, bool GEN>
-__global__ void __launch_bounds__(kTileThreads, 2)
+__global__ void __launch_bounds__(kTileThreads, 3)
     k_tile(float2 *__restrict__ psi, const __grid_constant__ TileParams P, const uint8_t *__restrict__ cbits) {
     tile_body<Off, GEN>(ParamProg{P}, psi, blockIdx.x, cbits);
 }
@@ -903,9 +773,9 @@ __global__ void __launch_bounds__(kTileThreads, 2)
 // Batched: CTA b finds its program by binary search in first[] (uniform over
 // the CTA) and runs that program's tile b - first[c] on the program's state.
 template <bool GEN>
-__global__ void __launch_bounds__(kTileThreads, 2)
+__global__ void __launch_bounds__(kTileThreads, 3)
     k_tile_batch(const TileProg *__restrict__ progs, const uint32_t *__restrict__ first, int n_progs,
-                 const TileOp *__restrict__ ops, const LayerGate *__restrict__ lg, const LinTerm *__restrict__ lin) {
+                 const TileOp *__restrict__ ops, const LayerGate *__restrict__ lg, const BitTerm *__restrict__ bt) {
     int lo = 0, hi = n_progs - 1;
     const uint32_t b = blockIdx.x;
     while (lo < hi) {  // the last c with first[c] <= b
@@ -914,11 +784,11 @@ __global__ void __launch_bounds__(kTileThreads, 2)
         else hi = mid - 1;
     }
     const TileProg &h = progs[lo];
-    tile_body<uint32_t, GEN>(PoolProg{h, ops, lg, lin}, h.psi, b - __ldg(&first[lo]), nullptr);
+    tile_body<uint32_t, GEN>(PoolProg{h, ops, lg, bt}, h.psi, b - __ldg(&first[lo]), nullptr);
 }
 
-// transposes (2^13 complex64) and pending sums (6 words per thread)
-constexpr int kTileSmem = ((int)(2 * sizeof(float)) << kTileQubits) + 6 * kTileThreads * 4;
+// transposes (2^13 complex64)
+constexpr int kTileSmem = (int)(2 * sizeof(float)) << kTileQubits;
 
 // the dynamic shared-memory attribute of kernel f, set once per device (host
 // threads of the serving loop may launch concurrently; setting it twice is harmless)
@@ -939,7 +809,7 @@ cudaError_t tile_smem_attr(F *f, std::atomic<bool> (&set)[64]) {
 // whether a program needs the general-op path of the kernel
 bool needs_general(const TileOp *ops, size_t n) {
     for (size_t i = 0; i < n; ++i)
-        if (ops[i].kind == TOP_U2 || ops[i].kind == TOP_PHASE || ops[i].kind == TOP_PAIR) return true;
+        if (ops[i].kind == TOP_U2 || ops[i].kind == TOP_PHASE || ops[i].kind == TOP_PHQ) return true;
     return false;
 }
 
@@ -962,22 +832,22 @@ cudaError_t launch_tile_t(void *psi, const TileParams &p, const uint8_t *cbits, 
 
 template <bool GEN>
 cudaError_t launch_tile_batch_g(const TileProg *progs, const uint32_t *first, int n_progs, uint32_t n_ctas,
-                                const TileOp *ops, const LayerGate *lg, const LinTerm *lin, cudaStream_t s) {
+                                const TileOp *ops, const LayerGate *lg, const BitTerm *bt, cudaStream_t s) {
     static std::atomic<bool> attr_set[64];
     const cudaError_t e = tile_smem_attr(k_tile_batch<GEN>, attr_set);
     if (e != cudaSuccess) return e;
-    k_tile_batch<GEN><<<n_ctas, kTileThreads, kTileSmem, s>>>(progs, first, n_progs, ops, lg, lin);
+    k_tile_batch<GEN><<<n_ctas, kTileThreads, kTileSmem, s>>>(progs, first, n_progs, ops, lg, bt);
     return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_tile_batch(const TileProg *progs, const uint32_t *first, int n_progs, uint32_t n_ctas,
-                              const TileOp *ops, const LayerGate *lg, const LinTerm *lin, bool general,
+                              const TileOp *ops, const LayerGate *lg, const BitTerm *bt, bool general,
                               cudaStream_t s) {
     if (n_progs <= 0 || n_ctas == 0) return cudaSuccess;
-    if (general) return launch_tile_batch_g<true>(progs, first, n_progs, n_ctas, ops, lg, lin, s);
-    return launch_tile_batch_g<false>(progs, first, n_progs, n_ctas, ops, lg, lin, s);
+    if (general) return launch_tile_batch_g<true>(progs, first, n_progs, n_ctas, ops, lg, bt, s);
+    return launch_tile_batch_g<false>(progs, first, n_progs, n_ctas, ops, lg, bt, s);
 }
 
 bool tile_ops_need_general(const TileOp *ops, size_t n) { return needs_general(ops, n); }

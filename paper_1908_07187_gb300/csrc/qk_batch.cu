@@ -357,8 +357,8 @@ struct qk_batch {
     size_t cap_lops = 0;
     qk::LayerGate *d_llg = nullptr;
     size_t cap_llg = 0;
-    qk::LinTerm *d_llin = nullptr;
-    size_t cap_llin = 0;
+    qk::BitTerm *d_lbt = nullptr;
+    size_t cap_lbt = 0;
     double plan_ms = 0.0;              // host planning time of the last run
     int large_launches = 0;            // batched tile launches of the last run
 };
@@ -486,7 +486,7 @@ qk_status run_large(qk_batch *b) {
         std::vector<qk::TileProg> progs;
         std::vector<qk::TileOp> ops;
         std::vector<qk::LayerGate> lg;
-        std::vector<qk::LinTerm> lin;
+        std::vector<qk::BitTerm> bt;
         qk_status st = QK_OK;
         std::string err;
     };
@@ -514,10 +514,10 @@ qk_status run_large(qk_batch *b) {
                 static_cast<qk::TileHead &>(h) = P;
                 h.op0 = (uint32_t)out.ops.size();
                 h.lg0 = (uint32_t)out.lg.size();
-                h.lin0 = (uint32_t)out.lin.size();
+                h.bt0 = (uint32_t)out.bt.size();
                 out.ops.insert(out.ops.end(), P.ops, P.ops + P.nops);
                 out.lg.insert(out.lg.end(), P.lg, P.lg + P.nlg);
-                out.lin.insert(out.lin.end(), P.lin, P.lin + P.nlin);
+                out.bt.insert(out.bt.end(), P.bt, P.bt + P.nbt);
                 out.progs.push_back(h);
                 return QK_OK;
             };
@@ -530,17 +530,17 @@ qk_status run_large(qk_batch *b) {
     std::vector<std::thread> th;
     for (int t = 0; t < nth; ++t) th.emplace_back(worker);
     for (auto &t : th) t.join();
-    size_t nops = 0, nlg = 0, nlin = 0, nprog = 0;
+    size_t nops = 0, nlg = 0, nbt = 0, nprog = 0;
     int maxp = 0;
-    std::vector<size_t> op_base(nl), lg_base(nl), lin_base(nl);
+    std::vector<size_t> op_base(nl), lg_base(nl), bt_base(nl);
     for (int i = 0; i < nl; ++i) {
         if (plans[i].st != QK_OK) return bfail(b, plans[i].st, "batch: circuit %d: %s", b->large[i].circ, plans[i].err.c_str());
         op_base[i] = nops;
         lg_base[i] = nlg;
-        lin_base[i] = nlin;
+        bt_base[i] = nbt;
         nops += plans[i].ops.size();
         nlg += plans[i].lg.size();
-        nlin += plans[i].lin.size();
+        nbt += plans[i].bt.size();
         nprog += plans[i].progs.size();
         b->large[i].npasses = (int)plans[i].progs.size();
         maxp = std::max(maxp, b->large[i].npasses);
@@ -552,7 +552,7 @@ qk_status run_large(qk_batch *b) {
     if ((s = grow(b, &b->d_loffs, &b->cap_loffs, (size_t)nl)) != QK_OK) return s;
     if ((s = grow(b, &b->d_lops, &b->cap_lops, std::max<size_t>(1, nops))) != QK_OK) return s;
     if ((s = grow(b, &b->d_llg, &b->cap_llg, std::max<size_t>(1, nlg))) != QK_OK) return s;
-    if ((s = grow(b, &b->d_llin, &b->cap_llin, std::max<size_t>(1, nlin))) != QK_OK) return s;
+    if ((s = grow(b, &b->d_lbt, &b->cap_lbt, std::max<size_t>(1, nbt))) != QK_OK) return s;
     // programs ordered by pass index; first[] splits each launch's grid
     std::vector<qk::TileProg> progs;
     progs.reserve(nprog);
@@ -567,7 +567,7 @@ qk_status run_large(qk_batch *b) {
             qk::TileProg h = plans[i].progs[k];
             h.op0 += (uint32_t)op_base[i];
             h.lg0 += (uint32_t)lg_base[i];
-            h.lin0 += (uint32_t)lin_base[i];
+            h.bt0 += (uint32_t)bt_base[i];
             h.psi = b->d_lstates + b->large[i].state_off;
             progs.push_back(h);
             first.push_back(acc);
@@ -578,15 +578,15 @@ qk_status run_large(qk_batch *b) {
     }
     std::vector<qk::TileOp> ops;
     std::vector<qk::LayerGate> lg;
-    std::vector<qk::LinTerm> lin;
+    std::vector<qk::BitTerm> bt;
     ops.reserve(nops);
     lg.reserve(nlg);
-    lin.reserve(nlin);
+    bt.reserve(nbt);
     std::vector<uint64_t> offs(nl);
     for (int i = 0; i < nl; ++i) {
         ops.insert(ops.end(), plans[i].ops.begin(), plans[i].ops.end());
         lg.insert(lg.end(), plans[i].lg.begin(), plans[i].lg.end());
-        lin.insert(lin.end(), plans[i].lin.begin(), plans[i].lin.end());
+        bt.insert(bt.end(), plans[i].bt.begin(), plans[i].bt.end());
         offs[i] = b->large[i].state_off;
     }
     b->plan_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -600,7 +600,7 @@ qk_status run_large(qk_batch *b) {
         !up(b->d_loffs, offs.data(), sizeof(uint64_t) * offs.size()) ||
         !up(b->d_lops, ops.data(), sizeof(qk::TileOp) * ops.size()) ||
         !up(b->d_llg, lg.data(), sizeof(qk::LayerGate) * lg.size()) ||
-        !up(b->d_llin, lin.data(), sizeof(qk::LinTerm) * lin.size()))
+        !up(b->d_lbt, bt.data(), sizeof(qk::BitTerm) * bt.size()))
         return bfail(b, QK_ECUDA, "batch: program upload failed");
     if (cudaMemsetAsync(b->d_lstates, 0, sizeof(float2) * b->large_amps, b->stream) != cudaSuccess)
         return bfail(b, QK_ECUDA, "batch: state reset failed");
@@ -616,7 +616,7 @@ qk_status run_large(qk_batch *b) {
             general = qk::tile_ops_need_general(ops.data() + h.op0, (size_t)h.nops);
         }
         const cudaError_t e = qk::launch_tile_batch(b->d_lprogs + launch[k].first, b->d_lfirst + launch[k].second, np,
-                                                    ctas[k], b->d_lops, b->d_llg, b->d_llin, general, b->stream);
+                                                    ctas[k], b->d_lops, b->d_llg, b->d_lbt, general, b->stream);
         if (e != cudaSuccess) return bfail(b, QK_ECUDA, "batch: tile launch failed: %s", cudaGetErrorString(e));
         ++b->large_launches;
     }
@@ -670,7 +670,7 @@ qk_status qk_batch_destroy(qk_batch *b) {
     if (!b) return QK_EINVAL;
     if (b->stream) {
         void *bufs[] = {b->d_ops, b->d_circs, b->d_states, b->d_cbits, b->d_lstates, b->d_lprogs,
-                        b->d_lfirst, b->d_loffs, b->d_lops, b->d_llg, b->d_llin};
+                        b->d_lfirst, b->d_loffs, b->d_lops, b->d_llg, b->d_lbt};
         for (void *q : bufs)
             if (q) cudaFreeAsync(q, b->stream);
         cudaStreamSynchronize(b->stream);

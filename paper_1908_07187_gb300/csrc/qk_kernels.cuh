@@ -280,7 +280,7 @@ constexpr int kTileQubits = 13;
 constexpr int kTileContig = 5;
 constexpr int kTileThreads = 256;
 constexpr int kTileMaxOps = 192;
-constexpr int kTileMaxLin = 512;
+constexpr int kTileMaxTerms = 768;
 // runs of consecutive fixed qubits: S holds 0..4 and eight more bits, which
 // split the rest into at most nine runs
 constexpr int kTileMaxRuns = 12;
@@ -288,73 +288,60 @@ constexpr int kTileMaxMats = 160;
 constexpr int kTileMaxConds = 4;
 enum TileArr : uint8_t { ARR_IO = 0, ARR_LO = 1, ARR_HI = 2 };
 // TOP_U2L: a layer of uncontrolled 2x2 gates on distinct register bits (k is
-// the bit mask), in pivot form; their coefficients are lg[first...] in bit order,
-// and bit b of rmask says that the gate on register bit b updates the pair's
-// stored |0> value first (LayerGate).  After the gates, a CZ between register
-// bits (k, l) for every bit set in tmask (bit cz_index(k, l) over the ten pairs,
-// see below).
-// TOP_PHASEL: a group of thread- or tile-dependent diagonal terms that all add to
-// one pending phase sum (register bit k, or the thread constant when k == 5):
-// lin[first, first + count), evaluated in place (see LinTerm); rval = 1 says that
-// bit k's qubit is stored flipped, so the sum lands on k = 0.  Diagonal terms
-// that are the same for every amplitude pair of a qubit (no thread or fixed-bit
-// condition) never reach the device: the planner folds them into the next layer
-// gate's coefficients or into the final flush.
-// TOP_PAIR: factor on the amplitudes whose register bits k and l (code k | l <<
-// 3) have the values in rval (bit 0: k, bit 1: l), under the op's thread /
-// fixed-bit conditions.
+// the bit mask); their descriptions are lg[first...] in bit order.  Before the gates, a
+// CZ between register bits (k, l) for every bit set in tmask (bit cz_index(k, l) over
+// the ten pairs, see below).  Bit b of rmask: the gate on register bit b updates the
+// pair's stored |0> value first; of rval: it turns the |1> value; of tval: a sign by
+// parity comes first; of count: phase terms come first (LayerGate).
 // TOP_PAIRNEG: an unconditional sign flip of the amplitudes whose register bits k
 // and l are both 1 (code k | l << 3): a CZ between two register bits.
-// TOP_PHASEB: a TOP_PHASEL group whose terms each test one bit (so every term is
-// "add turns where the bit is 1"; a term on a bit being 0 was split by the planner
-// into a constant it keeps and a negated bit-1 term): count thread-bit terms
-// followed by count2 tile-index-bit terms, BitTerm entries from index first of the
-// lin[] storage read as BitTerms (two per LinTerm slot); rval as for TOP_PHASEL.
-// TOP_PAIRU: a TOP_PAIR without thread, tile or classical condition (the common
-// case: a controlled phase between two register bits), always on the stored
-// pattern (1, 1): for qubits stored flipped the planner rewrites the factor as a
-// (1, 1) factor and uniform single-bit and constant phases.
+// TOP_PAIRU: factor on the amplitudes whose register bits k and l (code k | l << 3)
+// are both 1: a controlled phase between two register bits.
+// TOP_PHQ: a thread- and tile-dependent phase on register bit k = 1, from the BitTerms
+// [first, first + count) on thread bits and count2 more on tile-index bits (before a
+// general gate; layer gates carry their own).
+// TOP_U2, TOP_PHASE: controlled or conditioned 2x2 gate; factor on the amplitudes that
+// match the op's register, thread, tile and classical conditions.
 enum TileOpKind : uint8_t {
-    TOP_U2 = 0, TOP_PHASE = 1, TOP_XPOSE = 2, TOP_PHASEB = 3, TOP_U2L = 4, TOP_PAIR = 5, TOP_PHASEL = 6,
-    TOP_PAIRNEG = 7, TOP_PAIRU = 8
+    TOP_U2 = 0, TOP_PHASE = 1, TOP_XPOSE = 2, TOP_PHQ = 3, TOP_U2L = 4, TOP_PAIRNEG = 7, TOP_PAIRU = 8
 };
+// "add turns (2^-32 of a turn) where the bit is 1": a thread-bit index (lane 0..4, warp
+// 5..7) or a tile-index bit; in the final two-bit list b1 | b2 << 8, both bits of the
+// index thread bits + 256 * tile index
 struct BitTerm {
-    uint32_t bit;          // thread-bit index (lane 0..4, warp 5..7) or tile-index bit
+    uint32_t bit;
     uint32_t turns;
 };
 // the pairs k < l of register bits in the order (0,1) (0,2) (0,3) (0,4) (1,2)
 // (1,3) (1,4) (2,3) (2,4) (3,4): the bit of a TOP_U2L op's CZ mask
 __host__ __device__ constexpr int cz_index(int k, int l) { return k == 0 ? l - 1 : k == 1 ? l + 2 : k == 2 ? l + 4 : 9; }
 
-// A diagonal term of a TOP_PHASEL group: adds turns where the thread bits match
-// (tbits & tmask) == tval and the tile index matches (tile & fmask) == fval (its
-// bit b is the fixed qubit fixed[b]).
-struct LinTerm {
-    uint16_t tmask, tval;
-    uint32_t fmask, fval;
-    uint32_t turns;
-};
-
-// One gate of a TOP_U2L layer in pivot form.  The planner may keep a local
-// qubit's two values stored swapped ("flipped"); it picks the stored order of the
-// gate's output so that, with M the gate in stored order and the pending factor F
-// of the bit folded in, M diag(1, F) has its larger entries on the diagonal
-// (|M00| = |M11| >= |M10| = |M01|).  With a0 = M01 F / M00, a1 = M10 / (M11 F)
-// the true outputs are (M00 z0, M11 F z1) for z0 = y0 + a0 y1, z1 = y1 + a1 y0.
-// The device forms them in place from one value of the pair to the other, 8
-// FP32 FMAs per pair:
-//   zf = 0:  y1 += a1 y0,  then y0 += s a0 y1   (y0 ends as s z0, y1 as z1)
-//   zf = 1:  y0 += a0 y1,  then y1 += s a1 y0   (y0 ends as z0, y1 as s z1)
-// with s = 1 / (1 - a0 a1).  For a unitary M, a0 a1 = -|M01|^2 / |M00|^2, so s
-// = |M00|^2 is real and in [1/2, 1]; the planner keeps the leftover factor (M00 /
-// s and M11 F, or M00 and M11 F / s) as pending: a real scale and a phase for the
-// whole pass, and a factor of magnitude in [1/2, 2] on the bit's |1> (it picks zf
-// per gate so that the magnitude stays there).  The device uses c0 = C0 e and
-// c1 = C1 conj(e), with e the thread-dependent part of F; c[] holds C0 (s a0 or
-// a0) and C1 (a1 or s a1) as FFMA2 operand pairs (re, re), (im, im), (-im, -im).
+// One gate of a TOP_U2L layer.  The planner may keep a local qubit's two values stored
+// swapped ("flipped"); it picks the stored order of the gate's output so that, with M
+// the gate in stored order and F the pending factor of the bit, the larger entries are
+// on the diagonal.  With a0 = M01 F / M00 and a1 = M10 / (M11 F) the true outputs are
+// M00 (y0 + a0 y1) and M11 F (y1 + a1 y0), and a0 a1 is real and negative.  Turning y1
+// by e^{i phi} -- psi = arg a0 modulo pi, the sign goes into the updates -- makes both
+// updates real: three shears of (re, im) for the turn (3 FMAs per pair, none when phi =
+// 0), then, in place,
+//   zf = 0:  y1 += c1 y0,  then y0 += c0 y1;   zf = 1: the other order
+// (4 FMAs per pair).  7 FMAs per pair, against 8 for the same updates with complex
+// coefficients, every one in place.  (A turn as 1 + i tan(phi), its cosine kept pending,
+// is 2 FMAs but not in place: its register moves cost more, 103.8 ms of tile passes for
+// the 30-qubit step.)  The updates leave s = 1 / (1 - a0 a1) in [1/2, 1] on one value;
+// the planner picks zf so that the bit's pending magnitude stays near 1.
+// The diagonal terms that wait on the qubit (the other qubit a thread or tile-index
+// bit) come first, on the bit's |1>: a sign by the parity of the thread bits ts and
+// tile-index bits fs, and a phase from nt + ni BitTerms.
 struct LayerGate {
-    float2 c[6];           // C0r, C0i, -C0i, C1r, C1i, -C1i, each splatted
+    float2 h, s;           // -tan(phi / 2), sin(phi), splatted
+    float2 c0, c1;
+    uint32_t fs;
+    uint16_t ts, first;
+    uint8_t nt, ni;
+    uint16_t pad;
 };
+static_assert(sizeof(LayerGate) == 48, "LayerGate layout");
 
 struct TileOp {
     uint8_t kind;          // TileOpKind
@@ -362,27 +349,22 @@ struct TileOp {
     uint8_t rmask, rval;   // condition on register bits (5-bit register index space)
     uint16_t tmask, tval;  // condition on thread bits: bits 0..4 lane, 5..7 warp
     uint16_t cond;         // index into TileParams::conds, 0xffff = unconditional
-    uint16_t count;        // TOP_U2L: gates from lg[first]; TOP_PHASEL: terms from lin[first]
-    uint16_t first;
+    uint16_t count;
+    uint16_t first;        // TOP_U2L: gates from lg[first]; TOP_PHQ: terms from bt[first]
     uint16_t count2;
-    uint32_t hturns;       // TOP_U2: uniform pending turns of the target's qubit, added
-                           // to the thread's pending sum before the op
-    float hmag;            // TOP_U2: uniform pending magnitude of the target's |1>,
-                           // applied to the amplitudes before the op (1: none)
     uint64_t gmask, gval;  // condition on the tile's fixed (non-tile) physical bits
     union {
         float m[8];        // U2: m00, m01, m10, m11 as (re, im)
         struct {
-            float re, im;  // PHASE: factor f = exp(2 pi i turns / 2^32)
-            uint32_t turns;
+            float re, im;  // PHASE, PAIRU: factor
         } ph;
     };
 };
-// The tile kernel reads the fields the common op kinds need (kind, k, rval,
-// tmask, count, first, count2) as the op's first two 8-byte words, one op ahead.
-static_assert(offsetof(TileOp, kind) == 0 && offsetof(TileOp, k) == 1 && offsetof(TileOp, rval) == 3 &&
-                  offsetof(TileOp, tmask) == 4 && offsetof(TileOp, count2) == 14 &&
-                  offsetof(TileOp, count) == 10 && offsetof(TileOp, first) == 12 && offsetof(TileOp, hturns) == 16,
+// The tile kernel reads the fields the common op kinds need (kind, k, rmask, rval,
+// tmask, tval, count, first, count2) as the op's first two 8-byte words, one op ahead.
+static_assert(offsetof(TileOp, kind) == 0 && offsetof(TileOp, k) == 1 && offsetof(TileOp, rmask) == 2 &&
+                  offsetof(TileOp, rval) == 3 && offsetof(TileOp, tmask) == 4 && offsetof(TileOp, tval) == 6 &&
+                  offsetof(TileOp, count) == 10 && offsetof(TileOp, first) == 12 && offsetof(TileOp, count2) == 14,
               "TileOp head layout");
 static_assert(alignof(TileOp) >= 8, "TileOp head is read as 8-byte words");
 
@@ -415,20 +397,25 @@ struct TileHead {
     uint32_t fin_fixed[40];
     float fin_fixed_mag[40];
     int fin_flip;          // local qubits stored flipped at the end (bit b: local qubit b)
-    int nlg, nlin;         // entries of lg[] and lin[] in use
+    // diagonal terms that no gate of the plan called for (its last pass only): per
+    // register bit BitTerms from bt[fin_first[k]], fin_nt[k] on thread bits, then fin_ni[k]
+    // on tile-index bits; two-bit terms bt[fin2_first ...]
+    uint16_t fin_first[5], fin2_first, fin2_n;
+    uint8_t fin_nt[5], fin_ni[5];
+    int nlg, nbt;          // entries of lg[] and bt[] in use
 };
 
 // A whole pass program, passed as kernel parameters for one state.
 struct TileParams : TileHead {
     TileOp ops[kTileMaxOps];
     LayerGate lg[kTileMaxMats];
-    LinTerm lin[kTileMaxLin];
+    BitTerm bt[kTileMaxTerms];
 };
 
 // A pass program of one circuit in a batched launch: the header plus offsets
-// of its ops, layer gates and linear terms in device pools, and its state.
+// of its ops, layer gates and phase terms in device pools, and its state.
 struct TileProg : TileHead {
-    uint32_t op0, lg0, lin0, pad;
+    uint32_t op0, lg0, bt0, pad;
     float2 *psi;
 };
 static_assert(sizeof(TileParams) <= 32764, "tile program must fit in the kernel parameter space");
@@ -441,9 +428,9 @@ cudaError_t launch_tile(void *psi, const TileParams &p, const uint8_t *cbits, cu
 // general: some program holds general ops (see tile_ops_need_general); without
 // them a leaner instance of the kernel runs.
 cudaError_t launch_tile_batch(const TileProg *progs, const uint32_t *first, int n_progs, uint32_t n_ctas,
-                              const TileOp *ops, const LayerGate *lg, const LinTerm *lin, bool general,
+                              const TileOp *ops, const LayerGate *lg, const BitTerm *bt, bool general,
                               cudaStream_t s);
-// whether a pass program holds ops of the kinds TOP_U2, TOP_PHASE or TOP_PAIR
+// whether a pass program holds ops of the kinds TOP_U2, TOP_PHASE or TOP_PHQ
 bool tile_ops_need_general(const TileOp *ops, size_t n);
 
 // ---------------------------------------------------------------------------

@@ -12,12 +12,10 @@
 // gates are list-scheduled over the three register arrangements of the tile
 // kernel, inserting a transpose when no ready gate fits the current one.
 //
-// A last walk over the program (fold_program) turns each layer gate into pivot
-// form (LayerGate in qk_kernels.cuh) and keeps, in double precision, every
-// pending factor that is the same for all threads -- per local qubit (a phase and
-// a magnitude), plus a constant phase -- and the pass's real scale: those fold
-// into later gates' coefficients and the final flush, so the device never sees
-// them.
+// The program's builder (TileBuilder) keeps, in double precision, every single-qubit
+// diagonal factor -- one complex factor per qubit, and one for all amplitudes -- and the
+// diagonal terms on two qubits: a term waits until a gate acts on one of its qubits and
+// is applied there, so the device carries no phases from op to op.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -49,11 +47,14 @@ struct POp {
     const FusedOp *op;
     uint64_t nd;   // non-diagonal qubits
     uint64_t all;  // every qubit the op depends on
+    bool u2, cond; // what the walks over long lists ask, without touching the op
 };
 
 POp classify(const FusedOp &op) {
     POp p;
     p.op = &op;
+    p.u2 = op.kind == FusedOp::U2;
+    p.cond = op.cond.n != 0;
     if (op.kind == FusedOp::U2) {
         p.nd = 1ull << op.q;
         p.all = p.nd | op.cmask;
@@ -63,8 +64,6 @@ POp classify(const FusedOp &op) {
     }
     return p;
 }
-
-bool commute(const POp &a, const POp &b) { return !(a.nd & b.all) && !(b.nd & a.all); }
 
 bool same_cond(const Cond &a, const Cond &b) {
     if (a.n != b.n) return false;
@@ -137,82 +136,119 @@ uint32_t angle_turns(double x) {
 }
 double turns_angle(uint32_t t) { return 2.0 * M_PI * (double)t / 4294967296.0; }
 
-// local qubit of register bit k in an arrangement
-int local_of_reg(int arr, int k) { return arr == ARR_IO ? 5 + k : arr == ARR_LO ? k : 8 + k; }
-
-// Planner-only op kind: a diagonal term that is the same for every thread and
-// tile (no thread or fixed-bit condition) on register bit k (k == 5: constant),
-// ph.turns; fold_program absorbs it and it never reaches the device.
-constexpr uint8_t TOP_HOSTPH = 0x40;
-
 using cdm = std::complex<double>;
-struct Mat2 {
-    cdm m[4];
+// A diagonal term that is not yet in a program: f where (index & mask) == val.
+struct DTerm {
+    uint64_t mask, val;
+    cdm f;
+    const Cond *cond;
+    const FusedOp *src;      // the queued op that it is, if none of it became pending
 };
 
-// The program's pending state that is the same for every thread, in double
-// precision: mag[q] e^{i u[q]} the factor of local qubit q's stored |1> relative
-// to its stored |0>, u0 a constant phase, lam the real scale that the pivot form
-// leaves over, flip[q] whether q's values are stored swapped.
-struct UniformPending {
-    double u[kTileQubits] = {};     // phase of the pending factor on a local qubit's stored |1>
-    double mag[kTileQubits];        // its magnitude (in [1/2, 2])
-    double u0 = 0.0;
-    double lam = 1.0;
-    int flip[kTileQubits] = {};   // local qubit stored with its two values swapped
-    UniformPending() {
-        for (double &m : mag) m = 1.0;
+// What a pass program's builder keeps off the device.  Single-qubit diagonal factors
+// never reach it: F[q] is the pending complex factor of physical qubit q's |1>, lam the
+// one of every amplitude.  Diagonal terms on more qubits wait in terms until a gate
+// acts on one of their qubits and go out together there.
+struct PendingTerms {
+    cdm *F;
+    cdm &lam;
+    std::vector<DTerm> terms;
+
+    PendingTerms(cdm *f, cdm &l) : F(f), lam(l) {}
+
+    // a term of the queue: single-qubit and constant parts become pending factors, a
+    // two-qubit term keeps only its (1, 1) pattern
+    void diagonal(const POp &p) {
+        const FusedOp &op = *p.op;
+        DTerm t{op.mask, op.val, op.f, op.cond.n ? &op.cond : nullptr, &op};
+        const int k = __builtin_popcountll(t.mask);
+        if (t.cond || k > 2) {
+            terms.push_back(t);
+            return;
+        }
+        if (k == 0) {
+            lam *= t.f;
+            return;
+        }
+        const int a = __builtin_ctzll(t.mask), b = 63 - __builtin_clzll(t.mask);
+        const int va = (int)(t.val >> a) & 1, vb = (int)(t.val >> b) & 1;
+        const cdm inv = 1.0 / t.f;
+        if (k == 1) {
+            if (va) F[a] *= t.f;
+            else {
+                lam *= t.f;
+                F[a] *= inv;
+            }
+            return;
+        }
+        if (va && !vb) F[a] *= t.f;
+        if (!va && vb) F[b] *= t.f;
+        if (!va && !vb) {
+            lam *= t.f;
+            F[a] *= inv;
+            F[b] *= inv;
+        }
+        if (t.val != t.mask) t.src = nullptr;
+        if (va != vb) t.f = inv;
+        t.val = t.mask;
+        terms.push_back(t);
+    }
+    static bool is_pair(const DTerm &t) { return !t.cond && t.val == t.mask && __builtin_popcountll(t.mask) == 2; }
+    static bool is_sign(const DTerm &t) { return t.f == cdm(-1.0, 0.0); }
+    // the waiting terms as queue entries for a later pass; rewritten holds those that
+    // are not queued ops as they stand
+    void hand_on(std::vector<POp> &next, std::deque<FusedOp> &rewritten) const {
+        for (const DTerm &t : terms) {
+            if (t.src) {
+                next.push_back(classify(*t.src));
+                continue;
+            }
+            FusedOp o;
+            o.kind = FusedOp::PHASE;
+            o.mask = t.mask;
+            o.val = t.val;
+            o.f = t.f;
+            rewritten.push_back(o);
+            next.push_back(classify(rewritten.back()));
+        }
     }
 };
 
-// Pivot form of a layer gate on local qubit q (LayerGate in qk_kernels.cuh).  The
-// gate in stored order is W = U X^f (f: q stored flipped); the output is stored
-// flipped (f') when that puts the larger entries of M = X^f' W on the diagonal.
-// F = mag[q] e^{i u[q]} is the pending factor of q's stored |1>.  Returns zf, the
-// value of the pair the device updates first: the one that keeps the pending
-// magnitude of q's |1> within [1/2, 2] (zf = 0 multiplies it by s <= 1, zf = 1
-// divides it by s >= 1/2).
-int pivot_gate(const Mat2 &g, UniformPending &st, int q, LayerGate &out) {
-    cdm W[4] = {g.m[0], g.m[1], g.m[2], g.m[3]};
-    if (st.flip[q]) {  // U X: swap the columns
-        std::swap(W[0], W[1]);
-        std::swap(W[2], W[3]);
-    }
-    const bool fout = std::abs(W[0]) < std::abs(W[2]);
-    if (fout) {        // X W: swap the rows
+// How a 2x2 gate M on a qubit with pending factor f (on the stored |1>) is run: W is M
+// or, with sw, X M (the rows exchanged so that the larger entries are on the diagonal);
+// the true outputs are p0 and p1 times the values the device leaves.  a0 = W01 f / W00,
+// a1 = W10 / (W11 f); r0 = |a0|, r1 = |a1|, psi = arg a0, and a1 = -r1 e^{-i psi} for a
+// unitary M.  s = 1 / (1 + r0 r1) is what updating one value from the other in place
+// leaves on the value updated second.
+struct GateForm {
+    bool sw;
+    cdm p0, p1;
+    double r0, r1, psi, s;
+};
+GateForm gate_form(const cdm *M, cdm f) {
+    cdm W[4] = {M[0], M[1], M[2], M[3]};
+    GateForm g;
+    g.sw = std::abs(W[0]) < std::abs(W[2]);
+    if (g.sw) {
         std::swap(W[0], W[2]);
         std::swap(W[1], W[3]);
     }
-    const cdm m00 = W[0], m01 = W[1], m10 = W[2], m11 = W[3];
-    const cdm F = std::polar(st.mag[q], st.u[q]);
-    const cdm A0 = m01 * F / m00, A1 = m10 / (m11 * F);
-    // y1 += a1 y0 then y0 += s a0 y1 leaves y0 = s z0 (and the other order y1 =
-    // s z1) for s = 1 / (1 - a0 a1), real and in [1/2, 1] for a unitary gate
-    const cdm s = 1.0 / (1.0 - A0 * A1);
-    const int zf = st.mag[q] < 1.0 ? 1 : 0;
-    const cdm C0 = zf ? A0 : s * A0, C1 = zf ? s * A1 : A1;
-    const cdm P0 = zf ? m00 : m00 / s, P1 = zf ? m11 * F / s : m11 * F;   // the true outputs' factors
-    st.u0 += std::arg(P0);
-    st.lam *= std::abs(P0);
-    const cdm R = P1 / P0;
-    st.u[q] = std::arg(R);
-    st.mag[q] = std::abs(R);
-    st.flip[q] = fout ? 1 : 0;
-    const float a0r = (float)C0.real(), a0i = (float)C0.imag(), a1r = (float)C1.real(), a1i = (float)C1.imag();
-    out.c[0] = make_float2(a0r, a0r);
-    out.c[1] = make_float2(a0i, a0i);
-    out.c[2] = make_float2(-a0i, -a0i);
-    out.c[3] = make_float2(a1r, a1r);
-    out.c[4] = make_float2(a1i, a1i);
-    out.c[5] = make_float2(-a1i, -a1i);
-    return zf;
+    const cdm a0 = W[1] * f / W[0], a1 = W[2] / (W[3] * f);
+    g.r0 = std::abs(a0);
+    g.r1 = std::abs(a1);
+    g.psi = g.r0 != 0.0 || g.r1 != 0.0 ? std::arg(a0) : 0.0;
+    g.s = 1.0 / (1.0 + g.r0 * g.r1);
+    g.p0 = W[0];
+    g.p1 = W[3] * f;
+    return g;
+}
+// whether a0 a1 is real and not positive (GateForm): a matrix defined with a loose
+// tolerance need not be so
+bool real_form(const cdm *M, double tol) {
+    const cdm pr = M[1] * M[2] * std::conj(M[0] * M[3]);
+    return std::abs(pr.imag()) <= tol * std::abs(pr) && pr.real() <= 0.0;
 }
 
-// local qubits of the thread bits (0..4 lanes, 5..7 warps) in an arrangement
-int local_of_tbit(int arr, int t) {
-    if (t < 5) return arr == ARR_LO ? 5 + t : t;
-    return arr == ARR_HI ? 5 + (t - 5) : 10 + (t - 5);
-}
 // The gates one pass takes from rem for a qubit set S: in order, each gate
 // that commutes with every gate left behind before it, whose 2x2 target is in
 // S (with grow, a target joins S while S has room) and whose classical
@@ -237,10 +273,10 @@ void take_gates(const std::vector<POp> &rem, int n, const TakeLimits &lim, uint6
             break;
         }
         const POp &p = *it;
-        const bool is_u2 = p.op->kind == FusedOp::U2;
+        const bool is_u2 = p.u2;
         bool ok = (is_u2 ? n_u2 < lim.max_u2 : n_ph < lim.max_ph) && !(p.nd & allb) && !(p.all & ndb);
         if (ok && is_u2) {
-            const uint64_t t = 1ull << p.op->q;
+            const uint64_t t = p.nd;
             if (!(S & t)) {
                 if (grow && cnt < lim.tile_qubits) {
                     S |= t;
@@ -250,7 +286,7 @@ void take_gates(const std::vector<POp> &rem, int n, const TakeLimits &lim, uint6
                 }
             }
         }
-        if (ok && p.op->cond.n) {
+        if (ok && p.cond) {
             bool found = false;
             for (const auto &cd : conds) found = found || same_cond(cd, p.op->cond);
             if (!found) {
@@ -326,27 +362,13 @@ int smem_tile_qubits(int n, int prec) {
 // Qubits that every tile holds, for runs of 128 bytes in HBM; none for states in L2.
 int smem_tile_contig(int n) { return n >= 18 ? 3 : 0; }
 
-// A diagonal term that is not yet in a program: f where (index & mask) == val.
-struct DTerm {
-    uint64_t mask, val;
-    cdm f;
-    const Cond *cond;
-    const FusedOp *src;      // the queued op that it is, if none of it became pending
-};
-
-// Builds one pass's program from its gates in order.  Single-qubit diagonal factors
-// never reach the device: F[q] is the pending complex factor of physical qubit q's |1>,
-// lam the one of every amplitude.  Diagonal terms on more qubits wait in terms until a
-// gate acts on one of their qubits and go out together there.
-struct SmemTileBuilder {
+// Builds one pass's program from its gates in order.
+struct SmemTileBuilder : PendingTerms {
     SmemTileParams &P;
-    cdm *F;
-    cdm &lam;
     int local_of[64], tile_of[64];
-    std::vector<DTerm> terms;
     bool overflow = false;
 
-    SmemTileBuilder(SmemTileParams &p, cdm *f, cdm &l) : P(p), F(f), lam(l) {}
+    SmemTileBuilder(SmemTileParams &p, cdm *f, cdm &l) : PendingTerms(f, l), P(p) {}
 
     SmemTileOp *add(uint8_t kind, uint8_t q) {
         if (P.nops >= kSmemTileOps) {
@@ -379,46 +401,6 @@ struct SmemTileBuilder {
             if (same_cond(P.conds[k], c)) return (uint8_t)k;
         return kNoBit;
     }
-
-    // a term of the queue: single-qubit and constant parts become pending factors, a
-    // two-qubit term keeps only its (1, 1) pattern
-    void diagonal(const POp &p) {
-        const FusedOp &op = *p.op;
-        DTerm t{op.mask, op.val, op.f, op.cond.n ? &op.cond : nullptr, &op};
-        const int k = __builtin_popcountll(t.mask);
-        if (t.cond || k > 2) {
-            terms.push_back(t);
-            return;
-        }
-        if (k == 0) {
-            lam *= t.f;
-            return;
-        }
-        const int a = __builtin_ctzll(t.mask), b = 63 - __builtin_clzll(t.mask);
-        const int va = (int)(t.val >> a) & 1, vb = (int)(t.val >> b) & 1;
-        const cdm inv = 1.0 / t.f;
-        if (k == 1) {
-            if (va) F[a] *= t.f;
-            else {
-                lam *= t.f;
-                F[a] *= inv;
-            }
-            return;
-        }
-        if (va && !vb) F[a] *= t.f;
-        if (!va && vb) F[b] *= t.f;
-        if (!va && !vb) {
-            lam *= t.f;
-            F[a] *= inv;
-            F[b] *= inv;
-        }
-        if (t.val != t.mask) t.src = nullptr;
-        if (va != vb) t.f = inv;
-        t.val = t.mask;
-        terms.push_back(t);
-    }
-    static bool is_pair(const DTerm &t) { return !t.cond && t.val == t.mask && __builtin_popcountll(t.mask) == 2; }
-    static bool is_sign(const DTerm &t) { return t.f == cdm(-1.0, 0.0); }
 
     void single_term(const DTerm &t) {
         SmemTileOp *o = add(ST_PH, kNoBit);
@@ -526,26 +508,18 @@ struct SmemTileBuilder {
         F[b] = 1.0;
     }
 
-    // A 2x2 gate on physical qubit op.q.  Uncontrolled: with M = W or X W (rows
-    // exchanged when that puts the larger entries on the diagonal) and F the pending
-    // factor, the outputs are W00 (y0 + a0 y1) and W11 F (y1 + a1 y0) with a0 = W01 F /
-    // W00, a1 = W10 / (W11 F), and a0 a1 = -r0 r1 is real for a unitary M.  Turning y1
-    // (or y0) by psi = arg a0 makes both updates real; of e^{i psi} = i^k cos(phi) (1 +
-    // i tan(phi)), |phi| <= pi/4, only i^k (1 + i tan) is applied and the cosine stays
-    // pending.  Updating one value from the other in place leaves s = 1 / (1 + r0 r1)
-    // on the second one.  Which value is turned and which is updated first is chosen so
-    // that the pending magnitude stays near 1.
+    // A 2x2 gate on physical qubit op.q.  Uncontrolled (GateForm): turning y1 (or y0) by
+    // psi makes both updates real; of e^{i psi} = i^k cos(phi) (1 + i tan(phi)), |phi| <=
+    // pi/4, only i^k (1 + i tan) is applied and the cosine stays pending.  Which value is
+    // turned and which is updated first is chosen so that the pending magnitude stays
+    // near 1.
     void gate(const POp &p) {
         const FusedOp &op = *p.op;
         const int b = op.q;
         const uint8_t q = (uint8_t)local_of[b];
         const cdm *M = op.m;
         const bool is_x = M[0] == 0.0 && M[3] == 0.0 && M[1] == 1.0 && M[2] == 1.0;
-        // the update form below takes a0 a1 for real, which a matrix defined with a loose
-        // tolerance need not have
-        const cdm pr = M[1] * M[2] * std::conj(M[0] * M[3]);
-        const bool unitary = std::abs(pr.imag()) <= 0x1p-50 * std::abs(pr) && pr.real() <= 0.0;
-        if (op.cmask || op.cond.n || !unitary) {
+        if (op.cmask || op.cond.n || !real_form(M, 0x1p-50)) {
             emit_touching(b, nullptr, nullptr);
             materialise(b);
             SmemTileOp *o = add(is_x ? ST_X : ST_CU2, q);
@@ -563,18 +537,12 @@ struct SmemTileBuilder {
         SmemTileOp *o = add(ST_U2, q);
         o->lmask = sl;
         o->tmask = sg;
-        cdm W[4] = {M[0], M[1], M[2], M[3]};
-        const bool sw = std::abs(W[0]) < std::abs(W[2]);
-        if (sw) {
-            std::swap(W[0], W[2]);
-            std::swap(W[1], W[3]);
-            o->flags |= kU2Swap;
-        }
-        const cdm f = F[b], a0 = W[1] * f / W[0], a1 = W[2] / (W[3] * f);
-        const double r0 = std::abs(a0), r1 = std::abs(a1), s = 1.0 / (1.0 + r0 * r1);
-        cdm p0 = W[0], p1 = W[3] * f;
+        const GateForm g = gate_form(M, F[b]);
+        const bool sw = g.sw;
+        if (sw) o->flags |= kU2Swap;
+        const double r0 = g.r0, r1 = g.r1, s = g.s, psi = g.psi;
+        cdm p0 = g.p0, p1 = g.p1;
         if (r0 != 0.0 || r1 != 0.0) {
-            const double psi = std::arg(a0);
             const int k = (int)std::lround(psi / (M_PI / 2));
             const double phi = psi - k * (M_PI / 2), cs = std::cos(phi), tn = std::tan(phi);
             const cdm e = std::polar(1.0, psi);
@@ -621,7 +589,553 @@ struct SmemTileBuilder {
     }
 };
 
+// ---------------------------------------------------------------------------
+// register tiles (TileParams in qk_kernels.cuh)
+// ---------------------------------------------------------------------------
+
+constexpr uint32_t kHalf = 0x80000000u;   // half a turn
+
+// Builds one pass's program in the order the scheduler emits its gates (PendingTerms
+// holds what waits).  F is in terms of the qubits' true values; a local qubit may be
+// stored with its two values exchanged (flip).
+struct TileBuilder : PendingTerms {
+    TileParams &P;
+    int local_of[64], tile_of[64];
+    int flip[kTileQubits] = {};
+    int arr = ARR_IO;
+    int open = -1;           // index of the layer op that further gates may join, -1: none
+    bool overflow = false;
+
+    TileBuilder(TileParams &p, cdm *f, cdm &l) : PendingTerms(f, l), P(p) {}
+
+    TileOp &add(uint8_t kind) {
+        open = -1;
+        if (P.nops >= kTileMaxOps) {
+            overflow = true;
+            P.nops = 0;      // the program is thrown away
+        }
+        TileOp &o = P.ops[P.nops++];
+        std::memset(static_cast<void *>(&o), 0, sizeof o);
+        o.kind = kind;
+        o.cond = 0xffff;
+        return o;
+    }
+    void add_term(uint32_t bit, uint32_t turns) {
+        if (P.nbt >= kTileMaxTerms) {
+            overflow = true;
+            P.nbt = 0;
+        }
+        P.bt[P.nbt++] = BitTerm{bit, turns};
+    }
+    void transpose_to(int a) {
+        add(TOP_XPOSE).k = (uint8_t)a;
+        arr = a;
+    }
+    int flip_of(int b) const { return local_of[b] >= 0 ? flip[local_of[b]] : 0; }
+    // where physical qubit b is: 0 a register bit, 1 a thread bit, 2 a tile-index bit
+    int place(int b, int *pos) const {
+        if (local_of[b] < 0) {
+            *pos = tile_of[b];
+            return 2;
+        }
+        const int s = slot_of(arr, local_of[b], pos);
+        if (s == 2) *pos += 5;
+        return s == 0 ? 0 : 1;
+    }
+    // a phase on the stored |1> of qubit b
+    void stored_phase(int b, double x) {
+        if (flip_of(b)) {
+            lam *= std::polar(1.0, x);
+            F[b] *= std::polar(1.0, -x);
+        } else {
+            F[b] *= std::polar(1.0, x);
+        }
+    }
+    // e^{i th} where the true values of a and b are both 1, in stored values sa, sb: (sa ^
+    // fa)(sb ^ fb) = fa fb + fa (1 - 2 fb) sb + fb (1 - 2 fa) sa + (1 - 2 fa)(1 - 2 fb) sa
+    // sb.  The constant and the single-bit parts become pending; returns the turns left
+    // on the stored pattern (1, 1).
+    uint32_t stored_pair(int a, int b, const DTerm &t) {
+        const uint32_t T = is_sign(t) ? kHalf : angle_turns(std::arg(t.f));
+        const double th = turns_angle(T);
+        const int fa = flip_of(a), fb = flip_of(b);
+        if (fa && fb) lam *= std::polar(1.0, th);
+        if (fa) stored_phase(b, fb ? -th : th);
+        if (fb) stored_phase(a, fa ? -th : th);
+        return fa != fb ? 0u - T : T;
+    }
+    // an op's conditions in stored values
+    void conditions(TileOp &o, uint64_t mask, uint64_t val) {
+        for (uint64_t m = mask; m; m &= m - 1) {
+            const int b = __builtin_ctzll(m);
+            if (flip_of(b)) val ^= 1ull << b;
+        }
+        encode_cond(mask, val, arr, local_of, o);
+    }
+    void set_cond(TileOp &o, const Cond &c) {
+        for (int k = 0; k < P.n_conds; ++k)
+            if (same_cond(P.conds[k], c)) o.cond = (uint16_t)k;
+    }
+    void direct(uint64_t mask, uint64_t val, cdm f, const Cond *c) {
+        TileOp &o = add(TOP_PHASE);
+        conditions(o, mask, val);
+        if (c) set_cond(o, *c);
+        o.ph.re = (float)f.real();
+        o.ph.im = (float)f.imag();
+    }
+    void pair_op(int k, int l, uint32_t turns) {
+        if (turns == 0) return;
+        if (k > l) std::swap(k, l);
+        TileOp &o = add(turns == kHalf ? TOP_PAIRNEG : TOP_PAIRU);
+        o.k = (uint8_t)(k | (l << 3));
+        const double x = turns_angle(turns);
+        o.ph.re = (float)std::cos(x);
+        o.ph.im = (float)std::sin(x);
+    }
+
+    // what waits on qubit b (a register bit now), taken out of terms: register pairs
+    // (other bit, turns), thread and tile-index terms, and everything else
+    struct Touching {
+        std::vector<std::pair<int, uint32_t>> reg;
+        std::vector<BitTerm> thread, tile;
+        std::vector<DTerm> other;
+    };
+    void take_touching(int b, Touching &out) {
+        out.reg.clear();
+        out.thread.clear();
+        out.tile.clear();
+        out.other.clear();
+        size_t w = 0;
+        const uint64_t bb = 1ull << b;
+        auto put = [](std::vector<BitTerm> &v, uint32_t bit, uint32_t turns) {
+            for (BitTerm &t : v)
+                if (t.bit == bit) {
+                    t.turns += turns;
+                    return;
+                }
+            v.push_back(BitTerm{bit, turns});
+        };
+        for (size_t i = 0; i < terms.size(); ++i) {
+            const DTerm t = terms[i];
+            if (!(t.mask & bb)) {
+                terms[w++] = t;
+                continue;
+            }
+            if (!is_pair(t)) {
+                out.other.push_back(t);
+                continue;
+            }
+            const int d = __builtin_ctzll(t.mask & ~bb);
+            const uint32_t T = stored_pair(b, d, t);
+            int pos;
+            const int where = place(d, &pos);
+            if (where == 0) out.reg.push_back({pos, T});
+            else put(where == 1 ? out.thread : out.tile, (uint32_t)pos, T);
+        }
+        terms.resize(w);
+    }
+
+    // a 2x2 gate whose target is a register bit of the current arrangement
+    void gate(const POp &p) {
+        const FusedOp &op = *p.op;
+        const int b = op.q, lq = local_of[b];
+        int k;
+        place(b, &k);
+        static thread_local Touching T;
+        take_touching(b, T);
+        if (op.cmask || op.cond.n || !real_form(op.m, 1e-7)) {
+            for (const DTerm &t : T.other) direct(t.mask, t.val, t.f, t.cond);
+            for (const auto &r : T.reg) pair_op(k, r.first, r.second);
+            if (!T.thread.empty() || !T.tile.empty()) {
+                TileOp &o = add(TOP_PHQ);
+                o.k = (uint8_t)k;
+                o.first = (uint16_t)P.nbt;
+                o.count = (uint16_t)T.thread.size();
+                o.count2 = (uint16_t)T.tile.size();
+                for (const BitTerm &t : T.thread) add_term(t.bit, t.turns);
+                for (const BitTerm &t : T.tile) add_term(t.bit, t.turns);
+            }
+            if (F[b] != cdm(1.0, 0.0)) {
+                direct(1ull << b, 1ull << b, F[b], nullptr);
+                F[b] = 1.0;
+            }
+            TileOp &o = add(TOP_U2);
+            conditions(o, op.cmask, op.cmask);
+            if (op.cond.n) set_cond(o, op.cond);
+            o.k = (uint8_t)k;
+            for (int e = 0; e < 4; ++e) {   // X M X in stored order when the qubit is flipped
+                const cdm m = op.m[flip[lq] ? 3 - e : e];
+                o.m[2 * e] = (float)m.real();
+                o.m[2 * e + 1] = (float)m.imag();
+            }
+            return;
+        }
+        // joins the open layer unless its bit is in it, or a term with one of the
+        // layer's bits (put there after that bit's gate) or a factor has to come first
+        bool join = open >= 0 && !((P.ops[open].k >> k) & 1) && T.other.empty();
+        for (const auto &r : T.reg)
+            join = join && (r.second == kHalf || r.second == 0) && !((P.ops[open].k >> r.first) & 1);
+        if (!join) {
+            for (const DTerm &t : T.other) direct(t.mask, t.val, t.f, t.cond);
+            for (const auto &r : T.reg)
+                if (r.second != kHalf) pair_op(k, r.first, r.second);
+            TileOp &o = add(TOP_U2L);
+            o.first = (uint16_t)P.nlg;
+            open = P.nops - 1;
+        }
+        if (overflow || P.nlg >= kTileMaxMats) {
+            overflow = true;
+            return;
+        }
+        TileOp &o = P.ops[open];
+        for (const auto &r : T.reg)
+            if (r.second == kHalf) o.tmask ^= (uint16_t)(1u << cz_index(std::min(k, r.first), std::max(k, r.first)));
+        // the layer is the last one in lg: keep its gates in bit order
+        const int at = o.first + __builtin_popcount(o.k & ((1u << k) - 1));
+        for (int i = P.nlg; i > at; --i) P.lg[i] = P.lg[i - 1];
+        ++P.nlg;
+        o.k |= (uint8_t)(1u << k);
+        LayerGate &g = P.lg[at];
+        std::memset(static_cast<void *>(&g), 0, sizeof g);
+        // its waiting terms: half turns by parity, the rest as phase terms
+        for (const BitTerm &t : T.thread)
+            if (t.turns == kHalf) g.ts ^= (uint16_t)(1u << t.bit);
+        for (const BitTerm &t : T.tile)
+            if (t.turns == kHalf) g.fs ^= 1u << t.bit;
+        if (g.ts || g.fs) o.tval |= (uint16_t)(1u << k);
+        g.first = (uint16_t)P.nbt;
+        for (const BitTerm &t : T.thread)
+            if (t.turns != kHalf && t.turns != 0) {
+                add_term(t.bit, t.turns);
+                ++g.nt;
+            }
+        for (const BitTerm &t : T.tile)
+            if (t.turns != kHalf && t.turns != 0) {
+                add_term(t.bit, t.turns);
+                ++g.ni;
+            }
+        if (g.nt || g.ni) o.count |= (uint16_t)(1u << k);
+        pivot(op.m, b, lq, k, o, g);
+    }
+
+    // LayerGate's coefficients.  zf is chosen so that the pending magnitude of the qubit's
+    // |1> stays within [1/2, 2].
+    void pivot(const cdm *M, int b, int lq, int k, TileOp &o, LayerGate &g) {
+        cdm Ms[4] = {M[0], M[1], M[2], M[3]}, f = F[b];
+        if (flip[lq]) {                       // the stored input is the true one exchanged
+            std::swap(Ms[0], Ms[1]);
+            std::swap(Ms[2], Ms[3]);
+            lam *= f;
+            f = 1.0 / f;
+        }
+        const GateForm w = gate_form(Ms, f);
+        cdm p0 = w.p0, p1 = w.p1;
+        if (w.r0 != 0.0 || w.r1 != 0.0) {
+            const int turns = (int)std::lround(w.psi / M_PI);
+            const double phi = w.psi - turns * M_PI, sg = turns & 1 ? -1.0 : 1.0;
+            p1 *= std::polar(1.0, -phi);
+            double b0 = sg * w.r0, b1 = -sg * w.r1;
+            double r = std::abs(p1 / p0);
+            if (w.sw) r = 1.0 / r;
+            const bool zf = (r < 1.0) != w.sw;   // divide the smaller factor by s, or multiply the larger
+            if (zf) {
+                b1 *= w.s;
+                p1 /= w.s;
+                o.rmask |= (uint8_t)(1u << k);
+            } else {
+                b0 *= w.s;
+                p0 /= w.s;
+            }
+            auto splat = [](double x) { return make_float2((float)x, (float)x); };
+            if (std::abs(phi) > 0x1p-27) o.rval |= (uint8_t)(1u << k);   // below: less than a rounding error
+            g.h = splat(-std::tan(phi / 2));
+            g.s = splat(std::sin(phi));
+            g.c0 = splat(b0);
+            g.c1 = splat(b1);
+        }
+        flip[lq] = w.sw ? 1 : 0;
+        if (w.sw) std::swap(p0, p1);          // the true |0> and |1>
+        lam *= p0;
+        F[b] = p1 / p0;
+    }
+
+    // every waiting term as ops and as the final flush's terms
+    void finish_terms() {
+        std::vector<BitTerm> th[5], ti[5], two;
+        for (const DTerm &t : terms) {
+            if (!is_pair(t)) {
+                direct(t.mask, t.val, t.f, t.cond);
+                continue;
+            }
+            const int a = __builtin_ctzll(t.mask), b = 63 - __builtin_clzll(t.mask);
+            const uint32_t T = stored_pair(a, b, t);
+            int pa, pb;
+            const int wa = place(a, &pa), wb = place(b, &pb);
+            if (wa == 0 && wb == 0) pair_op(pa, pb, T);
+            else if (wa == 0) (wb == 1 ? th : ti)[pa].push_back(BitTerm{(uint32_t)pb, T});
+            else if (wb == 0) (wa == 1 ? th : ti)[pb].push_back(BitTerm{(uint32_t)pa, T});
+            else
+                two.push_back(BitTerm{(uint32_t)(wa == 2 ? pa + 8 : pa) | (uint32_t)(wb == 2 ? pb + 8 : pb) << 8, T});
+        }
+        terms.clear();
+        for (int k = 0; k < 5; ++k) {
+            if (th[k].size() > 255 || ti[k].size() > 255) overflow = true;
+            P.fin_first[k] = (uint16_t)P.nbt;
+            P.fin_nt[k] = (uint8_t)th[k].size();
+            P.fin_ni[k] = (uint8_t)ti[k].size();
+            for (const BitTerm &t : th[k]) add_term(t.bit, t.turns);
+            for (const BitTerm &t : ti[k]) add_term(t.bit, t.turns);
+        }
+        P.fin2_first = (uint16_t)P.nbt;
+        P.fin2_n = (uint16_t)two.size();
+        for (const BitTerm &t : two) add_term(t.bit, t.turns);
+    }
+};
+
 }  // namespace
+
+qk_status plan_passes(TilePlanner *planner, int n, const std::vector<FusedOp> &ops, const PassSink &sink,
+                      const char **err) {
+    *err = "";
+    std::vector<POp> rem;
+    rem.reserve(ops.size());
+    for (const auto &op : ops) rem.push_back(classify(op));
+
+    // take limits per pass; halved and retried when a program overflows the
+    // kernel-parameter budget (ops and grouped phase entries)
+    int max_u2 = 100, max_ph = 300;
+    static thread_local std::vector<POp> left, taken, next;
+    std::deque<FusedOp> rewritten;   // pair terms handed on without their single-qubit parts
+    // per physical qubit the pending factor of its |1>, and the one of all amplitudes,
+    // handed from pass to pass in FP64; only the plan's last pass applies them
+    cdm F[64], lam = 1.0;
+    for (cdm &f : F) f = 1.0;
+    std::vector<Cond> conds;
+    while (!rem.empty()) {
+        int n_u2 = 0, n_ph = 0;
+        const uint64_t S = choose_pass(rem, n, TakeLimits{kTileQubits, max_u2, max_ph}, kTileContig, conds, taken, left,
+                                       &n_u2, &n_ph);
+
+        static thread_local TileParams P;
+        std::memset(static_cast<TileHead *>(&P), 0, sizeof(TileHead));
+        P.n = n;
+        P.n_tiles = 1ull << (n - kTileQubits);
+        cdm F1[64], lam1 = lam;
+        std::copy(F, F + 64, F1);
+        TileBuilder B(P, F1, lam1);
+        int *const local_of = B.local_of;
+        for (int b = 0; b < 64; ++b) local_of[b] = B.tile_of[b] = -1;
+        {
+            int lb = 0, fb = 0;
+            for (int b = 0; b < n; ++b) {
+                if ((S >> b) & 1) {
+                    P.S[lb] = (int8_t)b;
+                    local_of[b] = lb++;
+                } else {
+                    B.tile_of[b] = fb;
+                    P.fixed[fb++] = (int8_t)b;
+                }
+            }
+            P.nfix = fb;
+            // runs of consecutive fixed qubits
+            P.nruns = 0;
+            for (int b = 0; b < fb;) {
+                int e = b + 1;
+                while (e < fb && P.fixed[e] == P.fixed[e - 1] + 1) ++e;
+                if (P.nruns >= kTileMaxRuns) {
+                    *err = "internal: too many fixed-qubit runs";
+                    return QK_EINVAL;
+                }
+                P.run_tlo[P.nruns] = (uint8_t)b;
+                P.run_len[P.nruns] = (uint8_t)(e - b);
+                P.run_plo[P.nruns] = (uint8_t)P.fixed[b];
+                ++P.nruns;
+                b = e;
+            }
+        }
+        P.n_conds = (int)conds.size();
+        for (int k = 0; k < P.n_conds; ++k) P.conds[k] = conds[k];
+
+        // ---- list-schedule the taken gates over the arrangements
+        const int m = (int)taken.size();
+        // What each op has to follow, qubit by qubit: a 2x2 gate comes after everything
+        // on its target since the last gate on it, any other touch after that gate.
+        // Successors of op i as a list in edges (next index in edges, or -1).
+        struct Edge {
+            int to, next;
+        };
+        static thread_local std::vector<Edge> edges;
+        static thread_local std::vector<int> npred, head, touch_next, ready;
+        edges.clear();
+        npred.assign(m, 0);
+        head.assign(m, -1);
+        int last_gate[64], touched[64];      // per qubit: the last gate on it; ops since then (a list)
+        for (int b = 0; b < 64; ++b) last_gate[b] = touched[b] = -1;
+        std::vector<Edge> &E = edges;
+        static thread_local std::vector<Edge> touches;
+        touches.clear();
+        auto edge = [&](int i, int j) {
+            E.push_back({j, head[i]});
+            head[i] = (int)E.size() - 1;
+            ++npred[j];
+        };
+        for (int j = 0; j < m; ++j) {
+            for (uint64_t q = taken[j].all; q; q &= q - 1) {
+                const int b = __builtin_ctzll(q);
+                if ((taken[j].nd >> b) & 1) {
+                    if (touched[b] < 0 && last_gate[b] >= 0) edge(last_gate[b], j);
+                    for (int t = touched[b]; t >= 0; t = touches[t].next) edge(touches[t].to, j);
+                    last_gate[b] = j;
+                    touched[b] = -1;
+                } else {
+                    if (last_gate[b] >= 0) edge(last_gate[b], j);
+                    touches.push_back({j, touched[b]});
+                    touched[b] = (int)touches.size() - 1;
+                }
+            }
+        }
+        // A diagonal term that is ready only starts to wait in the builder; a ready gate
+        // (at most one per qubit) is emitted when its target is a register bit.
+        ready.clear();
+        int ndone = 0;
+        static thread_local std::vector<int> stack;
+        auto settle = [&](int j) {           // op j has no predecessors left
+            stack.clear();
+            stack.push_back(j);
+            while (!stack.empty()) {
+                const int i = stack.back();
+                stack.pop_back();
+                if (taken[i].op->kind == FusedOp::U2) {
+                    ready.push_back(i);
+                    continue;
+                }
+                B.diagonal(taken[i]);
+                ++ndone;
+                for (int e = head[i]; e >= 0; e = E[e].next)
+                    if (--npred[E[e].to] == 0) stack.push_back(E[e].to);
+            }
+        };
+        static thread_local std::vector<int> start;
+        start.clear();
+        for (int j = 0; j < m; ++j)
+            if (npred[j] == 0) start.push_back(j);
+        for (int j : start) settle(j);
+        while (ndone < m && !B.overflow) {
+            bool progress = false;
+            for (size_t r = 0; r < ready.size();) {
+                const int j = ready[r];
+                if (!executable(taken[j], B.arr, local_of)) {
+                    ++r;
+                    continue;
+                }
+                ready.erase(ready.begin() + (long)r);
+                B.gate(taken[j]);
+                ++ndone;
+                progress = true;
+                for (int e = head[j]; e >= 0; e = E[e].next)
+                    if (--npred[E[e].to] == 0) settle(E[e].to);
+            }
+            if (ndone == m || progress) continue;
+            int best = -1, best_cnt = -1;
+            for (int a = 0; a < 3; ++a) {
+                if (a == B.arr) continue;
+                int cntr = 0;
+                for (int j : ready) cntr += executable(taken[j], a, local_of);
+                if (cntr > best_cnt) {
+                    best_cnt = cntr;
+                    best = a;
+                }
+            }
+            B.transpose_to(best);
+        }
+        const bool last = left.empty();
+        if (B.arr == ARR_LO) B.transpose_to(ARR_IO);   // stores take ARR_IO or ARR_HI
+        // Terms that no gate of this pass called for go to the front of what is left:
+        // they commute with everything taken after them, and with what was left behind
+        // before them.  (Their single-qubit parts are pending already.)
+        if (last || n_u2 == 0) B.finish_terms();
+        if (B.overflow) {
+            // too large for one launch: plan this pass again with fewer gates
+            if (max_u2 <= 1 && max_ph <= 1) {
+                *err = "internal: tile program overflow";
+                return QK_EINVAL;
+            }
+            max_u2 = std::max(1, max_u2 / 2);
+            max_ph = std::max(1, max_ph / 2);
+            continue;
+        }
+        P.fin_flip = 0;
+        for (int q = 0; q < kTileQubits; ++q) P.fin_flip |= B.flip[q] << q;
+        P.fin_fixed_mask = 0;
+        if (last) {   // everything pending, on the stored values
+            for (int q = 0; q < kTileQubits; ++q) {
+                cdm f = F1[(int)P.S[q]];
+                if (B.flip[q]) {
+                    lam1 *= f;
+                    f = 1.0 / f;
+                }
+                P.fin_turns[q] = angle_turns(std::arg(f));
+                P.fin_mag[q] = (float)std::abs(f);
+            }
+            for (int b = 0; b < P.nfix; ++b) {
+                const cdm f = F1[(int)P.fixed[b]];
+                P.fin_fixed[b] = angle_turns(std::arg(f));
+                P.fin_fixed_mag[b] = (float)std::abs(f);
+                if (P.fin_fixed[b] || P.fin_fixed_mag[b] != 1.f) P.fin_fixed_mask |= 1ull << b;
+            }
+            P.fin_turns[13] = angle_turns(std::arg(lam1));
+            P.fin_scale = (float)std::abs(lam1);
+        } else {
+            for (int q = 0; q < kTileQubits; ++q) {
+                P.fin_turns[q] = 0;
+                P.fin_mag[q] = 1.f;
+            }
+            P.fin_turns[13] = 0;
+            // the stored amplitudes are the true ones divided by lam: keep them within
+            // 2^24 of the true ones in FP32 (a factor in [2^-1/2, 2] per gate)
+            P.fin_scale = 1.f;
+            const double x = std::abs(lam1);
+            if (x < 0x1p-24 || x > 0x1p24) {
+                P.fin_scale = (float)x;
+                lam1 /= x;
+            }
+        }
+        // whether any phase factor the pass forms can be other than 1 or -1 (the kernel
+        // fills its phase table only then)
+        {
+            auto general = [](uint32_t t) { return t != 0u && t != kHalf; };
+            bool need = false;
+            for (int e = 0; e < P.nbt && !need; ++e) need = general(P.bt[e].turns);
+            for (int q = 0; q < 14; ++q) need = need || general(P.fin_turns[q]);
+            for (int b = 0; b < P.nfix; ++b)
+                if ((P.fin_fixed_mask >> b) & 1) need = need || general(P.fin_fixed[b]);
+            P.need_tab = need ? 1 : 0;
+        }
+        P.store_arr = B.arr;
+        next.clear();
+        B.hand_on(next, rewritten);
+        next.insert(next.end(), left.begin(), left.end());
+        if (planner->log) {
+            int cnt_k[9] = {0};  // by TileOpKind
+            for (int i = 0; i < P.nops; ++i) cnt_k[P.ops[i].kind]++;
+            std::fprintf(stderr,
+                         "[qk plan] pass S=%#llx gates=%d (u2 %d, phase %d) ops=%d u2=%d layers=%d layer_gates=%d "
+                         "phase_direct=%d phase_ops=%d terms=%d pairs=%d pair_signs=%d xpose=%d kept=%zu\n",
+                         (unsigned long long)S, m, n_u2, n_ph, P.nops, cnt_k[TOP_U2], cnt_k[TOP_U2L], P.nlg,
+                         cnt_k[TOP_PHASE], cnt_k[TOP_PHQ], P.nbt, cnt_k[TOP_PAIRU], cnt_k[TOP_PAIRNEG],
+                         cnt_k[TOP_XPOSE], B.terms.size());
+        }
+
+        const qk_status st = sink(P);
+        if (st != QK_OK) return st;
+        std::copy(F1, F1 + 64, F);
+        lam = lam1;
+        rem.swap(next);
+        max_u2 = 100;
+        max_ph = 300;
+    }
+    return QK_OK;
+}
 
 qk_status plan_smem_passes(TilePlanner *planner, int n, int prec, const std::vector<FusedOp> &ops,
                            const SmemPassSink &sink, const char **err) {
@@ -692,19 +1206,7 @@ qk_status plan_smem_passes(TilePlanner *planner, int n, int prec, const std::vec
             continue;
         }
         next.clear();
-        for (const DTerm &t : B.terms) {
-            if (t.src) {
-                next.push_back(classify(*t.src));
-                continue;
-            }
-            FusedOp o;
-            o.kind = FusedOp::PHASE;
-            o.mask = t.mask;
-            o.val = t.val;
-            o.f = t.f;
-            rewritten.push_back(o);
-            next.push_back(classify(rewritten.back()));
-        }
+        B.hand_on(next, rewritten);
         next.insert(next.end(), left.begin(), left.end());
         if (planner->log)
             std::fprintf(stderr, "[qk plan] c128 pass S=%#llx gates=%zu (u2 %d, phase %d) ops=%d factors=%d kept=%zu\n",
@@ -729,660 +1231,6 @@ qk_status plan_smem_passes(TilePlanner *planner, int n, int prec, const std::vec
 namespace {
 }  // namespace
 
-qk_status plan_passes(TilePlanner *planner, int n, const std::vector<FusedOp> &ops, const PassSink &sink,
-                      const char **err) {
-    *err = "";
-    std::vector<POp> rem;
-    rem.reserve(ops.size());
-    for (const auto &op : ops) rem.push_back(classify(op));
-
-    // take limits per pass; halved and retried when a program overflows the
-    // kernel-parameter budget (ops and grouped phase entries)
-    int max_u2 = 100, max_ph = 300;
-    std::vector<POp> left, taken;
-    // the uniform pending factors one pass leaves to the next (FP64): per physical
-    // qubit, on its |1> (a phase and a magnitude), plus a constant phase and a real
-    // scale; only the plan's last pass applies them to the amplitudes
-    double carry[64] = {0.0};
-    double carry_mag[64];
-    for (double &m : carry_mag) m = 1.0;
-    double carry_u0 = 0.0, carry_lam = 1.0;
-    std::vector<Cond> conds;
-    while (!rem.empty()) {
-        int n_u2 = 0, n_ph = 0;
-        const uint64_t S = choose_pass(rem, n, TakeLimits{kTileQubits, max_u2, max_ph}, kTileContig, conds, taken, left,
-                                       &n_u2, &n_ph);
-
-        static thread_local TileParams P;
-        std::memset(static_cast<TileHead *>(&P), 0, sizeof(TileHead));
-        P.n = n;
-        P.n_tiles = 1ull << (n - kTileQubits);
-        int local_of[64];
-        for (int b = 0; b < 64; ++b) local_of[b] = -1;
-        {
-            int lb = 0, fb = 0;
-            for (int b = 0; b < n; ++b) {
-                if ((S >> b) & 1) {
-                    P.S[lb] = (int8_t)b;
-                    local_of[b] = lb++;
-                } else {
-                    P.fixed[fb++] = (int8_t)b;
-                }
-            }
-            P.nfix = fb;
-            // runs of consecutive fixed qubits
-            P.nruns = 0;
-            for (int b = 0; b < fb;) {
-                int e = b + 1;
-                while (e < fb && P.fixed[e] == P.fixed[e - 1] + 1) ++e;
-                if (P.nruns >= kTileMaxRuns) {
-                    *err = "internal: too many fixed-qubit runs";
-                    return QK_EINVAL;
-                }
-                P.run_tlo[P.nruns] = (uint8_t)b;
-                P.run_len[P.nruns] = (uint8_t)(e - b);
-                P.run_plo[P.nruns] = (uint8_t)P.fixed[b];
-                ++P.nruns;
-                b = e;
-            }
-        }
-        P.n_conds = (int)conds.size();
-        for (int k = 0; k < P.n_conds; ++k) P.conds[k] = conds[k];
-
-        // ---- list-schedule the taken gates over the arrangements
-        const int m = (int)taken.size();
-        // dependency edges i -> j (i < j, not commuting) as flat successor lists:
-        // the successors of i are succ[succ_at[i] .. succ_at[i + 1])
-        static thread_local std::vector<int> npred, succ_at, succ, edge_i, edge_j;
-        npred.assign(m, 0);
-        succ_at.assign(m + 1, 0);
-        edge_i.clear();
-        edge_j.clear();
-        for (int j = 0; j < m; ++j)
-            for (int i = 0; i < j; ++i)
-                if (!commute(taken[i], taken[j])) {
-                    npred[j]++;
-                    succ_at[i + 1]++;
-                    edge_i.push_back(i);
-                    edge_j.push_back(j);
-                }
-        for (int i = 0; i < m; ++i) succ_at[i + 1] += succ_at[i];
-        succ.resize(edge_i.size());
-        {
-            static thread_local std::vector<int> fill;
-            fill.assign(succ_at.begin(), succ_at.end() - 1);
-            for (size_t e = 0; e < edge_i.size(); ++e) succ[fill[edge_i[e]]++] = edge_j[e];   // ascending j per i
-        }
-        std::vector<char> done(m, 0);
-        int ndone = 0, cur = ARR_IO, nops = 0;
-        static thread_local std::vector<TileOp> prog;
-        prog.assign(2 * (size_t)m + 2, TileOp{});
-        auto emit = [&](int j, int arr) {
-            const FusedOp &op = *taken[j].op;
-            TileOp &t = prog[nops++];
-            std::memset(&t, 0, sizeof t);
-            t.cond = 0xffff;
-            if (op.cond.n)
-                for (int k = 0; k < P.n_conds; ++k)
-                    if (same_cond(P.conds[k], op.cond)) t.cond = (uint16_t)k;
-            if (op.kind == FusedOp::U2) {
-                t.kind = TOP_U2;
-                int pos;
-                slot_of(arr, local_of[op.q], &pos);
-                t.k = (uint8_t)pos;
-                t.first = (uint16_t)j;   // the FP64 matrix: taken[j]
-                encode_cond(op.cmask, op.cmask, arr, local_of, t);
-                for (int e = 0; e < 4; ++e) {
-                    t.m[2 * e] = (float)op.m[e].real();
-                    t.m[2 * e + 1] = (float)op.m[e].imag();
-                }
-            } else {
-                t.kind = TOP_PHASE;
-                encode_cond(op.mask, op.val, arr, local_of, t);
-                t.ph.re = (float)op.f.real();
-                t.ph.im = (float)op.f.imag();
-                // the factor's angle as a fraction of a turn in 32-bit fixed point
-                double frac = std::arg(op.f) / (2.0 * M_PI);
-                if (frac < 0) frac += 1.0;
-                t.ph.turns = (uint32_t)(uint64_t)std::llround(frac * 4294967296.0);
-            }
-            done[j] = 1;
-            ++ndone;
-            for (int e = succ_at[j]; e < succ_at[j + 1]; ++e) npred[succ[e]]--;
-        };
-        while (ndone < m) {
-            bool progress = false;
-            for (int j = 0; j < m; ++j)
-                if (!done[j] && npred[j] == 0 && executable(taken[j], cur, local_of)) {
-                    emit(j, cur);
-                    progress = true;
-                }
-            if (ndone == m) break;
-            if (!progress) {
-                int best = -1, best_cnt = -1;
-                for (int a = 0; a < 3; ++a) {
-                    if (a == cur) continue;
-                    int cntr = 0;
-                    for (int j = 0; j < m; ++j)
-                        if (!done[j] && npred[j] == 0 && executable(taken[j], a, local_of)) ++cntr;
-                    if (cntr > best_cnt) {
-                        best_cnt = cntr;
-                        best = a;
-                    }
-                }
-                TileOp &t = prog[nops++];
-                std::memset(&t, 0, sizeof t);
-                t.kind = TOP_XPOSE;
-                t.k = (uint8_t)best;
-                t.cond = 0xffff;
-                cur = best;
-            }
-        }
-        if (cur == ARR_LO) {
-            TileOp &t = prog[nops++];
-            std::memset(&t, 0, sizeof t);
-            t.kind = TOP_XPOSE;
-            t.k = ARR_IO;
-            t.cond = 0xffff;
-            cur = ARR_IO;
-        }
-        // group runs of consecutive diagonal terms by the pending sum they feed
-        {
-            static thread_local TileOp out[2 * kTileMaxOps + 8];
-            int nout = 0, nlin = 0;
-            int fixed_index[64];   // physical qubit -> bit of the tile index
-            for (int b = 0; b < 64; ++b) fixed_index[b] = -1;
-            for (int b = 0; b < P.nfix; ++b) fixed_index[(int)P.fixed[b]] = b;
-            bool overflow = false;
-            for (int i = 0; i < nops && !overflow;) {
-                if (nout >= 2 * kTileMaxOps) {
-                    overflow = true;
-                    break;
-                }
-                if (prog[i].kind != TOP_PHASE) {
-                    out[nout++] = prog[i++];
-                    continue;
-                }
-                int j = i;
-                while (j < nops && prog[j].kind == TOP_PHASE) ++j;
-                // per pending sum (register bit 0..4, constant 5): entries that add turns
-                struct Term {
-                    uint16_t tmask, tval;
-                    uint32_t turns;
-                    uint64_t gmask, gval;
-                };
-                std::vector<Term> grp[6];
-                // terms on two register bits, reduced to the (1,1) pattern: key -> turns
-                struct PairKey {
-                    int code;
-                    uint16_t tmask, tval;
-                    uint64_t gmask, gval;
-                    uint32_t turns;
-                };
-                std::vector<PairKey> pairs;
-                auto add_entry = [&](int g, const TileOp &o, uint32_t turns) {
-                    Term e;
-                    e.tmask = o.tmask;
-                    e.tval = o.tval;
-                    e.gmask = o.gmask;
-                    e.gval = o.gval;
-                    e.turns = turns;
-                    grp[g].push_back(e);
-                };
-                for (int t = i; t < j; ++t) {
-                    const TileOp &o = prog[t];
-                    if (nout >= 2 * kTileMaxOps) {
-                        overflow = true;
-                        break;
-                    }
-                    const int pc = __builtin_popcount(o.rmask);
-                    const uint32_t T = o.ph.turns;
-                    if (o.cond != 0xffff || pc >= 3) {
-                        out[nout++] = o;   // applied directly
-                        continue;
-                    }
-                    if (pc == 0) {
-                        add_entry(5, o, T);
-                    } else if (pc == 1) {
-                        const int k = __builtin_ctz(o.rmask);
-                        if (o.rval) {
-                            add_entry(k, o, T);
-                        } else {  // f on bit k = 0:  f * (f^-1 on bit k = 1)
-                            add_entry(5, o, T);
-                            add_entry(k, o, 0u - T);
-                        }
-                    } else {
-                        // pattern (vk, vl) on register bits k < l as exact sums of a constant,
-                        // single-bit terms and a (1,1) pair term
-                        const int k = __builtin_ctz(o.rmask), l = 31 - __builtin_clz(o.rmask);
-                        const int vk = (o.rval >> k) & 1, vl = (o.rval >> l) & 1;
-                        uint32_t pair = T;
-                        if (vk && !vl) {
-                            add_entry(k, o, T);
-                            pair = 0u - T;
-                        } else if (!vk && vl) {
-                            add_entry(l, o, T);
-                            pair = 0u - T;
-                        } else if (!vk && !vl) {
-                            add_entry(5, o, T);
-                            add_entry(k, o, 0u - T);
-                            add_entry(l, o, 0u - T);
-                        }
-                        const int code = k | (l << 3);
-                        bool merged = false;
-                        for (auto &pk : pairs)
-                            if (pk.code == code && pk.tmask == o.tmask && pk.tval == o.tval && pk.gmask == o.gmask &&
-                                pk.gval == o.gval) {
-                                pk.turns += pair;
-                                merged = true;
-                                break;
-                            }
-                        if (!merged) pairs.push_back({code, o.tmask, o.tval, o.gmask, o.gval, pair});
-                    }
-                }
-                for (const auto &pk : pairs) {
-                    if (pk.turns == 0) continue;
-                    if (nout >= 2 * kTileMaxOps) {
-                        overflow = true;
-                        break;
-                    }
-                    TileOp &t = out[nout++];
-                    std::memset(&t, 0, sizeof t);
-                    t.cond = 0xffff;
-                    t.k = (uint8_t)pk.code;
-                    if (pk.tmask == 0 && pk.gmask == 0 && pk.turns == 0x80000000u) {
-                        t.kind = TOP_PAIRNEG;   // a CZ between two register bits
-                        continue;
-                    }
-                    t.kind = TOP_PAIR;
-                    t.rval = 3;   // both bits 1
-                    t.tmask = pk.tmask;
-                    t.tval = pk.tval;
-                    t.gmask = pk.gmask;
-                    t.gval = pk.gval;
-                    const double ang = 2.0 * M_PI * (double)pk.turns / 4294967296.0;
-                    t.ph.re = (float)std::cos(ang);
-                    t.ph.im = (float)std::sin(ang);
-                    t.ph.turns = pk.turns;
-                }
-                for (int g = 0; g < 6 && !overflow; ++g) {
-                    if (grp[g].empty()) continue;
-                    // split the group's terms: the same for every thread and tile
-                    // (kept by the planner), and the rest, each a linear term with
-                    // its thread-bit and tile-index conditions (TOP_PHASEL)
-                    uint32_t host_turns = 0;
-                    std::vector<LinTerm> lins;
-                    for (const Term &t : grp[g]) {
-                        if (t.gmask == 0 && t.tmask == 0) {
-                            host_turns += t.turns;
-                            continue;
-                        }
-                        uint32_t fm = 0, fv = 0;   // the fixed-qubit condition on tile-index bits
-                        for (uint64_t mk = t.gmask; mk; mk &= mk - 1) {
-                            const int pb = __builtin_ctzll(mk), tb = fixed_index[pb];
-                            fm |= 1u << tb;
-                            if ((t.gval >> pb) & 1) fv |= 1u << tb;
-                        }
-                        bool merged = false;
-                        for (auto &l : lins)
-                            if (l.tmask == t.tmask && l.tval == t.tval && l.fmask == fm && l.fval == fv) {
-                                l.turns += t.turns;
-                                merged = true;
-                                break;
-                            }
-                        if (!merged) {
-                            LinTerm l{};
-                            l.tmask = t.tmask;
-                            l.tval = t.tval;
-                            l.fmask = fm;
-                            l.fval = fv;
-                            l.turns = t.turns;
-                            lins.push_back(l);
-                        }
-                    }
-                    if (host_turns != 0) {
-                        if (nout >= 2 * kTileMaxOps) { overflow = true; break; }
-                        TileOp &t = out[nout++];
-                        std::memset(&t, 0, sizeof t);
-                        t.kind = TOP_HOSTPH;
-                        t.k = (uint8_t)g;
-                        t.cond = 0xffff;
-                        t.ph.turns = host_turns;
-                    }
-                    int nl = 0;
-                    for (const auto &l : lins) nl += l.turns != 0;
-                    if (nl) {
-                        if (nout >= 2 * kTileMaxOps || nlin + nl > kTileMaxLin) { overflow = true; break; }
-                        TileOp &t = out[nout++];
-                        std::memset(&t, 0, sizeof t);
-                        t.kind = TOP_PHASEL;
-                        t.k = (uint8_t)g;
-                        t.cond = 0xffff;
-                        t.first = (uint16_t)nlin;
-                        for (const auto &l : lins)
-                            if (l.turns != 0) P.lin[nlin++] = l;
-                        t.count = (uint16_t)(nlin - t.first);
-                    }
-                }
-                i = j;
-            }
-            if (overflow || nout > kTileMaxOps) {
-                // too large for one launch: plan this pass again with fewer gates
-                if (max_u2 <= 1 && max_ph <= 1) {
-                    *err = "internal: tile program overflow";
-                    return QK_EINVAL;
-                }
-                max_u2 = std::max(1, max_u2 / 2);
-                max_ph = std::max(1, max_ph / 2);
-                continue;
-            }
-            // merge runs of consecutive uncontrolled 2x2 gates on distinct
-            // register bits into layer ops (they commute with each other)
-            int nfin = 0, nmat = 0;
-            static thread_local uint16_t lg_mat[kTileMaxMats];   // layer gate -> taken[] index
-            for (int i = 0; i < nout && !overflow;) {
-                const TileOp &o = out[i];
-                const bool plain_u2 = o.kind == TOP_U2 && o.rmask == 0 && o.tmask == 0 && o.gmask == 0 &&
-                                      o.cond == 0xffff;
-                if (!plain_u2) {
-                    if (nfin >= kTileMaxOps) { overflow = true; break; }
-                    P.ops[nfin++] = out[i++];
-                    continue;
-                }
-                int bits = 0, j = i;
-                while (j < nout) {
-                    const TileOp &q = out[j];
-                    const bool ok = q.kind == TOP_U2 && q.rmask == 0 && q.tmask == 0 && q.gmask == 0 &&
-                                    q.cond == 0xffff && !(bits & (1 << q.k));
-                    if (!ok) break;
-                    bits |= 1 << q.k;
-                    ++j;
-                }
-                if (nfin >= kTileMaxOps || nmat + (j - i) > kTileMaxMats) { overflow = true; break; }
-                TileOp &t = P.ops[nfin++];
-                std::memset(&t, 0, sizeof t);
-                t.kind = TOP_U2L;
-                t.k = (uint8_t)bits;
-                t.cond = 0xffff;
-                t.first = (uint16_t)nmat;
-                t.count = (uint16_t)(j - i);
-                // the gates' FP64 matrices in register-bit order; fold_program turns
-                // them into pivot coefficients
-                for (int b = 0; b < 5; ++b)
-                    for (int q = i; q < j; ++q)
-                        if (out[q].k == b) lg_mat[nmat++] = out[q].first;
-                i = j;
-            }
-            if (overflow) {
-                if (max_u2 <= 1 && max_ph <= 1) {
-                    *err = "internal: tile program overflow";
-                    return QK_EINVAL;
-                }
-                max_u2 = std::max(1, max_u2 / 2);
-                max_ph = std::max(1, max_ph / 2);
-                continue;
-            }
-            // fold_program: walk the program in order, keeping the pending phases
-            // that are the same for every thread (and the scale and the stored bit
-            // order of each local qubit) in FP64; layer gates get their pivot
-            // coefficients, every other op's conditions are rewritten to the stored
-            // order, general gates take their target's uniform phase along to the
-            // device, and what is left goes to the final flush
-            {
-                UniformPending st;
-                for (int q = 0; q < kTileQubits; ++q) {
-                    st.u[q] = carry[(int)P.S[q]];
-                    st.mag[q] = carry_mag[(int)P.S[q]];
-                }
-                st.u0 = carry_u0;
-                st.lam = carry_lam;
-                int arr = ARR_IO, w = 0;
-                const double pi = M_PI;
-                for (int i = 0; i < nfin; ++i) {
-                    TileOp o = P.ops[i];
-                    // flipped register and thread bits in the current arrangement
-                    int rflip = 0, tflip = 0;
-                    for (int k = 0; k < 5; ++k) rflip |= st.flip[local_of_reg(arr, k)] << k;
-                    for (int t = 0; t < 8; ++t) tflip |= st.flip[local_of_tbit(arr, t)] << t;
-                    auto qk_of = [&](int k) { return local_of_reg(arr, k); };
-                    switch (o.kind) {
-                        case TOP_HOSTPH: {
-                            const double ang = turns_angle(o.ph.turns);
-                            if (o.k == 5) {
-                                st.u0 += ang;
-                            } else if (st.flip[qk_of(o.k)]) {  // on the stored |0>
-                                st.u0 += ang;
-                                st.u[qk_of(o.k)] -= ang;
-                            } else {
-                                st.u[qk_of(o.k)] += ang;
-                            }
-                            continue;   // never reaches the device
-                        }
-                        case TOP_XPOSE:
-                            arr = o.k;
-                            break;
-                        case TOP_U2L: {
-                            int idx = o.first;
-                            for (int b = 0; b < 5; ++b) {
-                                if (!((o.k >> b) & 1)) continue;
-                                const FusedOp &fo = *taken[lg_mat[idx]].op;
-                                const Mat2 g{{fo.m[0], fo.m[1], fo.m[2], fo.m[3]}};
-                                if (pivot_gate(g, st, qk_of(b), P.lg[idx])) o.rmask |= (uint8_t)(1u << b);
-                                ++idx;
-                            }
-                            break;
-                        }
-                        case TOP_PAIRNEG: {
-                            // (-1)^((a^fa)(b^fb)) = (-1)^(ab) (-1)^(fb a) (-1)^(fa b) (-1)^(fa fb)
-                            const int ka = o.k & 7, kb = o.k >> 3;
-                            const int fa = (rflip >> ka) & 1, fb = (rflip >> kb) & 1;
-                            if (fb) st.u[qk_of(ka)] += pi;
-                            if (fa) st.u[qk_of(kb)] += pi;
-                            if (fa && fb) st.u0 += pi;
-                            break;
-                        }
-                        case TOP_PAIR: {
-                            const int ka = o.k & 7, kb = o.k >> 3;
-                            const int fa = (rflip >> ka) & 1, fb = (rflip >> kb) & 1;
-                            o.tval ^= (uint16_t)(o.tmask & tflip);
-                            if (o.tmask == 0 && o.gmask == 0 && o.cond == 0xffff) {
-                                // e^{i th} where the true bits a = sa ^ fa, b = sb ^ fb are both
-                                // 1, in stored bits: (sa ^ fa)(sb ^ fb) = fa fb + fa (1 - 2 fb) sb
-                                // + fb (1 - 2 fa) sa + (1 - 2 fa)(1 - 2 fb) sa sb.  The stored
-                                // pattern (1, 1) takes +-th on the device; the constant and the
-                                // single-bit parts are uniform phases kept here.
-                                const double th = turns_angle(o.ph.turns);
-                                if (fa && fb) st.u0 += th;
-                                if (fa) st.u[qk_of(kb)] += fb ? -th : th;
-                                if (fb) st.u[qk_of(ka)] += fa ? -th : th;
-                                if (fa ^ fb) {
-                                    o.ph.turns = 0u - o.ph.turns;
-                                    o.ph.im = -o.ph.im;
-                                }
-                                o.rval = 3;
-                                o.kind = TOP_PAIRU;
-                            } else {
-                                o.rval = (uint8_t)(3 ^ (fa | (fb << 1)));
-                            }
-                            break;
-                        }
-                        case TOP_PHASEL: {
-                            for (int e = o.first; e < o.first + o.count; ++e)
-                                P.lin[e].tval ^= (uint16_t)(P.lin[e].tmask & tflip);
-                            o.rval = (uint8_t)(o.k < 5 ? (rflip >> o.k) & 1 : 0);
-                            // every term tests one bit: "turns where the bit is 1" terms
-                            // (TOP_PHASEB), a term on a bit being 0 split into a
-                            // constant kept here and a negated bit-1 term
-                            bool single = true;
-                            for (int e = o.first; e < o.first + o.count; ++e)
-                                single = single && __builtin_popcount(P.lin[e].tmask) + __builtin_popcount(P.lin[e].fmask) == 1;
-                            if (!single) break;
-                            std::vector<BitTerm> th, ti;
-                            uint32_t cst = 0;
-                            for (int e = o.first; e < o.first + o.count; ++e) {
-                                const LinTerm &L = P.lin[e];
-                                const bool thread = L.tmask != 0;
-                                const uint32_t b = thread ? (uint32_t)__builtin_ctz(L.tmask) : (uint32_t)__builtin_ctz(L.fmask);
-                                const uint32_t v = thread ? ((uint32_t)L.tval >> b) & 1u : (L.fval >> b) & 1u;
-                                uint32_t t = L.turns;
-                                if (!v) {
-                                    cst += t;
-                                    t = 0u - t;
-                                }
-                                (thread ? th : ti).push_back(BitTerm{b, t});
-                            }
-                            BitTerm *bt = reinterpret_cast<BitTerm *>(&P.lin[o.first]);
-                            for (size_t q = 0; q < th.size(); ++q) bt[q] = th[q];
-                            for (size_t q = 0; q < ti.size(); ++q) bt[th.size() + q] = ti[q];
-                            o.kind = TOP_PHASEB;
-                            o.first = (uint16_t)(2 * o.first);
-                            o.count = (uint16_t)th.size();
-                            o.count2 = (uint16_t)ti.size();
-                            if (cst) {   // the same for every thread and tile: kept here
-                                const double ang = turns_angle(cst);
-                                if (o.k == 5) {
-                                    st.u0 += ang;
-                                } else if (st.flip[qk_of(o.k)]) {
-                                    st.u0 += ang;
-                                    st.u[qk_of(o.k)] -= ang;
-                                } else {
-                                    st.u[qk_of(o.k)] += ang;
-                                }
-                            }
-                            break;
-                        }
-                        case TOP_PHASE:
-                            o.rval ^= (uint8_t)(o.rmask & rflip);
-                            o.tval ^= (uint16_t)(o.tmask & tflip);
-                            break;
-                        case TOP_U2: {
-                            const int q = qk_of(o.k);
-                            o.rval ^= (uint8_t)(o.rmask & rflip);
-                            o.tval ^= (uint16_t)(o.tmask & tflip);
-                            if (st.flip[q]) {  // X U X in stored order
-                                float t[8];
-                                std::memcpy(t, o.m, sizeof t);
-                                const int perm[4] = {3, 2, 1, 0};
-                                for (int e = 0; e < 4; ++e) {
-                                    o.m[2 * e] = t[2 * perm[e]];
-                                    o.m[2 * e + 1] = t[2 * perm[e] + 1];
-                                }
-                            }
-                            o.hturns = angle_turns(st.u[q]);
-                            o.hmag = (float)st.mag[q];
-                            st.u[q] = 0.0;
-                            st.mag[q] = 1.0;
-                            break;
-                        }
-                        default:
-                            break;
-                    }
-                    P.ops[w++] = o;
-                }
-                nfin = w;
-                // a CZ between register bits right after a layer op (nothing between
-                // them) becomes a bit of that op's CZ mask: one dispatch fewer
-                w = 0;
-                for (int i = 0; i < nfin; ++i) {
-                    const TileOp &o = P.ops[i];
-                    if (o.kind == TOP_PAIRNEG && w > 0 && P.ops[w - 1].kind == TOP_U2L) {
-                        P.ops[w - 1].tmask |= (uint16_t)(1u << cz_index(o.k & 7, o.k >> 3));
-                        continue;
-                    }
-                    P.ops[w++] = o;
-                }
-                nfin = w;
-                P.fin_flip = 0;
-                for (int q = 0; q < kTileQubits; ++q) P.fin_flip |= st.flip[q] << q;
-                P.fin_fixed_mask = 0;
-                if (left.empty()) {   // the plan's last pass applies everything pending
-                    for (int q = 0; q < kTileQubits; ++q) {
-                        P.fin_turns[q] = angle_turns(st.u[q]);
-                        P.fin_mag[q] = (float)st.mag[q];
-                    }
-                    P.fin_turns[13] = angle_turns(st.u0);
-                    P.fin_scale = (float)st.lam;
-                    for (int b = 0; b < P.nfix; ++b) {
-                        const uint32_t t = angle_turns(carry[(int)P.fixed[b]]);
-                        P.fin_fixed[b] = t;
-                        P.fin_fixed_mag[b] = (float)carry_mag[(int)P.fixed[b]];
-                        if (t || P.fin_fixed_mag[b] != 1.f) P.fin_fixed_mask |= 1ull << b;
-                    }
-                } else {              // hand the uniform part to the next pass
-                    for (int q = 0; q < kTileQubits; ++q) {
-                        // a qubit stored flipped has its factor F on |0>: F on |0> is F
-                        // overall times 1 / F on |1>
-                        const int pq = (int)P.S[q];
-                        if (st.flip[q]) {
-                            carry[pq] = -st.u[q];
-                            carry_mag[pq] = 1.0 / st.mag[q];
-                            st.u0 += st.u[q];
-                            st.lam *= st.mag[q];
-                        } else {
-                            carry[pq] = st.u[q];
-                            carry_mag[pq] = st.mag[q];
-                        }
-                        P.fin_turns[q] = 0;
-                        P.fin_mag[q] = 1.f;
-                    }
-                    carry_u0 = st.u0;
-                    P.fin_turns[13] = 0;
-                    // the stored amplitudes are the true ones divided by the scale
-                    // (a factor in [2^-1/2, 2] per gate): keep them within 2^24 of it
-                    // in FP32
-                    if (st.lam < 0x1p-24 || st.lam > 0x1p24) {
-                        P.fin_scale = (float)st.lam;
-                        carry_lam = 1.0;
-                    } else {
-                        P.fin_scale = 1.f;
-                        carry_lam = st.lam;
-                    }
-                }
-            }
-            nops = nfin;
-            P.nlg = nmat;
-            P.nlin = nlin;
-            // whether any phase factor the pass forms can be other than 1 or -1 (the
-            // kernel fills its phase table only then)
-            {
-                auto general = [](uint32_t t) { return t != 0u && t != 0x80000000u; };
-                bool need = false;
-                for (int i = 0; i < nops && !need; ++i) {
-                    const TileOp &o = P.ops[i];
-                    if (o.kind == TOP_U2 || o.kind == TOP_PHASE) need = true;
-                    if (o.kind == TOP_PHASEL)
-                        for (int e = o.first; e < o.first + o.count; ++e) need = need || general(P.lin[e].turns);
-                    if (o.kind == TOP_PHASEB) {
-                        const BitTerm *bt = reinterpret_cast<const BitTerm *>(&P.lin[0]) + o.first;
-                        for (int e = 0; e < o.count + o.count2; ++e) need = need || general(bt[e].turns);
-                    }
-                }
-                for (int q = 0; q < 14; ++q) need = need || general(P.fin_turns[q]);
-                for (int b = 0; b < P.nfix; ++b)
-                    if ((P.fin_fixed_mask >> b) & 1) need = need || general(P.fin_fixed[b]);
-                P.need_tab = need ? 1 : 0;
-            }
-        }
-        P.nops = nops;
-        P.store_arr = cur;
-        if (planner->log) {
-            int cnt_k[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // by TileOpKind
-            for (int i = 0; i < nops; ++i) cnt_k[P.ops[i].kind]++;
-            std::fprintf(stderr,
-                         "[qk plan] pass S=%#llx gates=%d (u2 %d, phase %d) ops=%d u2=%d layers=%d phase_direct=%d "
-                         "phase_groups=%d terms=%d pairs=%d pair_signs=%d xpose=%d store_arr=%d\n",
-                         (unsigned long long)S, m, n_u2, n_ph, nops, cnt_k[TOP_U2], cnt_k[TOP_U2L], cnt_k[TOP_PHASE],
-                         cnt_k[TOP_PHASEL], P.nlin, cnt_k[TOP_PAIR], cnt_k[TOP_PAIRNEG], cnt_k[TOP_XPOSE], cur);
-        }
-
-        const qk_status st = sink(P);
-        if (st != QK_OK) return st;
-        rem.swap(left);
-        max_u2 = 100;
-        max_ph = 300;
-    }
-    return QK_OK;
-}
 
 // A dense pass: S starts as the lowest qubits (runs of 128 bytes in HBM, 32 for states in
 // L2) and takes the targets of every gate, in order, that commutes with the gates left
