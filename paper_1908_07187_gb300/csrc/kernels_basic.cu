@@ -120,37 +120,21 @@ __global__ void __launch_bounds__(kThreads) k_u2(typename Amp<R>::T *psi, U2Args
 // the mask (two adjacent amplitudes per unit, one 16-byte vector).
 // With n_rphase > 0 the factor is exp(-2 pi i sum_l c_l / 2^(l+1)) from cbits.
 // ---------------------------------------------------------------------------
-template <typename R>
-__device__ __forceinline__ typename Amp<R>::T phase_factor(const PhaseArgs &a, const uint8_t *cbits) {
-    typename Amp<R>::T f;
-    if (a.n_rphase == 0) {
-        f.x = (R)a.f_re;
-        f.y = (R)a.f_im;
-        return f;
-    }
-    // fraction of a turn in 64-bit fixed point: sum_l c_l 2^-(l+1), l = 1..e
-    uint64_t turns = 0;
-    for (int l = 1; l <= a.n_rphase; ++l)
-        if (cbits[a.rphase_idx[l - 1]]) turns += 1ull << (63 - l);
-    const double frac = (double)turns * 0x1p-64;  // in [0, 1/2)
-    double s, c;
-    sincospi(-2.0 * frac, &s, &c);
-    f.x = (R)c;
-    f.y = (R)s;
-    return f;
-}
-
 template <typename R, int V>
 __global__ void __launch_bounds__(kThreads) k_phase(typename Amp<R>::T *psi, PhaseArgs a, const uint8_t *cbits) {
     using T = typename Amp<R>::T;
     if (a.cond.n && !cond_ok(a.cond, cbits)) return;
     // an angle from cbits is formed in FP64 once per block (GB300's FP64 rate is low)
-    __shared__ T s_f;
-    if (a.n_rphase) {
-        if (threadIdx.x == 0) s_f = phase_factor<R>(a, cbits);
-        __syncthreads();
+    __shared__ double2 s_om;
+    if (threadIdx.x < 32) {
+        double2 om = make_double2(a.f_re, a.f_im);
+        if (a.n_rphase) om = warp_rphase(a.rphase_idx, a.n_rphase, cbits);
+        if (threadIdx.x == 0) s_om = om;
     }
-    const T f = a.n_rphase ? s_f : phase_factor<R>(a, cbits);
+    __syncthreads();
+    T f;
+    f.x = (R)s_om.x;
+    f.y = (R)s_om.y;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < a.n_units; u += stride) {
         if constexpr (V == 1) {

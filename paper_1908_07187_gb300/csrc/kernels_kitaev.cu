@@ -61,21 +61,14 @@ __device__ __forceinline__ uint64_t source_index(uint64_t i, const KitaevArgs &a
     return src;
 }
 
-// exp(i theta), theta = -2 pi sum_l c_l / 2^(l+1) from the listed cbits (64-bit fixed point)
-__device__ __forceinline__ double2 rphase(const KitaevArgs &a, const uint8_t *cbits) {
-    uint64_t turns = 0;
-    for (int l = 1; l <= a.n_rphase; ++l)
-        if (cbits[a.rphase_idx[l - 1]]) turns += 1ull << (63 - l);
-    double s, c;
-    sincospi(-2.0 * ((double)turns * 0x1p-64), &s, &c);
-    return make_double2(c, s);
-}
-
-// the stage's phase factor, formed in FP64 by one thread per block (GB300's FP64
-// rate is low) and shared
+// the stage's phase factor, formed in FP64 by one warp per block (GB300's FP64 rate is
+// low) and shared
 __device__ __forceinline__ double2 block_rphase(const KitaevArgs &a, const uint8_t *cbits) {
     __shared__ double2 s_om;
-    if (threadIdx.x == 0) s_om = rphase(a, cbits);
+    if (threadIdx.x < 32) {
+        const double2 om = warp_rphase(a.rphase_idx, a.n_rphase, cbits);
+        if (threadIdx.x == 0) s_om = om;
+    }
     __syncthreads();
     return s_om;
 }
@@ -148,6 +141,167 @@ __global__ void __launch_bounds__(kThreads) k_kitaev_update(const typename Amp<R
     }
 }
 
+// The whole stage in one launch for states whose c = 0 half fits the register files:
+// each thread loads its amplitudes w and the gathered partners v once, the grid forms
+// the sums, the last block to arrive decides (partials added in a fixed order), and
+// after a grid barrier every thread updates its amplitudes from registers.  The two
+// kernels above read and gather everything twice and form the phase (FP64, about 2 us
+// of one thread's latency) in front of their loads; here the loads are in flight
+// meanwhile.  A cooperative launch, so all blocks are resident; the barrier's wait has a
+// limit, after which the error flag that qk_sync reports is set and the block returns.
+// KITAEV_FIGURES
+constexpr int kStageThreads = 512;
+constexpr int kStageBlocksPerSM = 2;
+constexpr int kStageWaitLimit = 1 << 22;   // polls of about 0.5 us: seconds
+
+__device__ __forceinline__ void fsum_merge(FSum &a, float hi, float lo) {
+    const float s = a.hi + hi;
+    const float bp = s - a.hi;
+    a.lo += lo + ((a.hi - (s - bp)) + (hi - bp));
+    a.hi = s;
+}
+
+template <typename R, int A>
+__global__ void __launch_bounds__(kStageThreads, kStageBlocksPerSM)
+    k_kitaev_stage(const typename Amp<R>::T *__restrict__ psi, typename Amp<R>::T *__restrict__ out,
+                   const __grid_constant__ KitaevArgs a, const uint8_t *cbits, double *partials, unsigned *bar, Decide dec,
+                   int *err) {
+    using T = typename Amp<R>::T;
+    __shared__ double2 s_om;
+    __shared__ double s_part[2][kStageThreads / 32];
+    __shared__ unsigned s_gen, s_last;
+    __shared__ R s_f[3];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint64_t step = (uint64_t)gridDim.x * kStageThreads, j0 = (uint64_t)blockIdx.x * kStageThreads + tid;
+    T w[A], v[A];
+#pragma unroll
+    for (int k = 0; k < A; ++k) {
+        const uint64_t j = j0 + k * step;
+        w[k].x = w[k].y = v[k].x = v[k].y = 0;
+        if (j < a.n_half) {
+            const uint64_t i = insert_zero(j, a.cpos);
+            w[k] = psi[i];
+            v[k] = psi[source_index(i, a)];
+        }
+    }
+    if (warp == 0) {
+        const double2 om = warp_rphase(a.rphase_idx, a.n_rphase, cbits);
+        if (lane == 0) s_om = om;
+    }
+    if (tid == 0) {
+        s_gen = *(volatile unsigned *)(bar + 1);   // the barrier's generation, before this block arrives
+    }
+    __syncthreads();
+    const R wr = (R)s_om.x, wi = (R)s_om.y;
+    FSum g0, g1;
+    double d0 = 0.0, d1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < A; ++k) {
+        const R tr = wr * v[k].x - wi * v[k].y, ti = wr * v[k].y + wi * v[k].x;
+        const R pr = w[k].x + tr, pi = w[k].y + ti, mr = w[k].x - tr, mi = w[k].y - ti;
+        v[k].x = tr;
+        v[k].y = ti;
+        if constexpr (sizeof(R) == 4) {
+            g0.add(pr * pr + pi * pi);
+            g1.add(mr * mr + mi * mi);
+        } else {
+            d0 += pr * pr + pi * pi;
+            d1 += mr * mr + mi * mi;
+        }
+    }
+    if constexpr (sizeof(R) == 4) {
+        // the warp's sums stay float pairs: an FP64 add per thread and step would cost more
+        for (int o = 16; o > 0; o >>= 1) {
+            fsum_merge(g0, __shfl_down_sync(0xffffffffu, g0.hi, o), __shfl_down_sync(0xffffffffu, g0.lo, o));
+            fsum_merge(g1, __shfl_down_sync(0xffffffffu, g1.hi, o), __shfl_down_sync(0xffffffffu, g1.lo, o));
+        }
+        if (lane == 0) {
+            d0 = g0.value();
+            d1 = g1.value();
+        }
+    } else {
+        for (int o = 16; o > 0; o >>= 1) {
+            d0 += __shfl_down_sync(0xffffffffu, d0, o);
+            d1 += __shfl_down_sync(0xffffffffu, d1, o);
+        }
+    }
+    if (lane == 0) {
+        s_part[0][warp] = d0;
+        s_part[1][warp] = d1;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        double s0 = lane < kStageThreads / 32 ? s_part[0][lane] : 0.0;
+        double s1 = lane < kStageThreads / 32 ? s_part[1][lane] : 0.0;
+        for (int o = kStageThreads / 64; o > 0; o >>= 1) {
+            s0 += __shfl_down_sync(0xffffffffu, s0, o);
+            s1 += __shfl_down_sync(0xffffffffu, s1, o);
+        }
+        if (lane == 0) {
+            partials[2 * blockIdx.x] = s0;
+            partials[2 * blockIdx.x + 1] = s1;
+            __threadfence();                       // the partials before the ticket
+            s_last = atomicAdd(bar, 1u) == gridDim.x - 1 ? 1u : 0u;
+        }
+        __syncwarp();
+        if (s_last) {
+            __threadfence();
+            double t0 = 0.0, t1 = 0.0;
+            for (int b = lane; b < (int)gridDim.x; b += 32) {
+                t0 += __ldcg(&partials[2 * b]);
+                t1 += __ldcg(&partials[2 * b + 1]);
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                t0 += __shfl_down_sync(0xffffffffu, t0, o);
+                t1 += __shfl_down_sync(0xffffffffu, t1, o);
+            }
+            if (lane == 0) {
+                const double tot = t0 + t1, p0 = tot > 0.0 ? t0 / tot : 1.0;
+                const int m = dec.u >= p0 ? 1 : 0;
+                const double pm = m ? t1 : t0;
+                volatile MeasSlot *sl = dec.slot;
+                sl->p0 = p0;
+                sl->m = m;
+                sl->scale = pm > 0.0 ? 1.0 / sqrt(pm) : 0.0;
+                if (dec.dest >= 0) dec.cbits[dec.dest] = (uint8_t)m;
+                *bar = 0;
+                __threadfence();                   // the decision before the next generation
+                atomicAdd(bar + 1, 1u);
+            }
+        } else if (lane == 0) {
+            int polls = 0;
+            while (*(volatile unsigned *)(bar + 1) == s_gen && ++polls < kStageWaitLimit) __nanosleep(64);
+            if (polls >= kStageWaitLimit) s_last = 2u;
+            __threadfence();
+        }
+        __syncwarp();
+        if (lane == 0 && s_last != 2u) {
+            const volatile MeasSlot *sl = dec.slot;
+            s_f[0] = (R)sl->scale;
+            s_f[1] = sl->m ? (R)-1 : (R)1;
+        }
+    }
+    __syncthreads();
+    if (s_last == 2u) {                            // the wait ran out: nothing is written
+        if (tid == 0) *err = 1;
+        return;
+    }
+    const R sc = s_f[0], sg = s_f[1];
+#pragma unroll
+    for (int k = 0; k < A; ++k) {
+        const uint64_t j = j0 + k * step;
+        if (j >= a.n_half) continue;
+        const uint64_t i = insert_zero(j, a.cpos);
+        T o, z;
+        o.x = (w[k].x + sg * v[k].x) * sc;
+        o.y = (w[k].y + sg * v[k].y) * sc;
+        z.x = 0;
+        z.y = 0;
+        out[i] = o;                                // control back at |0>
+        out[i | (1ull << a.cpos)] = z;
+    }
+}
+
 inline unsigned grid_for(uint64_t units, int sms) {
     uint64_t b = (units + kThreads - 1) / kThreads;
     const uint64_t cap = (uint64_t)sms * 16;
@@ -176,6 +330,50 @@ cudaError_t launch_kitaev_update(int prec, const void *psi, void *out, const Kit
         k_kitaev_update<double><<<grid_for(a.n_half, sms), kThreads, 0, s>>>((const double2 *)psi, (double2 *)out,
                                                                              a, cbits, slot);
     return cudaGetLastError();
+}
+
+// amplitudes per thread that the registers hold
+static int stage_max_amps(int prec) { return prec == 0 ? 8 : 4; }
+
+bool kitaev_stage_fits(int prec, uint64_t n_half, int sms) {
+    return n_half <= (uint64_t)sms * kStageBlocksPerSM * kStageThreads * stage_max_amps(prec);
+}
+
+template <typename R, int A>
+static cudaError_t stage_launch(const void *psi, void *out, const KitaevArgs &a, const uint8_t *cbits, double *partials,
+                                unsigned *bar, const Decide &d, int *err, unsigned grid, cudaStream_t s) {
+    using T = typename Amp<R>::T;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kStageThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeCooperative;
+    at.val.cooperative = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_kitaev_stage<R, A>, (const T *)psi, (T *)out, a, cbits, partials, bar, d, err);
+}
+
+template <typename R>
+static cudaError_t stage_r(const void *psi, void *out, const KitaevArgs &a, const uint8_t *cbits, double *partials,
+                           unsigned *bar, const Decide &d, int *err, int sms, cudaStream_t s) {
+    const uint64_t cap = (uint64_t)sms * kStageBlocksPerSM;
+    const uint64_t want = (a.n_half + kStageThreads - 1) / kStageThreads;
+    const unsigned grid = (unsigned)(want < cap ? want : cap);
+    const uint64_t per = (want + grid - 1) / grid;
+    if (per <= 1) return stage_launch<R, 1>(psi, out, a, cbits, partials, bar, d, err, grid, s);
+    if (per <= 2) return stage_launch<R, 2>(psi, out, a, cbits, partials, bar, d, err, grid, s);
+    if (per <= 4) return stage_launch<R, 4>(psi, out, a, cbits, partials, bar, d, err, grid, s);
+    if constexpr (sizeof(R) == 4) return stage_launch<R, 8>(psi, out, a, cbits, partials, bar, d, err, grid, s);
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_kitaev_stage(int prec, const void *psi, void *out, const KitaevArgs &a, const uint8_t *cbits,
+                                double *partials, unsigned *bar, const Decide &d, int *err, int sms, cudaStream_t s) {
+    if (!kitaev_stage_fits(prec, a.n_half, sms)) return cudaErrorInvalidValue;
+    return prec == 0 ? stage_r<float>(psi, out, a, cbits, partials, bar, d, err, sms, s)
+                     : stage_r<double>(psi, out, a, cbits, partials, bar, d, err, sms, s);
 }
 
 }  // namespace qk

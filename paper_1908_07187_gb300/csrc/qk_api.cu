@@ -120,7 +120,7 @@ struct qk_ctx {
 
     double *d_partials = nullptr;
     int *d_err = nullptr;          // set by a kernel whose bounded wait gave up
-    unsigned *d_counter = nullptr; // reduction ticket (zero between launches)
+    unsigned *d_counter = nullptr; // reduction ticket (zero between launches), then a grid barrier's two words
     int meas_blocks = 0;
     qk::MeasSlot *d_slots = nullptr;
     int slot_cap = 0;
@@ -631,8 +631,8 @@ qk_status qk_create(qk_ctx **out, qk_precision precision, void *cuda_stream, con
     if (dalloc(c, (void **)&c->d_partials,
                sizeof(double) * std::max<size_t>(qk::meas_partials(c->sms), 2 * (size_t)c->meas_blocks)) != cudaSuccess ||
         dalloc(c, (void **)&c->d_err, sizeof(int)) != cudaSuccess ||
-        dalloc(c, (void **)&c->d_counter, sizeof(unsigned)) != cudaSuccess ||
-        cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned), c->stream) != cudaSuccess ||
+        dalloc(c, (void **)&c->d_counter, 3 * sizeof(unsigned)) != cudaSuccess ||
+        cudaMemsetAsync(c->d_counter, 0, 3 * sizeof(unsigned), c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream) != cudaSuccess) {
         cudaGetLastError();
         qk_destroy(c);
@@ -1047,9 +1047,16 @@ qk_status qk_apply_kitaev_stage(qk_ctx *c, int control, int gate_id, const int *
     for (int l = 0; l < ncb; ++l) a.rphase_idx[l] = phase_cbits[l];
     a.n_half = 1ull << (c->n - 1);
     const double half = (double)c->amp * (double)a.n_half;
+    const qk::Decide d{c->d_counter, uniform, c->d_slots, c->d_cbits, dest};
+    if (qk::kitaev_stage_fits((int)c->prec, a.n_half, c->sms)) {
+        LaunchScope ls(c, 4, 4 * half);
+        CUDA_TRY(c, qk::launch_kitaev_stage((int)c->prec, c->d_state, c->d_scratch, a, c->d_cbits, c->d_partials,
+                                            c->d_counter + 1, d, c->d_err, c->sms, c->stream));
+        std::swap(c->d_state, c->d_scratch);
+        return QK_OK;
+    }
     {
         LaunchScope ls(c, 4, 2 * half);
-        const qk::Decide d{c->d_counter, uniform, c->d_slots, c->d_cbits, dest};
         // half the measurement grid: the stage's state sits in L2 and a longer grid
         // only adds partials for the deciding block to add
         CUDA_TRY(c, qk::launch_kitaev_reduce((int)c->prec, c->d_state, a, c->d_cbits, c->d_partials,
@@ -1203,7 +1210,7 @@ qk_status qk_sync(qk_ctx *c) {
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     if (err) {
         CUDA_TRY(c, cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
-        return fail(c, QK_ETIMEOUT, "a tensor-core pass gave up a bounded wait; the state is not valid");
+        return fail(c, QK_ETIMEOUT, "a kernel gave up a bounded wait; the state is not valid");
     }
     return QK_OK;
 }

@@ -148,6 +148,29 @@ struct FSum {
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
+// The semiclassical phase exp(i theta), theta = -2 pi sum_l c_l / 2^(l+1) over the listed
+// cbits, l = 1..n (64-bit fixed point), by one whole warp: a lane per cbit, so that
+// their loads are one latency and not n of them.  Valid in lane 0.
+__device__ __forceinline__ double2 warp_rphase(const int *idx, int n, const uint8_t *cbits) {
+    const int lane = (int)(threadIdx.x & 31);
+    uint32_t hi = 0, lo = 0;   // turns = sum of 2^(63 - l): bits 62 down to 1
+    for (int l = lane + 1; l <= n; l += 32)
+        if (cbits[idx[l - 1]]) {
+            if (l < 32) hi |= 1u << (31 - l);
+            else lo |= 1u << (63 - l);
+        }
+    hi = __reduce_or_sync(0xffffffffu, hi);
+    lo = __reduce_or_sync(0xffffffffu, lo);
+    double2 r = make_double2(1.0, 0.0);
+    if (lane == 0) {
+        const uint64_t turns = ((uint64_t)hi << 32) | lo;
+        double s, c;
+        sincospi(-2.0 * ((double)turns * 0x1p-64), &s, &c);
+        r = make_double2(c, s);
+    }
+    return r;
+}
+
 // Sum over the block of one double per thread, the FP64 additions done by warp 0
 // alone; sh holds blockDim.x doubles.  The result is valid in thread 0.
 __device__ __forceinline__ double block_sum_w0(double v, double *sh) {
@@ -549,6 +572,12 @@ cudaError_t launch_measure_round(int prec, const void *psi, const MeasArgs &a, M
                                  unsigned *counter, uint8_t *cbits, int sms, cudaStream_t s);
 cudaError_t launch_measure_collapse(int prec, void *psi, int n, const MeasArgs &a, const MeasSlot *slots, int sms,
                                     cudaStream_t s);
+// one stage in one cooperative launch, for states that fit the register files; bar: two
+// words, zero before the first launch (a ticket and a generation); err receives 1 if the
+// grid barrier's bounded wait gave up
+bool kitaev_stage_fits(int prec, uint64_t n_half, int sms);
+cudaError_t launch_kitaev_stage(int prec, const void *psi, void *out, const KitaevArgs &a, const uint8_t *cbits,
+                                double *partials, unsigned *bar, const Decide &d, int *err, int sms, cudaStream_t s);
 cudaError_t launch_kitaev_reduce(int prec, const void *psi, const KitaevArgs &a, const uint8_t *cbits,
                                  double *partials, int nblocks, const Decide &d, cudaStream_t s);
 cudaError_t launch_kitaev_update(int prec, const void *psi, void *out, const KitaevArgs &a, const uint8_t *cbits,
