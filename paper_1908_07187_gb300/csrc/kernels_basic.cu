@@ -171,26 +171,11 @@ __global__ void __launch_bounds__(kThreads) k_perm(const typename Amp<R>::T *__r
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n_amps; i += stride) {
         uint64_t src = i;
         if (active && (i & a.cmask) == a.cmask) {
-            uint64_t y = 0;
-            if (a.field.contig) {
-                y = field_get(i, a.field, a.w);
-            } else {
-                for (int b = 0; b < a.w; ++b) y = (y << 1) | ((i >> a.rpos[b]) & 1u);
-            }
-            uint64_t x = y;
-            if (a.kind == 0) {
-                if (y < a.N) x = mulmod_barrett(a.cinv, y, a.N, a.mu);
-            } else {
-                x = a.finv[y];
-            }
-            if (a.field.contig) {
-                src = field_put(src, x, a.field, a.w);
-            } else {
-                for (int b = 0; b < a.w; ++b) {
-                    const uint64_t bit = (x >> (a.w - 1 - b)) & 1u;
-                    src = (src & ~(1ull << a.rpos[b])) | (bit << a.rpos[b]);
-                }
-            }
+            const uint32_t y = reg_get<uint64_t>(i, a.field, a.rpos, a.w);
+            uint32_t x = y;
+            if (a.kind != 0) x = a.finv[y];
+            else if (y < a.mul.N) x = mul_mod(y, a.mul);
+            src = reg_put<uint64_t>(i, x, a.field, a.rpos, a.w);
         }
         out[i] = in[src];
     }
@@ -211,12 +196,7 @@ __global__ void __launch_bounds__(kThreads) k_modexp(const typename Amp<R>::T *_
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n_amps; i += stride) {
         uint64_t src = i;
         if (active) {
-            uint64_t y = 0;
-            if (a.field.contig) {
-                y = field_get(i, a.field, a.w);
-            } else {
-                for (int b = 0; b < a.w; ++b) y = (y << 1) | ((i >> a.rpos[b]) & 1u);
-            }
+            const uint32_t y = reg_get<uint64_t>(i, a.field, a.rpos, a.w);
             if (y < a.N) {
                 uint64_t m = 1;
                 for (int g = 0; g < a.ngroups; ++g) {
@@ -227,14 +207,7 @@ __global__ void __launch_bounds__(kThreads) k_modexp(const typename Amp<R>::T *_
                     m = g == 0 ? t : mulmod_barrett(m, t, a.N, a.mu);
                 }
                 const uint64_t x = mulmod_barrett(m, y, a.N, a.mu);
-                if (a.field.contig) {
-                    src = field_put(src, x, a.field, a.w);
-                } else {
-                    for (int b = 0; b < a.w; ++b) {
-                        const uint64_t bit = (x >> (a.w - 1 - b)) & 1u;
-                        src = (src & ~(1ull << a.rpos[b])) | (bit << a.rpos[b]);
-                    }
-                }
+                src = reg_put<uint64_t>(i, (uint32_t)x, a.field, a.rpos, a.w);
             }
         }
         out[i] = in[src];

@@ -894,9 +894,7 @@ qk_status qk_apply_gate(qk_ctx *c, int gate_id, const int *targets, int nt, cons
     a.cmask = cmask;
     a.n_amps = 1ull << c->n;
     a.kind = g.kind == 1 ? 0 : 1;
-    a.N = g.N;
-    a.cinv = g.cinv;
-    a.mu = g.kind == 1 ? (~0ull) / g.N : 0;
+    if (g.kind == 1) a.mul = qk::mul_const(g.cinv, g.N);
     a.finv = g.d_finv;
     a.cond = cond;
     {
@@ -1039,9 +1037,7 @@ qk_status qk_apply_kitaev_stage(qk_ctx *c, int control, int gate_id, const int *
     for (int t = 0; t < g.k; ++t) a.rpos[t] = c->l2p[targets[t]];
     a.field = qk::reg_field_of(a.rpos, g.k);
     a.kind = g.kind == 1 ? 0 : 1;
-    a.N = g.N;
-    a.cinv = g.cinv;
-    a.mu = g.kind == 1 ? (~0ull) / g.N : 0;
+    if (g.kind == 1) a.mul = qk::mul_const(g.cinv, g.N);
     a.finv = g.d_finv;
     a.n_rphase = ncb;
     for (int l = 0; l < ncb; ++l) a.rphase_idx[l] = phase_cbits[l];

@@ -69,14 +69,51 @@ inline RegField reg_field_of(const int *rpos, int w) {
     return f;
 }
 #ifdef __CUDACC__
-__device__ __forceinline__ uint64_t field_get(uint64_t i, const RegField &f, int w) {
-    const uint64_t v = (i >> f.p0) & ((1ull << w) - 1);
-    return f.rev ? (__brevll(v) >> (64 - w)) : v;
+// I: the index type, 32 bits where the state allows; register values have at most 30
+template <typename I>
+__device__ __forceinline__ uint32_t field_get(I i, const RegField &f, int w) {
+    const uint32_t v = (uint32_t)(i >> f.p0) & ((1u << w) - 1);
+    return f.rev ? __brev(v) >> (32 - w) : v;
 }
-__device__ __forceinline__ uint64_t field_put(uint64_t i, uint64_t x, const RegField &f, int w) {
-    const uint64_t v = f.rev ? (__brevll(x) >> (64 - w)) : x;
-    const uint64_t m = ((1ull << w) - 1) << f.p0;
-    return (i & ~m) | (v << f.p0);
+template <typename I>
+__device__ __forceinline__ I field_put(I i, uint32_t x, const RegField &f, int w) {
+    const uint32_t v = f.rev ? __brev(x) >> (32 - w) : x;
+    const I m = (I)((1u << w) - 1) << f.p0;
+    return (i & ~m) | ((I)v << f.p0);
+}
+// the value of a register on any bits (rpos[0] the most significant), and the index with
+// that value replaced
+template <typename I>
+__device__ __forceinline__ uint32_t reg_get(I i, const RegField &f, const int *rpos, int w) {
+    if (f.contig) return field_get<I>(i, f, w);
+    uint32_t y = 0;
+    for (int b = 0; b < w; ++b) y = (y << 1) | ((uint32_t)(i >> rpos[b]) & 1u);
+    return y;
+}
+template <typename I>
+__device__ __forceinline__ I reg_put(I i, uint32_t x, const RegField &f, const int *rpos, int w) {
+    if (f.contig) return field_put<I>(i, x, f, w);
+    for (int b = 0; b < w; ++b) {
+        const I bit = (x >> (w - 1 - b)) & 1u;
+        i = (i & ~((I)1 << rpos[b])) | (bit << rpos[b]);
+    }
+    return i;
+}
+#endif
+
+// x -> c x mod N by a constant c, for 32-bit x (Shoup's form: with s = floor(2^32 c / N),
+// q = floor(x s / 2^32) is the quotient or one less): two multiplies, a high multiply
+// and a subtraction, where a Barrett step on 64-bit products takes some thirty.
+struct MulConst {
+    uint32_t c, s, N;
+};
+inline MulConst mul_const(uint64_t c, uint64_t N) {   // c < N <= 2^30
+    return MulConst{(uint32_t)c, (uint32_t)((c << 32) / N), (uint32_t)N};
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ uint32_t mul_mod(uint32_t x, const MulConst &m) {
+    uint32_t r = x * m.c - __umulhi(x, m.s) * m.N;    // exact modulo 2^32, below 2 N
+    return r >= m.N ? r - m.N : r;
 }
 #endif
 
@@ -87,7 +124,7 @@ struct PermArgs {
     uint64_t cmask;
     uint64_t n_amps;
     int kind;             // 0 = mul-mod, 1 = table
-    uint64_t N, cinv, mu; // mul-mod: y -> cinv*y mod N for y < N, mu = floor((2^64-1)/N)
+    MulConst mul;         // mul-mod: y -> cinv * y mod N for y < N
     const uint32_t *finv; // table: inverse permutation
     Cond cond;
 };
@@ -268,7 +305,7 @@ struct KitaevArgs {
     int rpos[kMaxPermW];
     RegField field;
     int kind;             // 0 = mul-mod, 1 = table
-    uint64_t N, cinv, mu;
+    MulConst mul;
     const uint32_t *finv;
     int n_rphase;
     int rphase_idx[kMaxRphase];

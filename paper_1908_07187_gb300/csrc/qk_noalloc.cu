@@ -119,9 +119,7 @@ extern "C" qk_status qk_apply_perm_mulmod_noalloc(void *d_state, int n, qk_preci
     for (int b = 0; b < nc; ++b) a.cmask |= 1ull << controls[b];
     a.n_amps = 1ull << n;
     a.kind = 0;
-    a.N = N;
-    a.cinv = cinv;
-    a.mu = (~0ull) / N;
+    a.mul = qk::mul_const(cinv, N);
     a.finv = nullptr;
     a.cond.n = 0;
     cudaStream_t s = (cudaStream_t)cuda_stream;
