@@ -329,6 +329,16 @@ struct qk_batch {
     size_t cap_stage = 0;
     cudaEvent_t done = nullptr;
     cudaEvent_t start = nullptr;       // recorded once the host work of a run is done
+    // The launches of the small circuits go round these streams, beside the tile passes
+    // of the large ones; a run forks from and joins the batch's stream by events.
+    static constexpr int kSide = 4;
+    cudaStream_t side[kSide] = {};
+    cudaEvent_t fork = nullptr, join[kSide] = {};
+    // host copy of all small circuits' states and all cbits, taken when a second circuit
+    // of a run is read (one copy instead of two waits per circuit)
+    std::vector<unsigned char> h_states, h_cbits;
+    bool h_valid = false;
+    int reads = 0;                     // circuits read since the last run
     bool start_recorded = false;
     bool store_state = true;
     std::string err;
@@ -437,7 +447,9 @@ void form_raw_ops(std::vector<qk::BOp> &ops) {
             }
         }
     };
-    const size_t nth = n < (1u << 16) ? 1 : std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+    // about 0.1 us an op: a thread is worth its start from a few thousand ops on
+    const size_t nth = std::min<size_t>(std::max<size_t>(1, n >> 12),
+                                        std::max(1u, std::min(16u, std::thread::hardware_concurrency())));
     if (nth == 1) {
         work(0, n);
         return;
@@ -477,10 +489,21 @@ void append_fused(std::vector<qk::FusedOp> &out, const qk_gate_op &g) {
     }
 }
 
-// The circuits above 13 qubits: plan each into tile passes (host threads), pack
-// the pass programs into device pools ordered by pass index, set the states to
-// |0...0> and launch pass k of every circuit that has one in one batched launch.
-qk_status run_large(qk_batch *b) {
+// The circuits above 13 qubits: plan each into tile passes (host threads) and pack
+// the pass programs ordered by pass index; launch_large then uploads them, sets the
+// states to |0...0> and launches pass k of every circuit that has one in one batched
+// launch.
+struct LargeRun {
+    std::vector<qk::TileProg> progs;
+    std::vector<uint32_t> first;
+    std::vector<std::pair<size_t, size_t>> launch;   // per pass: first program, first[] index
+    std::vector<uint32_t> ctas;
+    std::vector<qk::TileOp> ops;
+    std::vector<qk::LayerGate> lg;
+    std::vector<qk::BitTerm> bt;
+    std::vector<uint64_t> offs;
+};
+qk_status plan_large(qk_batch *b, LargeRun &run) {
     const auto t0 = std::chrono::steady_clock::now();
     struct Plan {
         std::vector<qk::TileProg> progs;
@@ -554,11 +577,11 @@ qk_status run_large(qk_batch *b) {
     if ((s = grow(b, &b->d_llg, &b->cap_llg, std::max<size_t>(1, nlg))) != QK_OK) return s;
     if ((s = grow(b, &b->d_lbt, &b->cap_lbt, std::max<size_t>(1, nbt))) != QK_OK) return s;
     // programs ordered by pass index; first[] splits each launch's grid
-    std::vector<qk::TileProg> progs;
+    auto &progs = run.progs;
+    auto &first = run.first;
+    auto &launch = run.launch;
+    auto &ctas = run.ctas;
     progs.reserve(nprog);
-    std::vector<uint32_t> first;
-    std::vector<std::pair<size_t, size_t>> launch;   // (first program, first[] index)
-    std::vector<uint32_t> ctas;
     for (int k = 0; k < maxp; ++k) {
         launch.push_back({progs.size(), first.size()});
         uint32_t acc = 0;
@@ -576,13 +599,14 @@ qk_status run_large(qk_batch *b) {
         first.push_back(acc);
         ctas.push_back(acc);
     }
-    std::vector<qk::TileOp> ops;
-    std::vector<qk::LayerGate> lg;
-    std::vector<qk::BitTerm> bt;
+    auto &ops = run.ops;
+    auto &lg = run.lg;
+    auto &bt = run.bt;
+    auto &offs = run.offs;
     ops.reserve(nops);
     lg.reserve(nlg);
     bt.reserve(nbt);
-    std::vector<uint64_t> offs(nl);
+    offs.resize(nl);
     for (int i = 0; i < nl; ++i) {
         ops.insert(ops.end(), plans[i].ops.begin(), plans[i].ops.end());
         lg.insert(lg.end(), plans[i].lg.begin(), plans[i].lg.end());
@@ -590,8 +614,20 @@ qk_status run_large(qk_batch *b) {
         offs[i] = b->large[i].state_off;
     }
     b->plan_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-    if (cudaEventRecord(b->start, b->stream) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event record failed");
-    b->start_recorded = true;
+    return QK_OK;
+}
+
+// upload the plans, set the states to |0...0> and launch
+qk_status launch_large(qk_batch *b, const LargeRun &run) {
+    const auto &progs = run.progs;
+    const auto &first = run.first;
+    const auto &launch = run.launch;
+    const auto &ctas = run.ctas;
+    const auto &ops = run.ops;
+    const auto &lg = run.lg;
+    const auto &bt = run.bt;
+    const auto &offs = run.offs;
+    const int nl = (int)offs.size(), maxp = (int)launch.size();
     auto up = [&](void *dst, const void *src, size_t bytes) {
         return bytes == 0 || cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, b->stream) == cudaSuccess;
     };
@@ -658,7 +694,15 @@ qk_status qk_batch_create(qk_batch **out, void *cuda_stream) {
         }
         b->own_stream = true;
     }
-    if (cudaEventCreate(&b->done) != cudaSuccess || cudaEventCreate(&b->start) != cudaSuccess) {
+    bool ok = cudaEventCreate(&b->done) == cudaSuccess && cudaEventCreate(&b->start) == cudaSuccess &&
+              cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
+    int prio = 0;
+    ok = ok && cudaStreamGetPriority(b->stream, &prio) == cudaSuccess;
+    for (int k = 0; k < qk_batch::kSide && ok; ++k)
+        ok = cudaStreamCreateWithPriority(&b->side[k], cudaStreamNonBlocking, prio) == cudaSuccess &&
+             cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
         qk_batch_destroy(b);
         return QK_ECUDA;
     }
@@ -668,6 +712,8 @@ qk_status qk_batch_create(qk_batch **out, void *cuda_stream) {
 
 qk_status qk_batch_destroy(qk_batch *b) {
     if (!b) return QK_EINVAL;
+    for (cudaStream_t side : b->side)
+        if (side) cudaStreamSynchronize(side);
     if (b->stream) {
         void *bufs[] = {b->d_ops, b->d_circs, b->d_states, b->d_cbits, b->d_lstates, b->d_lprogs,
                         b->d_lfirst, b->d_loffs, b->d_lops, b->d_llg, b->d_lbt};
@@ -677,6 +723,11 @@ qk_status qk_batch_destroy(qk_batch *b) {
     }
     if (b->pool_held) qk::pool_release(b->device);   // after its blocks went back to the pool
     if (b->h_stage) cudaFreeHost(b->h_stage);
+    for (int k = 0; k < qk_batch::kSide; ++k) {
+        if (b->side[k]) cudaStreamDestroy(b->side[k]);
+        if (b->join[k]) cudaEventDestroy(b->join[k]);
+    }
+    if (b->fork) cudaEventDestroy(b->fork);
     if (b->done) cudaEventDestroy(b->done);
     if (b->start) cudaEventDestroy(b->start);
     if (b->own_stream) cudaStreamDestroy(b->stream);
@@ -696,6 +747,8 @@ qk_status qk_batch_clear(qk_batch *b) {
     b->large.clear();
     b->large_of.clear();
     b->large_amps = 0;
+    b->h_valid = false;
+    b->reads = 0;
     return QK_OK;
 }
 
@@ -888,30 +941,32 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
     b->start_recorded = false;
     b->plan_ms = 0.0;
     b->large_launches = 0;
-    // large circuits first: their planning is host work, after which the start
-    // event is recorded and everything else is enqueued back to back
+    b->h_valid = false;
+    b->reads = 0;
+    // host work first -- the large circuits' plans, the small ones' matrices -- then the
+    // start event, after which everything is enqueued back to back
+    LargeRun lr;
     if (!b->large.empty()) {
-        const qk_status ls = run_large(b);
+        const qk_status ls = plan_large(b, lr);
         if (ls != QK_OK) return ls;
-    } else {
-        if (cudaEventRecord(b->start, b->stream) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event record failed");
-        b->start_recorded = true;
     }
+    form_raw_ops(b->ops);
+    if (cudaEventRecord(b->start, b->stream) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event record failed");
+    b->start_recorded = true;
     qk_status s;
     if ((s = grow(b, &b->d_ops, &b->cap_ops, std::max<size_t>(1, b->ops.size()))) != QK_OK) return s;
     if ((s = grow(b, &b->d_circs, &b->cap_circs, std::max<size_t>(1, b->circs.size()))) != QK_OK) return s;
     if (b->store_state && (s = grow(b, &b->d_states, &b->cap_states, b->total_amps)) != QK_OK) return s;
     if ((s = grow(b, &b->d_cbits, &b->cap_cbits, std::max<size_t>(1, b->total_cb))) != QK_OK) return s;
-    // circuits of at most 13 qubits, sorted by size: one launch per qubit count (and
-    // per need of the second state buffer, which only mul-mod gathers use), each
-    // sized to its shared memory (small circuits then share an SM)
+    // circuits of at most 13 qubits, sorted by size, largest first: one launch per qubit
+    // count (and per need of the second state buffer, which only mul-mod gathers use),
+    // each sized to its shared memory (small circuits then share an SM)
     std::vector<qk::BCirc> sorted;
     for (const auto &c : b->circs)
         if (!(c.flags & 2u)) sorted.push_back(c);
     std::stable_sort(sorted.begin(), sorted.end(), [](const qk::BCirc &x, const qk::BCirc &y) {
-        return x.n != y.n ? x.n < y.n : (x.flags & 1u) < (y.flags & 1u);
+        return x.n != y.n ? x.n > y.n : (x.flags & 1u) < (y.flags & 1u);
     });
-    form_raw_ops(b->ops);
     // stage the program in pinned memory so that the copies are truly asynchronous
     const size_t ob = sizeof(qk::BOp) * b->ops.size(), cb = sizeof(qk::BCirc) * sorted.size();
     if (ob + cb > 0 && ob + cb > b->cap_stage) {
@@ -932,19 +987,40 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
             return bfail(b, QK_ECUDA, "batch: upload failed");
     }
     const size_t max_smem = sizeof(float2) * 2 * ((size_t)1 << b->max_n);
-    if (!sorted.empty() && max_smem > 48 * 1024 &&
+    if (!sorted.empty() && max_smem > 40 * 1024 &&
         cudaFuncSetAttribute(qk::k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem) != cudaSuccess)
         return bfail(b, QK_ECUDA, "batch: shared memory attribute failed");
-    for (size_t i = 0; i < sorted.size();) {
+    // The launches run beside each other and beside the tile passes: each is as long as
+    // its longest circuit and most leave SMs free.  (One after another on one stream, the
+    // 22 small circuits of a 60-circuit batch took 9.2 ms in four launches, in front of
+    // or behind 16 ms of tile passes.)
+    int used = 0;
+    if (!sorted.empty() && cudaEventRecord(b->fork, b->stream) != cudaSuccess)
+        return bfail(b, QK_ECUDA, "batch: event record failed");
+    qk_status st = QK_OK;
+    for (size_t i = 0; i < sorted.size() && st == QK_OK;) {
         size_t j = i;
         while (j < sorted.size() && sorted[j].n == sorted[i].n && (sorted[j].flags & 1u) == (sorted[i].flags & 1u))
             ++j;
+        const int k = used % qk_batch::kSide;
+        if (used < qk_batch::kSide && cudaStreamWaitEvent(b->side[k], b->fork, 0) != cudaSuccess)
+            st = bfail(b, QK_ECUDA, "batch: event wait failed");
         const size_t smem = sizeof(float2) * ((sorted[i].flags & 1u) ? 2 : 1) * ((size_t)1 << sorted[i].n);
-        qk::k_batch<<<(unsigned)(j - i), qk::kBThreads, smem, b->stream>>>(b->d_circs + i, b->d_ops, b->d_states,
-                                                                          b->d_cbits, b->store_state ? 1 : 0);
-        if (cudaGetLastError() != cudaSuccess) return bfail(b, QK_ECUDA, "batch: launch failed");
+        if (st == QK_OK) {
+            qk::k_batch<<<(unsigned)(j - i), qk::kBThreads, smem, b->side[k]>>>(b->d_circs + i, b->d_ops, b->d_states,
+                                                                                b->d_cbits, b->store_state ? 1 : 0);
+            if (cudaGetLastError() != cudaSuccess) st = bfail(b, QK_ECUDA, "batch: launch failed");
+        }
+        ++used;
         i = j;
     }
+    if (st == QK_OK && !b->large.empty()) st = launch_large(b, lr);
+    // the batch's stream continues after every side stream, also when a launch failed
+    for (int k = 0; k < std::min(used, (int)qk_batch::kSide); ++k)
+        if ((cudaEventRecord(b->join[k], b->side[k]) != cudaSuccess ||
+             cudaStreamWaitEvent(b->stream, b->join[k], 0) != cudaSuccess) && st == QK_OK)
+            st = bfail(b, QK_ECUDA, "batch: event wait failed");
+    if (st != QK_OK) return st;
     if (cudaEventRecord(b->done, b->stream) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event record failed");
     return QK_OK;
 }
@@ -985,9 +1061,27 @@ qk_status qk_batch_read(qk_batch *b, int circuit, uint8_t *cbits, int ncb, void 
     if (state && ((!large && !b->store_state) || bytes != sizeof(float2) << c.n))
         return bfail(b, QK_EINVAL, "batch: state not stored or wrong size (%zu bytes expected)", sizeof(float2) << c.n);
     if (cudaEventSynchronize(b->done) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event wait failed");
-    // reads on the batch's own stream (its run is complete: the event above)
-    if (ncb > 0 && !read_back(b, cbits, b->d_cbits + c.cb_off, ncb))
+    // A program that reads a second circuit reads many: all the small ones come over in
+    // one copy then (up to 64 MB of states), instead of two copies and waits for each.
+    const size_t all = b->store_state ? sizeof(float2) * b->total_amps : 0;
+    if (++b->reads == 2 && !b->h_valid && all <= (64u << 20)) {
+        b->h_states.resize(all);
+        b->h_cbits.resize(b->total_cb);
+        b->h_valid = (all == 0 || cudaMemcpyAsync(b->h_states.data(), b->d_states, all, cudaMemcpyDeviceToHost, b->stream) == cudaSuccess) &&
+                     (b->total_cb == 0 || cudaMemcpyAsync(b->h_cbits.data(), b->d_cbits, b->total_cb, cudaMemcpyDeviceToHost, b->stream) == cudaSuccess) &&
+                     cudaStreamSynchronize(b->stream) == cudaSuccess;
+        if (!b->h_valid) return bfail(b, QK_ECUDA, "batch: copy failed");
+    }
+    if (b->h_valid) {
+        if (ncb > 0) std::memcpy(cbits, b->h_cbits.data() + c.cb_off, (size_t)ncb);
+        if (state && !large) {
+            std::memcpy(state, b->h_states.data() + sizeof(float2) * c.state_off, bytes);
+            return QK_OK;
+        }
+    } else if (ncb > 0 && !read_back(b, cbits, b->d_cbits + c.cb_off, ncb)) {
         return bfail(b, QK_ECUDA, "batch: cbit copy failed");
+    }
+    // on the batch's own stream (its run is complete: the event above)
     const float2 *src = large ? b->d_lstates + b->large[b->large_of[circuit]].state_off : b->d_states + c.state_off;
     if (state && !read_back(b, state, src, bytes)) return bfail(b, QK_ECUDA, "batch: state copy failed");
     return QK_OK;
