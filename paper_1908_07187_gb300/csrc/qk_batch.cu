@@ -26,6 +26,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <thread>
@@ -339,6 +340,7 @@ struct qk_batch {
     std::vector<unsigned char> h_states, h_cbits;
     bool h_valid = false;
     int reads = 0;                     // circuits read since the last run
+    std::mutex read_mu;                // reads from several threads
     bool start_recorded = false;
     bool store_state = true;
     std::string err;
@@ -448,8 +450,9 @@ void form_raw_ops(std::vector<qk::BOp> &ops) {
         }
     };
     // about 0.1 us an op: a thread is worth its start from a few thousand ops on
-    const size_t nth = std::min<size_t>(std::max<size_t>(1, n >> 12),
-                                        std::max(1u, std::min(16u, std::thread::hardware_concurrency())));
+    // (and asking for the number of cores costs 18 us)
+    const size_t nth =
+        (n >> 12) < 2 ? 1 : std::min<size_t>(n >> 12, std::max(1u, std::min(16u, std::thread::hardware_concurrency())));
     if (nth == 1) {
         work(0, n);
         return;
@@ -994,24 +997,26 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
     // its longest circuit and most leave SMs free.  (One after another on one stream, the
     // 22 small circuits of a 60-circuit batch took 9.2 ms in four launches, in front of
     // or behind 16 ms of tile passes.)
-    int used = 0;
-    if (!sorted.empty() && cudaEventRecord(b->fork, b->stream) != cudaSuccess)
-        return bfail(b, QK_ECUDA, "batch: event record failed");
+    // Without tile passes the first launch stays on the batch's own stream, which has
+    // nothing else to run (a run of two launches: 7 event calls down to 4).
+    int used = 0;                      // launches on side streams
+    bool own = b->large.empty();
     qk_status st = QK_OK;
-    for (size_t i = 0; i < sorted.size() && st == QK_OK;) {
+    for (size_t i = 0; i < sorted.size() && st == QK_OK; own = false) {
         size_t j = i;
         while (j < sorted.size() && sorted[j].n == sorted[i].n && (sorted[j].flags & 1u) == (sorted[i].flags & 1u))
             ++j;
         const int k = used % qk_batch::kSide;
-        if (used < qk_batch::kSide && cudaStreamWaitEvent(b->side[k], b->fork, 0) != cudaSuccess)
-            st = bfail(b, QK_ECUDA, "batch: event wait failed");
-        const size_t smem = sizeof(float2) * ((sorted[i].flags & 1u) ? 2 : 1) * ((size_t)1 << sorted[i].n);
-        if (st == QK_OK) {
-            qk::k_batch<<<(unsigned)(j - i), qk::kBThreads, smem, b->side[k]>>>(b->d_circs + i, b->d_ops, b->d_states,
-                                                                                b->d_cbits, b->store_state ? 1 : 0);
-            if (cudaGetLastError() != cudaSuccess) st = bfail(b, QK_ECUDA, "batch: launch failed");
+        if ((i == 0 && (!own || j < sorted.size()) && cudaEventRecord(b->fork, b->stream) != cudaSuccess) ||
+            (!own && used < qk_batch::kSide && cudaStreamWaitEvent(b->side[k], b->fork, 0) != cudaSuccess)) {
+            st = bfail(b, QK_ECUDA, "batch: event failed");
+            break;
         }
-        ++used;
+        const size_t smem = sizeof(float2) * ((sorted[i].flags & 1u) ? 2 : 1) * ((size_t)1 << sorted[i].n);
+        qk::k_batch<<<(unsigned)(j - i), qk::kBThreads, smem, own ? b->stream : b->side[k]>>>(
+            b->d_circs + i, b->d_ops, b->d_states, b->d_cbits, b->store_state ? 1 : 0);
+        if (cudaGetLastError() != cudaSuccess) st = bfail(b, QK_ECUDA, "batch: launch failed");
+        if (!own) ++used;
         i = j;
     }
     if (st == QK_OK && !b->large.empty()) st = launch_large(b, lr);
@@ -1019,7 +1024,7 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
     for (int k = 0; k < std::min(used, (int)qk_batch::kSide); ++k)
         if ((cudaEventRecord(b->join[k], b->side[k]) != cudaSuccess ||
              cudaStreamWaitEvent(b->stream, b->join[k], 0) != cudaSuccess) && st == QK_OK)
-            st = bfail(b, QK_ECUDA, "batch: event wait failed");
+            st = bfail(b, QK_ECUDA, "batch: event failed");
     if (st != QK_OK) return st;
     if (cudaEventRecord(b->done, b->stream) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event record failed");
     return QK_OK;
@@ -1064,7 +1069,8 @@ qk_status qk_batch_read(qk_batch *b, int circuit, uint8_t *cbits, int ncb, void 
     // A program that reads a second circuit reads many: all the small ones come over in
     // one copy then (up to 64 MB of states), instead of two copies and waits for each.
     const size_t all = b->store_state ? sizeof(float2) * b->total_amps : 0;
-    if (++b->reads == 2 && !b->h_valid && all <= (64u << 20)) {
+    const std::lock_guard<std::mutex> lk(b->read_mu);
+    if (++b->reads == 2 && !b->h_valid && b->circs.size() > 2 && all <= (64u << 20)) {
         b->h_states.resize(all);
         b->h_cbits.resize(b->total_cb);
         b->h_valid = (all == 0 || cudaMemcpyAsync(b->h_states.data(), b->d_states, all, cudaMemcpyDeviceToHost, b->stream) == cudaSuccess) &&
