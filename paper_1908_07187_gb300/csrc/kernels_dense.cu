@@ -10,7 +10,8 @@
 // and clock).  Before, one thread formed one amplitude with two shared loads per
 // complex product, one gate per pass.  Measured in complex64: one gate on 24 qubits, k =
 // 2, 3, 4, 5, 6: 86, 84, 108, 144, 224 us (k = 6: 3670 before); a brickwork of 63 pair
-// gates on 22 qubits: 1383 -> 278 us.
+// gates on 22 qubits: 1383 -> 278 us.  In complex128, nine gates, k = 2 / 4 / 6: 892 -> 486,
+// 2154 -> 1364, 7006 -> 4876 us on 20 qubits and 98 -> 74, 130 -> 75, 342 -> 219 us on 8.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -44,7 +45,7 @@ __device__ __forceinline__ uint32_t lane_copy(uint32_t x) {
 }
 template <typename T, int RT>
 __device__ __forceinline__ void load_rows(T (&u)[RT], const T *p) {
-    if constexpr (sizeof(T) == 8) {
+    if constexpr (sizeof(T) == 8 && RT > 1) {
 #pragma unroll
         for (int i = 0; i < RT; i += 2) {
             const float4 a = *reinterpret_cast<const float4 *>(p + i);
@@ -57,47 +58,29 @@ __device__ __forceinline__ void load_rows(T (&u)[RT], const T *p) {
     }
 }
 
-// One or two 2-qubit gates (DenseOp::pair): a thread takes 16 amplitudes at a time, so
-// the state crosses shared memory once for both.  In complex64 a gate's matrix is held
+// One or two 2-qubit gates in complex64 (DenseOp::pair): a thread takes 16 amplitudes at
+// a time, so the state crosses shared memory once for both, and a gate's matrix is held
 // in registers for the four columns (read as kernel parameters per column, it kept the
 // constant path busy 60 % of the time).
-template <typename T>
 struct Mat2 {
-    static constexpr bool kRegs = sizeof(T) == 8;
-    T m[kRegs ? 16 : 1];
-    const T *p;
-    __device__ __forceinline__ explicit Mat2(const T *q) : p(q) {
-        if constexpr (kRegs) {
-#pragma unroll
-            for (int i = 0; i < 16; i += 2) {
-                const float4 a = *reinterpret_cast<const float4 *>(q + i);
-                m[i] = make_float2(a.x, a.y);
-                m[i + 1] = make_float2(a.z, a.w);
-            }
-        }
-    }
-    __device__ __forceinline__ T at(int i) const {
-        if constexpr (kRegs) return m[i];
-        else return p[i];
-    }
+    float2 m[16];
+    __device__ __forceinline__ explicit Mat2(const float2 *q) { load_rows(m, q); }
 };
-template <typename T>
-__device__ __forceinline__ void gate2(T &x0, T &x1, T &x2, T &x3, const Mat2<T> &m) {
-    T y[4];
-    const T x[4] = {x0, x1, x2, x3};
+__device__ __forceinline__ void gate2(float2 &x0, float2 &x1, float2 &x2, float2 &x3, const Mat2 &m) {
+    float2 y[4];
+    const float2 x[4] = {x0, x1, x2, x3};
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         y[r].x = y[r].y = 0;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) mac(y[r], m.at(4 * r + c), x[c]);
+        for (int c = 0; c < 4; ++c) mac(y[r], m.m[4 * r + c], x[c]);
     }
     x0 = y[0];
     x1 = y[1];
     x2 = y[2];
     x3 = y[3];
 }
-template <typename T>
-__device__ __forceinline__ void dense_two(T *A, const DenseOp &op, const T *mat, const T *next) {
+__device__ __forceinline__ void dense_two(float2 *A, const DenseOp &op, const float2 *mat, const float2 *next) {
     const int nf = op.nfree, ncol = 1 << op.ncs;
     const uint32_t t0 = lane_copy(op.ts[0]), t1 = lane_copy(op.ts[1]);
     const uint32_t c0 = lane_copy(op.cs[0]), c1 = lane_copy(op.cs[1]);
@@ -105,7 +88,7 @@ __device__ __forceinline__ void dense_two(T *A, const DenseOp &op, const T *mat,
         uint32_t s = op.ls;
         for (int b = 0; b < nf; ++b)
             if ((g >> b) & 1) s ^= op.fs[b];
-        T x[4][4];                                   // [column][register value]
+        float2 x[4][4];                              // [column][register value]
 #pragma unroll
         for (int c = 0; c < 4; ++c)
             if (c < ncol) {
@@ -114,13 +97,13 @@ __device__ __forceinline__ void dense_two(T *A, const DenseOp &op, const T *mat,
                 for (int r = 0; r < 4; ++r) x[c][r] = A[o ^ ((r & 1) ? t0 : 0u) ^ ((r & 2) ? t1 : 0u)];
             }
         {
-            const Mat2<T> m(mat);
+            const Mat2 m(mat);
 #pragma unroll
             for (int c = 0; c < 4; ++c)
                 if (c < ncol) gate2(x[c][0], x[c][1], x[c][2], x[c][3], m);
         }
         if (op.pair) {
-            const Mat2<T> m(next);
+            const Mat2 m(next);
 #pragma unroll
             for (int r = 0; r < 4; ++r) gate2(x[0][r], x[1][r], x[2][r], x[3][r], m);
         }
@@ -134,25 +117,28 @@ __device__ __forceinline__ void dense_two(T *A, const DenseOp &op, const T *mat,
     }
 }
 
-// One gate of k >= 3.  Column bits run over the op's free bits in their order: the
+// One gate (complex64: of k >= 3).  Column bits run over the op's free bits in their order: the
 // thread's column group takes the first ones, then the columns of one thread, then
 // rounds.  Ut holds the matrix transposed (Ut[c * G + r]).  A thread forms RT rows of CT
 // columns: with 4 x 4 the shared-memory loads of a step (their 128 bytes per clock into
-// registers) take as long as its FMAs, with 8 x 4 three quarters of it.
-template <typename R, int K>
+// registers) take as long as its FMAs, with 8 x 4 three quarters of it.  1 x 1 where the
+// tile has few columns, or threads would form rows and columns that are not there, and
+// in complex128, where a product's four FP64 FMAs take 64 cycles against 8 for its loads.
+template <typename R, int K, int RT, int CT>
 __device__ __forceinline__ void dense_gate(typename Amp<R>::T *A, const typename Amp<R>::T *Ut, const DenseOp &op) {
     using T = typename Amp<R>::T;
-    constexpr bool kF = sizeof(R) == 4;
-    constexpr int RT = kF && K >= 5 ? 8 : 4, G = 1 << K, RG = G / RT, CG = kThreads / RG, LCG = (RT == 8 ? 11 : 10) - K,
-                  CT = RT == 8 ? 4 : 2, LCT = RT == 8 ? 2 : 1;
+    constexpr int LRT = RT == 8 ? 3 : RT == 4 ? 2 : 0, LCT = CT == 4 ? 2 : CT == 2 ? 1 : 0;
+    constexpr int G = 1 << K, RG = G / RT, CG = kThreads / RG, LCG = 8 - (K - LRT);
     static_assert(CG == 1 << LCG, "column groups");
-    const int rg = threadIdx.x >> LCG, cg = threadIdx.x & (CG - 1);
     const int nf = op.nfree;
-    const bool live = nf >= LCG || cg < (1 << nf);
+    // fewer columns than column groups: the threads that have work stay in whole warps
+    const int lcg = nf < LCG ? nf : LCG;
+    const int rg = threadIdx.x >> lcg, cg = threadIdx.x & ((1 << lcg) - 1);
+    const bool live = rg < RG;
     uint32_t sb = op.ls;
 #pragma unroll
     for (int b = 0; b < LCG; ++b)
-        if (b < nf && ((cg >> b) & 1)) sb ^= op.fs[b];
+        if (b < lcg && ((cg >> b) & 1)) sb ^= op.fs[b];
     uint32_t ts[K];
 #pragma unroll
     for (int b = 0; b < K; ++b) ts[b] = lane_copy(op.ts[b]);
@@ -160,9 +146,9 @@ __device__ __forceinline__ void dense_gate(typename Amp<R>::T *A, const typename
     cs[0] = 0;
 #pragma unroll
     for (int j = 1; j < CT; ++j) cs[j] = 0;
-    const int ncol = nf <= LCG ? 1 : nf == LCG + 1 ? 2 : CT;
-    if (nf > LCG) {
-        cs[1] = lane_copy(op.fs[LCG]);
+    const int ncol = CT == 1 || nf <= LCG ? 1 : nf == LCG + 1 ? 2 : CT;
+    if (CT > 1 && nf > LCG) {
+        cs[CT > 1 ? 1 : 0] = lane_copy(op.fs[LCG]);
         if constexpr (CT == 4)
             if (nf > LCG + 1) {
                 cs[2] = lane_copy(op.fs[LCG + 1]);
@@ -181,7 +167,7 @@ __device__ __forceinline__ void dense_gate(typename Amp<R>::T *A, const typename
             for (int j = 0; j < CT; ++j) acc[i][j].x = acc[i][j].y = 0;
         constexpr int U = 2, LU = 1;               // steps unrolled
 #pragma unroll 1
-        for (int k0 = 0; k0 < G; k0 += U) {
+        for (int k0 = live ? 0 : G; k0 < G; k0 += U) {
             uint32_t o0 = s0;
 #pragma unroll
             for (int b = LU; b < K; ++b)
@@ -203,7 +189,7 @@ __device__ __forceinline__ void dense_gate(typename Amp<R>::T *A, const typename
         if (live) {
             uint32_t o0 = s0;
 #pragma unroll
-            for (int b = RT == 8 ? 3 : 2; b < K; ++b)
+            for (int b = LRT; b < K; ++b)
                 if (((rg * RT) >> b) & 1) o0 ^= ts[b];
 #pragma unroll
             for (int j = 0; j < CT; ++j) {
@@ -217,10 +203,17 @@ __device__ __forceinline__ void dense_gate(typename Amp<R>::T *A, const typename
     }
 }
 
+template <typename R, int K>                         // two gates at a time (dense_two)
+constexpr bool dense_pairs = sizeof(R) == 4 && K == 2;
+template <typename R, int K, int RT>
+constexpr int dense_ctas() {
+    return RT == 1 && !dense_pairs<R, K> ? 3 : sizeof(R) == 4 && (K == 3 || K == 4) ? 3 : 2;
+}
+
 // K: the k of every gate in the pass (one code path per kernel: with all of them in one
 // the compiler ran out of registers)
-template <typename R, int K>
-__global__ void __launch_bounds__(kThreads, sizeof(R) == 4 && (K == 3 || K == 4) ? 3 : 2)
+template <typename R, int K, int RT, int CT>
+__global__ void __launch_bounds__(kThreads, dense_ctas<R, K, RT>())
     k_dense(typename Amp<R>::T *__restrict__ psi, const __grid_constant__ DenseParams P,
             const uint8_t *__restrict__ cbits) {
     using T = typename Amp<R>::T;
@@ -237,13 +230,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 && (K == 3 || K == 4)
     for (int k = 0; k < 5; ++k) st[k] = 8 + k < P.m ? 1ull << P.S[8 + k] : 0ull;
     const int rounds = dim > kThreads ? (int)(dim / kThreads) : 1;
     const bool live = (uint32_t)tid < dim;
-    // every op's matrix (transposed for k > 2); a CTA runs over several tiles, so this is
+    // every op's matrix (transposed for dense_gate); a CTA runs over several tiles, so this is
     // paid once and the CTAs of an SM drift apart, one loading while the other computes
     constexpr int G = 1 << K;
     for (int o = 0; o < P.nops; ++o) {
         const T *gm = reinterpret_cast<const T *>(P.ops[o].mat);
         T *to = mats + o * (G * G);
-        for (int e = tid; e < G * G; e += kThreads) to[K == 2 ? e : (e & (G - 1)) * G + (e >> K)] = gm[e];
+        for (int e = tid; e < G * G; e += kThreads) to[dense_pairs<R, K> ? e : (e & (G - 1)) * G + (e >> K)] = gm[e];
     }
     unsigned condok = 0;
     for (int c = 0; c < P.n_conds; ++c) {
@@ -277,11 +270,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 && (K == 3 || K == 4)
             if (((uint32_t)tile & op.tmask) != op.tmask) continue;
             if (op.cond != 0xff && !((condok >> op.cond) & 1u)) continue;
             __syncthreads();                         // the tile and matrices, or the previous gate
-            if constexpr (K == 2) {
+            if constexpr (dense_pairs<R, K>) {
                 dense_two(A, op, mats + o * (G * G), mats + (op.pair ? o + 1 : o) * (G * G));
                 if (op.pair) ++o;
             } else {
-                dense_gate<R, K>(A, mats + o * (G * G), op);
+                dense_gate<R, K, RT, CT>(A, mats + o * (G * G), op);
             }
         }
         __syncthreads();
@@ -298,27 +291,34 @@ __global__ void __launch_bounds__(kThreads, sizeof(R) == 4 && (K == 3 || K == 4)
     }
 }
 
-template <typename R, int K>
+template <typename R, int K, int RT, int CT>
 cudaError_t dense_k(void *psi, const DenseParams &p, const uint8_t *cbits, int sms, cudaStream_t s) {
     using T = typename Amp<R>::T;
     const size_t sm = (sizeof(T) << p.m) + sizeof(T) * ((size_t)p.nops << (2 * K));
     if (sm > 47 * 1024) {
         const cudaError_t e =
-            cudaFuncSetAttribute(k_dense<R, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            cudaFuncSetAttribute(k_dense<R, K, RT, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
     }
-    const uint64_t cap = (uint64_t)sms * (sizeof(R) == 4 && (K == 3 || K == 4) ? 3 : 2);
-    k_dense<R, K><<<(unsigned)(p.n_tiles < cap ? p.n_tiles : cap), kThreads, sm, s>>>((T *)psi, p, cbits);
+    const uint64_t cap = (uint64_t)sms * dense_ctas<R, K, RT>();
+    k_dense<R, K, RT, CT><<<(unsigned)(p.n_tiles < cap ? p.n_tiles : cap), kThreads, sm, s>>>((T *)psi, p, cbits);
     return cudaGetLastError();
 }
+// 4 x 2 per thread takes 2^11 amplitudes for every thread to have columns, 8 x 4 2^13
 template <typename R>
 cudaError_t dense_r(void *psi, const DenseParams &p, const uint8_t *cbits, int sms, cudaStream_t s) {
+    constexpr bool kF = sizeof(R) == 4;
+    const bool big = kF && p.m >= (p.k >= 5 ? 13 : 11);
     switch (p.k) {
-        case 2: return dense_k<R, 2>(psi, p, cbits, sms, s);
-        case 3: return dense_k<R, 3>(psi, p, cbits, sms, s);
-        case 4: return dense_k<R, 4>(psi, p, cbits, sms, s);
-        case 5: return dense_k<R, 5>(psi, p, cbits, sms, s);
-        default: return dense_k<R, 6>(psi, p, cbits, sms, s);
+        case 2: return dense_k<R, 2, 1, 1>(psi, p, cbits, sms, s);
+        case 3: if constexpr (kF) if (big) return dense_k<R, 3, 4, 2>(psi, p, cbits, sms, s);
+                return dense_k<R, 3, 1, 1>(psi, p, cbits, sms, s);
+        case 4: if constexpr (kF) if (big) return dense_k<R, 4, 4, 2>(psi, p, cbits, sms, s);
+                return dense_k<R, 4, 1, 1>(psi, p, cbits, sms, s);
+        case 5: if constexpr (kF) if (big) return dense_k<R, 5, 8, 4>(psi, p, cbits, sms, s);
+                return dense_k<R, 5, 1, 1>(psi, p, cbits, sms, s);
+        default: if constexpr (kF) if (big) return dense_k<R, 6, 8, 4>(psi, p, cbits, sms, s);
+                return dense_k<R, 6, 1, 1>(psi, p, cbits, sms, s);
     }
 }
 

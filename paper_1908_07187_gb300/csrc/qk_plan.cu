@@ -1246,9 +1246,10 @@ qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const D
         static thread_local DenseParams P;
         std::memset(static_cast<void *>(&P), 0, offsetof(DenseParams, ops));
         // complex64 gates of 5 and 6 qubits form 8 rows per thread, which takes 2^13
-        // amplitudes to give every thread columns
+        // amplitudes to give every thread columns; smaller tiles for small states, so
+        // that there are tiles for all SMs (in complex128 a tile's FP64 work is the time)
         int m = prec != 0 ? 11 : rem[0]->k >= 5 ? 13 : 12;
-        if (n < 20) m = std::min(m, n >= 18 ? 11 : n >= 16 ? 10 : 9);
+        if (n < 20) m = std::min(m, prec != 0 ? (n >= 18 ? 10 : 8) : n >= 18 ? 11 : n >= 16 ? 10 : 9);
         m = std::min(m, n);
         const int contig = std::min(m, n >= 23 ? 4 : 2);
         uint64_t S = 0, left_t = 0, left_all = 0;
@@ -1325,7 +1326,7 @@ qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const D
             // through shared memory.  The first one's column bits are the second's register
             // bits (or, for one gate alone, its last free bits).
             const bool joined = P.nops >= 2 && P.ops[P.nops - 2].pair;
-            const bool free2 = it->k == 2 && !it->cmask && !it->cond.n;
+            const bool free2 = prec == 0 && it->k == 2 && !it->cmask && !it->cond.n;
             o.pair = 0;
             if (free2 && !joined && &it != &taken.back()) {
                 const DenseItem *nx = (&it)[1];
@@ -1349,7 +1350,7 @@ qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const D
                     placed |= 1u << b;
                     o.fs[o.nfree++] = (uint16_t)dense_slot(1u << b);
                 }
-            if (it->k == 2 && !o.pair)
+            if (prec == 0 && it->k == 2 && !o.pair)
                 while (o.ncs < 2 && o.nfree > 0) o.cs[o.ncs++] = o.fs[--o.nfree];
             o.mat = it->mat;
         }
