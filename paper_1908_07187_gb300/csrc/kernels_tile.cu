@@ -226,6 +226,35 @@ __device__ __forceinline__ void bit_negate(Regs &v) {
     }
 }
 
+// The turns of a layer gate's phase (LayerGate::slot), split into what the lane and what
+// the warp (with the tile index and the constant) contribute: formed once per CTA while
+// the tile's loads are in flight.  Summed term by term by every thread at its gate, they
+// were 15 % of a QFT pass (the four passes of the 30-qubit step that hold its QFT: 38.3 ms
+// with the sums, 32.6 ms with the tables and the turn folded in).
+__shared__ uint32_t s_lane_turns[kTileSlots][32], s_warp_turns[kTileSlots][kTileThreads / 32];
+
+template <typename Prog>
+__device__ __forceinline__ void fill_turns(const Prog &pr, int nlg, int lane, int warp, uint32_t tidx) {
+    for (int i = warp; i < nlg; i += kTileThreads / 32) {
+        const LayerGate &g = pr.lg(i);
+        if (g.slot >= kTileSlots) continue;
+        const uint2 *w = reinterpret_cast<const uint2 *>(pr.bt() + g.first);
+        uint32_t a = 0, b = __float_as_uint(g.h.x);
+        for (int e = 0; e < g.nt; ++e) {
+            const uint2 x = w[e];
+            const uint32_t y = ((((uint32_t)lane | (uint32_t)lane << 5) >> x.x) & 1u) * x.y;   // bits 5..7: warp = lane
+            if (x.x < 5) a += y;
+            else b += y;
+        }
+        for (int e = g.nt; e < g.nt + g.ni; ++e) {
+            const uint2 x = w[e];
+            b += ((tidx >> x.x) & 1u) * x.y;
+        }
+        s_lane_turns[g.slot][lane] = a;
+        if (lane < kTileThreads / 32) s_warp_turns[g.slot][lane] = b;
+    }
+}
+
 // turns of nt terms on thread bits and ni on tile-index bits (uniform over the CTA)
 __device__ __forceinline__ uint32_t sum_terms(const BitTerm *t, int nt, int ni, uint32_t tbits, uint32_t tidx) {
     uint32_t acc = 0, uacc = 0;
@@ -310,13 +339,13 @@ __device__ __forceinline__ void lift(Regs &v, float2 c0, float2 c1) {
 // One gate of a TOP_U2L layer on register bit K.  w: the op's flags for the gate (see
 // TOP_U2L), already shifted to bit 0.
 template <int K>
-__device__ __forceinline__ void layer_gate(Regs &v, const LayerGate &g, const BitTerm *bt, int zf, int on, int sign,
-                                           int terms, uint32_t tbits, uint32_t tidx) {
+__device__ __forceinline__ void layer_gate(Regs &v, const LayerGate &g, int zf, int on, int sign, int terms,
+                                           uint32_t tbits, uint32_t tidx) {
     if ((sign | terms) & 1) {
         bool neg = false;
         if (sign & 1) neg = ((__popc(tbits & g.ts) + __popc(tidx & g.fs)) & 1) != 0;
         if (terms & 1) {
-            const uint32_t t = sum_terms(bt + g.first, g.nt, g.ni, tbits, tidx);
+            const uint32_t t = s_lane_turns[g.slot][tbits & 31u] + s_warp_turns[g.slot][tbits >> 5];
             if (t == kHalfTurn) neg = !neg;
             else if (t != 0u) bit_factor<K>(v, turns_to_phase(t));
         }
@@ -550,20 +579,27 @@ __device__ __forceinline__ void general_op(Regs &v, const TileOp &op, const BitT
             default: u2_packed<4>(v, m00, m01, m10, m11, op.rmask, op.rval); break;
         }
     } else {  // TOP_PHASE: factor where (register index & rmask) == rval
-        const int rm = op.rmask, rv = op.rval;
-        const float2 f = make_float2(op.ph.re, op.ph.im);
+        // register bit 0 picks the halves that take part, the others the float2 values
+        const int hm = op.rmask & ~1, hv = op.rval & ~1;
+        const bool lo = !(op.rmask & 1) || !(op.rval & 1), hi = !(op.rmask & 1) || (op.rval & 1);
+        if (op.ph.re == -1.f && op.ph.im == 0.f) {
+            const uint32_t sl = lo ? kHalfTurn : 0u, sh = hi ? kHalfTurn : 0u;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            if (((2 * j) & rm) == rv) {
-                const float xr = v.R[j].x, xi = v.I[j].x;
-                v.R[j].x = xr * f.x - xi * f.y;
-                v.I[j].x = xr * f.y + xi * f.x;
-            }
-            if (((2 * j + 1) & rm) == rv) {
-                const float xr = v.R[j].y, xi = v.I[j].y;
-                v.R[j].y = xr * f.x - xi * f.y;
-                v.I[j].y = xr * f.y + xi * f.x;
-            }
+            for (int j = 0; j < 16; ++j)
+                if (((2 * j) & hm) == hv) {
+                    v.R[j] = make_float2(xor_sign(v.R[j].x, sl), xor_sign(v.R[j].y, sh));
+                    v.I[j] = make_float2(xor_sign(v.I[j].x, sl), xor_sign(v.I[j].y, sh));
+                }
+        } else {
+            const float2 fr = make_float2(lo ? op.ph.re : 1.f, hi ? op.ph.re : 1.f);
+            const float2 fi = make_float2(lo ? op.ph.im : 0.f, hi ? op.ph.im : 0.f), nfi = neg2(fi);
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (((2 * j) & hm) == hv) {
+                    const float2 A = v.R[j], B = v.I[j];
+                    v.R[j] = ffma2(nfi, B, __fmul2_rn(fr, A));
+                    v.I[j] = ffma2(fi, A, __fmul2_rn(fr, B));
+                }
         }
     }
 }
@@ -645,7 +681,10 @@ __device__ __forceinline__ void tile_body(const Prog &pr, float2 *__restrict__ p
         }
 
         // while the loads are in flight: the phase table, the classical conditions
-        if (P.need_tab) fill_turn_table();
+        if (P.need_tab) {
+            fill_turn_table();
+            fill_turns(pr, P.nlg, lane, warp, (uint32_t)tile);
+        }
         unsigned condok = 0;
         for (int c = 0; c < P.n_conds; ++c) {
             bool ok = true;
@@ -665,13 +704,12 @@ __device__ __forceinline__ void tile_body(const Prog &pr, float2 *__restrict__ p
                 case TOP_U2L: {
                     if (h.czmask()) cz_mask(v, h.czmask());
                     const LayerGate *lg = &pr.lg(h.first());
-                    const BitTerm *bt = pr.bt();
                     const int bits = h.k(), zf = h.rmask(), on = h.rval(), sg = h.tval(), tm = h.count();
-                    if (bits & 1) layer_gate<0>(v, *lg++, bt, zf, on, sg, tm, tbits, tidx);
-                    if (bits & 2) layer_gate<1>(v, *lg++, bt, zf >> 1, on >> 1, sg >> 1, tm >> 1, tbits, tidx);
-                    if (bits & 4) layer_gate<2>(v, *lg++, bt, zf >> 2, on >> 2, sg >> 2, tm >> 2, tbits, tidx);
-                    if (bits & 8) layer_gate<3>(v, *lg++, bt, zf >> 3, on >> 3, sg >> 3, tm >> 3, tbits, tidx);
-                    if (bits & 16) layer_gate<4>(v, *lg, bt, zf >> 4, on >> 4, sg >> 4, tm >> 4, tbits, tidx);
+                    if (bits & 1) layer_gate<0>(v, *lg++, zf, on, sg, tm, tbits, tidx);
+                    if (bits & 2) layer_gate<1>(v, *lg++, zf >> 1, on >> 1, sg >> 1, tm >> 1, tbits, tidx);
+                    if (bits & 4) layer_gate<2>(v, *lg++, zf >> 2, on >> 2, sg >> 2, tm >> 2, tbits, tidx);
+                    if (bits & 8) layer_gate<3>(v, *lg++, zf >> 3, on >> 3, sg >> 3, tm >> 3, tbits, tidx);
+                    if (bits & 16) layer_gate<4>(v, *lg, zf >> 4, on >> 4, sg >> 4, tm >> 4, tbits, tidx);
                     break;
                 }
                 case TOP_PAIRNEG:

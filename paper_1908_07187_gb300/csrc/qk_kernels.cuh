@@ -391,16 +391,19 @@ __host__ __device__ constexpr int cz_index(int k, int l) { return k == 0 ? l - 1
 // the 30-qubit step.)  The updates leave s = 1 / (1 - a0 a1) in [1/2, 1] on one value;
 // the planner picks zf so that the bit's pending magnitude stays near 1.
 // The diagonal terms that wait on the qubit (the other qubit a thread or tile-index
-// bit) come first, on the bit's |1>: a sign by the parity of the thread bits ts and
-// tile-index bits fs, and a phase from nt + ni BitTerms.
+// bit) come first, on the bit's |1>: when all are signs, by the parity of the thread bits
+// ts and tile-index bits fs; else a phase from nt + ni BitTerms.  The turn is part of that
+// phase then (h.x holds its 2^-32 turns as an integer, and the op's rval bit is clear).
 struct LayerGate {
     float2 h, s;           // -tan(phi / 2), sin(phi), splatted
     float2 c0, c1;
     uint32_t fs;
     uint16_t ts, first;
     uint8_t nt, ni;
-    uint16_t pad;
+    uint8_t slot;          // of the phase in the kernel's tables, 0xff: no phase
+    uint8_t pad;
 };
+constexpr int kTileSlots = 48;   // 7.5 KB: three CTAs still share an SM
 static_assert(sizeof(LayerGate) == 48, "LayerGate layout");
 
 struct TileOp {

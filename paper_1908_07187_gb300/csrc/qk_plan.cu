@@ -734,15 +734,19 @@ struct TileBuilder : PendingTerms {
     int local_of[64], tile_of[64];
     int flip[kTileQubits] = {};
     int arr = ARR_IO;
-    int open = -1;           // index of the layer op that further gates may join, -1: none
+    // Index of the layer op that further gates may join, -1: none, and the register bits
+    // that ops after it depend on (a gate on one of them cannot go before those ops) and
+    // act on.
+    int open = -1, since = 0, since_u2 = 0;
+    int slots = 0;           // of the kernel's tables of turns, in use
     bool overflow = false;
 
     TileBuilder(TileParams &p, cdm *f, cdm &l) : PendingTerms(f, l), P(p) {}
 
     TileOp &add(uint8_t kind) {
-        open = -1;
         if (P.nops >= kTileMaxOps) {
             overflow = true;
+            open = -1;
             P.nops = 0;      // the program is thrown away
         }
         TileOp &o = P.ops[P.nops++];
@@ -761,6 +765,7 @@ struct TileBuilder : PendingTerms {
     void transpose_to(int a) {
         add(TOP_XPOSE).k = (uint8_t)a;
         arr = a;
+        open = -1;
     }
     int flip_of(int b) const { return local_of[b] >= 0 ? flip[local_of[b]] : 0; }
     // where physical qubit b is: 0 a register bit, 1 a thread bit, 2 a tile-index bit
@@ -802,6 +807,7 @@ struct TileBuilder : PendingTerms {
             if (flip_of(b)) val ^= 1ull << b;
         }
         encode_cond(mask, val, arr, local_of, o);
+        since |= o.rmask;
     }
     void set_cond(TileOp &o, const Cond &c) {
         for (int k = 0; k < P.n_conds; ++k)
@@ -818,6 +824,7 @@ struct TileBuilder : PendingTerms {
         if (turns == 0) return;
         if (k > l) std::swap(k, l);
         TileOp &o = add(turns == kHalf ? TOP_PAIRNEG : TOP_PAIRU);
+        since |= 1 << k | 1 << l;
         o.k = (uint8_t)(k | (l << 3));
         const double x = turns_angle(turns);
         o.ph.re = (float)std::cos(x);
@@ -866,6 +873,20 @@ struct TileBuilder : PendingTerms {
         terms.resize(w);
     }
 
+    // a phase on register bit k from thread and tile-index terms, as an op
+    void phase_op(int k, Touching &T) {
+        if (T.thread.empty() && T.tile.empty()) return;
+        TileOp &o = add(TOP_PHQ);
+        since |= 1 << k;
+        o.k = (uint8_t)k;
+        o.first = (uint16_t)P.nbt;
+        o.count = (uint16_t)T.thread.size();
+        o.count2 = (uint16_t)T.tile.size();
+        for (const BitTerm &t : T.thread) add_term(t.bit, t.turns);
+        for (const BitTerm &t : T.tile) add_term(t.bit, t.turns);
+        T.thread.clear();
+        T.tile.clear();
+    }
     // a 2x2 gate whose target is a register bit of the current arrangement
     void gate(const POp &p) {
         const FusedOp &op = *p.op;
@@ -877,20 +898,14 @@ struct TileBuilder : PendingTerms {
         if (op.cmask || op.cond.n || !real_form(op.m, 1e-7)) {
             for (const DTerm &t : T.other) direct(t.mask, t.val, t.f, t.cond);
             for (const auto &r : T.reg) pair_op(k, r.first, r.second);
-            if (!T.thread.empty() || !T.tile.empty()) {
-                TileOp &o = add(TOP_PHQ);
-                o.k = (uint8_t)k;
-                o.first = (uint16_t)P.nbt;
-                o.count = (uint16_t)T.thread.size();
-                o.count2 = (uint16_t)T.tile.size();
-                for (const BitTerm &t : T.thread) add_term(t.bit, t.turns);
-                for (const BitTerm &t : T.tile) add_term(t.bit, t.turns);
-            }
+            phase_op(k, T);
             if (F[b] != cdm(1.0, 0.0)) {
                 direct(1ull << b, 1ull << b, F[b], nullptr);
                 F[b] = 1.0;
             }
             TileOp &o = add(TOP_U2);
+            since |= 1 << k;
+            since_u2 |= 1 << k;
             conditions(o, op.cmask, op.cmask);
             if (op.cond.n) set_cond(o, op.cond);
             o.k = (uint8_t)k;
@@ -901,11 +916,20 @@ struct TileBuilder : PendingTerms {
             }
             return;
         }
-        // joins the open layer unless its bit is in it, or a term with one of the
-        // layer's bits (put there after that bit's gate) or a factor has to come first
-        bool join = open >= 0 && !((P.ops[open].k >> k) & 1) && T.other.empty();
+        // its waiting terms: signs by parity when they are all it has, else a phase
+        bool signs = true;
+        for (const BitTerm &t : T.thread) signs = signs && (t.turns == kHalf || t.turns == 0);
+        for (const BitTerm &t : T.tile) signs = signs && (t.turns == kHalf || t.turns == 0);
+        if (!signs && slots == kTileSlots) {   // no room in the tables
+            phase_op(k, T);
+            signs = true;
+        }
+        // joins the open layer unless its bit is in it or in a later op, or a term with
+        // one of the layer's bits (put there after that bit's gate) or a factor has to
+        // come first
+        bool join = open >= 0 && !(((P.ops[open].k | since) >> k) & 1) && T.other.empty();
         for (const auto &r : T.reg)
-            join = join && (r.second == kHalf || r.second == 0) && !((P.ops[open].k >> r.first) & 1);
+            join = join && (r.second == kHalf || r.second == 0) && !(((P.ops[open].k | since_u2) >> r.first) & 1);
         if (!join) {
             for (const DTerm &t : T.other) direct(t.mask, t.val, t.f, t.cond);
             for (const auto &r : T.reg)
@@ -913,6 +937,7 @@ struct TileBuilder : PendingTerms {
             TileOp &o = add(TOP_U2L);
             o.first = (uint16_t)P.nlg;
             open = P.nops - 1;
+            since = since_u2 = 0;
         }
         if (overflow || P.nlg >= kTileMaxMats) {
             overflow = true;
@@ -928,24 +953,31 @@ struct TileBuilder : PendingTerms {
         o.k |= (uint8_t)(1u << k);
         LayerGate &g = P.lg[at];
         std::memset(static_cast<void *>(&g), 0, sizeof g);
-        // its waiting terms: half turns by parity, the rest as phase terms
-        for (const BitTerm &t : T.thread)
-            if (t.turns == kHalf) g.ts ^= (uint16_t)(1u << t.bit);
-        for (const BitTerm &t : T.tile)
-            if (t.turns == kHalf) g.fs ^= 1u << t.bit;
-        if (g.ts || g.fs) o.tval |= (uint16_t)(1u << k);
+        g.slot = 0xff;
         g.first = (uint16_t)P.nbt;
-        for (const BitTerm &t : T.thread)
-            if (t.turns != kHalf && t.turns != 0) {
-                add_term(t.bit, t.turns);
-                ++g.nt;
+        for (const BitTerm &t : T.thread) {
+            if (t.turns == 0) continue;
+            if (signs) {
+                g.ts ^= (uint16_t)(1u << t.bit);
+                continue;
             }
-        for (const BitTerm &t : T.tile)
-            if (t.turns != kHalf && t.turns != 0) {
-                add_term(t.bit, t.turns);
-                ++g.ni;
+            add_term(t.bit, t.turns);
+            ++g.nt;
+        }
+        for (const BitTerm &t : T.tile) {
+            if (t.turns == 0) continue;
+            if (signs) {
+                g.fs ^= 1u << t.bit;
+                continue;
             }
-        if (g.nt || g.ni) o.count |= (uint16_t)(1u << k);
+            add_term(t.bit, t.turns);
+            ++g.ni;
+        }
+        if (g.ts || g.fs) o.tval |= (uint16_t)(1u << k);
+        if (!signs) {
+            o.count |= (uint16_t)(1u << k);
+            g.slot = (uint8_t)slots++;
+        }
         pivot(op.m, b, lq, k, o, g);
     }
 
@@ -978,9 +1010,14 @@ struct TileBuilder : PendingTerms {
                 p0 /= w.s;
             }
             auto splat = [](double x) { return make_float2((float)x, (float)x); };
-            if (std::abs(phi) > 0x1p-27) o.rval |= (uint8_t)(1u << k);   // below: less than a rounding error
-            g.h = splat(-std::tan(phi / 2));
-            g.s = splat(std::sin(phi));
+            if ((o.count >> k) & 1) {
+                const uint32_t t = angle_turns(phi);
+                std::memcpy(&g.h.x, &t, sizeof t);
+            } else {
+                if (std::abs(phi) > 0x1p-27) o.rval |= (uint8_t)(1u << k);   // below: less than a rounding error
+                g.h = splat(-std::tan(phi / 2));
+                g.s = splat(std::sin(phi));
+            }
             g.c0 = splat(b0);
             g.c1 = splat(b1);
         }
