@@ -362,9 +362,12 @@ struct Rewriter {
         out.push_back(op);
     }
 };
-// whether any gate is controlled or follows another on its qubit
-bool rewrites(const std::vector<FusedOp> &ops) {
-    uint64_t open = 0;
+// Whether the queue is worth rewriting: any controlled gate, or enough gates that follow
+// another on their qubit.  Rewriting takes 0.03 us per op of the queue, a gate less saves
+// 0.2 ms of a pass over 30 qubits and in proportion (21-qubit layers and QFT, 744 ops and
+// a handful of such gates: 298 us, with rewriting 320).
+bool rewrites(const std::vector<FusedOp> &ops, int n) {
+    uint64_t open = 0, merges = 0;
     for (const FusedOp &op : ops) {
         if (op.kind == FusedOp::PHASE) {
             open &= ~op.mask;
@@ -374,10 +377,11 @@ bool rewrites(const std::vector<FusedOp> &ops) {
             open &= ~(op.cmask | 1ull << op.q);
             continue;
         }
-        if (op.cmask || ((open >> op.q) & 1)) return true;
+        if (op.cmask) return true;
+        merges += (open >> op.q) & 1;
         open |= 1ull << op.q;
     }
-    return false;
+    return (merges << n) > ((uint64_t)ops.size() << 17);
 }
 
 // The gates one pass takes from rem for a qubit set S: in order, each gate
@@ -1068,7 +1072,7 @@ qk_status plan_passes(TilePlanner *planner, int n, const std::vector<FusedOp> &o
     std::vector<POp> rem;
     std::vector<FusedOp> rewritten_ops;
     const std::vector<FusedOp> *list = &ops;
-    if (rewrites(ops)) {
+    if (rewrites(ops, n)) {
         Rewriter rw(rewritten_ops);
         for (const FusedOp &op : ops) rw.add(op);
         list = &rewritten_ops;
