@@ -665,6 +665,13 @@ qk_status launch_large(qk_batch *b, const LargeRun &run) {
 }  // namespace
 
 namespace {
+// side stream k and its event, made when first used
+bool side_stream(qk_batch *b, int k) {
+    int prio = 0;
+    return b->side[k] || (cudaStreamGetPriority(b->stream, &prio) == cudaSuccess &&
+                          (b->join[k] || cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming) == cudaSuccess) &&
+                          cudaStreamCreateWithPriority(&b->side[k], cudaStreamNonBlocking, prio) == cudaSuccess);
+}
 // device -> host copy on the batch's stream, complete on return
 bool read_back(qk_batch *b, void *dst, const void *src, size_t bytes) {
     return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, b->stream) == cudaSuccess &&
@@ -697,14 +704,8 @@ qk_status qk_batch_create(qk_batch **out, void *cuda_stream) {
         }
         b->own_stream = true;
     }
-    bool ok = cudaEventCreate(&b->done) == cudaSuccess && cudaEventCreate(&b->start) == cudaSuccess &&
-              cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
-    int prio = 0;
-    ok = ok && cudaStreamGetPriority(b->stream, &prio) == cudaSuccess;
-    for (int k = 0; k < qk_batch::kSide && ok; ++k)
-        ok = cudaStreamCreateWithPriority(&b->side[k], cudaStreamNonBlocking, prio) == cudaSuccess &&
-             cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming) == cudaSuccess;
-    if (!ok) {
+    if (cudaEventCreate(&b->done) != cudaSuccess || cudaEventCreate(&b->start) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         qk_batch_destroy(b);
         return QK_ECUDA;
@@ -1008,7 +1009,8 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
             ++j;
         const int k = used % qk_batch::kSide;
         if ((i == 0 && (!own || j < sorted.size()) && cudaEventRecord(b->fork, b->stream) != cudaSuccess) ||
-            (!own && used < qk_batch::kSide && cudaStreamWaitEvent(b->side[k], b->fork, 0) != cudaSuccess)) {
+            (!own && used < qk_batch::kSide &&
+             (!side_stream(b, k) || cudaStreamWaitEvent(b->side[k], b->fork, 0) != cudaSuccess))) {
             st = bfail(b, QK_ECUDA, "batch: event failed");
             break;
         }
