@@ -89,21 +89,17 @@ DIAGONAL = {"z", "s", "sdg", "t", "tdg", "p", "rz"}
 
 
 def tile_fp32_ops(ops, n: int, tile_launches: float) -> float:
-    """FP32 lane operations the fused tile passes execute for a gate list (an
-    FMA counts as one): an uncontrolled non-diagonal 1-qubit gate is a pivot-form
-    butterfly, 8 FMAs per amplitude pair; a
-    controlled one a full complex 2x2 product on the pairs where the controls
-    hold, 16 per pair; diagonal gates are folded into pending phases (no
-    per-gate arithmetic); each pass ends with one complex factor per amplitude
-    (4 operations).  Flushes at transposes are left out (sign flips are integer
-    work; general phase flushes occur only in the QFT passes), so this is a
-    lower bound."""
+    """FP32 lane operations of a gate list's fused tile passes (an FMA counts as one),
+    as if no tile were all zeros (such tiles are skipped): an uncontrolled non-diagonal
+    1-qubit gate is 7 FMAs per amplitude pair (three shears that turn one value, four
+    updates), a controlled one at least one such gate beside phases; diagonal gates
+    become pending factors and phases of other gates (not counted); each pass ends with
+    one complex factor per amplitude (4 operations)."""
     f = 0.0
     for op in ops:
         if op.kind == "swap" or op.kind in DIAGONAL:
             continue
-        c = len(op.controls)
-        f += (8.0 if c == 0 else 16.0) * 2.0 ** (n - c - 1)
+        f += 7.0 * 2.0 ** (n - 1)
     return f + 4.0 * 2.0 ** n * tile_launches
 
 
@@ -898,7 +894,8 @@ def main():
 
     # roofline for the kernel class with the largest device-time share: HBM,
     # the algorithmic bytes of one launch (a tile pass reads and writes the state
-    # once: 2^n x 8 B x 2) over the launch's average CUDA-event time
+    # once: 2^n x 8 B x 2; tiles of zeros, in a step's first passes, are only read)
+    # over the launch's average CUDA-event time
     top = max(prof, key=lambda k: prof[k]["ms"])
     rec = prof[top]
     peak, peak_kind = peaks()
@@ -915,7 +912,7 @@ def main():
                 "alg_bytes_per_launch": alg_bytes, "avg_launch_ms": round(1000.0 * per_launch_s, 4)}
     roofline_fp32 = None
     if top == "tile":
-        # the same passes against the FP32 lane rate, counting what the kernel executes
+        # the same passes against the FP32 lane rate
         sm_count = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
         sm_mhz = clk.get("sm_mhz") or 2070.0
         launches_step = rec["launches"] / args.steps
@@ -927,8 +924,8 @@ def main():
                          "ops_per_step": ops_step,
                          "peak_kind": f"derived: {sm_count} SMs x 128 FP32 lanes x {sm_mhz:.0f} MHz (median SM clock "
                                       "sampled during the timed region)",
-                         "count": "8 per amplitude pair per uncontrolled non-diagonal gate, 16 per acting pair per "
-                                  "controlled one, 4 per amplitude per pass (final phase and scale); lower bound"}
+                         "count": "7 per amplitude pair per non-diagonal gate, 4 per amplitude per pass (final phase "
+                                  "and scale), as if no tile were all zeros (those are skipped)"}
 
     # secondary measurements: a failure in one is recorded under its key and
     # the line is still printed
