@@ -11,10 +11,10 @@
 // arithmetic.  The tile width falls with the state (planner) so that small states
 // still spread over the SMs.  Measured against one pass per gate: a 23-qubit
 // complex128 circuit of 161 U3, 139 CZ and the QFT 33.0 -> 10.7 ms (six passes; the
-// FP64 unit's own time for its 5.2 G instructions per lane is 8.3 ms), the 12-qubit
-// complex128 circuit of 290 gates 1322 -> 333 us (bound by the latency of one short op
-// after another), a 10-qubit complex64 circuit of 175 gates, viewed and measured, 828
-// -> 158 us.
+// FP64 unit's own time for its 5.2 G instructions per lane is 8.3 ms) and to 6.0 ms with
+// tiles of zeros left alone, the 12-qubit complex128 circuit of 290 gates 1322 -> 318 us
+// (bound by the latency of one short op after another), a 10-qubit complex64 circuit of
+// 175 gates, viewed and measured, 828 -> 153 us.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -188,6 +188,15 @@ __global__ void __launch_bounds__(kMaxThreads, 3)
                 }
         }
     }
+    // The ops go to shared memory while the tile's loads are in flight: read from the
+    // kernel parameters, each one's first touch waited for the constant cache (12 qubits
+    // complex128 333 -> 318 us, 10 qubits complex64 159 -> 153, 12 qubits 275 -> 259).
+    // Through a generic address, so that lanes read neighbouring words.
+    const uint2 *src = reinterpret_cast<const uint2 *>(P.ops);
+    asm volatile("" : "+l"(src));
+    uint2 *staged = reinterpret_cast<uint2 *>(hi + 64);
+    for (int w = tid; w < P.nops * (int)(sizeof(SmemTileOp) / sizeof(uint2)); w += nt) staged[w] = src[w];
+    const SmemTileOp *ops = reinterpret_cast<const SmemTileOp *>(staged);
     unsigned condok = 0;
     for (int c = 0; c < P.n_conds; ++c) {
         bool ok = true;
@@ -200,7 +209,7 @@ __global__ void __launch_bounds__(kMaxThreads, 3)
     if (!__syncthreads_or(seen != 0u)) return;
 
     for (int o = 0; o < P.nops; ++o) {
-        const SmemTileOp &op = P.ops[o];
+        const SmemTileOp &op = ops[o];
         const int q = op.q;
         switch (op.kind) {
             case ST_U2: {
@@ -297,7 +306,7 @@ __global__ void __launch_bounds__(kMaxThreads, 3)
 template <typename R>
 static cudaError_t smem_tile_r(void *psi, const SmemTileParams &p, const uint8_t *cbits, unsigned nt, cudaStream_t s) {
     using T = typename Amp<R>::T;
-    const size_t sm = sizeof(T) * (((size_t)1 << p.m) + 128);
+    const size_t sm = sizeof(T) * (((size_t)1 << p.m) + 128) + sizeof(SmemTileOp) * (size_t)p.nops;
     if (sm > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(k_smem_tile<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;

@@ -538,6 +538,7 @@ struct SmemTileOp {
         float cf[8];                 // in complex64 programs
     };
 };
+static_assert(sizeof(SmemTileOp) % 8 == 0, "copied as 8-byte words");
 struct SmemTileParams {
     uint32_t n_tiles;
     int n, m, nfix;
