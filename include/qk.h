@@ -65,8 +65,9 @@ typedef enum { QK_C64 = 0, QK_C128 = 1 } qk_precision;
 
 /* Execution modes.  PLAIN: one kernel pass over the state per gate (the
  * unfused baseline).  FUSED: gates are queued; at a flush point a planner groups
- * runs of gates into shared-memory tile passes, so several gates cost one HBM
- * read+write of the state. */
+ * runs of gates (1-target gates, and dense gates of one size) into tile passes, so
+ * several gates cost one HBM read+write of the state, in both precisions and at any
+ * size. */
 typedef enum { QK_EXEC_PLAIN = 0, QK_EXEC_FUSED = 1 } qk_exec_mode;
 
 typedef struct {

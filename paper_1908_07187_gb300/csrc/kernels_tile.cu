@@ -23,7 +23,9 @@
 // so threads in flight count: without carried phases the kernel fits 80 registers and
 // three CTAs share an SM.  Tile passes of the 30-qubit layered step: 100.1 ms with
 // carried phases, complex updates and two CTAs per SM (128 registers), 95.5 ms with the
-// terms applied once, 75.3 ms with the third CTA.
+// terms applied once, 75.3 ms with the third CTA, 69.9 ms with phase sums from tables,
+// 42.8 ms with tiles of zeros left alone.  A full pass has the FMA pipe 57 % and issue 63 %
+// busy.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

@@ -334,9 +334,10 @@ struct RelabelArgs {
 constexpr int kTileQubits = 13;
 // Physical qubits 0 .. kTileContig-1 belong to every tile pass, so a warp's loads
 // and stores touch runs of 2^kTileContig contiguous amplitudes; the other tile
-// qubits are chosen freely by the planner.  With 3 the layered 30-qubit circuit
-// needs 10 passes instead of 15 but takes as long: the pass is bound by
-// instruction issue, and its HBM traffic already overlaps the gate arithmetic.
+// qubits are chosen freely by the planner.  With 4 or 3 passes hold more gates but
+// cost more transposes: the layered 30-qubit step 56.7 and 54.4 ms against 51.1, a
+// 26-qubit request 4.53 and 4.60 against 4.42; better only without a QFT (28 qubits 8.27
+// and 8.10 against 8.70).
 constexpr int kTileContig = 5;
 constexpr int kTileThreads = 256;
 constexpr int kTileMaxOps = 192;
