@@ -73,3 +73,28 @@ def test_permutations_stay_exact(n):
     want = np.zeros(1 << n, dtype=np.complex64)
     want[at] = 1.0
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("n", [13, 14])
+def test_more_phases_than_table_slots(n):
+    """Every gate with phase terms from other qubits: more of them in a pass than the
+    kernel's tables have slots."""
+    from paper_1908_07187_gb300 import qk
+
+    r = np.random.Generator(np.random.PCG64(n))
+    ops = []
+    for _ in range(9):
+        for q in range(n):
+            for d in (3, 5, 8):
+                ops.append(workloads.Op("p", (q,), controls=((q + d) % n,), params=(float(r.uniform(0, 6.28)),)))
+            ops.append(workloads.Op("u3", (q,), params=tuple(float(x) for x in r.uniform(0, 6.28, 3))))
+    psi = workloads.random_state(n, 2)
+    with qk.Context("c64") as ctx:
+        ctx.add_qubits(n)
+        ctx.set_state(psi)
+        qk.run_ops(ctx, ops)
+        got = ctx.get_state()
+    ref = oracle.OracleState(n, 0, psi)
+    for op in ops:
+        ref.apply_op(op)
+    assert np.max(np.abs(got - ref.psi)) <= 1e-5 * np.max(np.abs(ref.psi))
