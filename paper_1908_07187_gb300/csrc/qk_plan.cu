@@ -1070,7 +1070,7 @@ qk_status plan_passes(TilePlanner *planner, int n, const std::vector<FusedOp> &o
                       const char **err) {
     *err = "";
     std::vector<POp> rem;
-    std::vector<FusedOp> rewritten_ops;
+    static thread_local std::vector<FusedOp> rewritten_ops;
     const std::vector<FusedOp> *list = &ops;
     if (rewrites(ops, n)) {
         Rewriter rw(rewritten_ops);
