@@ -818,16 +818,21 @@ __device__ __forceinline__ void tile_body(const Prog &pr, float2 *__restrict__ p
 
 // one tile per CTA (a grid-stride loop would keep the tile's addressing state
 // live across iterations and push the kernel into spills)
-template <typename Off, bool GEN>
-__global__ void __launch_bounds__(kTileThreads, 3)
+// CTAS: resident CTAs per SM the registers are cut to.  Up to two tiles per SM a third
+// CTA has nothing to run, and the instance with 128 registers has no spills (a batch of
+// five circuits of 18 to 20 qubits: 3.33 -> 3.10 ms on the device; 14 to 21 qubits 0-3 % of
+// a whole call; above, three CTAs: 95.5 -> 75.3 ms of the 30-qubit step's passes).
+constexpr uint64_t kFewTiles = 2 * 152;
+template <typename Off, bool GEN, int CTAS>
+__global__ void __launch_bounds__(kTileThreads, CTAS)
     k_tile(float2 *__restrict__ psi, const __grid_constant__ TileParams P, const uint8_t *__restrict__ cbits) {
     tile_body<Off, GEN>(ParamProg{P}, psi, blockIdx.x, cbits);
 }
 
 // Batched: CTA b finds its program by binary search in first[] (uniform over
 // the CTA) and runs that program's tile b - first[c] on the program's state.
-template <bool GEN>
-__global__ void __launch_bounds__(kTileThreads, 3)
+template <bool GEN, int CTAS>
+__global__ void __launch_bounds__(kTileThreads, CTAS)
     k_tile_batch(const TileProg *__restrict__ progs, const uint32_t *__restrict__ first, int n_progs,
                  const TileOp *__restrict__ ops, const LayerGate *__restrict__ lg, const BitTerm *__restrict__ bt) {
     int lo = 0, hi = n_progs - 1;
@@ -867,12 +872,12 @@ bool needs_general(const TileOp *ops, size_t n) {
     return false;
 }
 
-template <typename Off, bool GEN>
+template <typename Off, bool GEN, int CTAS>
 cudaError_t launch_tile_g(void *psi, const TileParams &p, const uint8_t *cbits, cudaStream_t s) {
     static std::atomic<bool> attr_set[64];
-    const cudaError_t e = tile_smem_attr(k_tile<Off, GEN>, attr_set);
+    const cudaError_t e = tile_smem_attr(k_tile<Off, GEN, CTAS>, attr_set);
     if (e != cudaSuccess) return e;
-    k_tile<Off, GEN><<<(unsigned)p.n_tiles, kTileThreads, kTileSmem, s>>>((float2 *)psi, p, cbits);
+    k_tile<Off, GEN, CTAS><<<(unsigned)p.n_tiles, kTileThreads, kTileSmem, s>>>((float2 *)psi, p, cbits);
     return cudaGetLastError();
 }
 
@@ -880,17 +885,20 @@ template <typename Off>
 cudaError_t launch_tile_t(void *psi, const TileParams &p, const uint8_t *cbits, cudaStream_t s) {
     if (p.n_tiles == 0 || p.n_tiles > (1ull << 31) - 1) return cudaErrorInvalidValue;
     if (p.nops < 0 || p.nops > kTileMaxOps) return cudaErrorInvalidValue;
-    if (needs_general(p.ops, (size_t)p.nops)) return launch_tile_g<Off, true>(psi, p, cbits, s);
-    return launch_tile_g<Off, false>(psi, p, cbits, s);
+    const bool gen = needs_general(p.ops, (size_t)p.nops);
+    if constexpr (sizeof(Off) == 4)
+        if (p.n_tiles <= kFewTiles)
+            return gen ? launch_tile_g<Off, true, 2>(psi, p, cbits, s) : launch_tile_g<Off, false, 2>(psi, p, cbits, s);
+    return gen ? launch_tile_g<Off, true, 3>(psi, p, cbits, s) : launch_tile_g<Off, false, 3>(psi, p, cbits, s);
 }
 
-template <bool GEN>
+template <bool GEN, int CTAS>
 cudaError_t launch_tile_batch_g(const TileProg *progs, const uint32_t *first, int n_progs, uint32_t n_ctas,
                                 const TileOp *ops, const LayerGate *lg, const BitTerm *bt, cudaStream_t s) {
     static std::atomic<bool> attr_set[64];
-    const cudaError_t e = tile_smem_attr(k_tile_batch<GEN>, attr_set);
+    const cudaError_t e = tile_smem_attr(k_tile_batch<GEN, CTAS>, attr_set);
     if (e != cudaSuccess) return e;
-    k_tile_batch<GEN><<<n_ctas, kTileThreads, kTileSmem, s>>>(progs, first, n_progs, ops, lg, bt);
+    k_tile_batch<GEN, CTAS><<<n_ctas, kTileThreads, kTileSmem, s>>>(progs, first, n_progs, ops, lg, bt);
     return cudaGetLastError();
 }
 
@@ -900,8 +908,11 @@ cudaError_t launch_tile_batch(const TileProg *progs, const uint32_t *first, int 
                               const TileOp *ops, const LayerGate *lg, const BitTerm *bt, bool general,
                               cudaStream_t s) {
     if (n_progs <= 0 || n_ctas == 0) return cudaSuccess;
-    if (general) return launch_tile_batch_g<true>(progs, first, n_progs, n_ctas, ops, lg, bt, s);
-    return launch_tile_batch_g<false>(progs, first, n_progs, n_ctas, ops, lg, bt, s);
+    if (n_ctas <= kFewTiles)
+        return general ? launch_tile_batch_g<true, 2>(progs, first, n_progs, n_ctas, ops, lg, bt, s)
+                       : launch_tile_batch_g<false, 2>(progs, first, n_progs, n_ctas, ops, lg, bt, s);
+    return general ? launch_tile_batch_g<true, 3>(progs, first, n_progs, n_ctas, ops, lg, bt, s)
+                   : launch_tile_batch_g<false, 3>(progs, first, n_progs, n_ctas, ops, lg, bt, s);
 }
 
 bool tile_ops_need_general(const TileOp *ops, size_t n) { return needs_general(ops, n); }

@@ -33,8 +33,9 @@ def ops_for(n, style, seed):
     return ops
 
 
-@pytest.mark.parametrize("style", ["controls", "angles", "runs"])
-@pytest.mark.parametrize("n", [13, 14, 16])
+# 21 and 22 qubits: either side of the kernel's two register budgets
+@pytest.mark.parametrize("n,style", [(n, style) for n in (13, 14, 16) for style in ("controls", "angles", "runs")]
+                         + [(21, "controls"), (22, "controls")])
 def test_against_oracle(n, style):
     from paper_1908_07187_gb300 import qk
 
