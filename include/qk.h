@@ -293,9 +293,11 @@ qk_status qk_graph_destroy(qk_graph *g);
  * pass index of the large circuits) on the batch's stream without waiting;
  * qk_batch_done polls; qk_batch_read waits and copies a circuit's cbits and
  * final state (always kept for large circuits, for small ones if stored).  Add
- * ops to the most recently added circuit.  qk_batch_clear waits for a previous
+ * ops to the most recently added circuit.  Circuits may be added after a run; what
+ * can be read then is still that run's circuits.  qk_batch_clear waits for a previous
  * run and empties the batch.  Errors: QK_EINVAL (sizes, qubit lists, params),
- * QK_ENOTBIJECTIVE, QK_ESTATE (op before any circuit), QK_ENOMEM, QK_ECUDA;
+ * QK_ENOTBIJECTIVE, QK_ESTATE (op before any circuit, read of what the last run did
+ * not hold), QK_ENOMEM, QK_ECUDA;
  * message in qk_batch_last_error. */
 typedef struct qk_batch qk_batch;
 qk_status qk_batch_create(qk_batch **out, void *cuda_stream);

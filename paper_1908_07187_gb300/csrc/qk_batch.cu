@@ -341,6 +341,11 @@ struct qk_batch {
     bool h_valid = false;
     int reads = 0;                     // circuits read since the last run
     std::mutex read_mu;                // reads from several threads
+    // What the last run launched, which is what the device buffers hold: circuits may be
+    // added after it, and a read takes its sizes from here (0: nothing has run).
+    int run_circs = 0;
+    size_t run_amps = 0;
+    uint32_t run_cb = 0;
     bool start_recorded = false;
     bool store_state = true;
     std::string err;
@@ -753,6 +758,9 @@ qk_status qk_batch_clear(qk_batch *b) {
     b->large_amps = 0;
     b->h_valid = false;
     b->reads = 0;
+    b->run_circs = 0;
+    b->run_amps = 0;
+    b->run_cb = 0;
     return QK_OK;
 }
 
@@ -947,6 +955,7 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
     b->large_launches = 0;
     b->h_valid = false;
     b->reads = 0;
+    b->run_circs = 0;
     // host work first -- the large circuits' plans, the small ones' matrices -- then the
     // start event, after which everything is enqueued back to back
     LargeRun lr;
@@ -1029,6 +1038,9 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
             st = bfail(b, QK_ECUDA, "batch: event failed");
     if (st != QK_OK) return st;
     if (cudaEventRecord(b->done, b->stream) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event record failed");
+    b->run_circs = (int)b->circs.size();
+    b->run_amps = b->total_amps;
+    b->run_cb = b->total_cb;
     return QK_OK;
 }
 
@@ -1062,6 +1074,7 @@ int qk_batch_done(qk_batch *b) {
 qk_status qk_batch_read(qk_batch *b, int circuit, uint8_t *cbits, int ncb, void *state, size_t bytes) {
     if (!b) return QK_EINVAL;
     if (circuit < 0 || circuit >= (int)b->circs.size()) return bfail(b, QK_EINVAL, "batch: bad circuit index");
+    if (circuit >= b->run_circs) return bfail(b, QK_ESTATE, "batch: circuit %d is not in the last run", circuit);
     const qk::BCirc &c = b->circs[circuit];
     if (ncb < 0 || ncb > (int)c.ncb || (ncb > 0 && !cbits)) return bfail(b, QK_EINVAL, "batch: bad cbit count");
     const bool large = (c.flags & 2u) != 0;
@@ -1070,13 +1083,13 @@ qk_status qk_batch_read(qk_batch *b, int circuit, uint8_t *cbits, int ncb, void 
     if (cudaEventSynchronize(b->done) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event wait failed");
     // A program that reads a second circuit reads many: all the small ones come over in
     // one copy then (up to 64 MB of states), instead of two copies and waits for each.
-    const size_t all = b->store_state ? sizeof(float2) * b->total_amps : 0;
+    const size_t all = b->store_state ? sizeof(float2) * b->run_amps : 0;
     const std::lock_guard<std::mutex> lk(b->read_mu);
-    if (++b->reads == 2 && !b->h_valid && b->circs.size() > 2 && all <= (64u << 20)) {
+    if (++b->reads == 2 && !b->h_valid && b->run_circs > 2 && all <= (64u << 20)) {
         b->h_states.resize(all);
-        b->h_cbits.resize(b->total_cb);
+        b->h_cbits.resize(b->run_cb);
         b->h_valid = (all == 0 || cudaMemcpyAsync(b->h_states.data(), b->d_states, all, cudaMemcpyDeviceToHost, b->stream) == cudaSuccess) &&
-                     (b->total_cb == 0 || cudaMemcpyAsync(b->h_cbits.data(), b->d_cbits, b->total_cb, cudaMemcpyDeviceToHost, b->stream) == cudaSuccess) &&
+                     (b->run_cb == 0 || cudaMemcpyAsync(b->h_cbits.data(), b->d_cbits, b->run_cb, cudaMemcpyDeviceToHost, b->stream) == cudaSuccess) &&
                      cudaStreamSynchronize(b->stream) == cudaSuccess;
         if (!b->h_valid) return bfail(b, QK_ECUDA, "batch: copy failed");
     }
@@ -1098,6 +1111,7 @@ qk_status qk_batch_read(qk_batch *b, int circuit, uint8_t *cbits, int ncb, void 
 qk_status qk_batch_read_all_cbits(qk_batch *b, uint8_t *out, size_t n) {
     if (!b) return QK_EINVAL;
     if (n != b->total_cb || (n > 0 && !out)) return bfail(b, QK_EINVAL, "batch: need %u cbit bytes", b->total_cb);
+    if (n != b->run_cb) return bfail(b, QK_ESTATE, "batch: circuits with cbits were added since the last run");
     if (cudaEventSynchronize(b->done) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event wait failed");
     if (n > 0 && !read_back(b, out, b->d_cbits, n)) return bfail(b, QK_ECUDA, "batch: cbit copy failed");
     return QK_OK;
