@@ -735,10 +735,9 @@ static cudaError_t modexp_r(const void *in, void *out, const ModExpArgs &a, cons
         return cudaGetLastError();
     }
     const size_t sm = sizeof(T) << (t.w + t.cb);
-    if (sm > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_modexp_tiled<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = smem_limit(k_modexp_tiled<R>, (size_t)128 * 1024, limit);
+    if (e != cudaSuccess) return e;
     const uint64_t cap = (uint64_t)sms * (sm > 100 * 1024 ? 1 : sm > 48 * 1024 ? 3 : 6);
     k_modexp_tiled<R><<<(unsigned)(t.n_tiles < cap ? t.n_tiles : cap), kThreads, sm, s>>>((const T *)in, (T *)out, t, cbits);
     return cudaGetLastError();

@@ -295,11 +295,10 @@ template <typename R, int K, int RT, int CT>
 cudaError_t dense_k(void *psi, const DenseParams &p, const uint8_t *cbits, int sms, cudaStream_t s) {
     using T = typename Amp<R>::T;
     const size_t sm = (sizeof(T) << p.m) + sizeof(T) * ((size_t)p.nops << (2 * K));
-    if (sm > 47 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_dense<R, K, RT, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    static SmemLimit limit;
+    const cudaError_t e =
+        smem_limit(k_dense<R, K, RT, CT>, sizeof(T) * (((size_t)1 << kDenseMaxBits) + kDenseElems), limit);
+    if (e != cudaSuccess) return e;
     const uint64_t cap = (uint64_t)sms * dense_ctas<R, K, RT>();
     k_dense<R, K, RT, CT><<<(unsigned)(p.n_tiles < cap ? p.n_tiles : cap), kThreads, sm, s>>>((T *)psi, p, cbits);
     return cudaGetLastError();

@@ -307,10 +307,10 @@ template <typename R>
 static cudaError_t smem_tile_r(void *psi, const SmemTileParams &p, const uint8_t *cbits, unsigned nt, cudaStream_t s) {
     using T = typename Amp<R>::T;
     const size_t sm = sizeof(T) * (((size_t)1 << p.m) + 128) + sizeof(SmemTileOp) * (size_t)p.nops;
-    if (sm > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_smem_tile<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = smem_limit(
+        k_smem_tile<R>, sizeof(T) * (((size_t)1 << kSmemTileMax) + 128) + sizeof(SmemTileOp) * kSmemTileOps, limit);
+    if (e != cudaSuccess) return e;
     k_smem_tile<R><<<p.n_tiles, nt, sm, s>>>((T *)psi, p, cbits);
     return cudaGetLastError();
 }

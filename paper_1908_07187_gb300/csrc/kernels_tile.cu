@@ -29,7 +29,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
 #include <utility>
 
 #include "qk_kernels.cuh"
@@ -849,22 +848,6 @@ __global__ void __launch_bounds__(kTileThreads, CTAS)
 // transposes (2^13 complex64)
 constexpr int kTileSmem = (int)(2 * sizeof(float)) << kTileQubits;
 
-// the dynamic shared-memory attribute of kernel f, set once per device (host
-// threads of the serving loop may launch concurrently; setting it twice is harmless)
-template <typename F>
-cudaError_t tile_smem_attr(F *f, std::atomic<bool> (&set)[64]) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!set[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
-        if (e != cudaSuccess) return e;
-        set[dev].store(true, std::memory_order_release);
-    }
-    return cudaSuccess;
-}
-
 // whether a program needs the general-op path of the kernel
 bool needs_general(const TileOp *ops, size_t n) {
     for (size_t i = 0; i < n; ++i)
@@ -874,8 +857,8 @@ bool needs_general(const TileOp *ops, size_t n) {
 
 template <typename Off, bool GEN, int CTAS>
 cudaError_t launch_tile_g(void *psi, const TileParams &p, const uint8_t *cbits, cudaStream_t s) {
-    static std::atomic<bool> attr_set[64];
-    const cudaError_t e = tile_smem_attr(k_tile<Off, GEN, CTAS>, attr_set);
+    static SmemLimit limit;
+    const cudaError_t e = smem_limit(k_tile<Off, GEN, CTAS>, kTileSmem, limit);
     if (e != cudaSuccess) return e;
     k_tile<Off, GEN, CTAS><<<(unsigned)p.n_tiles, kTileThreads, kTileSmem, s>>>((float2 *)psi, p, cbits);
     return cudaGetLastError();
@@ -895,8 +878,8 @@ cudaError_t launch_tile_t(void *psi, const TileParams &p, const uint8_t *cbits, 
 template <bool GEN, int CTAS>
 cudaError_t launch_tile_batch_g(const TileProg *progs, const uint32_t *first, int n_progs, uint32_t n_ctas,
                                 const TileOp *ops, const LayerGate *lg, const BitTerm *bt, cudaStream_t s) {
-    static std::atomic<bool> attr_set[64];
-    const cudaError_t e = tile_smem_attr(k_tile_batch<GEN, CTAS>, attr_set);
+    static SmemLimit limit;
+    const cudaError_t e = smem_limit(k_tile_batch<GEN, CTAS>, kTileSmem, limit);
     if (e != cudaSuccess) return e;
     k_tile_batch<GEN, CTAS><<<n_ctas, kTileThreads, kTileSmem, s>>>(progs, first, n_progs, ops, lg, bt);
     return cudaGetLastError();

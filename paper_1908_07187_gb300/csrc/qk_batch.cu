@@ -999,9 +999,9 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
             cudaMemcpyAsync(b->d_circs, (char *)b->h_stage + ob, cb, cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
             return bfail(b, QK_ECUDA, "batch: upload failed");
     }
-    const size_t max_smem = sizeof(float2) * 2 * ((size_t)1 << b->max_n);
-    if (!sorted.empty() && max_smem > 40 * 1024 &&
-        cudaFuncSetAttribute(qk::k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem) != cudaSuccess)
+    static qk::SmemLimit limit;
+    if (!sorted.empty() &&
+        qk::smem_limit(qk::k_batch, sizeof(float2) * 2 * ((size_t)1 << qk::kBMaxQubits), limit) != cudaSuccess)
         return bfail(b, QK_ECUDA, "batch: shared memory attribute failed");
     // The launches run beside each other and beside the tile passes: each is as long as
     // its longest circuit and most leave SMs free.  (One after another on one stream, the

@@ -6,7 +6,29 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace qk {
+
+// The dynamic shared-memory limit of a kernel belongs to the function on its device and
+// not to the calling thread: set before a launch to that launch's size, a second thread
+// lowers it in between and the first one's launch is refused.  So it is set once per
+// device, to the most that any launch of the kernel asks for (twice by two threads at
+// once is harmless: the value is the same).
+struct SmemLimit {
+    std::atomic<bool> set[64] = {};
+};
+template <typename F>
+inline cudaError_t smem_limit(F *f, size_t most, SmemLimit &l) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (l.set[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e == cudaSuccess) l.set[dev].store(true, std::memory_order_release);
+    return e;
+}
 
 constexpr int kMaxPos = 24;        // sorted bit positions a launch may insert
 constexpr int kMaxCond = 16;       // classical-condition cbits per gate
