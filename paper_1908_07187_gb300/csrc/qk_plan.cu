@@ -242,9 +242,11 @@ GateForm gate_form(const cdm *M, cdm f) {
     g.p1 = W[3] * f;
     return g;
 }
-// whether a0 a1 is real and not positive (GateForm): a matrix defined with a loose
-// tolerance need not be so
+// whether a0 a1 is real and not positive, and both of them or neither is 0 (a phase taken
+// from a0 alone says nothing of a1 then): GateForm holds only so, and a matrix defined
+// with a loose tolerance need not be so
 bool real_form(const cdm *M, double tol) {
+    if ((M[1] == 0.0) != (M[2] == 0.0)) return false;
     const cdm pr = M[1] * M[2] * std::conj(M[0] * M[3]);
     return std::abs(pr.imag()) <= tol * std::abs(pr) && pr.real() <= 0.0;
 }

@@ -1,0 +1,56 @@
+"""One-qubit matrices that a wide unitarity tolerance lets in, among ordinary gates: the
+fused passes (both tile kinds, and the widths' edges) take them as they are, as one pass per
+gate does.  Bounds: a unit of the working precision per gate (40 gates), relative to the
+largest amplitude."""
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+SIZES = [("c128", 3), ("c128", 9), ("c128", 13), ("c64", 2), ("c64", 9), ("c64", 12), ("c64", 13), ("c64", 15)]
+TOL = {"c64": 40 * 2.0 ** -24, "c128": 40 * 2.0 ** -53}
+
+
+def both_modes(n, prec, ops):
+    """ops: (matrix, target, controls) in order; fused against plain."""
+    from paper_1908_07187_gb300 import qk
+
+    psi = workloads.random_state(n, 70 + n)
+    got = []
+    for mode in ("fused", "plain"):
+        with qk.Context(prec, mode) as ctx:
+            ctx.add_qubits(n)
+            ctx.set_state(psi)
+            for m, q, ctl in ops:
+                ctx.apply_gate(ctx.define_gate_matrix(m, tol=1e9), (q,), ctl)
+            got.append(ctx.get_state())
+    assert np.all(np.isfinite(got[0]))
+    assert np.max(np.abs(got[0] - got[1])) <= TOL[prec] * np.max(np.abs(got[1]))
+
+
+def among_gates(n, seed, special, often=3, most=40):
+    """40 gates, every third on average special(r), some controlled, with diagonal terms
+    between neighbours that wait over the gates."""
+    r = np.random.Generator(np.random.PCG64([n, seed]))
+    ops, used = [], 0
+    for _ in range(40):
+        q, d = (int(x) for x in r.permutation(n)[:2])
+        m, _ = np.linalg.qr(r.standard_normal((2, 2)) + 1j * r.standard_normal((2, 2)))
+        if used < most and r.integers(often) == 0:
+            m = special(r)
+            used += 1
+        ops.append((m, q, (d,) if r.random() < 0.3 else ()))
+        if r.random() < 0.5:
+            ops.append((np.diag([1, -1 if r.random() < 0.5 else np.exp(1j * r.uniform(0, 6))]), d, (q,)))
+    return ops
+
+
+@pytest.mark.parametrize("prec,n", SIZES)
+@pytest.mark.parametrize("lower", [False, True])
+def test_triangular(n, prec, lower):
+    def special(r):
+        m = np.diag(np.exp(1j * r.uniform(0, 6, 2)))
+        m[(1, 0) if lower else (0, 1)] = 0.3 * (r.standard_normal() + 1j * r.standard_normal())
+        return m
+    both_modes(n, prec, among_gates(n, 1 + lower, special))
