@@ -793,6 +793,10 @@ struct TileBuilder : PendingTerms {
             F[b] *= std::polar(1.0, x);
         }
     }
+    // Waiting pairs are kept as turns, which hold no magnitude: a pair from a diagonal
+    // matrix that is not unitary to an FP32 rounding error (defined with a wide tolerance)
+    // goes out as a direct factor instead.
+    static bool is_turn(const DTerm &t) { return is_pair(t) && std::abs(std::norm(t.f) - 1.0) <= 0x1p-23; }
     // e^{i th} where the true values of a and b are both 1, in stored values sa, sb: (sa ^
     // fa)(sb ^ fb) = fa fb + fa (1 - 2 fb) sb + fb (1 - 2 fa) sa + (1 - 2 fa)(1 - 2 fb) sa
     // sb.  The constant and the single-bit parts become pending; returns the turns left
@@ -865,7 +869,7 @@ struct TileBuilder : PendingTerms {
                 terms[w++] = t;
                 continue;
             }
-            if (!is_pair(t)) {
+            if (!is_turn(t)) {
                 out.other.push_back(t);
                 continue;
             }
@@ -1037,7 +1041,7 @@ struct TileBuilder : PendingTerms {
     void finish_terms() {
         std::vector<BitTerm> th[5], ti[5], two;
         for (const DTerm &t : terms) {
-            if (!is_pair(t)) {
+            if (!is_turn(t)) {
                 direct(t.mask, t.val, t.f, t.cond);
                 continue;
             }

@@ -54,3 +54,10 @@ def test_triangular(n, prec, lower):
         m[(1, 0) if lower else (0, 1)] = 0.3 * (r.standard_normal() + 1j * r.standard_normal())
         return m
     both_modes(n, prec, among_gates(n, 1 + lower, special))
+
+
+@pytest.mark.parametrize("prec,n", SIZES)
+def test_diagonal_of_any_magnitude(n, prec):
+    def special(r):
+        return np.diag(r.uniform(0.3, 1.8, 2) * np.exp(1j * r.uniform(0, 6, 2)))
+    both_modes(n, prec, among_gates(n, 3, special))
