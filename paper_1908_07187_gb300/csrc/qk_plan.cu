@@ -148,7 +148,10 @@ struct DTerm {
 // What a pass program's builder keeps off the device.  Single-qubit diagonal factors
 // never reach it: F[q] is the pending complex factor of physical qubit q's |1>, lam the
 // one of every amplitude.  Diagonal terms on more qubits wait in terms until a gate
-// acts on one of their qubits and go out together there.
+// acts on one of their qubits and go out together there.  Pending factors are divided
+// by, and a matrix defined with a wide tolerance may hold any entry, 0 among them: a
+// factor far from magnitude 1, or one that would take F[q] far from it, waits in terms
+// as it is, also on a single qubit.
 struct PendingTerms {
     cdm *F;
     cdm &lam;
@@ -162,7 +165,7 @@ struct PendingTerms {
         const FusedOp &op = *p.op;
         DTerm t{op.mask, op.val, op.f, op.cond.n ? &op.cond : nullptr, &op};
         const int k = __builtin_popcountll(t.mask);
-        if (t.cond || k > 2) {
+        if (t.cond || k > 2 || !moderate(t.f, 0x1p8) || !room(t.mask)) {
             terms.push_back(t);
             return;
         }
@@ -192,6 +195,17 @@ struct PendingTerms {
         if (va != vb) t.f = inv;
         t.val = t.mask;
         terms.push_back(t);
+    }
+    // |f| within [1 / lim, lim]; not so for 0 and NaN
+    static bool moderate(cdm f, double lim) {
+        const double a = std::norm(f);
+        return a >= 1.0 / (lim * lim) && a <= lim * lim;
+    }
+    // whether the pending factors of these qubits can take one more factor
+    bool room(uint64_t qubits) const {
+        for (; qubits; qubits &= qubits - 1)
+            if (!moderate(F[__builtin_ctzll(qubits)], 0x1p40)) return false;
+        return moderate(lam, 0x1p300);
     }
     static bool is_pair(const DTerm &t) { return !t.cond && t.val == t.mask && __builtin_popcountll(t.mask) == 2; }
     static bool is_sign(const DTerm &t) { return t.f == cdm(-1.0, 0.0); }
@@ -249,6 +263,18 @@ bool real_form(const cdm *M, double tol) {
     if ((M[1] == 0.0) != (M[2] == 0.0)) return false;
     const cdm pr = M[1] * M[2] * std::conj(M[0] * M[3]);
     return std::abs(pr.imag()) <= tol * std::abs(pr) && pr.real() <= 0.0;
+}
+
+// Whether M on a qubit with pending factor f can run in GateForm: its larger entries are
+// divided by, and their ratio becomes the next pending factor.  Not so for a singular
+// matrix, or one whose rows differ widely.  flipped: the two values are stored exchanged.
+bool has_pivots(const cdm *M, cdm f, bool flipped) {
+    const cdm a = flipped ? M[1] : M[0], b = flipped ? M[3] : M[2];
+    const bool sw = std::norm(a) < std::norm(b);
+    const double p = std::norm(sw ? b : a), nf = std::norm(f);
+    double d = std::norm(flipped ? (sw ? M[0] : M[2]) : (sw ? M[1] : M[3]));
+    d = flipped ? d / nf : d * nf;
+    return p > 0x1p-200 && d >= p * 0x1p-16 && d <= p * 0x1p16;
 }
 
 // M = V diag(e[0], e[1]) V^+ for a unitary M that is not a multiple of 1; false when M is
@@ -656,7 +682,7 @@ struct SmemTileBuilder : PendingTerms {
         const uint8_t q = (uint8_t)local_of[b];
         const cdm *M = op.m;
         const bool is_x = M[0] == 0.0 && M[3] == 0.0 && M[1] == 1.0 && M[2] == 1.0;
-        if (op.cmask || op.cond.n || !real_form(M, 0x1p-50)) {
+        if (op.cmask || op.cond.n || !real_form(M, 0x1p-50) || !has_pivots(M, F[b], false)) {
             emit_touching(b, nullptr, nullptr);
             materialise(b);
             SmemTileOp *o = add(is_x ? ST_X : ST_CU2, q);
@@ -905,7 +931,7 @@ struct TileBuilder : PendingTerms {
         place(b, &k);
         static thread_local Touching T;
         take_touching(b, T);
-        if (op.cmask || op.cond.n || !real_form(op.m, 1e-7)) {
+        if (op.cmask || op.cond.n || !real_form(op.m, 1e-7) || !has_pivots(op.m, F[b], flip[lq])) {
             for (const DTerm &t : T.other) direct(t.mask, t.val, t.f, t.cond);
             for (const auto &r : T.reg) pair_op(k, r.first, r.second);
             phase_op(k, T);

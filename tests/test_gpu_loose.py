@@ -61,3 +61,31 @@ def test_diagonal_of_any_magnitude(n, prec):
     def special(r):
         return np.diag(r.uniform(0.3, 1.8, 2) * np.exp(1j * r.uniform(0, 6, 2)))
     both_modes(n, prec, among_gates(n, 3, special))
+
+
+SINGULAR = {
+    "diagonal": lambda r: np.diag([1.0, 0.0] if r.random() < 0.5 else [0.0, 1.0]),
+    "projector": lambda r: np.outer(v := r.standard_normal(2) + 1j * r.standard_normal(2), v.conj()) / np.vdot(v, v),
+    "column": lambda r: np.linalg.qr(r.standard_normal((2, 2)))[0] * ([1, 0] if r.random() < 0.5 else [0, 1]),
+    "nilpotent": lambda r: np.array([[0, 1], [0, 0]] if r.random() < 0.5 else [[0, 0], [1, 0]]),
+    "rows": lambda r: np.linalg.qr(r.standard_normal((2, 2)))[0] * [[1], [2.0 ** -30]],
+}
+
+
+@pytest.mark.parametrize("prec,n", SIZES)
+@pytest.mark.parametrize("kind", list(SINGULAR))
+def test_singular_and_far_from_unitary(n, prec, kind):
+    """Three of them among the gates, or the state would soon be empty."""
+    both_modes(n, prec, among_gates(n, 4, SINGULAR[kind], often=6, most=3))
+
+
+@pytest.mark.parametrize("prec,n", [s for s in SIZES if s[0] == "c128" or s[1] == 2])   # 2^(63 n) fits the type
+def test_magnitudes_that_pile_up(n, prec):
+    """Each qubit scaled by 2^-9 on one value many times, turned by gates between, and back."""
+    ops, h = [], np.array([[1, 1], [1, -1]]) / np.sqrt(2)
+    for q in range(n):
+        ops += [(np.diag([1, 2.0 ** -9]), q, ())] * 6
+        ops += [(h, q, ()), (np.diag([1, 2.0 ** -9]), q, ()), (h, q, ())]
+    for q in range(n):
+        ops += [(np.diag([1, 2.0 ** 9]), q, ())] * 7
+    both_modes(n, prec, ops)
