@@ -343,9 +343,13 @@ struct Rewriter {
             out.push_back(o);
         } else {
             cdm *a = out[last[q]].m;
-            const cdm p[4] = {m[0] * a[0] + m[1] * a[2], m[0] * a[1] + m[1] * a[3],
-                              m[2] * a[0] + m[3] * a[2], m[2] * a[1] + m[3] * a[3]};
-            for (int e = 0; e < 4; ++e) a[e] = std::abs(p[e]) < 1e-15 ? cdm(0.0) : p[e];   // products that cancel
+            const auto dot = [](cdm x0, cdm y0, cdm x1, cdm y1) {   // 0 where the products cancel
+                const cdm u = x0 * y0, v = x1 * y1, p = u + v;
+                return std::norm(p) < 1e-30 * (std::norm(u) + std::norm(v)) ? cdm(0.0) : p;
+            };
+            const cdm p[4] = {dot(m[0], a[0], m[1], a[2]), dot(m[0], a[1], m[1], a[3]),
+                              dot(m[2], a[0], m[3], a[2]), dot(m[2], a[1], m[3], a[3])};
+            for (int e = 0; e < 4; ++e) a[e] = p[e];
         }
         const cdm *a = out[last[q]].m;
         if (a[0] != 0.0 && a[1] != 0.0 && a[2] != 0.0 && a[3] != 0.0) mixed |= 1ull << q;

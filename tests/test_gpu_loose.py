@@ -89,3 +89,11 @@ def test_magnitudes_that_pile_up(n, prec):
     for q in range(n):
         ops += [(np.diag([1, 2.0 ** 9]), q, ())] * 7
     both_modes(n, prec, ops)
+
+
+@pytest.mark.parametrize("n", [13, 15])
+def test_small_matrices_that_are_multiplied(n):
+    """Gates on one qubit that become one before the passes, each scaled by 2^-27."""
+    h = 2.0 ** -27 * np.array([[1, 1], [1j, -1j]]) / np.sqrt(2)
+    ops = [(h, 3, ()), (h, 3, ()), (np.array([[0.6, 0.8], [0.8, -0.6]]), 4, (3,)), (h, 3, ())]
+    both_modes(n, "c64", ops)
