@@ -1093,6 +1093,10 @@ qk_status qk_measure(qk_ctx *c, const int *qubits, int nq, const double *uniform
         for (int j = 0; j < ma.nb; ++j) {
             ma.u[j] = uniforms[k + j];
             ma.dest[j] = dest ? dest[k + j] : -1;
+            // a round's lanes write their cbits at once: of several outcomes for one cbit
+            // only the last is written, as one after another would leave it
+            for (int i = 0; i < j; ++i)
+                if (ma.dest[i] == ma.dest[j]) ma.dest[i] = -1;
         }
         LaunchScope ls(c, 5, (double)c->amp * (double)(1ull << (c->n - k)));
         CUDA_TRY(c, qk::launch_measure_round((int)c->prec, c->d_state, ma, c->d_slots, c->d_partials, c->d_counter,
