@@ -567,6 +567,7 @@ int ctx_sms(qk_ctx *c) { return c->sms; }
 int ctx_tile_qubits(qk_ctx *c) { return c->opt.tile_qubits; }
 cudaStream_t ctx_stream(qk_ctx *c) { return c->stream; }
 const uint8_t *ctx_cbits(qk_ctx *c) { return c->d_cbits; }
+qk_status ctx_run_plain(qk_ctx *c, const FusedOp &op) { return run_op_plain(c, op); }
 qk_status ctx_fail(qk_ctx *c, qk_status s, const char *msg) { return fail(c, s, "%s", msg); }
 void ctx_launch_begin(qk_ctx *c, int cls, double bytes, void **token) {
     *token = new LaunchScope(c, cls, bytes);

@@ -1576,10 +1576,39 @@ qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const D
     return QK_OK;
 }
 
+// Whether a queue that would go through tiles in shared memory is cheaper as one launch per
+// op: a pass reads and writes the whole state, a launch only the amplitudes that match its
+// controls, or its phase's bits.  Estimates in us, from complex128 on 26 qubits (2 GiB):
+// a pass 370, half as much again with a gate or phase on one qubit (FP64), a phase 500 and
+// a 2x2 gate 1030 times the fraction they match.  A launch takes 2.6, that of a pass, with
+// its program of 20 KB, 4.4.  One launch per op / one pass, complex128: CZ on 26 qubits 141 /
+// 380, T 253 / 582, X with two controls 264 / 371, with five 40 / 370, H 1034 / 743, three CZ
+// 453 / 395; one gate on 10 qubits, either type, 6.3 / 8.2, two 11.6 / 11.1.
+bool single_launches(int n, int prec, const std::vector<FusedOp> &ops) {
+    const double unit = std::ldexp(prec == 0 ? 0.5 : 1.0, n - 26);   // of the 2 GiB
+    double singles = 0.0;
+    bool wide = false;
+    for (const FusedOp &op : ops) {
+        const bool u2 = op.kind == FusedOp::U2;
+        const int bits = __builtin_popcountll(u2 ? op.cmask : op.mask);
+        wide = wide || bits + (u2 ? 1 : 0) <= 1;
+        singles += 2.6 + unit * std::ldexp(u2 ? 1030.0 : 500.0, -bits);
+        if (singles >= 4.4 + unit * 555.0) return false;
+    }
+    return singles < 4.4 + unit * (wide ? 555.0 : 370.0);
+}
+
 qk_status run_fused(TilePlanner *planner, qk_ctx *c, const std::vector<FusedOp> &ops) {
     const int n = ctx_n(c);
     const int prec = ctx_prec(c);
     if (prec != 0 || n < kTileQubits) {
+        if (single_launches(n, prec, ops)) {
+            for (const FusedOp &op : ops) {
+                const qk_status st = ctx_run_plain(c, op);
+                if (st != QK_OK) return st;
+            }
+            return QK_OK;
+        }
         const SmemPassSink launch = [&](SmemTileParams &P) -> qk_status {
             void *tok = nullptr;
             ctx_launch_begin(c, 0, (prec == 0 ? 2.0 * 8.0 : 2.0 * 16.0) * (double)(1ull << n), &tok);

@@ -52,7 +52,8 @@ using SmemPassSink = std::function<qk_status(SmemTileParams &)>;
 qk_status plan_smem_passes(TilePlanner *p, int n, int prec, const std::vector<FusedOp> &ops, const SmemPassSink &sink,
                            const char **err);
 // one of them with each pass launched on the context's stream: register tiles for
-// complex64 from 13 qubits on, tiles in shared memory otherwise
+// complex64 from 13 qubits on, tiles in shared memory otherwise, or one launch per op
+// where so few amplitudes are concerned that this is cheaper
 qk_status run_fused(TilePlanner *p, qk_ctx *c, const std::vector<FusedOp> &ops);
 
 // context hooks implemented in qk_api.cu
@@ -63,6 +64,7 @@ int ctx_sms(qk_ctx *c);
 int ctx_tile_qubits(qk_ctx *c);
 cudaStream_t ctx_stream(qk_ctx *c);
 const uint8_t *ctx_cbits(qk_ctx *c);
+qk_status ctx_run_plain(qk_ctx *c, const FusedOp &op);
 qk_status ctx_fail(qk_ctx *c, qk_status s, const char *msg);
 void ctx_launch_begin(qk_ctx *c, int cls, double bytes, void **token);
 void ctx_launch_end(void *token);
