@@ -1444,28 +1444,167 @@ qk_status plan_smem_passes(TilePlanner *planner, int n, int prec, const std::vec
 }
 
 namespace {
-}  // namespace
 
+// Tile qubits of a dense pass that enumerates n qubits: complex64 gates of 5 and 6 qubits
+// form 8 rows per thread, which takes 2^13 amplitudes to give every thread columns;
+// smaller tiles for small states, so that there are tiles for all SMs (in complex128 a
+// tile's FP64 work is the time).  One 6-qubit gate with a control on 20 qubits 24 us in
+// tiles of 2^13, 36 in 2^11; two of them with controls inside the tile on 18 qubits 24 and 17.
+int dense_tile_qubits(int n, int prec, int k, bool alone) {
+    if (prec != 0) return n >= 20 ? 11 : n >= 18 ? 10 : 8;
+    if (k >= 5 && n >= (alone ? 18 : 20)) return 13;
+    return n >= 20 ? 12 : n >= 18 ? 11 : n >= 16 ? 10 : 9;
+}
+// its qubits: the gates' targets and the lowest others that are not enumerated away
+uint64_t dense_tile_set(int n, int prec, int k, bool alone, uint64_t targets, uint64_t lone) {
+    const int m = dense_tile_qubits(n - __builtin_popcountll(lone), prec, k, alone);
+    uint64_t S = targets;
+    for (int b = 0; b < n && __builtin_popcountll(S) < m; ++b)
+        if (!((S | lone) >> b & 1)) S |= 1ull << b;
+    return S;
+}
+
+// The program of one dense pass over the given gates.  A pass of one controlled gate
+// enumerates only the tiles whose control bits are set.
+void dense_program(int n, int prec, const std::vector<const DenseItem *> &taken, DenseParams &P) {
+    std::memset(static_cast<void *>(&P), 0, offsetof(DenseParams, ops));
+    uint64_t S = 0;
+    for (const DenseItem *it : taken) {
+        S |= it->tmask;
+        bool known = !it->cond.n;
+        for (int k = 0; k < P.n_conds; ++k) known = known || same_cond(P.conds[k], it->cond);
+        if (!known) P.conds[P.n_conds++] = it->cond;
+    }
+    const uint64_t lone = taken.size() == 1 ? taken[0]->cmask : 0;   // enumerated only where set
+    S = dense_tile_set(n, prec, taken[0]->k, taken.size() == 1, S, lone);
+    P.m = __builtin_popcountll(S);
+    P.base = lone;
+    int local_of[64], tile_of[64];
+    for (int b = 0, lb = 0; b < n; ++b) {
+        local_of[b] = tile_of[b] = -1;
+        if ((S >> b) & 1) {
+            P.S[lb] = (int8_t)b;
+            local_of[b] = lb++;
+        } else if (!((lone >> b) & 1)) {
+            P.fixed[P.nfix] = (int8_t)b;
+            tile_of[b] = P.nfix++;
+        }
+    }
+    P.n_tiles = 1ull << P.nfix;
+    P.k = taken[0]->k;
+    for (const DenseItem *const &it : taken) {
+        DenseOp &o = P.ops[P.nops++];
+        std::memset(static_cast<void *>(&o), 0, sizeof o);
+        uint32_t used = 0;
+        for (int b = 0; b < it->k; ++b) {
+            const int lb = local_of[it->tpos[it->k - 1 - b]];
+            o.ts[b] = (uint16_t)dense_slot(1u << lb);
+            used |= 1u << lb;
+        }
+        o.cond = 0xff;
+        if (it->cond.n)
+            for (int k = 0; k < P.n_conds; ++k)
+                if (same_cond(P.conds[k], it->cond)) o.cond = (uint8_t)k;
+        for (uint64_t c = it->cmask & ~lone; c; c &= c - 1) {
+            const int b = __builtin_ctzll(c);
+            if (local_of[b] >= 0) {
+                o.ls ^= (uint16_t)dense_slot(1u << local_of[b]);
+                used |= 1u << local_of[b];
+            } else {
+                o.tmask |= 1u << tile_of[b];
+            }
+        }
+        // two 2-qubit gates in a row on other qubits, both unconditional: one round trip
+        // through shared memory.  The first one's column bits are the second's register
+        // bits (or, for one gate alone, its last free bits).
+        const bool joined = P.nops >= 2 && P.ops[P.nops - 2].pair;
+        const bool free2 = prec == 0 && it->k == 2 && !it->cmask && !it->cond.n;
+        o.pair = 0;
+        if (free2 && !joined && &it != &taken.back()) {
+            const DenseItem *nx = (&it)[1];
+            if (!nx->cmask && !nx->cond.n && !(nx->tmask & it->tmask)) {
+                o.pair = 1;
+                o.ncs = 2;
+                for (int b = 0; b < 2; ++b) {
+                    const int lb = local_of[nx->tpos[1 - b]];
+                    o.cs[b] = (uint16_t)dense_slot(1u << lb);
+                    used |= 1u << lb;
+                }
+            }
+        }
+        // free bits: lanes walk the first ones, so those go to distinct banks (bit mod 4)
+        uint32_t banks = 0, placed = used;
+        for (int pass = 0; pass < 2; ++pass)
+            for (int b = 0; b < P.m; ++b) {
+                if ((placed >> b) & 1u) continue;
+                if (pass == 0 && ((banks >> (b & 3)) & 1u)) continue;
+                banks |= 1u << (b & 3);
+                placed |= 1u << b;
+                o.fs[o.nfree++] = (uint16_t)dense_slot(1u << b);
+            }
+        if (prec == 0 && it->k == 2 && !o.pair)
+            while (o.ncs < 2 && o.nfree > 0) o.cs[o.ncs++] = o.fs[--o.nfree];
+        o.mat = it->mat;
+    }
+}
+
+// Whether the gates of a pass are cheaper in a pass each, which enumerates only the tiles
+// whose control bits are set, than in one over the whole state.  Estimates in us, from 24
+// qubits: traffic 45 (complex64) and 90, of which complex128's arithmetic hides most, and
+// which follows control bits only down to runs of 64 bytes; a gate of k qubits 10 + 2^k *
+// 3.4 and 2^k * 112; another launch 5.5.  In a shared pass a controlled gate keeps half its
+// time in complex64 (threads without columns); in complex128 its time follows the controls
+// inside the tile, but controls on tile-index bits leave it to few of an SM's CTAs, and the
+// tile with all of them set runs every gate in turn (chain).  Eight gates with four
+// controls on 24 qubits, gate by gate before / one pass / a pass each: complex64 k = 2 84 /
+// 149 / 71, k = 4 552 / 214 / 102, complex128 k = 4 1543 / 2875 / 1086 us; with one control,
+// complex64 k = 2, 394 / 180 in one pass.
+bool dense_apart(int n, int prec, const std::vector<const DenseItem *> &taken) {
+    uint64_t targets = 0, controls = 0;
+    for (const DenseItem *it : taken) {
+        targets |= it->tmask;
+        controls |= it->cmask;
+    }
+    if (taken.size() < 2 || !controls) return false;
+    const int k = taken[0]->k;
+    const uint64_t S = dense_tile_set(n, prec, k, false, targets, 0), run = prec == 0 ? 7u : 3u;
+    const double unit = std::ldexp(1.0, n - 24), traffic = unit * (prec == 0 ? 45.0 : 40.0);
+    const double gate = unit * (prec == 0 ? 10.0 + std::ldexp(3.4, k) : std::ldexp(112.0, k));
+    // complex128: a gate on one tile, beside others on its SM or by itself
+    const auto tile = [&](int bits, double rate) { return std::ldexp(1.0 / rate, bits + k + 2); };
+    const int m = __builtin_popcountll(S);
+    double joint = 2.5 + traffic, apart = 0.0, chain = 0.0;
+    for (const DenseItem *it : taken) {
+        const int nc = __builtin_popcountll(it->cmask), tc = __builtin_popcountll(it->cmask & ~S);
+        const double part = std::ldexp(traffic, -__builtin_popcountll(it->cmask & ~run)) + std::ldexp(gate, -nc);
+        apart += prec == 0 ? 5.5 + part
+                           : std::max(5.5 + part, 2.5 + tile(dense_tile_qubits(n - nc, prec, k, true), 2600.0));
+        if (prec == 0) {
+            joint += gate * (nc > 0 ? 0.5 : 1.0);
+        } else {
+            joint += std::ldexp(gate, tc - nc) * std::min(1.0, tc > 0 ? std::ldexp(5.0, -tc) : 1.0);
+            chain += std::ldexp(tile(m, tc > 0 ? 1300.0 : 2600.0), tc - nc);
+        }
+    }
+    return apart < 0.8 * std::max(joint, chain);
+}
+}  // namespace
 
 // A dense pass: S starts as the lowest qubits (runs of 128 bytes in HBM, 32 for states in
 // L2) and takes the targets of every gate, in order, that commutes with the gates left
-// behind, has the first one's k and still fits.  A pass of one controlled gate enumerates only the tiles whose
-// control bits are set.  Fewer amplitudes per tile for small states, so that there are
-// tiles for all SMs.
+// behind, has the first one's k and still fits; they go in one pass, or in one each where
+// that is cheaper (dense_apart).
 qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const DenseSink &sink) {
-    std::vector<const DenseItem *> rem, left, taken;
+    static thread_local std::vector<const DenseItem *> rem, left, taken, one(1);
+    static thread_local std::vector<Cond> conds;
+    rem.clear();
     for (const DenseItem &it : ops) rem.push_back(&it);
     while (!rem.empty()) {
         left.clear();
         taken.clear();
+        conds.clear();
         static thread_local DenseParams P;
-        std::memset(static_cast<void *>(&P), 0, offsetof(DenseParams, ops));
-        // complex64 gates of 5 and 6 qubits form 8 rows per thread, which takes 2^13
-        // amplitudes to give every thread columns; smaller tiles for small states, so
-        // that there are tiles for all SMs (in complex128 a tile's FP64 work is the time)
-        int m = prec != 0 ? 11 : rem[0]->k >= 5 ? 13 : 12;
-        if (n < 20) m = std::min(m, prec != 0 ? (n >= 18 ? 10 : 8) : n >= 18 ? 11 : n >= 16 ? 10 : 9);
-        m = std::min(m, n);
+        const int m = std::min(dense_tile_qubits(n, prec, rem[0]->k, false), n);
         const int contig = std::min(m, n >= 23 ? 4 : 2);
         uint64_t S = 0, left_t = 0, left_all = 0;
         int elems = 0;
@@ -1477,15 +1616,11 @@ qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const D
                       !(it->tmask & left_all) && !(all & left_t);
             // the first gate may use the room of the low qubits
             if (ok && __builtin_popcountll(S | it->tmask | (taken.empty() ? 0 : low)) > m) ok = false;
-            int ci = -1;
             if (ok && it->cond.n) {
-                for (int k = 0; k < P.n_conds; ++k)
-                    if (same_cond(P.conds[k], it->cond)) ci = k;
-                if (ci < 0 && P.n_conds >= kTileMaxConds) ok = false;
-                else if (ci < 0) {
-                    ci = P.n_conds++;
-                    P.conds[ci] = it->cond;
-                }
+                bool known = false;
+                for (const Cond &c : conds) known = known || same_cond(c, it->cond);
+                if (!known && (int)conds.size() >= kTileMaxConds) ok = false;
+                else if (!known) conds.push_back(it->cond);
             }
             if (!ok) {
                 left.push_back(it);
@@ -1497,80 +1632,18 @@ qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const D
             elems += 1 << (2 * it->k);
             taken.push_back(it);
         }
-        const uint64_t lone = taken.size() == 1 ? taken[0]->cmask : 0;   // enumerated only where set
-        for (int b = 0; b < n && __builtin_popcountll(S) < m; ++b)
-            if (!((S | lone) >> b & 1)) S |= 1ull << b;
-        P.m = __builtin_popcountll(S);
-        P.base = lone;
-        int local_of[64], tile_of[64];
-        for (int b = 0, lb = 0; b < n; ++b) {
-            local_of[b] = tile_of[b] = -1;
-            if ((S >> b) & 1) {
-                P.S[lb] = (int8_t)b;
-                local_of[b] = lb++;
-            } else if (!((lone >> b) & 1)) {
-                P.fixed[P.nfix] = (int8_t)b;
-                tile_of[b] = P.nfix++;
+        if (dense_apart(n, prec, taken)) {
+            for (const DenseItem *it : taken) {
+                one[0] = it;
+                dense_program(n, prec, one, P);
+                const qk_status st = sink(P);
+                if (st != QK_OK) return st;
             }
+        } else {
+            dense_program(n, prec, taken, P);
+            const qk_status st = sink(P);
+            if (st != QK_OK) return st;
         }
-        P.n_tiles = 1ull << P.nfix;
-        P.k = rem[0]->k;
-        for (const DenseItem *const &it : taken) {
-            DenseOp &o = P.ops[P.nops++];
-            std::memset(static_cast<void *>(&o), 0, sizeof o);
-            uint32_t used = 0;
-            for (int b = 0; b < it->k; ++b) {
-                const int lb = local_of[it->tpos[it->k - 1 - b]];
-                o.ts[b] = (uint16_t)dense_slot(1u << lb);
-                used |= 1u << lb;
-            }
-            o.cond = 0xff;
-            if (it->cond.n)
-                for (int k = 0; k < P.n_conds; ++k)
-                    if (same_cond(P.conds[k], it->cond)) o.cond = (uint8_t)k;
-            for (uint64_t c = it->cmask & ~lone; c; c &= c - 1) {
-                const int b = __builtin_ctzll(c);
-                if (local_of[b] >= 0) {
-                    o.ls ^= (uint16_t)dense_slot(1u << local_of[b]);
-                    used |= 1u << local_of[b];
-                } else {
-                    o.tmask |= 1u << tile_of[b];
-                }
-            }
-            // two 2-qubit gates in a row on other qubits, both unconditional: one round trip
-            // through shared memory.  The first one's column bits are the second's register
-            // bits (or, for one gate alone, its last free bits).
-            const bool joined = P.nops >= 2 && P.ops[P.nops - 2].pair;
-            const bool free2 = prec == 0 && it->k == 2 && !it->cmask && !it->cond.n;
-            o.pair = 0;
-            if (free2 && !joined && &it != &taken.back()) {
-                const DenseItem *nx = (&it)[1];
-                if (!nx->cmask && !nx->cond.n && !(nx->tmask & it->tmask)) {
-                    o.pair = 1;
-                    o.ncs = 2;
-                    for (int b = 0; b < 2; ++b) {
-                        const int lb = local_of[nx->tpos[1 - b]];
-                        o.cs[b] = (uint16_t)dense_slot(1u << lb);
-                        used |= 1u << lb;
-                    }
-                }
-            }
-            // free bits: lanes walk the first ones, so those go to distinct banks (bit mod 4)
-            uint32_t banks = 0, placed = used;
-            for (int pass = 0; pass < 2; ++pass)
-                for (int b = 0; b < P.m; ++b) {
-                    if ((placed >> b) & 1u) continue;
-                    if (pass == 0 && ((banks >> (b & 3)) & 1u)) continue;
-                    banks |= 1u << (b & 3);
-                    placed |= 1u << b;
-                    o.fs[o.nfree++] = (uint16_t)dense_slot(1u << b);
-                }
-            if (prec == 0 && it->k == 2 && !o.pair)
-                while (o.ncs < 2 && o.nfree > 0) o.cs[o.ncs++] = o.fs[--o.nfree];
-            o.mat = it->mat;
-        }
-        const qk_status st = sink(P);
-        if (st != QK_OK) return st;
         rem.swap(left);
     }
     return QK_OK;
