@@ -26,6 +26,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -335,11 +336,15 @@ struct qk_batch {
     static constexpr int kSide = 4;
     cudaStream_t side[kSide] = {};
     cudaEvent_t fork = nullptr, join[kSide] = {};
-    // host copy of all small circuits' states and all cbits, taken when a second circuit
-    // of a run is read (one copy instead of two waits per circuit)
-    std::vector<unsigned char> h_states, h_cbits;
-    bool h_valid = false;
-    int reads = 0;                     // circuits read since the last run
+    // Read-ahead (read_window): host copy of circuits [win_first, win_first + win_count), of
+    // their cbits and, with win_states, the small ones' states; the circuit after the last
+    // read, and how many the last window was asked to hold
+    static constexpr size_t kWindow = 4u << 20;
+    std::unique_ptr<unsigned char[]> win;
+    size_t win_cbits = 0, win_amp0 = 0;
+    int win_first = 0, win_count = 0;
+    bool win_states = false;
+    int read_next = 0, ahead = 0;
     std::mutex read_mu;                // reads from several threads
     // What the last run launched, which is what the device buffers hold: circuits may be
     // added after it, and a read takes its sizes from here (0: nothing has run).
@@ -682,6 +687,52 @@ bool read_back(qk_batch *b, void *dst, const void *src, size_t bytes) {
     return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, b->stream) == cudaSuccess &&
            cudaStreamSynchronize(b->stream) == cudaSuccess;
 }
+bool in_window(const qk_batch *b, int circuit, bool state) {
+    return circuit >= b->win_first && circuit < b->win_first + b->win_count && (b->win_states || !state);
+}
+// Read a circuit's cbits and (small ones) its state.  Each copy is a wait of about 10 us,
+// and programs read circuits in order: a read just after the last one takes the following
+// circuits along, four times as many as the window before, up to kWindow bytes: 256
+// circuits of 6 MB cost six waits (2.33 ms in all, 2.25 with everything in one copy), and
+// reading two circuits costs the bytes of three more.  Any other read copies its own
+// circuit only.  states: whether this program reads states at all.
+qk_status read_window(qk_batch *b, int circuit, uint8_t *cbits, int ncb, void *state, size_t bytes, bool states) {
+    const int gap = circuit - b->read_next;
+    b->ahead = b->ahead > 0 && gap >= 0 && gap <= b->ahead ? std::min(4 * b->ahead, 1 << 20) : 1;
+    const int want = std::min(b->ahead, b->run_circs - circuit);
+    const qk::BCirc &c = b->circs[circuit];
+    b->win_count = 0;
+    // the small circuits' states lie one after another, and so do all cbits
+    size_t amps = 0, ncbits = 0, amp0 = 0;
+    int count = 0;
+    for (; count < want; ++count) {
+        const qk::BCirc &x = b->circs[circuit + count];
+        const size_t more = states && !(x.flags & 2u) ? (size_t)1 << x.n : 0;
+        if (sizeof(float2) * (amps + more) + ncbits + x.ncb > qk_batch::kWindow) break;
+        if (more && amps == 0) amp0 = x.state_off;
+        amps += more;
+        ncbits += x.ncb;
+    }
+    if (count > 1 && !b->win) b->win.reset(new (std::nothrow) unsigned char[qk_batch::kWindow]);
+    if (count <= 1 || !b->win) {
+        if (ncb > 0 && !read_back(b, cbits, b->d_cbits + c.cb_off, ncb)) return bfail(b, QK_ECUDA, "batch: cbit copy failed");
+        if (state && !read_back(b, state, b->d_states + c.state_off, bytes))
+            return bfail(b, QK_ECUDA, "batch: state copy failed");
+        return QK_OK;
+    }
+    unsigned char *h = b->win.get();
+    const size_t sb = sizeof(float2) * amps;
+    if ((sb > 0 && cudaMemcpyAsync(h, b->d_states + amp0, sb, cudaMemcpyDeviceToHost, b->stream) != cudaSuccess) ||
+        (ncbits > 0 && cudaMemcpyAsync(h + sb, b->d_cbits + c.cb_off, ncbits, cudaMemcpyDeviceToHost, b->stream) != cudaSuccess) ||
+        cudaStreamSynchronize(b->stream) != cudaSuccess)
+        return bfail(b, QK_ECUDA, "batch: copy failed");
+    b->win_first = circuit;
+    b->win_count = count;
+    b->win_states = states;
+    b->win_cbits = sb;
+    b->win_amp0 = amp0;
+    return QK_OK;
+}
 }  // namespace
 
 extern "C" {
@@ -756,8 +807,8 @@ qk_status qk_batch_clear(qk_batch *b) {
     b->large.clear();
     b->large_of.clear();
     b->large_amps = 0;
-    b->h_valid = false;
-    b->reads = 0;
+    b->win_count = 0;
+    b->ahead = 0;
     b->run_circs = 0;
     b->run_amps = 0;
     b->run_cb = 0;
@@ -953,8 +1004,8 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
     b->start_recorded = false;
     b->plan_ms = 0.0;
     b->large_launches = 0;
-    b->h_valid = false;
-    b->reads = 0;
+    b->win_count = 0;
+    b->ahead = 0;
     b->run_circs = 0;
     // host work first -- the large circuits' plans, the small ones' matrices -- then the
     // start event, after which everything is enqueued back to back
@@ -1081,30 +1132,23 @@ qk_status qk_batch_read(qk_batch *b, int circuit, uint8_t *cbits, int ncb, void 
     if (state && ((!large && !b->store_state) || bytes != sizeof(float2) << c.n))
         return bfail(b, QK_EINVAL, "batch: state not stored or wrong size (%zu bytes expected)", sizeof(float2) << c.n);
     if (cudaEventSynchronize(b->done) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event wait failed");
-    // A program that reads a second circuit reads many: all the small ones come over in
-    // one copy then (up to 64 MB of states), instead of two copies and waits for each.
-    const size_t all = b->store_state ? sizeof(float2) * b->run_amps : 0;
     const std::lock_guard<std::mutex> lk(b->read_mu);
-    if (++b->reads == 2 && !b->h_valid && b->run_circs > 2 && all <= (64u << 20)) {
-        b->h_states.resize(all);
-        b->h_cbits.resize(b->run_cb);
-        b->h_valid = (all == 0 || cudaMemcpyAsync(b->h_states.data(), b->d_states, all, cudaMemcpyDeviceToHost, b->stream) == cudaSuccess) &&
-                     (b->run_cb == 0 || cudaMemcpyAsync(b->h_cbits.data(), b->d_cbits, b->run_cb, cudaMemcpyDeviceToHost, b->stream) == cudaSuccess) &&
-                     cudaStreamSynchronize(b->stream) == cudaSuccess;
-        if (!b->h_valid) return bfail(b, QK_ECUDA, "batch: copy failed");
-    }
-    if (b->h_valid) {
-        if (ncb > 0) std::memcpy(cbits, b->h_cbits.data() + c.cb_off, (size_t)ncb);
-        if (state && !large) {
-            std::memcpy(state, b->h_states.data() + sizeof(float2) * c.state_off, bytes);
-            return QK_OK;
+    const bool small = state && !large;
+    if (small || ncb > 0) {
+        if (!in_window(b, circuit, small)) {
+            const qk_status st = read_window(b, circuit, cbits, ncb, small ? state : nullptr, bytes, state != nullptr);
+            if (st != QK_OK) return st;
         }
-    } else if (ncb > 0 && !read_back(b, cbits, b->d_cbits + c.cb_off, ncb)) {
-        return bfail(b, QK_ECUDA, "batch: cbit copy failed");
+        if (in_window(b, circuit, small)) {
+            const unsigned char *h = b->win.get();
+            if (ncb > 0) std::memcpy(cbits, h + b->win_cbits + (c.cb_off - b->circs[b->win_first].cb_off), (size_t)ncb);
+            if (small) std::memcpy(state, h + sizeof(float2) * (c.state_off - b->win_amp0), bytes);
+        }
     }
+    b->read_next = circuit + 1;
     // on the batch's own stream (its run is complete: the event above)
-    const float2 *src = large ? b->d_lstates + b->large[b->large_of[circuit]].state_off : b->d_states + c.state_off;
-    if (state && !read_back(b, state, src, bytes)) return bfail(b, QK_ECUDA, "batch: state copy failed");
+    if (state && large && !read_back(b, state, b->d_lstates + b->large[b->large_of[circuit]].state_off, bytes))
+        return bfail(b, QK_ECUDA, "batch: state copy failed");
     return QK_OK;
 }
 
