@@ -173,6 +173,11 @@ struct DDC {
     DDC(DD r, DD i) : re(r), im(i) {}
     explicit DDC(cdm z) : re{z.real(), 0.0}, im{z.imag(), 0.0} {}
     explicit operator cdm() const { return {re.h, im.h}; }
+    DDC &operator/=(DD x) {
+        re = re / x;
+        im = im / x;
+        return *this;
+    }
     DDC &operator*=(const DDC &b) {
         const DD r = re * b.re - im * b.im;
         im = re * b.im + im * b.re;
@@ -182,9 +187,7 @@ struct DDC {
     DDC &operator/=(const DDC &b) {
         const DD n = b.re * b.re + b.im * b.im;
         *this *= DDC(b.re, -b.im);
-        re = re / n;
-        im = im / n;
-        return *this;
+        return *this /= n;
     }
 };
 inline DDC operator*(DDC a, const DDC &b) { return a *= b; }
@@ -200,6 +203,10 @@ template <typename X> struct RealOf { using T = double; };
 template <> struct RealOf<DDC> { using T = DD; };
 inline DD real_from(double x, DD) { return {x, 0.0}; }
 inline double real_from(double x, double) { return x; }
+template <typename X> X turned(const X &z, int k) {   // i^k z
+    const auto r = real_of(z), m = imag_of(z);
+    return (k & 3) == 0 ? z : (k & 3) == 1 ? X(-m, r) : (k & 3) == 2 ? X(-r, -m) : X(m, -r);
+}
 
 // A diagonal term that is not yet in a program: f where (index & mask) == val.
 struct DTerm {
@@ -792,9 +799,8 @@ struct SmemTileBuilder : PendingTerms<X> {
             X a0 = X(W[1]) * F[b] / p0, a1 = X(W[2]) / p1;
             const cdm dir(a0);
             const int k = std::abs(dir.real()) >= std::abs(dir.imag()) ? (dir.real() >= 0.0 ? 0 : 2) : dir.imag() > 0.0 ? 1 : 3;
-            const X quarter[4] = {X(1.0), X(cdm(0.0, 1.0)), X(-1.0), X(cdm(0.0, -1.0))};
-            a0 *= quarter[(4 - k) & 3];
-            a1 *= quarter[k];
+            a0 = turned(a0, 4 - k);
+            a1 = turned(a1, k);
             // a0 = i^k c (1 + i t), a1 = i^-k g (1 - i t): t from the mean of both directions,
             // since a matrix is unitary only to rounding, and c and g along it
             const double w0 = 1.0 / std::sqrt(std::norm(cdm(a0))), w1 = 1.0 / std::sqrt(std::norm(cdm(a1)));
@@ -825,9 +831,10 @@ struct SmemTileBuilder : PendingTerms<X> {
             o->c[0] = t;
             o->c[1] = rounded(b0);
             o->c[2] = rounded(b1);
-            if (side == 0) p1 /= X(cdm(1.0, t)) * quarter[k];
-            else p0 /= X(cdm(1.0, -t)) * quarter[(4 - k) & 3];
-            const X left(num(1.0) + num(o->c[1]) * num(o->c[2]), num(0.0));
+            // 1 / u = i^-k (1 - i t) / (1 + t^2)
+            if (side == 0) p1 = turned(p1 * X(cdm(1.0, -t)), 4 - k) /= sq;
+            else p0 = turned(p0 * X(cdm(1.0, t)), k) /= sq;
+            const R left = num(1.0) + num(o->c[1]) * num(o->c[2]);
             if (first0) p1 /= left;
             else p0 /= left;
             o->flags |= (uint8_t)(k | kU2Lift);
