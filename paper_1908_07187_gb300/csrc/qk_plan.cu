@@ -237,7 +237,7 @@ struct PendingTerms {
         const FusedOp &op = *p.op;
         DTerm t{op.mask, op.val, op.f, op.cond.n ? &op.cond : nullptr, &op};
         const int k = __builtin_popcountll(t.mask);
-        if (t.cond || k > 2 || !moderate(t.f, 0x1p8) || !room(t.mask)) {
+        if (t.cond || k > 2 || (k == 2 && t.val == t.mask) || !moderate(t.f, 0x1p8) || !room(t.mask)) {
             terms.push_back(t);
             return;
         }
@@ -263,7 +263,7 @@ struct PendingTerms {
             F[a] /= f;
             F[b] /= f;
         }
-        if (t.val != t.mask) t.src = nullptr;
+        t.src = nullptr;
         if (va != vb) t.f = 1.0 / t.f;
         t.val = t.mask;
         terms.push_back(t);
