@@ -303,7 +303,7 @@ struct PendingTerms {
 // How a 2x2 gate M on a qubit with pending factor f (on the stored |1>) is run: W is M
 // or, with sw, X M (the rows exchanged so that the larger entries are on the diagonal);
 // the true outputs are p0 and p1 times the values the device leaves.  a0 = W01 f / W00,
-// a1 = W10 / (W11 f); r0 = |a0|, r1 = |a1|, psi = arg a0, and a1 = -r1 e^{-i psi} for a
+// a1 = W10 / (W11 f); r0 = |a0|, r1 = |a1|, a0 = r0 e^{i psi} and a1 = -r1 e^{-i psi} for a
 // unitary M.  s = 1 / (1 + r0 r1) is what updating one value from the other in place
 // leaves on the value updated second.
 struct GateForm {
@@ -322,7 +322,9 @@ GateForm gate_form(const cdm *M, cdm f) {
     const cdm a0 = W[1] * f / W[0], a1 = W[2] / (W[3] * f);
     g.r0 = std::abs(a0);
     g.r1 = std::abs(a1);
-    g.psi = g.r0 != 0.0 || g.r1 != 0.0 ? std::arg(a0) : 0.0;
+    // the mean of what the two say (real_form: not far apart), so that either is off by half
+    // of what a matrix lacks
+    g.psi = g.r0 != 0.0 && g.r1 != 0.0 ? std::arg(a0 * g.r1 - std::conj(a1) * g.r0) : 0.0;
     g.s = 1.0 / (1.0 + g.r0 * g.r1);
     g.p0 = W[0];
     g.p1 = W[3] * f;

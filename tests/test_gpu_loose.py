@@ -97,3 +97,35 @@ def test_small_matrices_that_are_multiplied(n):
     h = 2.0 ** -27 * np.array([[1, 1], [1j, -1j]]) / np.sqrt(2)
     ops = [(h, 3, ()), (h, 3, ()), (np.array([[0.6, 0.8], [0.8, -0.6]]), 4, (3,)), (h, 3, ())]
     both_modes(n, "c64", ops)
+
+
+def test_direction_between_the_entries():
+    """Register tiles turn a gate by one angle; a matrix whose off-diagonal entries ask for
+    angles 9e-8 apart gets the one between, so either entry is off by half of that.  The mean
+    over 400 gates, rounding (2^-25 each) averaged down to 2e-9."""
+    from paper_1908_07187_gb300 import qk
+
+    n, d, off = 13, 9e-8, []
+    r = np.random.Generator(np.random.PCG64(8))
+    with qk.Context("c64") as ctx:
+        ctx.add_qubits(n)
+        for _ in range(400):
+            c = np.cos(r.uniform(0.1, 0.7))          # the larger entries on the diagonal
+            a, b = np.exp(1j * r.uniform(0, 6, 2))
+            s = np.sqrt(1 - c * c)
+            m = np.array([[c, -b * s], [a * s * np.exp(1j * d), a * b * c]])
+            ctx.reset()
+            ctx.apply_gate(ctx.define_gate_matrix(m, tol=1e-6), (6,))
+            off.append(np.imag(ctx.get_state()[1 << 6] / m[1, 0]))
+    assert abs(np.mean(off)) <= d / 2 + 4e-9
+
+
+@pytest.mark.parametrize("prec,n", SIZES)
+@pytest.mark.parametrize("noise", [1e-3, 1e-7, "float32"])
+def test_nearly_unitary(n, prec, noise):
+    def special(r):
+        u = np.linalg.qr(r.standard_normal((2, 2)) + 1j * r.standard_normal((2, 2)))[0]
+        if noise == "float32":
+            return u.astype(np.complex64).astype(np.complex128)
+        return u + noise * (r.standard_normal((2, 2)) + 1j * r.standard_normal((2, 2)))
+    both_modes(n, prec, among_gates(n, 5, special))
