@@ -290,7 +290,8 @@ qk_status qk_graph_destroy(qk_graph *g);
  * qk_batch_run plans it into fused tile passes (on the host's cores) and runs
  * pass k of every such circuit in one batched launch.  qk_batch_run uploads the
  * programs and launches (one launch per distinct small-circuit size, one per
- * pass index of the large circuits) on the batch's stream without waiting;
+ * pass index of the large circuits) on the batch's stream without waiting (but
+ * for the uploads of a run before it, whose staging memory it writes again);
  * qk_batch_done polls; qk_batch_read waits and copies a circuit's cbits and
  * final state (always kept for large circuits, for small ones if stored).  Add
  * ops to the most recently added circuit.  Circuits may be added after a run; what

@@ -326,9 +326,10 @@ struct qk_batch {
     size_t cap_states = 0;
     uint8_t *d_cbits = nullptr;
     size_t cap_cbits = 0;
-    // pinned staging for the uploads (valid until the next run)
+    // pinned staging for the uploads; the next run writes it again once they are done (staged)
     void *h_stage = nullptr;
     size_t cap_stage = 0;
+    cudaEvent_t staged = nullptr;
     cudaEvent_t done = nullptr;
     cudaEvent_t start = nullptr;       // recorded once the host work of a run is done
     // The launches of the small circuits go round these streams, beside the tile passes
@@ -761,6 +762,7 @@ qk_status qk_batch_create(qk_batch **out, void *cuda_stream) {
         b->own_stream = true;
     }
     if (cudaEventCreate(&b->done) != cudaSuccess || cudaEventCreate(&b->start) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         qk_batch_destroy(b);
@@ -788,6 +790,7 @@ qk_status qk_batch_destroy(qk_batch *b) {
         if (b->join[k]) cudaEventDestroy(b->join[k]);
     }
     if (b->fork) cudaEventDestroy(b->fork);
+    if (b->staged) cudaEventDestroy(b->staged);
     if (b->done) cudaEventDestroy(b->done);
     if (b->start) cudaEventDestroy(b->start);
     if (b->own_stream) cudaStreamDestroy(b->stream);
@@ -1033,6 +1036,8 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
     });
     // stage the program in pinned memory so that the copies are truly asynchronous
     const size_t ob = sizeof(qk::BOp) * b->ops.size(), cb = sizeof(qk::BCirc) * sorted.size();
+    // a run before this one may still wait on the stream for its copies from there
+    if (b->h_stage && cudaEventSynchronize(b->staged) != cudaSuccess) return bfail(b, QK_ECUDA, "batch: event wait failed");
     if (ob + cb > 0 && ob + cb > b->cap_stage) {
         if (b->h_stage) cudaFreeHost(b->h_stage);
         b->h_stage = nullptr;
@@ -1047,7 +1052,8 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
         std::memcpy(b->h_stage, b->ops.data(), ob);
         std::memcpy((char *)b->h_stage + ob, sorted.data(), cb);
         if (cudaMemcpyAsync(b->d_ops, b->h_stage, ob, cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
-            cudaMemcpyAsync(b->d_circs, (char *)b->h_stage + ob, cb, cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
+            cudaMemcpyAsync(b->d_circs, (char *)b->h_stage + ob, cb, cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
+            cudaEventRecord(b->staged, b->stream) != cudaSuccess)
             return bfail(b, QK_ECUDA, "batch: upload failed");
     }
     static qk::SmemLimit limit;
