@@ -819,9 +819,10 @@ __device__ __forceinline__ void tile_body(const Prog &pr, float2 *__restrict__ p
 // live across iterations and push the kernel into spills)
 // CTAS: resident CTAs per SM the registers are cut to.  Up to two tiles per SM a third
 // CTA has nothing to run, and the instance with 128 registers has no spills (a batch of
-// five circuits of 18 to 20 qubits: 3.33 -> 3.10 ms on the device; 14 to 21 qubits 0-3 % of
-// a whole call; above, three CTAs: 95.5 -> 75.3 ms of the 30-qubit step's passes).
-constexpr uint64_t kFewTiles = 2 * 152;
+// five circuits of 18 to 20 qubits 3.33 -> 3.10 ms on the device, 2.97 with the kernel that
+// carried phases; 14 to 21 qubits 0-3 % of a whole call; above, three CTAs: 95.5 -> 75.3 ms
+// of the 30-qubit step's passes).
+inline bool few_tiles(uint64_t tiles, int sms) { return tiles <= 2 * (uint64_t)sms; }
 template <typename Off, bool GEN, int CTAS>
 __global__ void __launch_bounds__(kTileThreads, CTAS)
     k_tile(float2 *__restrict__ psi, const __grid_constant__ TileParams P, const uint8_t *__restrict__ cbits) {
@@ -865,12 +866,12 @@ cudaError_t launch_tile_g(void *psi, const TileParams &p, const uint8_t *cbits, 
 }
 
 template <typename Off>
-cudaError_t launch_tile_t(void *psi, const TileParams &p, const uint8_t *cbits, cudaStream_t s) {
+cudaError_t launch_tile_t(void *psi, const TileParams &p, const uint8_t *cbits, int sms, cudaStream_t s) {
     if (p.n_tiles == 0 || p.n_tiles > (1ull << 31) - 1) return cudaErrorInvalidValue;
     if (p.nops < 0 || p.nops > kTileMaxOps) return cudaErrorInvalidValue;
     const bool gen = needs_general(p.ops, (size_t)p.nops);
     if constexpr (sizeof(Off) == 4)
-        if (p.n_tiles <= kFewTiles)
+        if (few_tiles(p.n_tiles, sms))
             return gen ? launch_tile_g<Off, true, 2>(psi, p, cbits, s) : launch_tile_g<Off, false, 2>(psi, p, cbits, s);
     return gen ? launch_tile_g<Off, true, 3>(psi, p, cbits, s) : launch_tile_g<Off, false, 3>(psi, p, cbits, s);
 }
@@ -889,9 +890,9 @@ cudaError_t launch_tile_batch_g(const TileProg *progs, const uint32_t *first, in
 
 cudaError_t launch_tile_batch(const TileProg *progs, const uint32_t *first, int n_progs, uint32_t n_ctas,
                               const TileOp *ops, const LayerGate *lg, const BitTerm *bt, bool general,
-                              cudaStream_t s) {
+                              int sms, cudaStream_t s) {
     if (n_progs <= 0 || n_ctas == 0) return cudaSuccess;
-    if (n_ctas <= kFewTiles)
+    if (few_tiles(n_ctas, sms))
         return general ? launch_tile_batch_g<true, 2>(progs, first, n_progs, n_ctas, ops, lg, bt, s)
                        : launch_tile_batch_g<false, 2>(progs, first, n_progs, n_ctas, ops, lg, bt, s);
     return general ? launch_tile_batch_g<true, 3>(progs, first, n_progs, n_ctas, ops, lg, bt, s)
@@ -900,10 +901,10 @@ cudaError_t launch_tile_batch(const TileProg *progs, const uint32_t *first, int 
 
 bool tile_ops_need_general(const TileOp *ops, size_t n) { return needs_general(ops, n); }
 
-cudaError_t launch_tile(void *psi, const TileParams &p, const uint8_t *cbits, cudaStream_t s) {
+cudaError_t launch_tile(void *psi, const TileParams &p, const uint8_t *cbits, int sms, cudaStream_t s) {
     // 32-bit element offsets inside a tile reach 2^32 amplitudes
-    if (p.n <= 32) return launch_tile_t<uint32_t>(psi, p, cbits, s);
-    return launch_tile_t<uint64_t>(psi, p, cbits, s);
+    if (p.n <= 32) return launch_tile_t<uint32_t>(psi, p, cbits, sms, s);
+    return launch_tile_t<uint64_t>(psi, p, cbits, sms, s);
 }
 
 }  // namespace qk

@@ -564,7 +564,6 @@ void *ctx_state(qk_ctx *c) { return c->d_state; }
 int ctx_n(qk_ctx *c) { return c->n; }
 int ctx_prec(qk_ctx *c) { return (int)c->prec; }
 int ctx_sms(qk_ctx *c) { return c->sms; }
-int ctx_tile_qubits(qk_ctx *c) { return c->opt.tile_qubits; }
 cudaStream_t ctx_stream(qk_ctx *c) { return c->stream; }
 const uint8_t *ctx_cbits(qk_ctx *c) { return c->d_cbits; }
 qk_status ctx_run_plain(qk_ctx *c, const FusedOp &op) { return run_op_plain(c, op); }

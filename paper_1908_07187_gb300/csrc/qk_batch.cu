@@ -666,7 +666,7 @@ qk_status launch_large(qk_batch *b, const LargeRun &run) {
             general = qk::tile_ops_need_general(ops.data() + h.op0, (size_t)h.nops);
         }
         const cudaError_t e = qk::launch_tile_batch(b->d_lprogs + launch[k].first, b->d_lfirst + launch[k].second, np,
-                                                    ctas[k], b->d_lops, b->d_llg, b->d_lbt, general, b->stream);
+                                                    ctas[k], b->d_lops, b->d_llg, b->d_lbt, general, b->sms, b->stream);
         if (e != cudaSuccess) return bfail(b, QK_ECUDA, "batch: tile launch failed: %s", cudaGetErrorString(e));
         ++b->large_launches;
     }

@@ -320,7 +320,7 @@ inline size_t meas_partials(int sms) { return (size_t)meas_max_blocks(sms) << 6;
 
 // One fused Kitaev stage (kernels_kitaev.cu): control qubit at physical bit
 // cpos, register of w qubits at rpos[] (rpos[0] = MSB), permutation f given by
-// its inverse (mul-mod: cinv, N, mu; table: finv), phase from cbits.
+// its inverse (mul-mod: mul; table: finv), phase from cbits.
 struct KitaevArgs {
     int cpos;
     int w;
@@ -466,7 +466,6 @@ struct TileHead {
     // len) land on physical bits [plo, plo + len)
     int nruns;
     uint8_t run_tlo[kTileMaxRuns], run_len[kTileMaxRuns], run_plo[kTileMaxRuns];
-    int store_arr;
     int n_conds;
     Cond conds[kTileMaxConds];
     int nops;
@@ -506,7 +505,7 @@ struct TileProg : TileHead {
 };
 static_assert(sizeof(TileParams) <= 32764, "tile program must fit in the kernel parameter space");
 
-cudaError_t launch_tile(void *psi, const TileParams &p, const uint8_t *cbits, cudaStream_t s);
+cudaError_t launch_tile(void *psi, const TileParams &p, const uint8_t *cbits, int sms, cudaStream_t s);
 // Pass k of many circuits in one launch: CTA b runs tile (b - first[c]) of
 // program c, where first[] (n_progs + 1 entries, ascending, first[0] = 0) splits
 // the grid; programs are in n-qubit order so that the 32-bit offset kernel serves
@@ -515,7 +514,7 @@ cudaError_t launch_tile(void *psi, const TileParams &p, const uint8_t *cbits, cu
 // them a leaner instance of the kernel runs.
 cudaError_t launch_tile_batch(const TileProg *progs, const uint32_t *first, int n_progs, uint32_t n_ctas,
                               const TileOp *ops, const LayerGate *lg, const BitTerm *bt, bool general,
-                              cudaStream_t s);
+                              int sms, cudaStream_t s);
 // whether a pass program holds ops of the kinds TOP_U2, TOP_PHASE or TOP_PHQ
 bool tile_ops_need_general(const TileOp *ops, size_t n);
 

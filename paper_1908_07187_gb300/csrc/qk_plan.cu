@@ -1419,7 +1419,6 @@ qk_status plan_passes(TilePlanner *planner, int n, const std::vector<FusedOp> &o
                 if ((P.fin_fixed_mask >> b) & 1) need = need || general(P.fin_fixed[b]);
             P.need_tab = need ? 1 : 0;
         }
-        P.store_arr = B.arr;
         next.clear();
         B.hand_on(next, rewritten);
         next.insert(next.end(), left.begin(), left.end());
@@ -1809,7 +1808,7 @@ qk_status run_fused(TilePlanner *planner, qk_ctx *c, const std::vector<FusedOp> 
             cudaEventRecord(ev0, ctx_stream(c));
         }
         ctx_launch_begin(c, 0, 2.0 * 8.0 * (double)(1ull << n), &tok);
-        cudaError_t e = launch_tile(ctx_state(c), P, ctx_cbits(c), ctx_stream(c));
+        cudaError_t e = launch_tile(ctx_state(c), P, ctx_cbits(c), ctx_sms(c), ctx_stream(c));
         ctx_launch_end(tok);
         if (e != cudaSuccess) return ctx_fail(c, QK_ECUDA, cudaGetErrorString(e));
         if (planner->log) {

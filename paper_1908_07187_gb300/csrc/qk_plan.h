@@ -61,7 +61,6 @@ void *ctx_state(qk_ctx *c);
 int ctx_n(qk_ctx *c);
 int ctx_prec(qk_ctx *c);
 int ctx_sms(qk_ctx *c);
-int ctx_tile_qubits(qk_ctx *c);
 cudaStream_t ctx_stream(qk_ctx *c);
 const uint8_t *ctx_cbits(qk_ctx *c);
 qk_status ctx_run_plain(qk_ctx *c, const FusedOp &op);
