@@ -23,6 +23,7 @@
 #include <complex>
 #include <cstring>
 #include <deque>
+#include <tuple>
 #include <vector>
 
 #include "qk_plan.h"
@@ -42,6 +43,17 @@ TilePlanner *make_planner() {
 void free_planner(TilePlanner *p) { delete p; }
 
 namespace {
+
+// Storage that a thread keeps from plan to plan is given back after a queue far beyond the
+// default length of 4096 ops.
+template <typename... V>
+struct GiveBack {
+    std::tuple<V &...> kept;
+    explicit GiveBack(V &...v) : kept(v...) {}
+    ~GiveBack() {
+        std::apply([](V &...v) { ((v.capacity() > (1u << 16) ? V().swap(v) : void()), ...); }, kept);
+    }
+};
 
 struct POp {
     const FusedOp *op;
@@ -1213,6 +1225,7 @@ qk_status plan_passes(TilePlanner *planner, int n, const std::vector<FusedOp> &o
     // kernel-parameter budget (ops and grouped phase entries)
     int max_u2 = 100, max_ph = 300;
     static thread_local std::vector<POp> left, taken, next;
+    const GiveBack trim(rewritten_ops, left, taken, next);
     std::deque<FusedOp> rewritten;   // pair terms handed on without their single-qubit parts
     // per physical qubit the pending factor of its |1>, and the one of all amplitudes,
     // handed from pass to pass in FP64; only the plan's last pass applies them
@@ -1450,6 +1463,7 @@ qk_status smem_passes(TilePlanner *planner, int n, int prec, const std::vector<F
                       const char **err) {
     *err = "";
     static thread_local std::vector<POp> rem, left, taken, next;
+    const GiveBack trim(rem, left, taken, next);
     rem.clear();
     for (const auto &op : ops) rem.push_back(classify(op));
     const int m = smem_tile_qubits(n, prec);
@@ -1702,6 +1716,7 @@ bool dense_apart(int n, int prec, const std::vector<const DenseItem *> &taken) {
 qk_status plan_dense(int n, int prec, const std::vector<DenseItem> &ops, const DenseSink &sink) {
     static thread_local std::vector<const DenseItem *> rem, left, taken, one(1);
     static thread_local std::vector<Cond> conds;
+    const GiveBack trim(rem, left, taken);
     rem.clear();
     for (const DenseItem &it : ops) rem.push_back(&it);
     while (!rem.empty()) {
