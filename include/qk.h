@@ -67,7 +67,8 @@ typedef enum { QK_C64 = 0, QK_C128 = 1 } qk_precision;
  * unfused baseline).  FUSED: gates are queued; at a flush point a planner groups
  * runs of gates (1-target gates, and dense gates of one size) into tile passes, so
  * several gates cost one HBM read+write of the state, in both precisions and at any
- * size. */
+ * size (a queue that concerns a small part of the state takes single launches where
+ * that is cheaper). */
 typedef enum { QK_EXEC_PLAIN = 0, QK_EXEC_FUSED = 1 } qk_exec_mode;
 
 typedef struct {
@@ -135,7 +136,8 @@ qk_status qk_add_cbits(qk_ctx *ctx, int n, int *first_cbit_out);
  * relabelling pass first moves them there (the qubit map records the move, no
  * extra memory beyond the context's gather buffer).  Other dense gates run on
  * CUDA cores in the working precision.  qk_sync reports QK_ETIMEOUT if a
- * tensor-core pass hit its bounded wait. */
+ * tensor-core pass hit its bounded wait.  Matrices that are not unitary to rounding
+ * are applied as they are, singular ones too. */
 qk_status qk_define_gate_matrix(qk_ctx *ctx, int k, const double *u, double unitarity_tol, int *gate_id);
 
 /* Define a gate "as a function" (Q-Kit section, command 4; QuModExpUaj of
@@ -199,8 +201,10 @@ qk_status qk_apply_rphase_cbits(qk_ctx *ctx, int target, const int *cbits, int n
  * `control` with `uniform` into dest_cbit; X(control) if the outcome is 1.
  * Precondition: `control` is |0> (every amplitude with the control bit set is
  * zero), which holds at the start and after every stage.  The result equals the
- * six separate calls; the stage costs two passes over the control = 0 half (the
- * reduction's last block takes the decision).  Stream-ordered, no host round trip.
+ * six separate calls.  One cooperative launch where the control = 0 half fits the
+ * registers of the resident blocks (up to 21 qubits in complex64, 20 in complex128; its
+ * grid barrier's wait is bounded: qk_sync reports QK_ETIMEOUT if it gave up), two passes over that half above
+ * (the reduction's last block takes the decision).  Stream-ordered, no host round trip.
  * Errors: QK_EINVAL (bad ids, lists or uniform), QK_ENOMEM, QK_ECUDA. */
 qk_status qk_apply_kitaev_stage(qk_ctx *ctx, int control, int perm_gate_id, const int *targets, int nt,
                                 const int *phase_cbits, int ncb, double uniform, int dest_cbit);
