@@ -696,7 +696,7 @@ bool in_window(const qk_batch *b, int circuit, bool state) {
 // circuits along, four times as many as the window before, up to kWindow bytes: 256
 // circuits of 6 MB cost six waits (2.33 ms in all, 2.25 with everything in one copy), and
 // reading two circuits costs the bytes of three more.  Any other read copies its own
-// circuit only.  states: whether this program reads states at all.
+// circuit only.  states: whether the run stored states and this program reads them.
 qk_status read_window(qk_batch *b, int circuit, uint8_t *cbits, int ncb, void *state, size_t bytes, bool states) {
     const int gap = circuit - b->read_next;
     b->ahead = b->ahead > 0 && gap >= 0 && gap <= b->ahead ? std::min(4 * b->ahead, 1 << 20) : 1;
@@ -1142,7 +1142,8 @@ qk_status qk_batch_read(qk_batch *b, int circuit, uint8_t *cbits, int ncb, void 
     const bool small = state && !large;
     if (small || ncb > 0) {
         if (!in_window(b, circuit, small)) {
-            const qk_status st = read_window(b, circuit, cbits, ncb, small ? state : nullptr, bytes, state != nullptr);
+            const qk_status st = read_window(b, circuit, cbits, ncb, small ? state : nullptr, bytes,
+                                             state && b->store_state);
             if (st != QK_OK) return st;
         }
         if (in_window(b, circuit, small)) {

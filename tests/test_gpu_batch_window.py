@@ -76,3 +76,25 @@ def test_two_reads_do_not_copy_the_batch():
         assert b.read(i)[1][8] == 1
     assert resident() - before < 16 << 20
     b.close()
+
+
+def test_runs_that_store_no_small_states():
+    """Large circuits' states are always kept; reading them in order, with cbits, takes no
+    states of small circuits along from a run that stored none."""
+    from paper_1908_07187_gb300 import qk
+
+    b = qk.Batch()
+    for i in range(60):
+        n = 14 if i % 2 else 13
+        b.add_ops(n, 2, [workloads.Op("x", (i % n,))])
+    b.run(store_states=False)
+    for i in range(60):
+        bits, psi = b.read(i, state=i % 2 == 1)
+        assert list(bits) == [0, 0]
+        if i % 2:
+            assert abs(psi[1 << (i % 14)]) == 1 and np.count_nonzero(psi) == 1
+        else:
+            with pytest.raises(qk.QKError) as e:
+                b.read(i)
+            assert e.value.status == qk.QK_EINVAL
+    b.close()
