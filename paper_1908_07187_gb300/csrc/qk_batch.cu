@@ -1025,6 +1025,11 @@ qk_status qk_batch_run(qk_batch *b, int store_states) {
     if ((s = grow(b, &b->d_circs, &b->cap_circs, std::max<size_t>(1, b->circs.size()))) != QK_OK) return s;
     if (b->store_state && (s = grow(b, &b->d_states, &b->cap_states, b->total_amps)) != QK_OK) return s;
     if ((s = grow(b, &b->d_cbits, &b->cap_cbits, std::max<size_t>(1, b->total_cb))) != QK_OK) return s;
+    // no kernel writes the cbits of a large circuit: it measures nothing
+    for (const auto &L : b->large)
+        if (b->circs[L.circ].ncb > 0 &&
+            cudaMemsetAsync(b->d_cbits + b->circs[L.circ].cb_off, 0, b->circs[L.circ].ncb, b->stream) != cudaSuccess)
+            return bfail(b, QK_ECUDA, "batch: cbit reset failed");
     // circuits of at most 13 qubits, sorted by size, largest first: one launch per qubit
     // count (and per need of the second state buffer, which only mul-mod gathers use),
     // each sized to its shared memory (small circuits then share an SM)

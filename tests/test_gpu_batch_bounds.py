@@ -70,3 +70,21 @@ def test_circuits_added_after_a_run(before):
         b.read(0)
     assert e.value.status == qk.QK_ESTATE
     b.close()
+
+
+def test_large_circuits_have_cbits_of_0():
+    from paper_1908_07187_gb300 import qk
+
+    b = qk.Batch()
+    for _ in range(8):                               # cbits of 1 in the buffer
+        b.add_ops(4, 4, [workloads.Op("x", (q,)) for q in range(4)] + [
+            workloads.Op("measure", (0, 1, 2, 3), uniforms=(0.5,) * 4, cbits=(0, 1, 2, 3))])
+    b.run()
+    assert list(b.read_all_cbits()) == [1] * 32
+    b.clear()
+    for i in range(8):
+        b.add_ops(14 if i % 2 else 3, 4, [workloads.Op("x", (0,))])
+    b.run()
+    assert list(b.read_all_cbits()) == [0] * 32
+    assert all(list(b.read(i)[0]) == [0] * 4 for i in range(8))
+    b.close()
